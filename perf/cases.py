@@ -231,6 +231,56 @@ def run(s):
     return out
 
 
+def _rotate(q, lens, case):
+    """Pseudo queries [B, Hq, N, d] at positions L_b + i, rotate-half pairs, in 64 bits."""
+    c = torch.arange(D // 2, dtype=torch.float64, device="cuda")
+    theta = case["rope_base"] ** (-2.0 * c / D) if case["rope"] == "plain" else None
+    if theta is None:                                    # the Llama-3.1 frequencies: base 5e5, factor 8, 1 and 4, 8192
+        theta = 5.0e5 ** (-2.0 * c / D)
+        turns = 8192 * theta / (2.0 * math.pi)
+        mix = (turns - 1.0) / 3.0
+        theta = torch.where(turns > 4.0, theta, torch.where(turns < 1.0, theta / 8.0, (1.0 - mix) * theta / 8.0 + mix * theta))
+    start = torch.tensor(lens, dtype=torch.float64, device="cuda")
+    at = start[:, None] + torch.arange(q.shape[2], dtype=torch.float64, device="cuda")
+    angle = (at[:, :, None] * theta)[:, None]
+    cos, sin, (x, y) = angle.cos(), angle.sin(), q.double().split(D // 2, dim=3)
+    return torch.cat([x * cos - y * sin, y * cos + x * sin], dim=3)
+
+
+def exact(case, seed):
+    """The same pass in 64 bits: softmax over the prompt and the synthetic keys that a pseudo query sees,
+    summed per KV head; the best rows in ascending order."""
+    s = prepare(case, seed)
+    lens, keep, cu, H, N = s["lens"], s["keep"], s["cu_rows"], case["kv_heads"], case["window"]
+    one = case["entry"] in ("evict", "steps")
+    out = {"k": torch.zeros_like(s["k_out"]), "v": torch.zeros_like(s["v_out"]), "idx": torch.zeros_like(s["idx"])}
+    if one:
+        out["scores"] = torch.zeros((H, sum(lens)), dtype=torch.float64, device="cuda")
+    for l, (q, k, v) in enumerate([(s["q"], s["k"], s["v"])] if one else zip(s["q"], s["k"], s["v"])):
+        q, k, v = q.cuda(), k.cuda(), v.cuda()
+        rot = _rotate(q, lens, case)
+        if case["entry"] == "steps":
+            rot = rot.to(q.dtype).double()               # the step between hands them on in the cache's type
+        at, at_p = 0, 0
+        for L, K, lo, qb in zip(lens, keep, cu, rot):
+            for h in range(H):
+                logits = qb.view(H, -1, D)[h] @ k[h, lo:lo + L + N].double().T / math.sqrt(D)
+                unseen = torch.ones((N, N), dtype=torch.bool, device="cuda").triu(1)
+                logits.view(-1, N, L + N)[:, :, L:].masked_fill_(unseen, -math.inf)
+                score = logits.softmax(1)[:, :L].sum(0)
+                chosen = score
+                if case["pool"]:
+                    chosen = torch.nn.functional.max_pool1d(score[None], case["pool"], 1, case["pool"] // 2)[0]
+                idx = chosen.sort(descending=True, stable=True).indices[:K].sort().values
+                out["idx"][l, h, at:at + K] = idx
+                out["k"][l, h, at:at + K] = k[h, lo + idx]
+                out["v"][l, h, at:at + K] = v[h, lo + idx]
+                if one:
+                    out["scores"][h, at_p:at_p + L] = score
+            at, at_p = at + K, at_p + L
+    return out
+
+
 def work(case):
     """K once, the kept rows of K and V read and written, queries, indices, scores; one contraction of the
     pseudo queries with every key (the exponentials are not counted)."""
