@@ -201,13 +201,16 @@ dapq_status check_view(dapq_ctx* ctx, const dapq_cache_view* cv, bool need_v, bo
   return DAPQ_OK;
 }
 
-// The tensor-core scorer takes bf16 caches whose query block is at least half an MMA tile high;
-// everything else (fp32 storage, tiny windows, views TMA cannot describe, syn_mass requests)
-// goes to the CUDA-core scorer.
+// The fp16 tensor-core scorer takes bf16 caches whose query block is at least half an MMA tile high; fp32 storage
+// and smaller query blocks go to the one that splits its operands (run_score); views TMA cannot describe and
+// syn_mass requests to the CUDA-core scorer.
 bool wants_umma(const dapq_ctx* ctx) {
   return ctx->shape.dtype == DAPQ_BF16 && !(ctx->shape.flags & DAPQ_FLAG_CUDA_CORE_SCORER) &&
          ctx->dims.group * ctx->dims.n_pseudo >= 64;
 }
+
+// ... and the one with split operands what the other does not take, unless the context asks for the CUDA cores.
+bool wants_split(const dapq_ctx* ctx) { return !(ctx->shape.flags & DAPQ_FLAG_CUDA_CORE_SCORER) && !wants_umma(ctx); }
 
 dapq_status run_score_umma(dapq_ctx* ctx, const UmmaPlan& plan, const SeqTable& t, const float* lse_in,
                            float* scores, int64_t score_stride, float* lse_out, cudaStream_t s) {
@@ -229,11 +232,19 @@ dapq_status run_score_qg(dapq_ctx* ctx, const QgPlan& plan, const SeqTable& t, c
 // the contexts that ask for that part in either sweep.
 bool wants_lo(const dapq_ctx* ctx) { return (ctx->shape.flags & (DAPQ_FLAG_Q_LO_SWEEP1 | DAPQ_FLAG_Q_LO_SWEEP2)) != 0; }
 
+// fp32 arithmetic on unrounded queries: on the tensor cores with split operands, or on the CUDA cores where the
+// context asks for them, the attention mass of the synthetic keys is wanted, or TMA cannot describe the view.
 dapq_status run_score(dapq_ctx* ctx, int q_dtype, const void* q_rot, const CacheDev& cd, const SeqTable& t,
                       const float* lse_in, float* scores, int64_t score_stride, float* lse_out,
-                      float* syn_mass, cudaStream_t s) {
-  cudaError_t e = launch_score_fma(ctx->shape.dtype, q_dtype, q_rot, cd, t, ctx->dims, lse_in, ctx->part, ctx->max_chunks, ctx->n_sm,
-                                   ctx->lse2, scores, score_stride, lse_out, syn_mass, s, &ctx->log);
+                      float* syn_mass, bool after_rope, cudaStream_t s) {
+  cudaError_t e;
+  SplitPlan plan;
+  if (wants_split(ctx) && !syn_mass && split_plan(ctx->shape.dtype, cd, t, ctx->dims, ctx->n_sm, &plan))
+    e = launch_score_split(plan, q_dtype, q_rot, t, ctx->dims, lse_in, ctx->part, ctx->slots, scores, score_stride, lse_out,
+                           ctx->status, ctx->wait_limit, after_rope, s, &ctx->log);
+  else
+    e = launch_score_fma(ctx->shape.dtype, q_dtype, q_rot, cd, t, ctx->dims, lse_in, ctx->part, ctx->max_chunks, ctx->n_sm,
+                         ctx->lse2, scores, score_stride, lse_out, syn_mass, s, &ctx->log);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "score kernels");
   return DAPQ_OK;
 }
@@ -326,8 +337,8 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
   ok = ok && cudaMalloc(&ctx->idx, (size_t)sh->n_kv_heads * rows * sizeof(int32_t)) == cudaSuccess;
   if (sh->pool_mode != DAPQ_POOL_NONE)
     ok = ok && cudaMalloc(&ctx->pooled, (size_t)sh->n_kv_heads * rows * sizeof(float)) == cudaSuccess;
-  if (sh->dtype == DAPQ_BF16 && qg_groups(ctx->dims) > 1)
-    ok = ok && cudaMalloc(&ctx->slots, (size_t)qg_groups(ctx->dims) * sh->n_kv_heads * rows * sizeof(float)) == cudaSuccess;
+  const int n_slots = wants_umma(ctx) ? qg_groups(ctx->dims) : (wants_split(ctx) ? split_groups(ctx->dims) : 1);
+  if (n_slots > 1) ok = ok && cudaMalloc(&ctx->slots, (size_t)n_slots * sh->n_kv_heads * rows * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMemcpy(ctx->inv_freq, freq, sizeof(freq), cudaMemcpyHostToDevice) == cudaSuccess;
   ok = ok && cudaMemset(ctx->status, 0, sizeof(int)) == cudaSuccess;
   if (!ok) { cudaGetLastError(); return bail(DAPQ_ERR_CUDA, "workspace allocation failed"); }
@@ -473,7 +484,8 @@ dapq_status dapq_score(dapq_ctx* ctx, const void* q_rot, const dapq_cache_view* 
         return run_score_qg(ctx, plan, t, lse_in, scores, t.cu_prompt[t.batch], lse_out, false, (cudaStream_t)stream);
     }
   }
-  return run_score(ctx, ctx->shape.dtype, q_rot, cd, t, lse_in, scores, t.cu_prompt[t.batch], lse_out, syn_mass, (cudaStream_t)stream);
+  return run_score(ctx, ctx->shape.dtype, q_rot, cd, t, lse_in, scores, t.cu_prompt[t.batch], lse_out, syn_mass, false,
+                   (cudaStream_t)stream);
 }
 
 dapq_status dapq_topk_select(dapq_ctx* ctx, const float* scores, const int32_t* cu_prompt_host,
@@ -569,11 +581,11 @@ dapq_status evict_impl(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* 
     if (e != cudaSuccess) return cuda_fail(ctx, e, "rope kernel");
     st = run_score_umma(ctx, plan, t, nullptr, scores, score_stride, nullptr, s);
   } else {
-    // CUDA-core scorer: reads the rotated queries unrounded (fp32)
+    // the rotated queries unrounded (fp32)
     e = launch_rope(ctx->shape.dtype, kRopeOutF32, 0, q_pre, ctx->q_rot, ctx->inv_freq, t, ctx->dims, after_own_compaction, s,
                     &ctx->log);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "rope kernel");
-    st = run_score(ctx, DAPQ_F32, ctx->q_rot, cd, t, nullptr, scores, score_stride, nullptr, nullptr, s);
+    st = run_score(ctx, DAPQ_F32, ctx->q_rot, cd, t, nullptr, scores, score_stride, nullptr, nullptr, true, s);
   }
   if (st != DAPQ_OK) return st;
   st = run_select(ctx, scores, score_stride, idx, idx_stride, t, s);

@@ -170,6 +170,9 @@ cudaError_t launch_score_umma(const UmmaPlan& plan, const SeqTable& t, const Dim
 // the sequences' keys into chunks of whole tiles with ctas_per_chunk CTAs working on every chunk.
 bool encode_tile_map(CUtensorMap* map, const void* base, bool f16, int rank, const uint64_t* dims,
                      const uint64_t* strides_bytes, int box_rows);
+// fp32 tensor [H, rows, 128], boxes of box_cols (up to 32) channels x box_rows rows, 128-byte swizzle.
+bool encode_rows_map_f32(CUtensorMap* map, const void* base, const uint64_t* dims, const uint64_t* strides_bytes, int box_cols,
+                         int box_rows);
 bool plan_chunks(const SeqTable& t, int extra_keys, int tile_keys, int ctas_per_chunk, int n_sm, ChunkTable* ct,
                  double cta_cost = 3.0);
 
@@ -191,6 +194,25 @@ bool qg_plan(const void* q, int q_is_f16, const CacheDev& cv, const SeqTable& t,
 cudaError_t launch_score_qg(const QgPlan& plan, const SeqTable& t, const Dims& dm, const float* lse_in, float2* part,
                             float* slots, float* scores, int64_t score_stride, float* lse_out, const float* ref, int* status,
                             long long wait_limit, bool after_own_kernel, cudaStream_t s, LaunchLog* log);
+
+// Sum of n_slots score arrays of `count` values that lie one behind the other, in slot order.
+cudaError_t launch_slots_sum(const float* slots, int n_slots, float* scores, int64_t count, cudaStream_t s, LaunchLog* log);
+
+// Tensor-core scorer with unrounded operands (score_split.cu).  split_plan returns false when the view cannot be
+// described to TMA; split_groups: score slots that sweep 2 needs (one per 128 query rows of a KV head).
+struct SplitPlan {
+  CUtensorMap tm_k;
+  ChunkTable ct1, ct2;
+  int32_t key_parts;                      // 3: fp32 keys, 1: bf16 keys
+  int32_t R, n_qgroups;                   // query rows per sub-group (16 .. 64), sub-groups of a KV head
+  int32_t n_sub2, n_qgroups2;             // sub-groups per CTA in sweep 2, CTAs per chunk there
+  int32_t n_ring1, n_ring2, n_stage1, n_stage2, smem1, smem2;
+};
+int split_groups(const Dims& dm);
+bool split_plan(int dtype, const CacheDev& cv, const SeqTable& t, const Dims& dm, int n_sm, SplitPlan* plan);
+cudaError_t launch_score_split(const SplitPlan& plan, int q_dtype, const void* q, const SeqTable& t, const Dims& dm,
+                               const float* lse_in, float2* part, float* slots, float* scores, int64_t score_stride, float* lse_out,
+                               int* status, long long wait_limit, bool after_own_kernel, cudaStream_t s, LaunchLog* log);
 
 cudaError_t launch_topk(const float* scores, int64_t score_stride, int32_t* idx, int64_t idx_stride,
                         const SeqTable& t, int n_kv_heads, cudaStream_t s, LaunchLog* log);

@@ -100,6 +100,16 @@ bool encode_tile_map(CUtensorMap* map, const void* base, bool f16, int rank, con
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool encode_rows_map_f32(CUtensorMap* map, const void* base, const uint64_t* dims, const uint64_t* strides_bytes, int box_cols,
+                         int box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t gdim[3] = {dims[0], dims[1], dims[2]}, gstride[2] = {strides_bytes[0], strides_bytes[1]};
+  const cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1}, estr[3] = {1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Cut every sequence's keys (prompt, plus the synthetic rows if asked) into chunks of whole tiles;
 // ctas_per_chunk CTAs work on every chunk (KV heads x query groups).  cta_cost: what a CTA spends besides
 // its tiles (set-up, first loads, drain), in units of one tile's work.
@@ -175,6 +185,19 @@ bool qg_plan(const void* q, int q_is_f16, const CacheDev& cv, const SeqTable& t,
          encode_tile_map(&plan->tm_q, q, q_is_f16 != 0, 2, qd, qs, 128);
 }
 
+cudaError_t launch_slots_sum(const float* slots, int n_slots, float* scores, int64_t count, cudaStream_t s, LaunchLog* log) {
+  cudaError_t e;
+  log->begin(kKindSlotSum, s);
+  if (count % 4 == 0 && ((uintptr_t)slots & 15u) == 0 && ((uintptr_t)scores & 15u) == 0)
+    e = launch_pdl(score_slots_sum_kernel, dim3((unsigned)((count / 4 + 255) / 256)), dim3(256), 0, s, 1,
+                   (const float4*)slots, n_slots, count / 4, (float4*)scores, count / 4);
+  else
+    e = launch_pdl(score_slots_sum1_kernel, dim3((unsigned)((count + 255) / 256)), dim3(256), 0, s, 1, slots, n_slots, count, scores,
+                   count);
+  log->end(s);
+  return e;
+}
+
 cudaError_t launch_score_qg(const QgPlan& plan, const SeqTable& t, const Dims& dm, const float* lse_in, float2* part,
                             float* slots, float* scores, int64_t score_stride, float* lse_out, const float* ref, int* status,
                             long long wait_limit, bool after_own_kernel, cudaStream_t s, LaunchLog* log) {
@@ -229,18 +252,7 @@ cudaError_t launch_score_qg(const QgPlan& plan, const SeqTable& t, const Dims& d
     e = plan.q_is_f16 ? run(rowstat_kernel<true>, colsum_kernel<true, false>, kSmemBytes)
                       : run(rowstat_kernel<false>, colsum_kernel<false, false>, kSmemBytes);
   if (e != cudaSuccess) return e;
-  if (plan.n_qgroups2 > 1) {
-    const int64_t count = (int64_t)dm.n_kv_heads * score_stride;
-    log->begin(kKindSlotSum, s);
-    if (count % 4 == 0 && a.slot_stride % 4 == 0 && ((uintptr_t)slots & 15u) == 0 && ((uintptr_t)scores & 15u) == 0)
-      e = launch_pdl(score_slots_sum_kernel, dim3((unsigned)((count / 4 + 255) / 256)), dim3(256), 0, s, 1,
-                     (const float4*)slots, plan.n_qgroups2, a.slot_stride / 4, (float4*)scores, count / 4);
-    else
-      e = launch_pdl(score_slots_sum1_kernel, dim3((unsigned)((count + 255) / 256)), dim3(256), 0, s, 1, (const float*)slots,
-                     plan.n_qgroups2, a.slot_stride, scores, count);
-    log->end(s);
-    if (e != cudaSuccess) return e;
-  }
+  if (plan.n_qgroups2 > 1 && (e = launch_slots_sum(slots, plan.n_qgroups2, scores, a.slot_stride, s, log)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

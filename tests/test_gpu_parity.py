@@ -840,3 +840,66 @@ def test_logits_far_above_and_below_the_first_key(dq, where):
         ctx = _ctx(dq, w, flags=flags)
         _check_evict(w, data, _gpu_evict(dq, w, data, ctx), ref)
         dq.dapq_destroy(ctx)
+
+
+# ------------------------------------------- the scorer with split operands (fp32 caches, small query blocks)
+# Rows of a KV head at the edges of its sub-groups (16 / 32 / 48 / 64 rows, two per CTA in sweep 2, several score
+# slots beyond 128 rows), prompts at the edges of its 128-key tiles, synthetic rows that begin a tile of their own,
+# one and several chunks per sequence.
+SPLIT_CASES = [
+    ("f32", 1, 1, 1, (1, 127, 128, 129)), ("f32", 1, 1, 17, (111, 112, 2049)), ("f32", 3, 1, 16, (384,)),
+    ("f32", 2, 1, 32, (640, 300)), ("f32", 5, 1, 13, (257,)), ("f32", 4, 2, 64, (500, 3)), ("f32", 3, 1, 64, (1000,)),
+    ("f32", 7, 1, 64, (390, 129)), ("f32", 16, 2, 128, (260,)), ("f32", 8, 8, 31, (9000,)),
+    ("bf16", 1, 1, 1, (1, 127, 128, 129)), ("bf16", 2, 2, 63, (640, 1)), ("bf16", 3, 1, 11, (255, 256, 257)),
+    ("bf16", 16, 16, 32, (5000,)), ("bf16", 4, 4, 48, (2100, 800)), ("bf16", 1, 1, 32, (40000,)),
+]
+
+
+@pytest.mark.parametrize("dtype,hq,hkv,n,lens", SPLIT_CASES)
+def test_split_operand_scorer(dq, dtype, hq, hkv, n, lens):
+    """dapq_evict's scores against the oracle, and against the same call on the CUDA cores.  Bound: a logit is a sum
+    of exact bf16 products with fp32 roundings of at most 2^-23 of its largest partial sum in some 16 steps, and
+    |q||k|/sqrt(d) log2(e) stays below 25 for these N(0, 1) operands: 16 * 2^-23 * 25 = 4.8e-5 in base 2, 3.3e-5
+    relative, plus 2^-21 for two exponentials and the sums (measured: 2e-6)."""
+    w = _small(lens=lens, keep=tuple(max(1, L // 3) for L in lens), dtype=dtype, n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n,
+               n_needles=0, outlier_channels=0)
+    data = gi.draw_layer(w, 0, "cpu")
+    ref = util.oracle_evict(w, data)
+    got = _gpu_evict(dq, w, data)
+    _check_evict(w, data, got, ref)
+    ctx = _ctx(dq, w, flags=dq.DAPQ_FLAG_CUDA_CORE_SCORER)
+    cores = _gpu_evict(dq, w, data, ctx)
+    dq.dapq_destroy(ctx)
+    for b in range(w.batch):
+        cols = slice(w.cu_prompt[b], w.cu_prompt[b + 1])
+        for other in (ref["scores"][b], cores["scores"][:, cols]):
+            assert np.all(np.abs(got["scores"][:, cols] - other) <= 4e-5 * np.abs(other) + 1e-30)
+
+
+@pytest.mark.parametrize("dtype,hq,n", [("f32", 8, 64), ("bf16", 2, 20)])
+@pytest.mark.parametrize("where", [3, 700, 1290])
+def test_split_operand_scorer_far_logits(dq, dtype, hq, n, where):
+    """One key whose logit lies about 150 above the bulk for one row (and tens above or below it for the others),
+    early, in the middle and among the last tiles: the running maximum has to follow it."""
+    w = _small(lens=(1300,), keep=(40,), dtype=dtype, n_q_heads=hq, n_kv_heads=2, n_pseudo=n, n_needles=0, outlier_channels=0)
+    data = gi.draw_layer(w, 0, "cpu")
+    q_rot = util.oracle_q_rot(w, data)[0]
+    for h in range(w.n_kv_heads):
+        u = q_rot[h * w.group, 7]
+        data["k"][h, where] = (150.0 * np.sqrt(128.0) * u / (u.norm() ** 2)).to(w.torch_dtype())
+    _check_evict(w, data, _gpu_evict(dq, w, data), util.oracle_evict(w, data))
+
+
+def test_split_operand_scorer_wait_limit(dq):
+    """A device-side wait that runs out: the call returns, the status says so once, and the context works again."""
+    for dtype, hkv in (("f32", 2), ("bf16", 8)):
+        w = _small(lens=(3000,), keep=(100,), dtype=dtype, n_q_heads=8, n_kv_heads=hkv, n_pseudo=32, n_needles=0, outlier_channels=0)
+        data = gi.draw_layer(w, 0, "cpu")
+        ctx = _ctx(dq, w)
+        dq.dapq_set_wait_limit(ctx, 1)
+        with pytest.raises(dq.DapqError) as e:
+            _gpu_evict(dq, w, data, ctx)
+        assert e.value.status == dq.DAPQ_ERR_TIMEOUT
+        dq.dapq_set_wait_limit(ctx, 0)
+        _check_evict(w, data, _gpu_evict(dq, w, data, ctx), util.oracle_evict(w, data))
+        dq.dapq_destroy(ctx)
