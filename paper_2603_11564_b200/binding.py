@@ -8,8 +8,10 @@ no fallback: a missing library raises ImportError at first use.
 """
 from __future__ import annotations
 
+import array
 import ctypes as C
 import os
+import struct
 from typing import Optional, Sequence
 
 import numpy as np
@@ -65,7 +67,7 @@ def load_library() -> C.CDLL:
     if not os.path.exists(_LIB_PATH):
         raise ImportError(f"{_LIB_PATH} not found: build it with `python -m paper_2603_11564_b200.build`")
     lib = C.CDLL(_LIB_PATH)
-    vp, i32p, f32p = C.c_void_p, C.POINTER(C.c_int32), C.c_void_p
+    vp = i32p = f32p = view = ptrs = C.c_void_p    # (plain addresses: the cheapest conversion that ctypes has)
     lib.dapq_create.argtypes = [C.POINTER(vp), C.POINTER(dapq_shape), C.c_int]
     lib.dapq_create.restype = C.c_int
     lib.dapq_destroy.argtypes = [vp]
@@ -86,24 +88,24 @@ def load_library() -> C.CDLL:
     lib.dapq_profile_read.restype = C.c_int
     lib.dapq_rope_pseudo_q.argtypes = [vp, vp, i32p, C.c_int32, vp, vp]
     lib.dapq_rope_pseudo_q.restype = C.c_int
-    lib.dapq_score.argtypes = [vp, vp, C.POINTER(dapq_cache_view), f32p, f32p, f32p, f32p, vp]
+    lib.dapq_score.argtypes = [vp, vp, view, f32p, f32p, f32p, f32p, vp]
     lib.dapq_score.restype = C.c_int
     lib.dapq_topk_select.argtypes = [vp, f32p, i32p, i32p, C.c_int32, vp, vp]
     lib.dapq_topk_select.restype = C.c_int
-    lib.dapq_compact_kv.argtypes = [vp, C.POINTER(dapq_cache_view), vp, i32p, vp, vp, vp]
+    lib.dapq_compact_kv.argtypes = [vp, view, vp, i32p, vp, vp, vp]
     lib.dapq_compact_kv.restype = C.c_int
-    lib.dapq_evict.argtypes = [vp, vp, C.POINTER(dapq_cache_view), i32p, vp, vp, vp, f32p, vp]
+    lib.dapq_evict.argtypes = [vp, vp, view, i32p, vp, vp, vp, f32p, vp]
     lib.dapq_evict.restype = C.c_int
-    lib.dapq_evict_layers.argtypes = [vp, C.c_int32, C.POINTER(vp), C.POINTER(dapq_cache_view), i32p, C.c_int64,
-                                      C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), vp]
+    lib.dapq_evict_layers.argtypes = [vp, C.c_int32, ptrs, view, i32p, C.c_int64,
+                                      ptrs, ptrs, ptrs, vp]
     lib.dapq_evict_layers.restype = C.c_int
     lib.dapq_evict_layers_host.argtypes = lib.dapq_evict_layers.argtypes
     lib.dapq_evict_layers_host.restype = C.c_int
-    lib.dapq_evict_host.argtypes = [vp, vp, C.POINTER(dapq_cache_view), i32p, vp, vp, vp, vp]
+    lib.dapq_evict_host.argtypes = [vp, vp, view, i32p, vp, vp, vp, vp]
     lib.dapq_evict_host.restype = C.c_int
     lib.dapq_recall.argtypes = [vp, vp, vp, i32p, i32p, C.c_int32, f32p, vp]
     lib.dapq_recall.restype = C.c_int
-    lib.dapq_score_static.argtypes = [C.POINTER(dapq_shape), C.c_int, vp, C.POINTER(dapq_cache_view), f32p, vp,
+    lib.dapq_score_static.argtypes = [C.POINTER(dapq_shape), C.c_int, vp, view, f32p, vp,
                                       C.c_char_p, C.c_size_t]
     lib.dapq_score_static.restype = C.c_int
     _lib = lib
@@ -111,8 +113,15 @@ def load_library() -> C.CDLL:
 
 
 def _i32(seq: Sequence[int]):
+    """Host int32 array of `seq` and its address."""
+    if type(seq) in (list, tuple):
+        try:
+            arr = array.array("i", seq)
+            return arr, arr.buffer_info()[0]
+        except (TypeError, OverflowError):
+            pass                                   # what only numpy converts (or refuses)
     arr = np.ascontiguousarray(np.asarray(seq, dtype=np.int32))
-    return arr, arr.ctypes.data_as(C.POINTER(C.c_int32))
+    return arr, arr.ctypes.data
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -121,6 +130,8 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
+        if torch.cuda.is_initialized():            # the current stream without a Stream object (3 us) around it
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
         return torch.cuda.current_stream().cuda_stream or None
     return getattr(stream, "cuda_stream", stream) or None
 
@@ -130,22 +141,23 @@ def _check(ctx, st: int) -> None:
         raise DapqError(st, load_library().dapq_last_error(ctx).decode())
 
 
+_VIEW = struct.Struct("@PPqqqqPPii")               # dapq_cache_view, field by field
+assert _VIEW.size == C.sizeof(dapq_cache_view)
+
+
 def _view(k: torch.Tensor, v: Optional[torch.Tensor], cu_rows, prompt_len):
-    """dapq_cache_view of [H_kv, R, d] tensors (any head / row strides, d contiguous)."""
-    assert k.dim() == 3 and k.stride(2) == 1
+    """dapq_cache_view of [H_kv, R, d] tensors (any head / row strides, d contiguous): its bytes, and the host
+    arrays that they point to (to be kept until the call returns).  Packed at once: filling a ctypes structure and
+    converting its pointers took 6 of a call's 37 us, more than the launches of a short layer leave room for."""
+    ks = k.stride()
+    assert len(ks) == 3 and ks[2] == 1
+    vp, vs = 0, (0, 0, 1)
+    if v is not None:
+        vp, vs = v.data_ptr(), v.stride()
+        assert len(vs) == 3 and vs[2] == 1
     cu, cu_p = _i32(cu_rows)
     pl, pl_p = _i32(prompt_len)
-    view = dapq_cache_view()
-    view.k = k.data_ptr()
-    view.k_head_stride, view.k_row_stride = k.stride(0), k.stride(1)
-    if v is not None:
-        assert v.dim() == 3 and v.stride(2) == 1
-        view.v = v.data_ptr()
-        view.v_head_stride, view.v_row_stride = v.stride(0), v.stride(1)
-    view.cu_rows_host, view.prompt_len_host = cu_p, pl_p
-    view.batch = len(pl)
-    view._keep = (cu, pl, k, v)
-    return view
+    return _VIEW.pack(k.data_ptr(), vp, ks[0], ks[1], vs[0], vs[1], cu_p, pl_p, len(pl), 0), (cu, pl)
 
 
 def dapq_create(n_q_heads: int, n_kv_heads: int, n_pseudo: int, max_batch: int, max_total_rows: int,
@@ -223,8 +235,8 @@ def dapq_rope_pseudo_q(ctx, q_pre: torch.Tensor, pos_start: Sequence[int], q_rot
 def dapq_score(ctx, q_rot: torch.Tensor, k: torch.Tensor, cu_rows, prompt_len, scores: torch.Tensor,
                lse_in: Optional[torch.Tensor] = None, lse_out: Optional[torch.Tensor] = None,
                syn_mass: Optional[torch.Tensor] = None, stream=None) -> None:
-    view = _view(k, None, cu_rows, prompt_len)
-    _check(ctx, load_library().dapq_score(ctx, q_rot.data_ptr(), C.byref(view), _ptr(lse_in), scores.data_ptr(),
+    view, keep_alive = _view(k, None, cu_rows, prompt_len)
+    _check(ctx, load_library().dapq_score(ctx, q_rot.data_ptr(), view, _ptr(lse_in), scores.data_ptr(),
                                           _ptr(lse_out), _ptr(syn_mass), _stream(stream)))
 
 
@@ -237,9 +249,9 @@ def dapq_topk_select(ctx, scores: torch.Tensor, cu_prompt, k_keep, idx_out: torc
 
 def dapq_compact_kv(ctx, k: torch.Tensor, v: torch.Tensor, cu_rows, prompt_len, idx: torch.Tensor, k_keep,
                     k_out: torch.Tensor, v_out: torch.Tensor, stream=None) -> None:
-    view = _view(k, v, cu_rows, prompt_len)
+    view, keep_alive = _view(k, v, cu_rows, prompt_len)
     kk, kk_p = _i32(k_keep)
-    _check(ctx, load_library().dapq_compact_kv(ctx, C.byref(view), idx.data_ptr(), kk_p, k_out.data_ptr(),
+    _check(ctx, load_library().dapq_compact_kv(ctx, view, idx.data_ptr(), kk_p, k_out.data_ptr(),
                                                v_out.data_ptr(), _stream(stream)))
 
 
@@ -254,9 +266,9 @@ def dapq_recall(ctx, idx_gold: torch.Tensor, idx_pred: torch.Tensor, prompt_len,
 def dapq_evict(ctx, q_pre: torch.Tensor, k: torch.Tensor, v: torch.Tensor, cu_rows, prompt_len, k_keep,
                k_out: torch.Tensor, v_out: torch.Tensor, idx_out: Optional[torch.Tensor] = None,
                scores_out: Optional[torch.Tensor] = None, stream=None) -> None:
-    view = _view(k, v, cu_rows, prompt_len)
+    view, keep_alive = _view(k, v, cu_rows, prompt_len)
     kk, kk_p = _i32(k_keep)
-    _check(ctx, load_library().dapq_evict(ctx, q_pre.data_ptr(), C.byref(view), kk_p, k_out.data_ptr(),
+    _check(ctx, load_library().dapq_evict(ctx, q_pre.data_ptr(), view, kk_p, k_out.data_ptr(),
                                           v_out.data_ptr(), _ptr(idx_out), _ptr(scores_out), _stream(stream)))
 
 
@@ -265,17 +277,13 @@ def dapq_evict_layers(ctx, q_pre: Sequence[torch.Tensor], k: Sequence[torch.Tens
                       idx_out: Optional[Sequence[torch.Tensor]] = None, stream=None, host: bool = False) -> None:
     """k_keep: one budget row [batch] for all layers, or one row per layer [n_layers][batch]."""
     n = len(k)
-    views = (dapq_cache_view * n)()
-    keep_alive = []
-    for l in range(n):
-        view = _view(k[l], v[l], cu_rows, prompt_len)
-        keep_alive.append(view)
-        C.memmove(C.byref(views, l * C.sizeof(dapq_cache_view)), C.byref(view), C.sizeof(dapq_cache_view))
+    packed = [_view(k[l], v[l], cu_rows, prompt_len) for l in range(n)]
+    views = b"".join(p[0] for p in packed)
     budgets = np.asarray(k_keep, dtype=np.int32)
     assert budgets.ndim == 1 or (budgets.ndim == 2 and budgets.shape[0] == n)
     kk, kk_p = _i32(budgets.reshape(-1))
     stride = budgets.shape[1] if budgets.ndim == 2 else 0
-    arr = lambda ts: (C.c_void_p * n)(*[t.data_ptr() for t in ts])
+    arr = lambda ts: struct.pack("@%dP" % n, *[t.data_ptr() for t in ts], *[0] * (n - len(ts)))
     idx_arr = arr(idx_out) if idx_out is not None else None
     fn = load_library().dapq_evict_layers_host if host else load_library().dapq_evict_layers
     _check(ctx, fn(ctx, n, arr(q_pre), views, kk_p, stride, arr(k_out), arr(v_out), idx_arr, _stream(stream)))
@@ -292,9 +300,9 @@ def dapq_evict_host(ctx, q_pre: torch.Tensor, k: torch.Tensor, v: torch.Tensor, 
     """All tensors are HOST tensors (pinned for full copy speed); returns after the results landed."""
     for t in (q_pre, k, v, k_out, v_out):
         assert not t.is_cuda
-    view = _view(k, v, cu_rows, prompt_len)
+    view, keep_alive = _view(k, v, cu_rows, prompt_len)
     kk, kk_p = _i32(k_keep)
-    _check(ctx, load_library().dapq_evict_host(ctx, q_pre.data_ptr(), C.byref(view), kk_p, k_out.data_ptr(),
+    _check(ctx, load_library().dapq_evict_host(ctx, q_pre.data_ptr(), view, kk_p, k_out.data_ptr(),
                                                v_out.data_ptr(), _ptr(idx_out), _stream(stream)))
 
 
@@ -310,9 +318,9 @@ def dapq_score_static(n_q_heads: int, n_kv_heads: int, n_pseudo: int, dtype: int
     sh = dapq_shape(n_q_heads=n_q_heads, n_kv_heads=n_kv_heads, head_dim=head_dim, n_pseudo=n_pseudo,
                     max_batch=len(prompt_len), dtype=dtype, max_total_rows=int(cu_rows[-1]), rope_base=1.0,
                     softmax_scale=softmax_scale)
-    view = _view(k, None, cu_rows, prompt_len)
+    view, keep_alive = _view(k, None, cu_rows, prompt_len)
     err = C.create_string_buffer(512)
-    st = load_library().dapq_score_static(C.byref(sh), device, q_rot.data_ptr(), C.byref(view), scores.data_ptr(),
+    st = load_library().dapq_score_static(C.byref(sh), device, q_rot.data_ptr(), view, scores.data_ptr(),
                                           _stream(stream), err, len(err))
     if st != DAPQ_OK:
         raise DapqError(st, err.value.decode())
