@@ -257,6 +257,31 @@ def test_topk_score_distributions(dq, case):
     dq.dapq_destroy(ctx)
 
 
+@pytest.mark.parametrize("lens", [(1, 2, 3, 4093, 4094), (4095,), (8190, 5), (16381,), (32766, 1, 2), (65533,), (65537,), (131070,)])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+def test_topk_heads_between_16_byte_boundaries(dq, lens, offset):
+    """Heads whose first score lies 0 to 3 scores behind a 16-byte boundary, at the lengths where a thread's keys or
+    a CTA's slice just do, or just do not, hold the head and what lies before it."""
+    rng = np.random.default_rng(17 + offset)
+    H, keep = 5, tuple(max(1, L // 5) for L in lens)
+    w = _small(lens=lens, keep=keep, n_q_heads=H, n_kv_heads=H, n_pseudo=4, n_needles=0, outlier_channels=0)
+    T = w.total_prompt
+    s = rng.lognormal(0.0, 1.0, size=(H, T)).astype(np.float32)
+    s[1] = np.round(s[1] * 4) / 4                          # ties
+    buf = torch.full((H * T + offset,), 9e9, dtype=torch.float32, device="cuda")
+    buf[offset:] = torch.from_numpy(s).reshape(-1).cuda()
+    ctx = _ctx(dq, w)
+    idx = torch.full((H, int(w.cu_keep[-1])), -1, dtype=torch.int32, device="cuda")
+    dq.dapq_topk_select(ctx, buf[offset:], w.cu_prompt, keep, idx)
+    torch.cuda.synchronize()
+    got = idx.cpu().numpy()
+    for b in range(len(lens)):
+        for h in range(H):
+            ref = orc.topk_select(s[h, w.cu_prompt[b]:w.cu_prompt[b + 1]].astype(np.float64), keep[b])
+            np.testing.assert_array_equal(got[h, w.cu_keep[b]:w.cu_keep[b + 1]], ref, err_msg=f"b={b} h={h}")
+    dq.dapq_destroy(ctx)
+
+
 # --------------------------------------------------------------------------- dapq_compact_kv
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_compact_bit_exact_given_oracle_indices(dq, dtype):
