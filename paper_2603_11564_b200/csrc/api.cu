@@ -31,6 +31,7 @@ struct dapq_ctx {
   float* slots = nullptr;        // [query groups, H_kv, max_total_rows] (sized for groups of 256 query rows; used when sweep 2 has more than one group)
   long long wait_limit = 0;      // cycles a device-side wait may take (0: the default, about a second)
   int32_t* idx = nullptr;        // [H_kv, max_total_rows]
+  PruneBuffers prune = {};       // the pruned selection (sums == nullptr: not available)
   // staging for the host-buffer entry points (allocated on first use): two sets, so that the copies of one
   // layer run beside the kernels of the layer before
   struct HostStage {
@@ -249,6 +250,13 @@ dapq_status run_score(dapq_ctx* ctx, int q_dtype, const void* q_rot, const Cache
   return DAPQ_OK;
 }
 
+void free_prune(PruneBuffers* pr) {
+  void* bufs[] = {pr->part_m, pr->sums, pr->cand, pr->hist};
+  for (void* p : bufs)
+    if (p) cudaFree(p);
+  *pr = PruneBuffers{};
+}
+
 // Eq. 5 on the scores, or on their pooled image if the context asks for pooling.
 dapq_status run_select(dapq_ctx* ctx, const float* scores, int64_t score_stride, int32_t* idx, int64_t idx_stride,
                        const SeqTable& t, cudaStream_t s) {
@@ -342,6 +350,20 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
   ok = ok && cudaMemcpy(ctx->inv_freq, freq, sizeof(freq), cudaMemcpyHostToDevice) == cudaSuccess;
   ok = ok && cudaMemset(ctx->status, 0, sizeof(int)) == cudaSuccess;
   if (!ok) { cudaGetLastError(); return bail(DAPQ_ERR_CUDA, "workspace allocation failed"); }
+  if (wants_umma(ctx) && !wants_lo(ctx) && !(sh->flags & DAPQ_FLAG_Q_BF16) && sh->pool_mode == DAPQ_POOL_NONE &&
+      qg_groups(ctx->dims) <= kPruneSums && prune_available()) {
+    PruneBuffers& pr = ctx->prune;
+    const bool got = cudaMalloc(&pr.part_m, part_elems * sizeof(float2)) == cudaSuccess &&
+                     cudaMalloc(&pr.sums, kPruneSums * (sh->n_kv_heads * rows + 4) * sizeof(float)) == cudaSuccess &&
+                     cudaMalloc(&pr.cand, (size_t)sh->n_kv_heads * rows * sizeof(int32_t)) == cudaSuccess &&
+                     cudaMalloc(&pr.hist, (size_t)sh->max_batch * sh->n_kv_heads * kPruneHist * sizeof(uint32_t)) == cudaSuccess;
+    if (!got) {                                                 // no room: the two full sweeps need none of these
+      cudaGetLastError();
+      free_prune(&pr);
+    }
+    pr.part_s = ctx->part;
+    pr.ref = ctx->lse2;
+  }
   *out = ctx;
   return DAPQ_OK;
 }
@@ -353,6 +375,7 @@ void dapq_destroy(dapq_ctx* ctx) {
     void* bufs[] = {ctx->inv_freq, ctx->status, ctx->q_rot, ctx->part, ctx->lse2, ctx->scores, ctx->pooled, ctx->slots, ctx->idx};
     for (void* p : bufs)
       if (p) cudaFree(p);
+    free_prune(&ctx->prune);
     for (auto& st : ctx->hs) {
       void* sb[] = {st.q, st.k, st.v, st.ko, st.vo, st.idx};
       for (void* p : sb)
@@ -570,7 +593,15 @@ dapq_status evict_impl(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* 
     e = launch_rope(ctx->shape.dtype, qplan.q_is_f16 ? kRopeOutF16 : kRopeOutBf16, 0, q_pre, ctx->q_rot, ctx->inv_freq, t,
                     ctx->dims, after_own_compaction, s, &ctx->log, &ref);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "rope kernel");
-    st = run_score_qg(ctx, qplan, t, nullptr, scores, score_stride, nullptr, true, s);
+    PrunePlan pplan;
+    if (!scores_out && ctx->prune.sums && prune_plan(qplan, cd, t, ctx->dims, ctx->n_sm, &pplan)) {
+      // nobody reads the scores: only those that can be among the K largest are computed
+      e = launch_prune(pplan, cd, t, ctx->dims, ctx->prune, ctx->slots, scores, score_stride, ctx->status, ctx->wait_limit, s,
+                       &ctx->log);
+      if (e != cudaSuccess) return cuda_fail(ctx, e, "pruned score kernels");
+    } else {
+      st = run_score_qg(ctx, qplan, t, nullptr, scores, score_stride, nullptr, true, s);
+    }
   } else if (wants_umma(ctx) && wants_lo(ctx) && umma_plan(ctx->q_rot, 1, lo_rows, cd, t, ctx->dims, ctx->n_sm, &plan)) {
     // older tensor-core scorer: rotated queries as a bf16 pair hi + lo, the lo part added by a second MMA
     // pass in the sweeps that the flags name

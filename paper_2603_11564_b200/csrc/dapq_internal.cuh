@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "dapq.h"
 
@@ -214,6 +215,29 @@ cudaError_t launch_score_split(const SplitPlan& plan, int q_dtype, const void* q
                                const float* lse_in, float2* part, float* slots, float* scores, int64_t score_stride, float* lse_out,
                                int* status, long long wait_limit, bool after_own_kernel, cudaStream_t s, LaunchLog* log);
 
+// ---- the pruned selection: dapq_evict without score output (score_prune.cu) ----------------------------------
+constexpr int kPruneSums = 4;              // partial sums per key
+constexpr int kPruneBins = 2048, kPruneHist = kPruneBins + 4;   // histogram of a head's lower bounds, then its candidate count
+struct PrunePlan {
+  QgPlan qg;                               // the full scorer's plan; sweep 2's cut serves the candidates
+  CUtensorMap tm_s;                        // every 16th key
+  SeqTable ts;                             // the sequences of the sample
+  ChunkTable ct_s, ct_m;                   // chunks of the sample's sweep and of the one-pass sweep
+  int32_t n_stages_m, per_cta, gather_ctas;
+};
+struct PruneBuffers {                      // device workspace
+  float2 *part_s, *part_m;                 // umma_part_elems each
+  float* ref;                              // [B, H_q, N]: first the rotation's reference logits, then the estimates
+  float* sums;                             // kPruneSums * (H_kv * max_total_rows rounded up to 4)
+  int32_t* cand;                           // [H_kv][max_total_rows]
+  uint32_t* hist;                          // [max_batch, H_kv][kPruneHist]
+};
+bool prune_available();
+bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const Dims& dm, int n_sm, PrunePlan* plan);
+// scores: [H_kv][score_stride], those of keys that cannot be selected are negative; slots as for launch_score_qg.
+cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTable& t, const Dims& dm, const PruneBuffers& buf,
+                         float* slots, float* scores, int64_t score_stride, int* status, long long wait_limit,
+                         cudaStream_t s, LaunchLog* log);
 cudaError_t launch_topk(const float* scores, int64_t score_stride, int32_t* idx, int64_t idx_stride,
                         const SeqTable& t, int n_kv_heads, cudaStream_t s, LaunchLog* log);
 

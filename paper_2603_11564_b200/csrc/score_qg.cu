@@ -201,7 +201,7 @@ cudaError_t launch_slots_sum(const float* slots, int n_slots, float* scores, int
 cudaError_t launch_score_qg(const QgPlan& plan, const SeqTable& t, const Dims& dm, const float* lse_in, float2* part,
                             float* slots, float* scores, int64_t score_stride, float* lse_out, const float* ref, int* status,
                             long long wait_limit, bool after_own_kernel, cudaStream_t s, LaunchLog* log) {
-  Args a;
+  Args a = {};
   a.n_pseudo = dm.n_pseudo;
   a.group = dm.group;
   a.n_q_heads = dm.n_q_heads;

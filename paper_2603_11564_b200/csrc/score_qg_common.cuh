@@ -16,6 +16,7 @@ constexpr int kGroupRows = 256;                // most query rows a CTA keeps re
 constexpr int kEpiGroups = 4;                  // epilogue groups of 4 warps (128 TMEM lanes each)
 constexpr int kConvWarps = 4;                  // warps that convert the K tiles in place
 constexpr int kFirstEpiWarp = 2 + kConvWarps;
+constexpr int kThreadsOne = 24 * 32;             // the one-pass form of sweep 2: whole groups of four warps per role
 constexpr int kEpiThreads = kEpiGroups * 128;
 constexpr int kThreads1 = (kFirstEpiWarp + 4 * kEpiGroups) * 32;        // sweep 1: 22 warps
 constexpr int kThreads2 = kThreads1 + 32;                               // sweep 2: one more warp sums the groups' partials
@@ -83,6 +84,17 @@ struct Args {
   float* scores;             // [n_qgroups][H_kv][score_stride] when n_qgroups > 1 (one slot per group), else [H_kv][score_stride]
   int64_t score_stride, slot_stride;
   int* status;
+  // the pruned selection (score_prune.cu)
+  int32_t sampled;           // sweep 1 over a sample of the prompt: no synthetic keys
+  float log2_sample;         // one-pass sweep: log2 of the sample's stride
+  int32_t sum_groups;        // one-pass sweep: partial column sums kept per CTA (1, 2 or 4), in slots like the scores
+  float2* part_out;          // one-pass sweep: its own partials (`part` holds the sample's)
+  float* ref_out;            // one-pass sweep: [B, H_q, N] the estimate of each row's log-sum-exp that it worked with
+  uint32_t* hist;            // [B, H_kv][kPruneHist] histogram and candidate count of every head (one-pass sweep: cleared)
+  const int32_t* cand;       // [H_kv][score_stride] candidate positions, sequence b's from column cu_prompt[b] on
+  int32_t gather_ctas;       // CTAs per (sequence, KV head, query group) of the sweep over the candidates
+  const void* k;             // the keys, for the loads that TMA does not do
+  int64_t k_head_stride, k_row_stride;
 };
 
 // This CTA's work: sequence, tile range, first cache row, its query group.
@@ -97,7 +109,7 @@ __device__ __forceinline__ Work cta_work(const SeqTable& t, const ChunkTable& ct
   const int kvh = blockIdx.y;
   w.b = find_segment(ct.cu_chunk, t.batch, w.chunk);
   w.L = t.prompt_len[w.b];
-  const int n_keys = w.L + (with_synthetic ? a.n_pseudo : 0);
+  const int n_keys = w.L + (with_synthetic && !a.sampled ? a.n_pseudo : 0);
   const int n_tiles = (n_keys + tile_keys - 1) / tile_keys;
   w.t0 = (w.chunk - ct.cu_chunk[w.b]) * ct.chunk_tiles;
   w.nt = min(n_tiles, w.t0 + ct.chunk_tiles) - w.t0;

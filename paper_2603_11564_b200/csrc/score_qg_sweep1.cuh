@@ -228,7 +228,8 @@ rowstat_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // running max (raw dot product) and sum of this thread's row of block 0 / block 1
     float m_raw0 = -CUDART_INF_F, z0 = 0.f, m_raw1 = -CUDART_INF_F, z1 = 0.f;
     RowSum rs0, rs1;                                            // ... or, with reference logits, the rows' sums
-    const int i_q0 = (w.qgrp * a.rows_g + r) % N, i_q1 = (w.qgrp * a.rows_g + 128 + r) % N;   // pseudo-query indices
+    // pseudo-query indices (sampled: the keys end with the prompt)
+    const int i_q0 = a.sampled ? -1 : (w.qgrp * a.rows_g + r) % N, i_q1 = a.sampled ? -1 : (w.qgrp * a.rows_g + 128 + r) % N;
     if (kFold) {
       // The [256 x 16] operand: row i holds -r_i as an fp16 pair in channels 0 and 1 (zeros elsewhere, also
       // for rows beyond the group); the operand of ones carries its two ones in BOTH 16-byte halves of every

@@ -928,3 +928,92 @@ def test_split_operand_scorer_wait_limit(dq):
         dq.dapq_set_wait_limit(ctx, 0)
         _check_evict(w, data, _gpu_evict(dq, w, data, ctx), util.oracle_evict(w, data))
         dq.dapq_destroy(ctx)
+
+
+# --------------------------------------------------------- the retained set without the scores (pruned selection)
+# At the smallest sizes that take it (1e8 query-key pairs): 1, 2, 3 and 4 query groups with full and ragged ends, one and
+# two score slots, odd lengths, ragged batches, budgets from one row to a quarter of a prompt.
+PRUNE_CASES = [
+    # H_q, H_kv, N, lengths, budgets
+    (32, 8, 32, (98000,), (983,)), (32, 8, 64, (49003,), (1,)), (28, 4, 64, (60001,), (15000,)), (64, 8, 128, (16411,), (500,)),
+    (12, 4, 100, (90003,), (5000,)), (6, 1, 128, (131072,), (1310,)), (5, 1, 104, (200001,), (9000,)),
+    (32, 8, 32, (30001, 9000, 2049, 30000, 37003), (3000, 900, 200, 2000, 40)), (32, 8, 32, (8192,) * 13, (256,) * 13),
+]
+
+
+@pytest.mark.parametrize("hq,hkv,n,lens,keep", PRUNE_CASES)
+@pytest.mark.parametrize("keys", ["plain", "outliers", "far", "equal"])
+def test_pruned_selection_matches_the_full_sweeps(dq, hq, hkv, n, lens, keep, keys):
+    """dapq_evict without scores_out against the same call with it (both full sweeps).  The two score a candidate with
+    log-sum-exps that were summed in another order (some 1e-6 apart): the sets may differ only in keys whose
+    score lies within 1e-5 of the K-th.  keys: N(0, 1); four channels x 8; three keys whose logit for one row of a
+    head lies 150 above the bulk and that the sample misses (its row sums leave the float range); all keys equal."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(hq * 1000 + n)
+    w = _small(lens=lens, keep=keep, n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0)
+    q = torch.randn((w.batch, hq, n, 128), generator=g, device="cuda").bfloat16()
+    k = torch.randn((hkv, w.total_rows, 128), generator=g, device="cuda")
+    ctx = _ctx(dq, w)
+    if keys == "outliers":
+        k[:, :, [3, 40, 77, 100]] *= 8
+    elif keys == "far":
+        rot = torch.empty_like(q)
+        dq.dapq_rope_pseudo_q(ctx, q, list(lens), rot)
+        for h in range(hkv):
+            for pos in (0, lens[0] // 2 // 16 * 16, lens[0] // 16 * 16):       # (the sample takes rows 7, 23, ...)
+                u = rot[0, h * (hq // hkv), pos % n].float()
+                k[h, pos] = 150.0 * 128 ** 0.5 * u / u.norm() ** 2
+    elif keys == "equal":
+        k[:] = k[:, :1]
+    k = k.bfloat16()
+    v = torch.randn(k.shape, generator=g, device="cuda", dtype=torch.bfloat16)
+    KT = int(w.cu_keep[-1])
+
+    def call(scores):
+        idx = torch.full((hkv, KT), -1, dtype=torch.int32, device="cuda")
+        ko, vo = (torch.zeros((hkv, KT, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        before = dq.dapq_launch_count(ctx)
+        dq.dapq_evict(ctx, q, k, v, w.cu_rows, list(lens), list(keep), ko, vo, idx, scores)
+        dq.dapq_poll_status(ctx)
+        return idx, ko, vo, dq.dapq_launch_count(ctx) - before
+
+    scores = torch.empty((hkv, w.total_prompt), dtype=torch.float32, device="cuda")
+    full, _, _, n_full = call(scores)
+    idx, ko, vo, n_pruned = call(None)
+    assert n_pruned > n_full                                                   # the pruned selection ran
+    assert torch.equal(call(None)[0], idx)                                     # and gives the same set again
+    for b in range(w.batch):
+        o, e, p = int(w.cu_keep[b]), int(w.cu_keep[b + 1]), int(w.cu_prompt[b])
+        for h in range(hkv):
+            x, y = full[h, o:e].long(), idx[h, o:e].long()
+            assert bool((y[1:] > y[:-1]).all()) and int(y[0]) >= 0 and int(y[-1]) < lens[b]
+            rows = y + int(w.cu_rows[b])
+            assert torch.equal(ko[h, o:e], k[h, rows]) and torch.equal(vo[h, o:e], v[h, rows])
+            if not torch.equal(x, y):
+                s = scores[h, p:p + lens[b]]
+                kth = s[x].min()
+                other = torch.tensor(sorted(set(x.tolist()) ^ set(y.tolist())), device="cuda")
+                assert bool(((s[other] - kth).abs() <= 1e-5 * kth).all()), (b, h, len(other))
+    dq.dapq_destroy(ctx)
+
+
+def test_pruned_selection_wait_limit(dq):
+    """A device-side wait of the pruned selection that runs out: status once, and the context works again."""
+    hq, hkv, n, L, K = 28, 4, 64, 60001, 2000
+    w = _small(lens=(L,), keep=(K,), n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0)
+    q, k, v = (torch.randn(s, device="cuda").bfloat16() for s in ((1, hq, n, 128), (hkv, L + n, 128), (hkv, L + n, 128)))
+    ctx = _ctx(dq, w)
+    outs = [[torch.zeros((hkv, K, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2)] + [torch.zeros((hkv, K), dtype=torch.int32, device="cuda")]
+            for _ in range(2)]
+    dq.dapq_evict(ctx, q, k, v, w.cu_rows, [L], [K], *outs[0])
+    dq.dapq_poll_status(ctx)
+    dq.dapq_set_wait_limit(ctx, 1)
+    dq.dapq_evict(ctx, q, k, v, w.cu_rows, [L], [K], *outs[1])
+    with pytest.raises(dq.DapqError) as e:
+        dq.dapq_poll_status(ctx)
+    assert e.value.status == dq.DAPQ_ERR_TIMEOUT
+    dq.dapq_set_wait_limit(ctx, 0)
+    dq.dapq_evict(ctx, q, k, v, w.cu_rows, [L], [K], *outs[1])
+    dq.dapq_poll_status(ctx)
+    assert all(torch.equal(x, y) for x, y in zip(*outs))
+    dq.dapq_destroy(ctx)
