@@ -222,8 +222,8 @@ struct PrunePlan {
   QgPlan qg;                               // the full scorer's plan; sweep 2's cut serves the candidates
   CUtensorMap tm_s;                        // every 16th key
   SeqTable ts;                             // the sequences of the sample
-  ChunkTable ct_s, ct_m;                   // chunks of the sample's sweep and of the one-pass sweep
-  int32_t n_stages_m, per_cta, gather_ctas;
+  ChunkTable ct_s, ct_m, ct_g;             // chunks of the sample's sweep and of the one-pass sweep; CTAs per candidate list
+  int32_t n_stages_m, per_cta;
 };
 struct PruneBuffers {                      // device workspace
   float2 *part_s, *part_m;                 // umma_part_elems each

@@ -15,10 +15,13 @@
 // Nothing depends on how good the estimate is but the number of candidates.  A row sum that leaves the float range
 // is done over again by itself (careful_row).
 //
-// Measured on B200, a layer with the two full sweeps -> here (prompts whose relevant passages stand out: candidates = K):
-// 128 k, 8 KV heads x 1024 query rows 690 -> 460 us; 128 k, 4 x 448 rows 182 -> 139; 8 ragged prompts of 8 to 31 k,
-// 8 x 128 rows 187 -> 154; 40 x 8 k 365 -> 301; 32 k, 8 x 256 rows 64 -> 65 (2 us more for each of the two more
-// launches, and the sample and the bounds at their start-up times): hence the least number of query-key pairs below.
+// Measured on B200, a layer with the two full sweeps -> here, on prompts whose relevant passages stand out (candidates = K):
+// 128 k, 8 KV heads x 1024 query rows 690 -> 460 us; 128 k, 4 x 448 rows 182 -> 139; 40 prompts of 8 k, 8 x 128 rows 365 -> 301;
+// 32 k, 8 x 256 rows 64 -> 65 (four more launches, the sample and the bounds at their start-up times).  On N(0, 1) keys, which
+// stand out by nothing, a fifth to a quarter of them are candidates at 128 k (704 -> 605 us with outlier channels, 188 ->
+// 162), but a sample of a few hundred keys bounds nothing: 8 prompts of 4 to 32 k that keep a tenth of their rows 206 -> 285.
+// Hence the conditions in prune_plan: enough query-key pairs, and a budget of at most a sixteenth of a prompt (an
+// eighth of a long one), so that the threshold lies in the tail of the scores.
 #include "score_qg_sweep1.cuh"
 #include "score_qg_sweep2.cuh"
 
@@ -54,13 +57,18 @@ __device__ __forceinline__ int bound_bin(float lo) {
   return lo < 3e38f ? min(max(x, 0), kPruneBins - 1) : 0;       // (a sum beyond the float range bounds nothing from below)
 }
 
+// Scores between the 16-byte boundary before a head's first score and that score.
+__device__ __forceinline__ int head_lead(const SeqTable& t, const BoundArgs& a, int b, int kvh) {
+  return (int)(((int64_t)kvh * a.score_stride + t.cu_prompt[b]) & 3);
+}
+
 // The kBoundKeys positions of this thread begin at a 16-byte boundary of the head's arrays, whatever the head's offset.
 struct BoundSpan {
   int base, v0, nv;
   int64_t at;                              // of position 0, in the arrays
   __device__ __forceinline__ BoundSpan(const SeqTable& t, const BoundArgs& a, int b, int kvh, int tile) {
     at = (int64_t)kvh * a.score_stride + t.cu_prompt[b];
-    base = tile * kBoundTile + (int)threadIdx.x * kBoundKeys - (int)(at & 3);
+    base = tile * kBoundTile + (int)threadIdx.x * kBoundKeys - head_lead(t, a, b, kvh);
     v0 = max(0, -base);
     nv = max(0, min(kBoundKeys, t.prompt_len[b] - base));
   }
@@ -95,7 +103,7 @@ bound_hist_kernel(const __grid_constant__ SeqTable t, const __grid_constant__ Ch
   __shared__ uint32_t f_min[kPruneSums], f_max[kPruneSums];
   const int tid = threadIdx.x, kvh = blockIdx.y, b = blockIdx.z, H = gridDim.y;
   pdl_trigger();
-  if ((int)blockIdx.x * kBoundTile >= t.prompt_len[b] + 3) return;
+  if ((int)blockIdx.x * kBoundTile - head_lead(t, a, b, kvh) >= t.prompt_len[b]) return;
   for (int x = tid; x < kPruneBins; x += kBoundThreads) hist[x] = 0u;
   if (tid < kPruneSums) { f_min[tid] = 0x7f800000u; f_max[tid] = 0u; }
   __syncthreads();
@@ -127,7 +135,7 @@ bound_hist_kernel(const __grid_constant__ SeqTable t, const __grid_constant__ Ch
     int eg = 3;
     while (eg > 0 && (rr >> 4) < (eg * nch) / 4) --eg;          // the epilogue group that held the row's column
     const int g = qg * a.per_cta + (a.per_cta == 4 ? eg : (a.per_cta == 2 ? eg >> 1 : 0));
-    atomicMin(&f_min[g], __float_as_uint(f));
+    atomicMin(&f_min[g], __float_as_uint(f));                    // (positive floats order like their bit patterns)
     atomicMax(&f_max[g], __float_as_uint(f));
   }
   __syncthreads();
@@ -166,7 +174,7 @@ bound_list_kernel(const __grid_constant__ SeqTable t, const BoundArgs a) {
   __shared__ uint32_t list_at;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, kvh = blockIdx.y, b = blockIdx.z, H = gridDim.y;
   pdl_trigger();
-  if ((int)blockIdx.x * kBoundTile >= t.prompt_len[b] + 3) return;
+  if ((int)blockIdx.x * kBoundTile - head_lead(t, a, b, kvh) >= t.prompt_len[b]) return;
   pdl_wait();
   const BoundSpan sp(t, a, b, kvh, blockIdx.x);
   float hi[kBoundKeys];
@@ -245,10 +253,10 @@ bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const D
   double pairs = 0.0;
   for (int b = 0; b < t.batch; ++b) {
     const int L = t.prompt_len[b], K = t.cu_keep[b + 1] - t.cu_keep[b];
-    if (L < 2048 || L > 8 * 32 * 1024 - 4 || K > L / 4) return false;
+    if (L < 2048 || K > L / (L < 65536 ? 16 : 8)) return false;
     pairs += (double)rows * dm.n_kv_heads * L;
   }
-  if (pairs < 1e8) return false;                                // (6.7e7: even, 1.5e8: a sixth less; see above)
+  if (pairs < 1e8) return false;
   plan->qg = qg;
   plan->per_cta = kPruneSums / qg.n_qgroups;
   // ---- the sample: rows kSamplePhase, kSamplePhase + 16, ... of the cache, seen as a tensor of its own
@@ -273,8 +281,17 @@ bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const D
   if (plan->n_stages_m < 2) return false;
   if (!plan_chunks(ts, 0, kTile1, dm.n_kv_heads * qg.n_qgroups, n_sm, &plan->ct_s, 3.0)) return false;
   if (!plan_chunks(t, dm.n_pseudo, kTile2, dm.n_kv_heads * qg.n_qgroups, n_sm, &plan->ct_m, 6.0)) return false;
-  const int lists = t.batch * dm.n_kv_heads * qg.n_qgroups2;
-  plan->gather_ctas = n_sm > lists ? n_sm / lists : 1;
+  // ---- the candidates: a wave of CTAs shared out by the prompts' lengths
+  int64_t total = 0, upto = 0;
+  for (int b = 0; b < t.batch; ++b) total += t.prompt_len[b];
+  const int per_head = n_sm / (dm.n_kv_heads * qg.n_qgroups2);
+  memset(&plan->ct_g, 0, sizeof(ChunkTable));
+  for (int b = 0; b < t.batch; ++b) {
+    upto += t.prompt_len[b];
+    const int to = (int)(per_head * upto / total), least = plan->ct_g.cu_chunk[b] + 1;
+    plan->ct_g.cu_chunk[b + 1] = to > least ? to : least;
+  }
+  plan->ct_g.n_chunks = plan->ct_g.cu_chunk[t.batch];
   return true;
 }
 
@@ -361,7 +378,6 @@ cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTab
   // 4: the candidates' scores
   a.part = buf.part_m;
   a.cand = buf.cand;
-  a.gather_ctas = plan.gather_ctas;
   a.n_qgroups = plan.qg.n_qgroups2;
   a.rows_g = plan.qg.rows_g2;
   a.n_stages = plan.qg.n_stages2;
@@ -371,8 +387,8 @@ cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTab
     cudaError_t e2 = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e2 != cudaSuccess) return e2;
     log->begin(kKindSweep2, s);
-    e2 = launch_pdl(kernel, dim3(a.gather_ctas * a.n_qgroups, dm.n_kv_heads, t.batch), dim3(kThreads2), smem, s, 1, plan.qg.tm_k2, plan.qg.tm_q,
-                    t, plan.qg.ct2, plan.ct_m, a);
+    e2 = launch_pdl(kernel, dim3(plan.ct_g.n_chunks * a.n_qgroups, dm.n_kv_heads), dim3(kThreads2), smem, s, 1, plan.qg.tm_k2, plan.qg.tm_q,
+                    t, plan.ct_g, plan.ct_m, a);
     log->end(s);
     return e2;
   };

@@ -92,7 +92,6 @@ struct Args {
   float* ref_out;            // one-pass sweep: [B, H_q, N] the estimate of each row's log-sum-exp that it worked with
   uint32_t* hist;            // [B, H_kv][kPruneHist] histogram and candidate count of every head (one-pass sweep: cleared)
   const int32_t* cand;       // [H_kv][score_stride] candidate positions, sequence b's from column cu_prompt[b] on
-  int32_t gather_ctas;       // CTAs per (sequence, KV head, query group) of the sweep over the candidates
   const void* k;             // the keys, for the loads that TMA does not do
   int64_t k_head_stride, k_row_stride;
 };

@@ -83,8 +83,9 @@ __device__ __forceinline__ float colsum_job(uint32_t taddr, const float* lse_s, 
 //   kOnePass (score_prune.cu) the log-sum-exp is an estimate from a sample of the keys.  Every exponential is added
 //            twice: to its key's sum and to its query's, so that one pass yields the exact log-sum-exp and the scores up
 //            to the estimates' errors;
-//   kGather  the keys of a candidate list instead of a chunk, read by the converting warps; rows' log-sum-exp from
-//            the one-pass sweep's partials.
+//   kGather  the keys of a candidate list instead of a chunk; rows' log-sum-exp from the one-pass sweep's partials.
+//            A list of most of the prompt gives way to the whole prompt, whose tiles come in larger pieces (a listed tile
+//            takes about 0.85 us to gather, a job of 256 query rows 1.1).
 enum : int { kPlain = 0, kOnePass = 1, kGather = 2 };
 template <int kForm> struct Layout2 {
   // (kOnePass: its epilogue keeps 64 sums per thread and takes registers from the other roles; that works on whole
@@ -273,44 +274,55 @@ __device__ __forceinline__ void one_pass_epilogue(const Args& a, const Work& w, 
   }
 }
 
-// The K tiles of a candidate list, converted to fp16 on their way to shared memory (kConvWarps warps).  The rows
-// lie anywhere, so these warps read them themselves, 16 bytes per lane and eight loads in flight, and write the
-// layout that a TMA box would have left.  Slots beyond the list read its last row: nobody stores their scores.
-__device__ __forceinline__ void gather_tiles(const Work& w, const Args& a, int n_cand, int cand_base, int kvh, uint32_t sbase,
+// The K tiles of a candidate list, to shared memory and from bf16 to fp16 there (kConvWarps warps).  The rows lie
+// anywhere, so these warps copy them themselves, 16 bytes per lane, asynchronously and up to S tiles ahead, into the
+// layout that a TMA box would have left; a lane converts what it has copied.  (Single rows by TMA gather took 75
+// cycles per 128 bytes.)  Slots beyond the list take its last row: nobody stores their scores.
+__device__ __forceinline__ void gather_tiles(const Work& w, const Args& a, int n_cand, const int32_t* cand, int kvh, uint32_t sbase,
                                              const Bars& bars, int cw, const Waiter& wt) {
   using T = TileGeo<kTile2>;
-  const int lane = threadIdx.x & 31, S = a.n_stages, piece = lane & 15;
-  const uint32_t ring = sbase + (uint32_t)w.mb * 2u * 128u * 128u;
-  const int32_t* cand = a.cand + (int64_t)kvh * a.score_stride + cand_base;
-  const __nv_bfloat16* kb = reinterpret_cast<const __nv_bfloat16*>(a.k) + (int64_t)kvh * a.k_head_stride + (int64_t)w.row_base * a.k_row_stride;
-  Ring rs(S);
-  for (int ti = 0; ti < w.nt; ++ti, rs.next()) {
-    const int s = rs.i;
-    const int own = __ldg(cand + min((w.chunk + ti * a.gather_ctas) * kTile2 + cw * 32 + lane, n_cand - 1));
-    if (rs.wrapped && !__all_sync(0xffffffffu, wt.wait(bars.k_empty(s), rs.phase ^ 1u))) break;
-    const uint32_t dst = ring + s * T::kStage + (piece >> 3) * T::kHalf;
+  const int lane = threadIdx.x & 31, S = a.n_stages, piece = lane & 15, r0 = cw * 32 + (lane >> 4);
+  const uint32_t ring = sbase + (uint32_t)w.mb * 2u * 128u * 128u + (piece >> 3) * T::kHalf + r0 * 128;
+  const __nv_bfloat16* kb = reinterpret_cast<const __nv_bfloat16*>(a.k) + (int64_t)kvh * a.k_head_stride + (int64_t)w.row_base * a.k_row_stride + piece * 8;
+  // (row r0 + 2 i of the tile: its 16-byte pieces are permuted by the row's lowest three bits)
+  auto slot_at = [&](int s, int i) { return ring + s * T::kStage + i * 256 + (((piece & 7) ^ ((r0 + 2 * i) & 7)) << 4); };
+  auto issue = [&](int ti) {
+    if (ti < w.nt) {
+      const int own = __ldg(cand + min((w.t0 + ti) * kTile2 + cw * 32 + lane, n_cand - 1));
 #pragma unroll
-    for (int i0 = 0; i0 < 16; i0 += 8) {                        // two rows per round: 16 lanes each
-      uint4 v[8];
+      for (int i = 0; i < 16; ++i)
+        cp_async16(slot_at(ti % S, i), kb + (int64_t)__shfl_sync(0xffffffffu, own, 2 * i + (lane >> 4)) * a.k_row_stride);
+    }
+    cp_async_commit();
+  };
+  for (int ti = 0; ti < S; ++ti) issue(ti);
+  for (int ti = 0; ti < w.nt; ++ti) {
+    // tile ti has landed: S + ti - 1 groups have been committed by now (S before the first tile)
+    if (S == 2) cp_async_wait<0>(); else if (S == 3) cp_async_wait<1>(); else cp_async_wait<2>();
+    __syncwarp();
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int j = __shfl_sync(0xffffffffu, own, (i0 + i) * 2 + (lane >> 4));
-        v[i] = __ldg(reinterpret_cast<const uint4*>(kb + (int64_t)j * a.k_row_stride) + piece);
-      }
+    for (int i0 = 0; i0 < 16; i0 += 4) {
+      uint4 v[4];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int r = cw * 32 + (i0 + i) * 2 + (lane >> 4);
-        v[i].x = bf16x2_to_f16x2(v[i].x);
-        v[i].y = bf16x2_to_f16x2(v[i].y);
-        v[i].z = bf16x2_to_f16x2(v[i].z);
-        v[i].w = bf16x2_to_f16x2(v[i].w);
-        sts128(dst + r * 128 + (((piece & 7) ^ (r & 7)) << 4), v[i]);
+      for (int u = 0; u < 4; ++u) v[u] = lds128(slot_at(ti % S, i0 + u));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        v[u].x = bf16x2_to_f16x2(v[u].x);
+        v[u].y = bf16x2_to_f16x2(v[u].y);
+        v[u].z = bf16x2_to_f16x2(v[u].z);
+        v[u].w = bf16x2_to_f16x2(v[u].w);
+        sts128(slot_at(ti % S, i0 + u), v[u]);
       }
     }
     fence_proxy_async();
     __syncwarp();
-    if (lane == 0) mbar_arrive(bars.k_conv(s));
+    if (lane == 0) mbar_arrive(bars.k_conv(ti % S));
+    if (ti >= 1 && ti - 1 + S < w.nt) {                         // the slot of the tile before is free once its MMAs have retired
+      if (!__all_sync(0xffffffffu, wt.wait(bars.k_empty((ti - 1) % S), ((ti - 1) / S) & 1))) break;
+    }
+    if (ti >= 1) issue(ti - 1 + S);
   }
+  cp_async_wait<0>();                                           // (no copy in flight when the CTA returns)
 }
 
 // kNarrow (kOnePass): groups of up to 128 query rows.  kWide: the CTA keeps up to 512 query rows resident and runs two jobs per K tile (query columns 0..255 and
@@ -335,17 +347,22 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
   constexpr int kFirstEpi = Lay::first_epi;
   const int kvh = blockIdx.y;
   Work w;
-  int n_cand = 0;                                               // kGather: the candidates of this (sequence, head)
+  int n_cand = 0;                                               // kGather: candidates of this (sequence, head)
+  bool listed = kForm == kGather;                               // ... and whether the tiles are made of them
   if constexpr (kForm == kGather) {
     pdl_wait();
-    w.b = blockIdx.z;
-    w.chunk = blockIdx.x / a.n_qgroups;                         // this CTA takes every gather_ctas-th tile from here
-    w.qgrp = blockIdx.x - w.chunk * a.n_qgroups;
+    const int cta = blockIdx.x / a.n_qgroups;
+    w.qgrp = blockIdx.x - cta * a.n_qgroups;
+    w.b = find_segment(ct.cu_chunk, t.batch, cta);
+    w.chunk = cta - ct.cu_chunk[w.b];
+    const int n_ctas = ct.cu_chunk[w.b + 1] - ct.cu_chunk[w.b];
     w.L = t.prompt_len[w.b];
     n_cand = (int)a.hist[(w.b * a.n_kv_heads + kvh) * kPruneHist + kPruneBins];
     if (n_cand == t.cu_keep[w.b + 1] - t.cu_keep[w.b]) return;  // as many as are kept: they need no scores
-    w.t0 = 0;
-    w.nt = ((n_cand + kTile2 - 1) / kTile2 - w.chunk + a.gather_ctas - 1) / a.gather_ctas;
+    listed = kWide ? 8 * (int64_t)n_cand <= 7 * (int64_t)w.L : 3 * (int64_t)n_cand <= 2 * (int64_t)w.L;
+    const int n_tiles = ((listed ? n_cand : w.L) + kTile2 - 1) / kTile2, per = (n_tiles + n_ctas - 1) / n_ctas;
+    w.t0 = w.chunk * per;
+    w.nt = min(per, n_tiles - w.t0);
     w.row_base = t.cu_rows[w.b];
     w.qrow_base = (w.b * a.n_q_heads + kvh * a.group) * a.n_pseudo;
     w.rows = min(a.rows_g, a.rows_total - w.qgrp * a.rows_g);
@@ -383,7 +400,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
   // (behind this library's own sweep 1 or rotation kernel, keys and queries were complete before that kernel
   // got past its wait: both go out at once)
   const uint32_t tmem_base = cta_prologue<Smem>(smem, sbase, bars, [&] {
-    if (kForm == kGather) tma_queries(&tm_q, w, a, sbase, bars);
+    if (listed) tma_queries(&tm_q, w, a, sbase, bars);
     else if (a.early_loads) tma_first<kTile2, true>(&tm_k, &tm_q, w, a, sbase, bars, kvh);
   });
   // UMMA N: only the query columns that exist; job 1 (kWide) holds the rows from 256 on
@@ -526,8 +543,8 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     if constexpr (kForm == kOnePass && !kNarrow) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
     if (warp == 0) {
       if (lane == 0) {
-        if constexpr (kForm == kGather) {
-          drain_wait(bars.q_full(), 0, kWaitLimit);               // (the only copy of this form has landed)
+        if (listed) {
+          drain_wait(bars.q_full(), 0, kWaitLimit);             // (the only TMA copy of this form has landed)
         } else {
           if (!a.early_loads) tma_first<kTile2, true>(&tm_k, &tm_q, w, a, sbase, bars, kvh);
           tma_producer<kTile2, false, true>(&tm_k, &tm_q, w, a, sbase, bars, kvh, wt);
@@ -571,7 +588,8 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
         mma_drain(bars);
       }
     } else if (warp < 2 + kConvWarps) {
-      if constexpr (kForm == kGather) gather_tiles(w, a, n_cand, t.cu_prompt[b], kvh, sbase, bars, warp - 2, wt);
+      if (listed)
+        gather_tiles(w, a, n_cand, a.cand + (int64_t)kvh * a.score_stride + t.cu_prompt[b], kvh, sbase, bars, warp - 2, wt);
       else if (kConvert) convert_tiles<kTile2>(w, a, sbase, bars, warp - 2, wt);
     } else if (warp == Lay::sum_warp) {
       // ====================================================================== sum of the four groups
@@ -585,8 +603,8 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
   #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int r = q * 32 + lane;
-          if constexpr (kForm == kGather) {
-            const int c = (w.chunk + ti * a.gather_ctas) * kTile2 + r;
+          if (listed) {
+            const int c = (w.t0 + ti) * kTile2 + r;
             const float v = ((e[r] + e[128 + r]) + e[256 + r]) + e[384 + r];
             if (c < n_cand) out[cand[c]] = v;
           } else {

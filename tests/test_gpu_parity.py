@@ -932,12 +932,12 @@ def test_split_operand_scorer_wait_limit(dq):
 
 # --------------------------------------------------------- the retained set without the scores (pruned selection)
 # At the smallest sizes that take it (1e8 query-key pairs): 1, 2, 3 and 4 query groups with full and ragged ends, one and
-# two score slots, odd lengths, ragged batches, budgets from one row to a quarter of a prompt.
+# two score slots, odd lengths, ragged batches, budgets from one row to a sixteenth of a prompt.
 PRUNE_CASES = [
     # H_q, H_kv, N, lengths, budgets
-    (32, 8, 32, (98000,), (983,)), (32, 8, 64, (49003,), (1,)), (28, 4, 64, (60001,), (15000,)), (64, 8, 128, (16411,), (500,)),
+    (32, 8, 32, (98000,), (983,)), (32, 8, 64, (49003,), (1,)), (28, 4, 64, (60001,), (3750,)), (64, 8, 128, (16411,), (500,)),
     (12, 4, 100, (90003,), (5000,)), (6, 1, 128, (131072,), (1310,)), (5, 1, 104, (200001,), (9000,)),
-    (32, 8, 32, (30001, 9000, 2049, 30000, 37003), (3000, 900, 200, 2000, 40)), (32, 8, 32, (8192,) * 13, (256,) * 13),
+    (32, 8, 32, (30001, 9000, 2049, 30000, 37003), (1875, 500, 100, 1000, 40)), (32, 8, 32, (8192,) * 13, (256,) * 13),
 ]
 
 
