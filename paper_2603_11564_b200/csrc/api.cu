@@ -21,6 +21,8 @@ struct dapq_ctx {
   int64_t max_chunks = 0;
   int64_t q_rows_max = 0;        // max_batch * H_q * N
   // device workspace
+  void* owned[24] = {};          // its allocations
+  int n_owned = 0;
   double* inv_freq = nullptr;    // [d/2]
   int* status = nullptr;         // device status word
   void* q_rot = nullptr;         // [max_batch, H_q, N, d]
@@ -111,6 +113,37 @@ dapq_status cuda_fail(dapq_ctx* ctx, cudaError_t e, const char* what) {
     cudaError_t e_ = (call);                                        \
     if (e_ != cudaSuccess) return cuda_fail((ctx), e_, #call);      \
   } while (0)
+
+// Device buffers allocated together: as one block, cut up at 256-byte boundaries, where a block of its own for each
+// would cost up to a millisecond apiece (large ones), or each by itself, where the driver has small blocks at hand.
+struct Arena {
+  struct Part { void** p; size_t bytes; };
+  Part parts[12];
+  int n = 0;
+  size_t size = 0;
+  template <typename T> void add(T** p, size_t bytes) {
+    parts[n++] = {reinterpret_cast<void**>(p), (bytes + 255) & ~(size_t)255};
+    size += parts[n - 1].bytes;
+  }
+  bool allocate(dapq_ctx* ctx) {
+    const bool together = size >= (4u << 20);
+    char* at = nullptr;
+    if (together) {
+      if (cudaMalloc(&at, size) != cudaSuccess) return false;
+      ctx->owned[ctx->n_owned++] = at;
+    }
+    for (int i = 0; i < n; ++i) {
+      if (together) {
+        *parts[i].p = at;
+        at += parts[i].bytes;
+      } else {
+        if (cudaMalloc(parts[i].p, parts[i].bytes) != cudaSuccess) return false;
+        ctx->owned[ctx->n_owned++] = *parts[i].p;
+      }
+    }
+    return true;
+  }
+};
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -250,13 +283,6 @@ dapq_status run_score(dapq_ctx* ctx, int q_dtype, const void* q_rot, const Cache
   return DAPQ_OK;
 }
 
-void free_prune(PruneBuffers* pr) {
-  void* bufs[] = {pr->part_m, pr->sums, pr->cand, pr->hist};
-  for (void* p : bufs)
-    if (p) cudaFree(p);
-  *pr = PruneBuffers{};
-}
-
 // Eq. 5 on the scores, or on their pooled image if the context asks for pooling.
 dapq_status run_select(dapq_ctx* ctx, const float* scores, int64_t score_stride, int32_t* idx, int64_t idx_stride,
                        const SeqTable& t, cudaStream_t s) {
@@ -335,31 +361,34 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
   const size_t part_umma = (size_t)umma_part_elems(sh->max_batch, sh->n_q_heads, sh->n_kv_heads, sh->n_pseudo);
   if (part_umma > part_elems) part_elems = part_umma;
   const size_t rows = (size_t)sh->max_total_rows;
-  bool ok = true;
-  ok = ok && cudaMalloc(&ctx->inv_freq, sizeof(freq)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->status, sizeof(int)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->q_rot, (size_t)sh->max_batch * hq_n * kHeadDim * sizeof(float)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->part, part_elems * sizeof(float2)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->lse2, ((size_t)sh->max_batch * hq_n + 32) * sizeof(float)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->scores, (size_t)sh->n_kv_heads * rows * sizeof(float)) == cudaSuccess;
-  ok = ok && cudaMalloc(&ctx->idx, (size_t)sh->n_kv_heads * rows * sizeof(int32_t)) == cudaSuccess;
-  if (sh->pool_mode != DAPQ_POOL_NONE)
-    ok = ok && cudaMalloc(&ctx->pooled, (size_t)sh->n_kv_heads * rows * sizeof(float)) == cudaSuccess;
   const int n_slots = wants_umma(ctx) ? qg_groups(ctx->dims) : (wants_split(ctx) ? split_groups(ctx->dims) : 1);
-  if (n_slots > 1) ok = ok && cudaMalloc(&ctx->slots, (size_t)n_slots * sh->n_kv_heads * rows * sizeof(float)) == cudaSuccess;
+  const size_t score_bytes = (size_t)sh->n_kv_heads * rows * sizeof(float);
+  Arena ar;
+  ar.add(&ctx->inv_freq, sizeof(freq));
+  ar.add(&ctx->status, sizeof(int));
+  ar.add(&ctx->q_rot, (size_t)sh->max_batch * hq_n * kHeadDim * sizeof(float));
+  ar.add(&ctx->part, part_elems * sizeof(float2));
+  ar.add(&ctx->lse2, ((size_t)sh->max_batch * hq_n + 32) * sizeof(float));
+  ar.add(&ctx->scores, score_bytes);
+  ar.add(&ctx->idx, (size_t)sh->n_kv_heads * rows * sizeof(int32_t));
+  if (sh->pool_mode != DAPQ_POOL_NONE) ar.add(&ctx->pooled, score_bytes);
+  if (n_slots > 1) ar.add(&ctx->slots, n_slots * score_bytes);
+  bool ok = ar.allocate(ctx);
   ok = ok && cudaMemcpy(ctx->inv_freq, freq, sizeof(freq), cudaMemcpyHostToDevice) == cudaSuccess;
   ok = ok && cudaMemset(ctx->status, 0, sizeof(int)) == cudaSuccess;
   if (!ok) { cudaGetLastError(); return bail(DAPQ_ERR_CUDA, "workspace allocation failed"); }
   if (wants_umma(ctx) && !wants_lo(ctx) && !(sh->flags & DAPQ_FLAG_Q_BF16) && sh->pool_mode == DAPQ_POOL_NONE &&
-      qg_groups(ctx->dims) <= kPruneSums && prune_available()) {
+      qg_groups(ctx->dims) <= kPruneSums && (double)hq_n * rows >= kPruneLeastPairs && prune_available()) {
+    // (no room: the two full sweeps need none of these)
     PruneBuffers& pr = ctx->prune;
-    const bool got = cudaMalloc(&pr.part_m, part_elems * sizeof(float2)) == cudaSuccess &&
-                     cudaMalloc(&pr.sums, kPruneSums * (sh->n_kv_heads * rows + 4) * sizeof(float)) == cudaSuccess &&
-                     cudaMalloc(&pr.cand, (size_t)sh->n_kv_heads * rows * sizeof(int32_t)) == cudaSuccess &&
-                     cudaMalloc(&pr.hist, (size_t)sh->max_batch * sh->n_kv_heads * kPruneHist * sizeof(uint32_t)) == cudaSuccess;
-    if (!got) {                                                 // no room: the two full sweeps need none of these
+    Arena pa;
+    pa.add(&pr.part_m, part_elems * sizeof(float2));
+    pa.add(&pr.sums, kPruneSums * (score_bytes + 16));
+    pa.add(&pr.cand, (size_t)sh->n_kv_heads * rows * sizeof(int32_t));
+    pa.add(&pr.hist, (size_t)sh->max_batch * sh->n_kv_heads * kPruneHist * sizeof(uint32_t));
+    if (!pa.allocate(ctx)) {
       cudaGetLastError();
-      free_prune(&pr);
+      pr.sums = nullptr;
     }
     pr.part_s = ctx->part;
     pr.ref = ctx->lse2;
@@ -372,10 +401,7 @@ void dapq_destroy(dapq_ctx* ctx) {
   if (!ctx) return;
   {
     DeviceGuard guard(ctx->device);
-    void* bufs[] = {ctx->inv_freq, ctx->status, ctx->q_rot, ctx->part, ctx->lse2, ctx->scores, ctx->pooled, ctx->slots, ctx->idx};
-    for (void* p : bufs)
-      if (p) cudaFree(p);
-    free_prune(&ctx->prune);
+    for (int i = 0; i < ctx->n_owned; ++i) cudaFree(ctx->owned[i]);
     for (auto& st : ctx->hs) {
       void* sb[] = {st.q, st.k, st.v, st.ko, st.vo, st.idx};
       for (void* p : sb)

@@ -85,8 +85,8 @@ struct LaunchLog {
 // and its writes are visible (pdl_wait): its launch is then prepared, and its CTAs' set-up done,
 // while the predecessor still runs.  The short kernels that precede a long one (rotation,
 // selection) also signal at their start that the next kernel may be scheduled (pdl_trigger); the
-// sweeps do not: their successors' CTAs would only sit on the SMs the next sweep needs (measured:
-// slower).  The compaction signals at its start too: in dapq_evict_layers the next layer's
+// second sweeps do not: their successors' CTAs would only sit on the SMs the next sweep needs (measured:
+// slower); the first sweeps do where a CTA's run is short (see there).  The compaction signals at its start too: in dapq_evict_layers the next layer's
 // rotation, which touches nothing the compaction or the selection before it use, runs beside
 // them and waits at its END, so that the kernels after it stay ordered behind the compaction.
 // Both instructions are no-ops for a kernel launched the ordinary way.
@@ -217,6 +217,7 @@ cudaError_t launch_score_split(const SplitPlan& plan, int q_dtype, const void* q
 
 // ---- the pruned selection: dapq_evict without score output (score_prune.cu) ----------------------------------
 constexpr int kPruneSums = 4;              // partial sums per key
+constexpr double kPruneLeastPairs = 1e8;   // query-key pairs of a call below which the full sweeps are as fast
 constexpr int kPruneBins = 2048, kPruneHist = kPruneBins + 4;   // histogram of a head's lower bounds, then its candidate count
 struct PrunePlan {
   QgPlan qg;                               // the full scorer's plan; sweep 2's cut serves the candidates

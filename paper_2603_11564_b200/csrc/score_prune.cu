@@ -256,7 +256,7 @@ bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const D
     if (L < 2048 || K > L / (L < 65536 ? 16 : 8)) return false;
     pairs += (double)rows * dm.n_kv_heads * L;
   }
-  if (pairs < 1e8) return false;
+  if (pairs < kPruneLeastPairs) return false;
   plan->qg = qg;
   plan->per_cta = kPruneSums / qg.n_qgroups;
   // ---- the sample: rows kSamplePhase, kSamplePhase + 16, ... of the cache, seen as a tensor of its own
