@@ -588,7 +588,9 @@ TopkShape plan_topk(int heads, int max_len, int n_sm, int max_lead) {
     const int ctas = heads * n_cta;
     const int per_sm = (kpt <= 16 && ctas > n_sm) ? 2 : 1;
     const int waves = (ctas + n_sm * per_sm - 1) / (n_sm * per_sm);
-    const double cost = waves * ((n_cta == 1 ? 5.0 : 7.0) + 0.2 * kpt);
+    // (the cluster instances that fit two CTAs on an SM have 32 registers and take a third longer: 24 heads of up to 20 k keys
+    // 10.7 us with eight CTAs a head and two on an SM, 8.7 with four; 64 heads of 8 to 31 k keys 14.1 with four, 12.2 with two)
+    const double cost = waves * ((n_cta == 1 ? 5.0 : 7.0) + 0.2 * kpt) * (n_cta > 1 && per_sm == 2 ? 1.35 : 1.0);
     if (best.n_cta == 0 || cost < best_cost) { best = {n_cta, kpt, per_sm}; best_cost = cost; }
   }
   return best;
