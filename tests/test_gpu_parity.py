@@ -88,6 +88,35 @@ def test_rope_parity(dq, dtype, interleaved):
     dq.dapq_destroy(ctx)
 
 
+@pytest.mark.parametrize("interleaved", [False, True])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_rope_of_a_large_batch(dq, dtype, interleaved):
+    """65 sequences x 33 queries: enough blocks that each takes four queries, the last one a single one; 11 heads."""
+    B, N, H = 65, 33, 11
+    w = _small(lens=(8,) * B, keep=(1,) * B, dtype=dtype, n_q_heads=H, n_kv_heads=1, n_pseudo=N, rope_base=5.0e5, n_needles=0, outlier_channels=0)
+    ctx = _ctx(dq, w, flags=dq.DAPQ_FLAG_ROPE_INTERLEAVED if interleaved else 0)
+    q = torch.randn((B, H, N, 128), generator=torch.Generator().manual_seed(3)).to(w.torch_dtype())
+    pos = [(b * 2017) % 131072 for b in range(B)]
+    out = torch.empty_like(q, device="cuda")
+    dq.dapq_rope_pseudo_q(ctx, q.cuda(), pos, out)
+    torch.cuda.synchronize()
+    got = util.to_f64(out)
+    tol = 2.0 ** -8 if dtype == "bf16" else 2.0 ** -22                        # one rounding of the type; fp32: four (of the angles too)
+    for b in range(B):
+        ref = orc.rope_pseudo_q(util.to_f64(q[b]), pos[b], w.rope_base, interleaved=interleaved)
+        assert np.all(np.abs(got[b] - ref) <= tol * np.abs(ref) + 1e-7), b
+    dq.dapq_destroy(ctx)
+
+
+def test_evict_of_a_large_batch_of_short_prompts(dq):
+    """The same blocks with the reference logits of the first sweep (bf16, 132 query rows per KV head)."""
+    rng = np.random.default_rng(8)
+    lens = tuple(int(x) for x in rng.integers(1, 90, 65))
+    w = _small(lens=lens, keep=tuple(max(1, L // 3) for L in lens), n_q_heads=8, n_kv_heads=2, n_pseudo=33, n_needles=0, outlier_channels=0)
+    data = gi.draw_layer(w, 0, "cpu")
+    _check_evict(w, data, _gpu_evict(dq, w, data), util.oracle_evict(w, data))
+
+
 # --------------------------------------------------------------------------------- dapq_score
 SCORE_CASES = [
     # dtype, H_q, H_kv, N, prompt lengths
