@@ -84,7 +84,7 @@ struct LaunchLog {
 // waits, before its first access to global memory, until the kernel before it has completed
 // and its writes are visible (pdl_wait): its launch is then prepared, and its CTAs' set-up done,
 // while the predecessor still runs.  The short kernels that precede a long one (rotation,
-// selection) also signal at their start that the next kernel may be scheduled (pdl_trigger); the
+// behind its own wait, and selection) also signal early that the next kernel may be scheduled (pdl_trigger); the
 // second sweeps do not: their successors' CTAs would only sit on the SMs the next sweep needs (measured:
 // slower); the first sweeps do where a CTA's run is short (see there).  The compaction signals at its start too: in dapq_evict_layers the next layer's
 // rotation, which touches nothing the compaction or the selection before it use, runs beside

@@ -48,8 +48,11 @@ rope_pseudo_q_kernel(const T* __restrict__ q_pre, TO* __restrict__ q_rot,
   // late_wait: the kernel before this one in the stream neither writes q_pre nor still reads q_rot
   // (it is the compaction of the layer before), so the rotation runs beside it; the wait at the end
   // keeps this grid, and with it everything launched after it, ordered behind that kernel.
-  pdl_trigger();
+  // (the trigger comes behind the wait: the first sweep reads keys ahead of its own wait, so it may not start before
+  // whatever wrote them has completed.  With late_wait the keys were complete before an earlier layer's rotation got past
+  // its wait.)
   if (!late_wait) pdl_wait();
+  pdl_trigger();
   const int i0 = blockIdx.x * kQ, b = blockIdx.y, c = threadIdx.x;
   const int h = blockIdx.z * kHeadsPerBlock + threadIdx.y, n = min(kQ, n_pseudo - i0);
   const bool active = h < n_q_heads;
