@@ -80,7 +80,8 @@ enum { DAPQ_MAX_BATCH = 128, DAPQ_MAX_PSEUDO = 128, DAPQ_HEAD_DIM = 128, DAPQ_MA
 typedef enum { DAPQ_POOL_NONE = 0, DAPQ_POOL_MAX = 1, DAPQ_POOL_AVG = 2 } dapq_pool_mode;
 
 /* dapq_shape.flags.  DAPQ_FLAG_CUDA_CORE_SCORER keeps the scorer on the CUDA-core kernels
- * (fp32 arithmetic on unrounded rotated queries) even where the tensor-core path applies.
+ * (fp32 arithmetic on unrounded rotated queries) even where a tensor-core path applies: the one below, or, for
+ * fp32 caches and fewer than 64 query rows per KV head, the one that splits unrounded operands into bf16 parts.
  * DAPQ_FLAG_ROPE_INTERLEAVED: the rotation pairs channel 2c with 2c + 1 instead of c with
  * c + d/2 (Section 4.1 only says "RoPE"; the rotate-half pairing of the paper's Llama and Qwen
  * models is the default; the cache's keys must have been rotated with the same pairing).
@@ -162,7 +163,9 @@ DAPQ_API dapq_status dapq_set_wait_limit(dapq_ctx* ctx, int64_t cycles);
  * kernel launch is bracketed by CUDA events on its stream; dapq_profile(ctx, 1) also clears
  * the totals.  dapq_profile_read synchronises `stream` and returns, per kernel kind, the
  * summed device time in milliseconds and the number of launches since profiling was
- * enabled.  ms_out / count_out: host [DAPQ_PROF_KINDS], in the order of dapq_prof_kind. */
+ * enabled.  ms_out / count_out: host [DAPQ_PROF_KINDS], in the order of dapq_prof_kind.  Where only the keys that can be
+ * selected are scored: LSE_MERGE is the sample sweep, SWEEP1 the pass over all keys, SWEEP2 the candidates' scores, and the
+ * two kernels that make the candidate list count as TOPK. */
 typedef enum {
   DAPQ_PROF_ROPE = 0, DAPQ_PROF_SWEEP1 = 1, DAPQ_PROF_LSE_MERGE = 2, DAPQ_PROF_SWEEP2 = 3,
   DAPQ_PROF_TOPK = 4, DAPQ_PROF_COMPACT = 5, DAPQ_PROF_POOL = 6, DAPQ_PROF_RECALL = 7, DAPQ_PROF_SLOT_SUM = 8,
@@ -226,7 +229,9 @@ DAPQ_API dapq_status dapq_recall(dapq_ctx* ctx, const int32_t* idx_gold, const i
                         float* recall_out, void* stream);
 
 /* Figure 1, the whole eviction step for one layer: rotate to positions L_b + i, score,
- * select, compact.  idx_out, scores_out may be NULL (kept in the workspace). */
+ * select, compact.  idx_out, scores_out may be NULL (kept in the workspace).  Without scores_out (and without pooling)
+ * large calls with budgets that are small against their prompts compute the scores of those keys only that can be
+ * among the K largest: the same set, chosen by exact bounds, in less time. */
 DAPQ_API dapq_status dapq_evict(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* cache,
                        const int32_t* k_keep_host, void* k_out, void* v_out, int32_t* idx_out,
                        float* scores_out, void* stream);
