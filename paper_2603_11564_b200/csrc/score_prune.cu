@@ -16,12 +16,14 @@
 // is done over again by itself (careful_row).
 //
 // Measured on B200, a layer with the two full sweeps -> here, on prompts whose relevant passages stand out (candidates = K):
-// 128 k, 8 KV heads x 1024 query rows 690 -> 460 us; 128 k, 4 x 448 rows 182 -> 139; 40 prompts of 8 k, 8 x 128 rows 365 -> 301;
-// 32 k, 8 x 256 rows 64 -> 65 (four more launches, the sample and the bounds at their start-up times).  On N(0, 1) keys, which
-// stand out by nothing, a fifth to a quarter of them are candidates at 128 k (704 -> 605 us with outlier channels, 188 ->
-// 162), but a sample of a few hundred keys bounds nothing: 8 prompts of 4 to 32 k that keep a tenth of their rows 206 -> 285.
-// Hence the conditions in prune_plan: enough query-key pairs, and a budget of at most a sixteenth of a prompt (an
-// eighth of a long one), so that the threshold lies in the tail of the scores.
+// 128 k, 8 KV heads x 1024 query rows 690 -> 460 us; 128 k, 4 x 448 rows 182 -> 139; 32 k, 8 x 256 rows 64 -> 65 (four more
+// launches, the sample and the bounds at their start-up times).  On N(0, 1) keys, which stand out by nothing, a fifth to a
+// quarter of them are candidates at 128 k (704 -> 605 us with outlier channels, 188 -> 162), and a sample of 2 k keys is
+// the least that bounds anything: 8 prompts of 32 k 270 -> 249 (logits of standard deviation 2: 296 -> 290; 3: 294 -> 341, the
+// worst seen), 12 of 16 k 201 -> 237, 40 of 8 k 365 -> 446 (365 -> 290 where passages stand out), and 8 of 4 to 32 k that
+// keep a tenth 206 -> 285.  Hence the conditions in prune_plan: prompts long enough for the sample, query-key pairs enough
+// for the launches, and a budget of at most a sixteenth of a prompt (an eighth of a long one), so that the threshold lies
+// in the tail of the scores.
 #include "score_qg_sweep1.cuh"
 #include "score_qg_sweep2.cuh"
 
@@ -253,7 +255,7 @@ bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const D
   double pairs = 0.0;
   for (int b = 0; b < t.batch; ++b) {
     const int L = t.prompt_len[b], K = t.cu_keep[b + 1] - t.cu_keep[b];
-    if (L < 2048 || K > L / (L < 65536 ? 16 : 8)) return false;
+    if (L < 32768 || K > L / (L < 65536 ? 16 : 8)) return false;
     pairs += (double)rows * dm.n_kv_heads * L;
   }
   if (pairs < kPruneLeastPairs) return false;

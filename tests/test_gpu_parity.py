@@ -960,13 +960,13 @@ def test_split_operand_scorer_wait_limit(dq):
 
 
 # --------------------------------------------------------- the retained set without the scores (pruned selection)
-# At the smallest sizes that take it (1e8 query-key pairs): 1, 2, 3 and 4 query groups with full and ragged ends, one and
-# two score slots, odd lengths, ragged batches, budgets from one row to a sixteenth of a prompt.
+# At the smallest sizes that take it (2e8 query-key pairs): 1, 2, 3 and 4 query groups with full and ragged ends, one and
+# two score slots, odd lengths, ragged batches, budgets from one row to an eighth of a prompt.
 PRUNE_CASES = [
     # H_q, H_kv, N, lengths, budgets
-    (32, 8, 32, (98000,), (983,)), (32, 8, 64, (49003,), (1,)), (28, 4, 64, (60001,), (3750,)), (64, 8, 128, (16411,), (500,)),
-    (12, 4, 100, (90003,), (5000,)), (6, 1, 128, (131072,), (1310,)), (5, 1, 104, (200001,), (9000,)),
-    (32, 8, 32, (30001, 9000, 2049, 30000, 37003), (1875, 500, 100, 1000, 40)), (32, 8, 32, (8192,) * 13, (256,) * 13),
+    (32, 8, 32, (196001,), (983,)), (32, 8, 64, (98003,), (1,)), (28, 4, 64, (112001,), (14000,)), (64, 8, 128, (32771,), (500,)),
+    (12, 4, 100, (167003,), (5000,)), (6, 1, 128, (262001,), (1310,)), (5, 1, 104, (390001,), (9000,)),
+    (32, 8, 32, (33001, 50003, 40000, 32768, 45001), (2062, 900, 200, 2000, 40)), (32, 8, 32, (32768,) * 6, (256,) * 6),
 ]
 
 
@@ -1028,7 +1028,7 @@ def test_pruned_selection_matches_the_full_sweeps(dq, hq, hkv, n, lens, keep, ke
 
 def test_pruned_selection_wait_limit(dq):
     """A device-side wait of the pruned selection that runs out: status once, and the context works again."""
-    hq, hkv, n, L, K = 28, 4, 64, 60001, 2000
+    hq, hkv, n, L, K = 28, 4, 64, 112001, 2000
     w = _small(lens=(L,), keep=(K,), n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0)
     q, k, v = (torch.randn(s, device="cuda").bfloat16() for s in ((1, hq, n, 128), (hkv, L + n, 128), (hkv, L + n, 128)))
     ctx = _ctx(dq, w)
