@@ -159,11 +159,11 @@ __device__ __forceinline__ float2 careful_row(const Args& a, uint32_t q_row, uin
 }
 
 // The one-pass form's epilogue loop and the merge of its row sums.  kPieces: pieces of 16 query columns per thread (2 for
-// groups of up to 128 rows, else 4).
+// groups of up to 128 rows, else 4).  sums: [rows] floats of this CTA's own (the lse merge is done with them).
 template <int kPieces>
 __device__ __forceinline__ void one_pass_epilogue(const Args& a, const Work& w, const Bars& bars, const Waiter& wt, int L, int nt, int kvh,
                                                   uint32_t sbase, uint32_t lane_addr, int acc_cols, int n_acc, int p0, int np, bool full,
-                                                  int eg, int quad, int lane, float* lse_s, float* exch, uint32_t q_half) {
+                                                  int eg, int quad, int lane, float* lse_s, float* sums, float* exch, uint32_t q_half) {
   const int r = quad * 32 + lane, N = a.n_pseudo, col0 = p0 * 16;
   float2 z[8 * kPieces];                                        // this thread's columns over the keys of its lane
 #pragma unroll
@@ -247,28 +247,31 @@ __device__ __forceinline__ void one_pass_epilogue(const Args& a, const Work& w, 
     }
     if (hi) c += n;
   }
-  // the four quadrants through shared memory (the ring behind the queries: every MMA that read it has retired)
-  float* red = reinterpret_cast<float*>(__cvta_shared_to_generic(sbase + 2 * q_half));   // [4][256]
+  // The four quadrants through shared memory (the ring behind the queries: every MMA that read it has retired, unless a
+  // wait ran out: then copies and conversions may still land there, and what is read back is as undefined as the results).
+  // No decision that a barrier hangs on comes from the ring: whether a row is done over again is agreed on by all
+  // epilogue threads at once, never in a CTA one of whose epilogue warps gave up (the others' waits are over by then),
+  // and which rows from `sums`, which no other role writes.
+  float* red = reinterpret_cast<float*>(__cvta_shared_to_generic(sbase + 2 * q_half));   // [4][256], then the scratch of careful_row
   if (c * 2 < np * 16) *reinterpret_cast<float2*>(red + quad * 256 + col0 + c * 2) = z[0];
   const int te = eg * 128 + r;
-  float* sum = red + 4 * 256;                                   // [256], then the scratch of careful_row, then `whole`
-  int* again = reinterpret_cast<int*>(sum + 256 + 64);          // some row has to be done over again
-  if (te == 0) *again = 0;
-  epilogue_sync();
+  const bool gave_up = epilogue_any(wt.aborting());
+  float sum = 0.f;
   if (te < w.rows) {
-    sum[te] = (red[te] + red[256 + te]) + (red[512 + te] + red[768 + te]);
-    if (!(sum[te] < 1e37f) && !wt.aborting()) atomicOr(again, 1);   // (true for inf and NaN)
+    sum = (red[te] + red[256 + te]) + (red[512 + te] + red[768 + te]);
+    sums[te] = sum;
+    float2* out = a.part_out + ((int64_t)w.chunk * a.n_kv_heads + kvh) * a.rows_pad + w.qgrp * a.rows_g;
+    out[te] = make_float2(lse_s[te], sum);
   }
-  epilogue_sync();
-  float2* out = a.part_out + ((int64_t)w.chunk * a.n_kv_heads + kvh) * a.rows_pad + w.qgrp * a.rows_g;
-  if (te < w.rows) out[te] = make_float2(lse_s[te], sum[te]);
-  if (*again) {                                                 // (the same for every epilogue warp)
+  const bool again = epilogue_any(!(sum < 1e37f));              // (inf and NaN too)
+  if (again && !gave_up) {
     const __nv_bfloat16* k = reinterpret_cast<const __nv_bfloat16*>(a.k) + (int64_t)kvh * a.k_head_stride + (int64_t)w.row_base * a.k_row_stride;
+    float2* out = a.part_out + ((int64_t)w.chunk * a.n_kv_heads + kvh) * a.rows_pad + w.qgrp * a.rows_g;
     const int j0 = w.t0 * kTile2, j1 = j0 + nt * kTile2;
     for (int row = 0; row < w.rows; ++row) {
-      if (sum[row] < 1e37f) continue;
+      if (sums[row] < 1e37f) continue;
       const float2 v = careful_row(a, sbase + (row >> 7) * 128 * 128 + (row & 127) * 128, q_half, row & 7, k, j0, j1,
-                                   L + (w.qgrp * a.rows_g + row) % N, reinterpret_cast<float2*>(sum + 256), te);
+                                   L + (w.qgrp * a.rows_g + row) % N, reinterpret_cast<float2*>(red + 4 * 256), te);
       if (te == 0) out[row] = v;
     }
   }
@@ -505,7 +508,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     const bool full = (p0 + np) * 16 <= min(w.rows, kGroupRows);    // no column of this warp's pieces lies beyond the group
     const bool full1 = (p1 + np1) * 16 <= w.rows - kGroupRows;
     if constexpr (kForm == kOnePass) {
-      one_pass_epilogue<(kForm == kOnePass && kNarrow) ? 2 : 4>(a, w, bars, wt, L, nt, kvh, sbase, lane_addr, acc_cols, n_acc, p0, np, full, eg, quad, lane, lse_s, exch, q_half);
+      one_pass_epilogue<(kForm == kOnePass && kNarrow) ? 2 : 4>(a, w, bars, wt, L, nt, kvh, sbase, lane_addr, acc_cols, n_acc, p0, np, full, eg, quad, lane, lse_s, aux, exch, q_half);
     } else {
       bool ok = true;
       Ring ra(n_acc);

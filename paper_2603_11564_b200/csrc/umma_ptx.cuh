@@ -218,6 +218,18 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 }
 // Barrier among the 16 epilogue warps only (the producer warps never join it).
 __device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
+// The same barrier, and whether `p` holds in any of its threads: the same answer for all of them, from no memory that
+// another role could write.
+__device__ __forceinline__ bool epilogue_any(bool p) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, 1, 512, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(any) : "r"((uint32_t)p) : "memory");
+  return any != 0u;
+}
 
 // Descriptor of the operand `bytes` further on in shared memory (the start-address field is
 // in 16-byte units in the low bits and never carries out of it for addresses below 256 KB).

@@ -1046,3 +1046,37 @@ def test_pruned_selection_wait_limit(dq):
     dq.dapq_poll_status(ctx)
     assert all(torch.equal(x, y) for x, y in zip(*outs))
     dq.dapq_destroy(ctx)
+
+
+@pytest.mark.parametrize("cycles", [1, 20, 40, 60, 100])
+def test_pruned_selection_gives_up_anywhere(dq, cycles):
+    """Limits at which some waits of a CTA run out and others do not, with rows whose sums leave the float range: no
+    role may hang on a barrier that another one, having given up, does not reach; and the context works again."""
+    hq, hkv, n, L, K = 28, 4, 64, 112001, 2000
+    w = _small(lens=(L,), keep=(K,), n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0)
+    q, v = (torch.randn(s, device="cuda").bfloat16() for s in ((1, hq, n, 128), (hkv, L + n, 128)))
+    k = torch.randn((hkv, L + n, 128), device="cuda")
+    ctx = _ctx(dq, w)
+    rot = torch.empty_like(q)
+    dq.dapq_rope_pseudo_q(ctx, q, [L], rot)
+    for h in range(hkv):
+        u = rot[0, h * (hq // hkv), 5].float()
+        k[h, L // 2 // 16 * 16] = 150.0 * 128 ** 0.5 * u / u.norm() ** 2
+    k = k.bfloat16()
+    outs = [[torch.zeros((hkv, K, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2)] + [torch.zeros((hkv, K), dtype=torch.int32, device="cuda")]
+            for _ in range(2)]
+    layers = lambda o: dq.dapq_evict_layers(ctx, [q] * 4, [k] * 4, [v] * 4, w.cu_rows, [L], [K], [o[0]] * 4, [o[1]] * 4, [o[2]] * 4)
+    layers(outs[0])
+    dq.dapq_poll_status(ctx)
+    for _ in range(3):
+        dq.dapq_set_wait_limit(ctx, cycles)
+        layers(outs[1])
+        try:
+            dq.dapq_poll_status(ctx)
+        except dq.DapqError as e:
+            assert e.status == dq.DAPQ_ERR_TIMEOUT
+        dq.dapq_set_wait_limit(ctx, 0)
+        layers(outs[1])
+        dq.dapq_poll_status(ctx)
+        assert all(torch.equal(x, y) for x, y in zip(*outs))
+    dq.dapq_destroy(ctx)
