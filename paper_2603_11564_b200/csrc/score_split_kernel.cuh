@@ -11,7 +11,10 @@
 // count, are kept in two halves (channels 0-63 and 64-127):
 //   columns [0, R)   q0.k0 over channels 0-63      [3R, 4R)  q0.k0 over channels 64-127
 //           [R, 2R)  the products of order 2^-8    [2R, 3R)  those of order 2^-16
-// and the epilogue adds the four columns of a logit in fp32.  Both sweeps use this layout:
+// and the epilogue adds the four columns of a logit in fp32.  The queries are multiplied by softmax scale * log2(e) before
+// they are split: what the epilogue adds up is the base-2 logit, the same number in both sweeps whatever its size (a
+// product formed and rounded in one sweep and fused into the subtraction in the other differs by half an ulp of the logit,
+// which an exponential of logits beyond 2^24 turns into any value).  Both sweeps use this layout:
 //   sweep 1  a thread keeps a running maximum and sum for a quarter of the query columns over the keys of its
 //            lane; the lanes are merged once, at the end of the CTA's chunk;
 //   sweep 2  a thread sums its key's exponentials over all query columns: one score, no exchange.
@@ -93,7 +96,7 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
 }
-// The four blocks of P columns from `taddr` on, summed: x[e] = the raw dot product of column e.  `release` gives
+// The four blocks of P columns from `taddr` on, summed: x[e] = the logit of column e.  `release` gives
 // the accumulator back once its `last` columns are in registers.
 template <int kR, int P, class Release>
 __device__ __forceinline__ void load_logits(uint32_t taddr, float (&x)[P], bool last, Release release) {
@@ -117,6 +120,11 @@ __device__ __forceinline__ void load_logits(uint32_t taddr, float (&x)[P], bool 
 
 __device__ __forceinline__ float4 as_float4(uint4 v) {
   return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+}
+
+// Two words of packed bf16 values as fp32.
+__device__ __forceinline__ float4 from_bf16(uint32_t a, uint32_t b) {
+  return as_float4(make_uint4(a << 16, a & 0xffff0000u, b << 16, b & 0xffff0000u));
 }
 
 // (maximum, sum of exp2) of two disjoint sets of logits -> of their union (either may be empty: sum 0).
@@ -341,23 +349,24 @@ split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ S
     const int te = threadIdx.x - Ro::first_epi * 32;              // 0 .. 511
     const int eg = te >> 7, quad = warp & 3, r = quad * 32 + lane;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
-    const float c = a.scale_log2e;
     pdl_wait();                                                   // the rotation kernel (sweep 1) wrote the queries (partials)
     // (sweep 2 reads nothing that is not complete by now ahead of its own wait; its CTAs set up as this sweep's leave: 2 k
     // fp32 keys 24.0 -> 22.0 us a layer, 32 heads of 16 k bf16 keys 69.9 -> 68.0)
     if (!kSweep2) pdl_trigger();
-    // ---- the CTA's queries in three parts
+    // ---- the CTA's queries, scaled, in three parts
+    const float c = a.scale_log2e;
+    auto scaled = [c](float4 v) { return make_float4(v.x * c, v.y * c, v.z * c, v.w * c); };
     for (int x = te; x < n_sub * kR * 16; x += kEpiWarps * 32) {
       const int row = x >> 4, ch = x & 15, sub = row / kR, rr = row - sub * kR, h = ch >> 3;
       uint4 p[3];
       if (row >= rows) {
         p[0] = p[1] = p[2] = make_uint4(0u, 0u, 0u, 0u);
       } else if (a.q_bf16) {
-        p[0] = __ldg(reinterpret_cast<const uint4*>(a.q) + ((int64_t)qrow_base + row) * 16 + ch);
-        p[1] = p[2] = make_uint4(0u, 0u, 0u, 0u);
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(a.q) + ((int64_t)qrow_base + row) * 16 + ch);
+        split8(scaled(from_bf16(v.x, v.y)), scaled(from_bf16(v.z, v.w)), p);
       } else {
         const float4* src = reinterpret_cast<const float4*>(a.q) + ((int64_t)qrow_base + row) * 32 + ch * 2;
-        split8(__ldg(src), __ldg(src + 1), p);
+        split8(scaled(__ldg(src)), scaled(__ldg(src + 1)), p);
       }
       const uint32_t at = sbase + sub * Ro::query_bytes(kR) + h * 3 * kR * 128 + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4);
 #pragma unroll
@@ -393,7 +402,7 @@ split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ S
           load_logits<kR, P>(lane_addr + ra.i * kAcc + c0 + p, x, p + P == C, release);
 #pragma unroll
           for (int e = 0; e < P; ++e) {
-            float s = x[e] * c;
+            float s = x[e];
             if (masked && beyond > (row0 + c0 + p + e) % N) s = -CUDART_INF_F;
             // one exponential per logit: the smaller of (logit, running maximum) against the larger
             const float dlt = s - m[p + e], f = ex2(-fabsf(dlt));
@@ -504,7 +513,7 @@ split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ S
             const float4 l0 = *reinterpret_cast<const float4*>(lse_s + sub * kR + p), l1 = *reinterpret_cast<const float4*>(lse_s + sub * kR + p + 4);
             const float ls[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e & 3] += ex2(fmaf(x[e], c, ls[e]));
+            for (int e = 0; e < 8; ++e) acc[e & 3] += ex2(x[e] + ls[e]);
           }
         }
         if (!ok) break;

@@ -944,6 +944,25 @@ def test_split_operand_scorer_far_logits(dq, dtype, hq, n, where):
     _check_evict(w, data, _gpu_evict(dq, w, data), util.oracle_evict(w, data))
 
 
+@pytest.mark.parametrize("dtype,hq,hkv", [("f32", 8, 2), ("bf16", 2, 2)])
+@pytest.mark.parametrize("size", [1e4, 1e6, 1e10, 1e20, 1e30])
+def test_split_operand_scorer_huge_logits(dq, dtype, hq, hkv, size):
+    """A key of that size in every channel has the largest logit of about half of the rows, alone, and weight 0 in the
+    others: its score is the number of those rows.  Both sweeps have to see the same logit to the last bit: half an ulp
+    of a logit of 2^33 is 2^9, and 2^(2^9) no float.  The other keys share what is left, as on the CUDA cores."""
+    w = _small(lens=(2000,), keep=(100,), dtype=dtype, n_q_heads=hq, n_kv_heads=hkv, n_pseudo=32, n_needles=0, outlier_channels=0)
+    data = gi.draw_layer(w, 0, "cpu")
+    data["k"][0, 700] = size
+    rows = util.oracle_q_rot(w, data)[0, :w.group].reshape(-1, 128).numpy() @ util.to_f64(data["k"][0, 700])
+    got, cores = _gpu_evict(dq, w, data), None
+    ctx = _ctx(dq, w, flags=dq.DAPQ_FLAG_CUDA_CORE_SCORER)
+    cores = _gpu_evict(dq, w, data, ctx)
+    dq.dapq_destroy(ctx)
+    assert abs(got["scores"][0, 700] - int((rows > 0).sum())) <= 1e-4
+    assert np.all(np.abs(got["scores"] - cores["scores"]) <= 4e-5 * np.abs(cores["scores"]) + 1e-30)
+    np.testing.assert_array_equal(got["idx"], cores["idx"])
+
+
 def test_split_operand_scorer_wait_limit(dq):
     """A device-side wait that runs out: the call returns, the status says so once, and the context works again."""
     for dtype, hkv in (("f32", 2), ("bf16", 8)):
