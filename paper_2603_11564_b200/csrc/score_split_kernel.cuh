@@ -1,10 +1,14 @@
 // The tensor-core scorer that loses nothing of 32-bit queries and keys (Section 4.2, Eq. 4); host side and
 // the reasons for its shape in score_split.cu.
 //
-// Every fp32 number is the exact sum of three bf16 numbers (8 + 8 + 8 significant bits, split by truncation),
-// and a product of two bf16 numbers is exact in fp32, so q.k is a short sum of bf16 MMAs:
+// Every fp32 number is the exact sum of three bf16 numbers (the nearest one, the one nearest to what is left, and the
+// rest), and a product of two bf16 numbers is exact in fp32, so q.k is a short sum of bf16 MMAs:
 //   bf16 keys   q0.k + q1.k + q2.k                                   (nothing left out)
-//   fp32 keys   q0.k0 + (q1.k0 + q0.k1) + (q2.k0 + q1.k1 + q0.k2)    (what is left out is below 2^-23 |q||k|)
+//   fp32 keys   q0.k0 + (q1.k0 + q0.k1) + (q2.k0 + q1.k1 + q0.k2)
+// What is left out for fp32 keys, q1.k2 + q2.k1 + q2.k2, is at most (2^-24 + 2^-34) |q||k|: |q1| <= 2^-8 |q| and
+// |q2| <= 2^-17 |q| by rounding to nearest (truncated parts have the sign of their number and twice the size each: up to
+// 2^-21 |q||k|, always of the product's own sign).  Its sign is either one, 0.05 * 2^-23 |q||k| in root mean square on
+// N(0, 1) operands (truncated: 0.50), where one rounding of fp32 is 0.29 * 2^-23 of its result.
 // The three parts of the R query rows are stacked along N ([q0; q1; q2], N = 3 R), so that one MMA per k-step
 // multiplies all of them with a part of K.  D[key, query]: keys on tensor-memory lanes, and the products of one
 // order of magnitude share R accumulator columns; the leading products, whose roundings are the ones that
@@ -76,20 +80,30 @@ struct Args {
 };
 
 // Two fp32 values -> their three bf16 parts, packed in pairs (lower half: a).
-__device__ __forceinline__ void split2(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
-  const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
-  p0 = __byte_perm(ua, ub, 0x7632);
-  const float ra = a - __uint_as_float(ua & 0xffff0000u), rb = b - __uint_as_float(ub & 0xffff0000u);
-  const uint32_t va = __float_as_uint(ra), vb = __float_as_uint(rb);
-  p1 = __byte_perm(va, vb, 0x7632);
-  const float sa = ra - __uint_as_float(va & 0xffff0000u), sb = rb - __uint_as_float(vb & 0xffff0000u);
-  p2 = __byte_perm(__float_as_uint(sa), __float_as_uint(sb), 0x7632);
+// kNearest (fp32 keys): values beyond the largest bf16 number keep it as their first part (the others hold the rest); an
+// infinity ends up in the third part, and its products are infinite, of their sign, as in fp32.  Otherwise (bf16 keys:
+// all products are formed) by truncation: the parts of a query have one sign, and an infinite key meets no
+// infinities of both signs.  NaN stays NaN.
+__device__ __forceinline__ uint32_t nearest_bf16x2(float a, float b) {
+  uint32_t r;
+  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
 }
+template <bool kNearest>
+__device__ __forceinline__ void split2(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
+  auto part = [](float x, float y) { return kNearest ? nearest_bf16x2(x, y) : __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632); };
+  p0 = part(a, b);
+  const float ra = a - __uint_as_float(p0 << 16), rb = b - __uint_as_float(p0 & 0xffff0000u);
+  p1 = part(ra, rb);
+  const float sa = ra - __uint_as_float(p1 << 16), sb = rb - __uint_as_float(p1 & 0xffff0000u);
+  p2 = __byte_perm(__float_as_uint(sa), __float_as_uint(sb), 0x7632);   // (at most eight significant bits)
+}
+template <bool kNearest>
 __device__ __forceinline__ void split8(const float4& x, const float4& y, uint4 (&p)[3]) {
-  split2(x.x, x.y, p[0].x, p[1].x, p[2].x);
-  split2(x.z, x.w, p[0].y, p[1].y, p[2].y);
-  split2(y.x, y.y, p[0].z, p[1].z, p[2].z);
-  split2(y.z, y.w, p[0].w, p[1].w, p[2].w);
+  split2<kNearest>(x.x, x.y, p[0].x, p[1].x, p[2].x);
+  split2<kNearest>(x.z, x.w, p[0].y, p[1].y, p[2].y);
+  split2<kNearest>(y.x, y.y, p[0].z, p[1].z, p[2].z);
+  split2<kNearest>(y.z, y.w, p[0].w, p[1].w, p[2].w);
 }
 
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
@@ -331,7 +345,7 @@ split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ S
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             uint4 p[3];
-            split8(as_float4(x[i][0]), as_float4(x[i][1]), p);
+            split8<true>(as_float4(x[i][0]), as_float4(x[i][1]), p);
 #pragma unroll
             for (int e = 0; e < 3; ++e) sts128(at + i * 1024 + e * kPart, p[e]);
           }
@@ -363,10 +377,10 @@ split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ S
         p[0] = p[1] = p[2] = make_uint4(0u, 0u, 0u, 0u);
       } else if (a.q_bf16) {
         const uint4 v = __ldg(reinterpret_cast<const uint4*>(a.q) + ((int64_t)qrow_base + row) * 16 + ch);
-        split8(scaled(from_bf16(v.x, v.y)), scaled(from_bf16(v.z, v.w)), p);
+        split8<kF32>(scaled(from_bf16(v.x, v.y)), scaled(from_bf16(v.z, v.w)), p);
       } else {
         const float4* src = reinterpret_cast<const float4*>(a.q) + ((int64_t)qrow_base + row) * 32 + ch * 2;
-        split8(scaled(__ldg(src)), scaled(__ldg(src + 1)), p);
+        split8<kF32>(scaled(__ldg(src)), scaled(__ldg(src + 1)), p);
       }
       const uint32_t at = sbase + sub * Ro::query_bytes(kR) + h * 3 * kR * 128 + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4);
 #pragma unroll

@@ -963,6 +963,31 @@ def test_split_operand_scorer_huge_logits(dq, dtype, hq, hkv, size):
     np.testing.assert_array_equal(got["idx"], cores["idx"])
 
 
+def test_split_operand_scorer_products_of_full_fractions(dq):
+    """Operands whose three bf16 parts are all as large as they can be.  One channel, so that nothing but the products left
+    out and the additions of a logit's four columns counts: at most 2^-24 of the logit for those, three roundings of 2^-24
+    for these, once more for the key that it is compared with, 2^-22 for the exponentials: 2 * 4 * 2^-24 * 2080 + 2^-21."""
+    n_keys, scale = 512, float(np.float32(np.log(2.0)))            # (scale * log2(e) = 1 to the last bit: q enters unscaled)
+    assert np.float32(np.float64(np.float32(scale)) * 1.4426950408889634) == 1.0
+    rng = np.random.default_rng(11)
+    full = np.float32(1.0) + np.float32(2.0 ** -7) - np.float32(2.0 ** -23) * rng.integers(1, 4000, n_keys + 1).astype(np.float32)
+    full = (full.view(np.uint32) | np.uint32(0x7f7f)).view(np.float32)         # parts of ones in every place
+    k = torch.zeros((1, n_keys + 1, 128))
+    k[0, :n_keys, 0] = torch.from_numpy(full[:n_keys]) * 2048
+    k[0, ::2, 0] = 2048.0                                          # every other key: a power of two, nothing left out
+    q = torch.zeros((1, 1, 1, 128))
+    q[0, 0, 0, 0] = float(full[-1])
+    ctx = dq.dapq_create(1, 1, 1, 1, n_keys + 1, dq.DAPQ_F32, 1e4, softmax_scale=scale)
+    scores = torch.empty((1, n_keys), device="cuda")
+    dq.dapq_score(ctx, q.cuda(), k.cuda(), [0, n_keys + 1], [n_keys], scores)
+    dq.dapq_poll_status(ctx)
+    dq.dapq_destroy(ctx)
+    logit = util.to_f64(k)[0, :n_keys, 0] * float(full[-1])
+    got, base = np.log2(scores[0].cpu().double().numpy()), 2.0 * (n_keys // 4)
+    err = (got - got[0]) - (logit - logit[0])
+    assert np.abs(err).max() <= 2 * 4 * 2.0 ** -24 * 2080 + 2.0 ** -21
+
+
 def test_split_operand_scorer_wait_limit(dq):
     """A device-side wait that runs out: the call returns, the status says so once, and the context works again."""
     for dtype, hkv in (("f32", 2), ("bf16", 8)):
