@@ -373,13 +373,13 @@ split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ S
     for (int x = te; x < n_sub * kR * 16; x += kEpiWarps * 32) {
       const int row = x >> 4, ch = x & 15, sub = row / kR, rr = row - sub * kR, h = ch >> 3;
       uint4 p[3];
-      if (row >= rows) {
-        p[0] = p[1] = p[2] = make_uint4(0u, 0u, 0u, 0u);
-      } else if (a.q_bf16) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(a.q) + ((int64_t)qrow_base + row) * 16 + ch);
+      const int64_t src_row = (int64_t)qrow_base + min(row, rows - 1);   // (rows that do not exist repeat the last one: zeros
+                                                                         // would make NaN of an infinite key, here as in its sums)
+      if (a.q_bf16) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(a.q) + src_row * 16 + ch);
         split8<kF32>(scaled(from_bf16(v.x, v.y)), scaled(from_bf16(v.z, v.w)), p);
       } else {
-        const float4* src = reinterpret_cast<const float4*>(a.q) + ((int64_t)qrow_base + row) * 32 + ch * 2;
+        const float4* src = reinterpret_cast<const float4*>(a.q) + src_row * 32 + ch * 2;
         split8<kF32>(scaled(__ldg(src)), scaled(__ldg(src + 1)), p);
       }
       const uint32_t at = sbase + sub * Ro::query_bytes(kR) + h * 3 * kR * 128 + rr * 128 + (((ch & 7) ^ (rr & 7)) << 4);

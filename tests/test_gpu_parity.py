@@ -988,6 +988,37 @@ def test_split_operand_scorer_products_of_full_fractions(dq):
     assert np.abs(err).max() <= 2 * 4 * 2.0 ** -24 * 2080 + 2.0 ** -21
 
 
+@pytest.mark.parametrize("edit", ["-inf", "inf", "nan", "lowest", "largest", "above_bf16"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_split_operand_scorer_infinities_and_limits(dq, dtype, edit):
+    """40 keys with an infinite, undefined or largest finite value in one channel, one query row: as on the CUDA cores."""
+    big = torch.finfo(torch.float32 if dtype == "f32" else torch.bfloat16).max
+    value = {"-inf": -np.inf, "inf": np.inf, "nan": np.nan, "lowest": -big, "largest": big, "above_bf16": 3.3999e38 if dtype == "f32" else big}[edit]
+    w = _small(lens=(700,), keep=(40,), dtype=dtype, n_q_heads=1, n_kv_heads=1, n_pseudo=1, n_needles=0, outlier_channels=0)
+    data = gi.draw_layer(w, 0, "cpu")
+    q = util.oracle_q_rot(w, data)[0, 0, 0]
+    c = int(torch.argmax(q))                                       # positive: -inf and the lowest value mask the key
+    data["k"][0, 100:140, c] = value
+    if edit in ("lowest", "largest", "above_bf16"):
+        data["k"][0, 100:140, :c], data["k"][0, 100:140, c + 1:] = 0, 0
+    got = _gpu_evict(dq, w, data)
+    ctx = _ctx(dq, w, flags=dq.DAPQ_FLAG_CUDA_CORE_SCORER)
+    cores = _gpu_evict(dq, w, data, ctx)
+    dq.dapq_destroy(ctx)
+    finite = np.isfinite(cores["scores"])                          # (a product above the float range is inf there, and may stay below it here)
+    np.testing.assert_allclose(got["scores"][finite], cores["scores"][finite], rtol=4e-5, atol=1e-30)
+    if edit in ("inf", "nan"):
+        assert np.isnan(got["scores"]).all() and np.isnan(cores["scores"]).all()
+    if edit in ("-inf", "lowest"):
+        assert np.isfinite(got["scores"]).all() and (got["scores"][0, 100:140] == 0).all() and got["scores"].sum() > 0.9
+    if edit in ("largest", "above_bf16"):                          # (inf on the CUDA cores; times the scale it stays a number here)
+        np.testing.assert_array_equal(got["scores"][0, 100:140], got["scores"][0, 100])
+        assert 0.024 < got["scores"][0, 100] <= 1                  # (40 added to a sum of 2^1e38 may round to nothing)
+        np.testing.assert_array_equal(got["idx"][0], np.arange(100, 140))
+    else:
+        np.testing.assert_array_equal(got["idx"], cores["idx"])
+
+
 def test_split_operand_scorer_wait_limit(dq):
     """A device-side wait that runs out: the call returns, the status says so once, and the context works again."""
     for dtype, hkv in (("f32", 2), ("bf16", 8)):
