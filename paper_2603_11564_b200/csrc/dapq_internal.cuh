@@ -218,7 +218,8 @@ cudaError_t launch_score_split(const SplitPlan& plan, int q_dtype, const void* q
 // ---- the pruned selection: dapq_evict without score output (score_prune.cu) ----------------------------------
 constexpr int kPruneSums = 4;              // partial sums per key
 constexpr double kPruneLeastPairs = 2e8;   // query-key pairs of a call below which the full sweeps are as fast
-constexpr int kPruneBins = 2048, kPruneHist = kPruneBins + 4;   // histogram of a head's lower bounds, then its candidate count
+// histogram of a head's lower bounds, its candidate count, the largest magnitude of its rows' log-sum-exps (bits of a float)
+constexpr int kPruneBins = 2048, kPruneHist = kPruneBins + 4;
 struct PrunePlan {
   QgPlan qg;                               // the full scorer's plan; sweep 2's cut serves the candidates
   CUtensorMap tm_s;                        // every 16th key

@@ -102,12 +102,13 @@ struct BoundSpan {
 __global__ void __launch_bounds__(kBoundThreads)
 bound_hist_kernel(const __grid_constant__ SeqTable t, const __grid_constant__ ChunkTable ct, const BoundArgs a) {
   __shared__ uint32_t hist[kPruneBins];
-  __shared__ uint32_t f_min[kPruneSums], f_max[kPruneSums];
+  __shared__ uint32_t f_min[kPruneSums], f_max[kPruneSums], lse_max;
   const int tid = threadIdx.x, kvh = blockIdx.y, b = blockIdx.z, H = gridDim.y;
   pdl_trigger();
   if ((int)blockIdx.x * kBoundTile - head_lead(t, a, b, kvh) >= t.prompt_len[b]) return;
   for (int x = tid; x < kPruneBins; x += kBoundThreads) hist[x] = 0u;
   if (tid < kPruneSums) { f_min[tid] = 0x7f800000u; f_max[tid] = 0u; }
+  if (tid == 0) lse_max = 0u;
   __syncthreads();
   pdl_wait();
   const BoundSpan sp(t, a, b, kvh, blockIdx.x);
@@ -131,7 +132,8 @@ bound_hist_kernel(const __grid_constant__ SeqTable t, const __grid_constant__ Ch
         m = mm;
       }
     }
-    const float f = exp2f(a.ref[((int64_t)b * H + kvh) * a.rows_total + row] - (m + log2f(z)));
+    const float lse = m + log2f(z), f = exp2f(a.ref[((int64_t)b * H + kvh) * a.rows_total + row] - lse);
+    if (blockIdx.x == 0) atomicMax(&lse_max, __float_as_uint(fabsf(lse)));   // (NaN above infinity above all numbers)
     const int qg = row / a.rows_g, rr = row - qg * a.rows_g;
     const int nch = (min(a.rows_g, a.rows_total - qg * a.rows_g) + 15) >> 4;
     int eg = 3;
@@ -163,6 +165,7 @@ bound_hist_kernel(const __grid_constant__ SeqTable t, const __grid_constant__ Ch
   uint32_t* out = a.hist + (int64_t)(b * H + kvh) * kPruneHist;
   for (int x = tid; x < kPruneBins; x += kBoundThreads)
     if (hist[x]) atomicAdd(out + x, hist[x]);
+  if (tid == 0 && blockIdx.x == 0) out[kPruneBins + 1] = lse_max;
 }
 
 // The candidates: keys whose upper bound reaches the lower edge of the bin that holds the K-th largest lower bound.
@@ -185,6 +188,7 @@ bound_list_kernel(const __grid_constant__ SeqTable t, const BoundArgs a) {
   const int top = kPruneBins - 1 - kPer * tid;                   // this thread's highest bin
   const uint4 h4 = *reinterpret_cast<const uint4*>(hist + top - 3);
   const uint32_t h[4] = {h4.w, h4.z, h4.y, h4.x};
+  const float lse_max = __uint_as_float(hist[kPruneBins + 1]);
   // inclusive prefix over the block, in thread order (every warp sums the totals of the warps before it by itself)
   auto prefix = [&](uint32_t mine, uint32_t* sums, uint32_t* total) {
     uint32_t incl = mine;
@@ -217,9 +221,12 @@ bound_list_kernel(const __grid_constant__ SeqTable t, const BoundArgs a) {
       if (c >= K) break;
       --bin;
     }
-    // with a margin for the roundings of either side: 2^-10 of the score, ten times what the polynomial exponentials,
-    // the fp16 pairs of the references and the sums amount to
-    edge = bin > 0 ? __uint_as_float(((uint32_t)bin + kBinBase) << 18) * (1.f - 0x1p-10f) : 0.f;
+    // with a margin for the roundings of either side: 2^-10 of the score, ten times what the polynomial exponentials and
+    // the sums amount to, and 2^-20 of the largest log-sum-exp for what grows with the logits: an fp16 pair holds one
+    // to 2^-23 of it (that of an estimate is the one the bounds use, that of the candidates' sweep is not known here), and the
+    // MMA that subtracts it from a dot product of its size rounds to 2^-24 of that or, with fewer bits kept, 2^-23
+    const float margin = 0x1p-10f + 0x1p-20f * lse_max;
+    edge = bin > 0 ? __uint_as_float(((uint32_t)bin + kBinBase) << 18) * (1.f - margin) : 0.f;   // (NaN or negative: all keys)
   }
   __syncthreads();
   const float floor_ = edge;
