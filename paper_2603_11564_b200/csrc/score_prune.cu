@@ -139,8 +139,11 @@ bound_hist_kernel(const __grid_constant__ SeqTable t, const __grid_constant__ Ch
     int eg = 3;
     while (eg > 0 && (rr >> 4) < (eg * nch) / 4) --eg;          // the epilogue group that held the row's column
     const int g = qg * a.per_cta + (a.per_cta == 4 ? eg : (a.per_cta == 2 ? eg >> 1 : 0));
-    atomicMin(&f_min[g], __float_as_uint(f));                    // (positive floats order like their bit patterns)
-    atomicMax(&f_max[g], __float_as_uint(f));
+    // (positive floats order like their bit patterns; a factor below the normal range keeps no bits that a bound could
+    // rely on: at least 0 and at most the range's lower end)
+    constexpr float kTiny = 0x1p-126f;
+    atomicMin(&f_min[g], __float_as_uint(f < kTiny ? 0.f : f));
+    atomicMax(&f_max[g], __float_as_uint(f < kTiny ? kTiny : f));
   }
   __syncthreads();
   float hi[kBoundKeys], lo[kBoundKeys];
