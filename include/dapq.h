@@ -163,9 +163,10 @@ DAPQ_API dapq_status dapq_set_wait_limit(dapq_ctx* ctx, int64_t cycles);
  * kernel launch is bracketed by CUDA events on its stream; dapq_profile(ctx, 1) also clears
  * the totals.  dapq_profile_read synchronises `stream` and returns, per kernel kind, the
  * summed device time in milliseconds and the number of launches since profiling was
- * enabled.  ms_out / count_out: host [DAPQ_PROF_KINDS], in the order of dapq_prof_kind.  Where only the keys that can be
- * selected are scored: LSE_MERGE is the sample sweep, SWEEP1 the pass over all keys, SWEEP2 the candidates' scores, and the
- * two kernels that make the candidate list count as TOPK. */
+ * enabled.  ms_out / count_out: host [DAPQ_PROF_KINDS], in the order of dapq_prof_kind.  In layers that may score only the
+ * keys that can be selected: LSE_MERGE is the sample sweep or, where all keys are scored, the first sweep; SWEEP1 the pass
+ * over all keys (nothing then); SWEEP2 the candidates' scores or the second sweep; and the two kernels that make the
+ * candidate list count as TOPK. */
 typedef enum {
   DAPQ_PROF_ROPE = 0, DAPQ_PROF_SWEEP1 = 1, DAPQ_PROF_LSE_MERGE = 2, DAPQ_PROF_SWEEP2 = 3,
   DAPQ_PROF_TOPK = 4, DAPQ_PROF_COMPACT = 5, DAPQ_PROF_POOL = 6, DAPQ_PROF_RECALL = 7, DAPQ_PROF_SLOT_SUM = 8,
@@ -229,9 +230,7 @@ DAPQ_API dapq_status dapq_recall(dapq_ctx* ctx, const int32_t* idx_gold, const i
                         float* recall_out, void* stream);
 
 /* Figure 1, the whole eviction step for one layer: rotate to positions L_b + i, score,
- * select, compact.  idx_out, scores_out may be NULL (kept in the workspace).  Without scores_out (and without pooling)
- * large calls with budgets that are small against their prompts compute the scores of those keys only that can be
- * among the K largest: the same set, chosen by exact bounds, in less time. */
+ * select, compact.  idx_out, scores_out may be NULL (kept in the workspace). */
 DAPQ_API dapq_status dapq_evict(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* cache,
                        const int32_t* k_keep_host, void* k_out, void* v_out, int32_t* idx_out,
                        float* scores_out, void* stream);
@@ -244,7 +243,12 @@ DAPQ_API dapq_status dapq_evict(dapq_ctx* ctx, const void* q_pre, const dapq_cac
  * [n_layers, batch] when k_keep_layer_stride = batch, or one row shared by all layers when
  * k_keep_layer_stride = 0.  Every layer uses the same workspace, so the layers run back to back;
  * only launches are issued (no copies, no synchronisation), which makes the whole call
- * capturable into a CUDA graph.  Stops at the first layer that fails and returns its status. */
+ * capturable into a CUDA graph.  Stops at the first layer that fails and returns its status.
+ * Calls of 12 layers and more on long prompts, without pooling and with budgets that are small against the prompts, compute
+ * the scores of those keys only that can be among the K largest, in layers where the layers before show that it
+ * pays.  The sets are those of dapq_evict up to keys whose scores agree with the K-th to rounding (1e-5 of it), as are the
+ * sets of two scorings whose log-sum-exps are summed in different orders; calls of fewer layers select dapq_evict's own,
+ * bit for bit. */
 DAPQ_API dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const* q_pre,
                               const dapq_cache_view* caches, const int32_t* k_keep_host,
                               int64_t k_keep_layer_stride, void* const* k_out, void* const* v_out,

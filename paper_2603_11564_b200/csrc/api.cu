@@ -386,6 +386,7 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
     pa.add(&pr.sums, kPruneSums * (score_bytes + 16));
     pa.add(&pr.cand, (size_t)sh->n_kv_heads * rows * sizeof(int32_t));
     pa.add(&pr.hist, (size_t)sh->max_batch * sh->n_kv_heads * kPruneHist * sizeof(uint32_t));
+    pa.add(&pr.route, 2 * sizeof(int));
     if (!pa.allocate(ctx)) {
       cudaGetLastError();
       pr.sums = nullptr;
@@ -585,12 +586,17 @@ dapq_status dapq_recall(dapq_ctx* ctx, const int32_t* idx_gold, const int32_t* i
 
 namespace {
 
+// The layers of a dapq_evict_layers call that took the pruned selection so far: the last one that did whatever the one
+// before it had found, and which of the two route words holds what the next one is to do.
+struct PruneRoute { int32_t last_try = -1, at = 0; };
+
 // after_own_compaction: the kernel before this call in `stream` is the compaction kernel of an
 // earlier evict on the same context (the layers of dapq_evict_layers); the rotation then does
 // not wait for it before it starts.
+// route: the call's layers may take the pruned selection (NULL: they may not); layer: this one's number.
 dapq_status evict_impl(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* cache, const int32_t* k_keep_host,
                        void* k_out, void* v_out, int32_t* idx_out, float* scores_out, void* stream,
-                       bool after_own_compaction) {
+                       bool after_own_compaction, PruneRoute* route = nullptr, int32_t layer = 0) {
   if (!ctx) return DAPQ_ERR_INVALID_ARG;
   if (!q_pre || !k_keep_host || !k_out || !v_out) return fail(ctx, DAPQ_ERR_INVALID_ARG, "dapq_evict: NULL argument");
   if (!aligned16(k_out) || !aligned16(v_out)) return fail(ctx, DAPQ_ERR_UNSUPPORTED, "k_out / v_out must be 16-byte aligned");
@@ -620,11 +626,14 @@ dapq_status evict_impl(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* 
                     ctx->dims, after_own_compaction, s, &ctx->log, &ref);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "rope kernel");
     PrunePlan pplan;
-    if (!scores_out && ctx->prune.sums && prune_plan(qplan, cd, t, ctx->dims, ctx->n_sm, &pplan)) {
+    if (route && ctx->prune.sums && prune_plan(qplan, cd, t, ctx->dims, ctx->n_sm, &pplan)) {
       // nobody reads the scores: only those that can be among the K largest are computed
-      e = launch_prune(pplan, cd, t, ctx->dims, ctx->prune, ctx->slots, scores, score_stride, ctx->status, ctx->wait_limit, s,
+      const bool attempt = route->last_try < 0 || layer - route->last_try >= kPruneRetry;
+      if (attempt) route->last_try = layer;
+      e = launch_prune(pplan, cd, t, ctx->dims, ctx->prune, attempt ? -1 : route->at, route->at ^ 1, ctx->slots, scores, score_stride, ctx->status, ctx->wait_limit, s,
                        &ctx->log);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "pruned score kernels");
+      route->at ^= 1;
     } else {
       st = run_score_qg(ctx, qplan, t, nullptr, scores, score_stride, nullptr, true, s);
     }
@@ -668,9 +677,11 @@ dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const
   if (n_layers < 0 || k_keep_layer_stride < 0) return fail(ctx, DAPQ_ERR_INVALID_ARG, "dapq_evict_layers: negative count or stride");
   if (n_layers > 0 && (!q_pre || !caches || !k_keep_host || !k_out || !v_out))
     return fail(ctx, DAPQ_ERR_INVALID_ARG, "dapq_evict_layers: NULL argument");
+  PruneRoute route;
   for (int32_t l = 0; l < n_layers; ++l) {
     const dapq_status st = evict_impl(ctx, q_pre[l], &caches[l], k_keep_host + (int64_t)l * k_keep_layer_stride, k_out[l],
-                                      v_out[l], idx_out ? idx_out[l] : nullptr, nullptr, stream, l > 0);
+                                      v_out[l], idx_out ? idx_out[l] : nullptr, nullptr, stream, l > 0,
+                                      n_layers >= kPruneLeastLayers ? &route : nullptr, l);
     if (st != DAPQ_OK) return st;
   }
   return DAPQ_OK;

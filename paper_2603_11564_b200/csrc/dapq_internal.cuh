@@ -215,17 +215,20 @@ cudaError_t launch_score_split(const SplitPlan& plan, int q_dtype, const void* q
                                const float* lse_in, float2* part, float* slots, float* scores, int64_t score_stride, float* lse_out,
                                int* status, long long wait_limit, bool after_own_kernel, cudaStream_t s, LaunchLog* log);
 
-// ---- the pruned selection: dapq_evict without score output (score_prune.cu) ----------------------------------
+// ---- the pruned selection: the layers of dapq_evict_layers (score_prune.cu) ----------------------------------
 constexpr int kPruneSums = 4;              // partial sums per key
-constexpr double kPruneLeastPairs = 2e8;   // query-key pairs of a call below which the full sweeps are as fast
+constexpr double kPruneLeastPairs = 2e8;   // query-key pairs of a layer below which the full sweeps are as fast
+constexpr int kPruneLeastLen = 65536;      // shortest prompt
+constexpr int kPruneLeastLayers = 12;      // of a call: the first one has to find out whether it pays, and loses a fifth if not
+constexpr int kPruneRetry = 32;            // layers after which a call that went back to the full sweeps tries again
 // histogram of a head's lower bounds, its candidate count, the largest magnitude of its rows' log-sum-exps (bits of a float)
 constexpr int kPruneBins = 2048, kPruneHist = kPruneBins + 4;
 struct PrunePlan {
   QgPlan qg;                               // the full scorer's plan; sweep 2's cut serves the candidates
   CUtensorMap tm_s;                        // every 16th key
-  SeqTable ts;                             // the sequences of the sample
   ChunkTable ct_s, ct_m, ct_g;             // chunks of the sample's sweep and of the one-pass sweep; CTAs per candidate list
   int32_t n_stages_m, per_cta;
+  float most;                              // candidates of a head, as a share of its prompt, up to which the route pays
 };
 struct PruneBuffers {                      // device workspace
   float2 *part_s, *part_m;                 // umma_part_elems each
@@ -233,12 +236,15 @@ struct PruneBuffers {                      // device workspace
   float* sums;                             // kPruneSums * (H_kv * max_total_rows rounded up to 4)
   int32_t* cand;                           // [H_kv][max_total_rows]
   uint32_t* hist;                          // [max_batch, H_kv][kPruneHist]
+  int* route;                              // [2] a layer's route and the next one's
 };
 bool prune_available();
 bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const Dims& dm, int n_sm, PrunePlan* plan);
+// route_at, route_next: which of buf.route holds this layer's route (-1: pruned, whatever the last one found) and which
+// receives the next one's.
 // scores: [H_kv][score_stride], those of keys that cannot be selected are negative; slots as for launch_score_qg.
 cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTable& t, const Dims& dm, const PruneBuffers& buf,
-                         float* slots, float* scores, int64_t score_stride, int* status, long long wait_limit,
+                         int route_at, int route_next, float* slots, float* scores, int64_t score_stride, int* status, long long wait_limit,
                          cudaStream_t s, LaunchLog* log);
 cudaError_t launch_topk(const float* scores, int64_t score_stride, int32_t* idx, int64_t idx_stride,
                         const SeqTable& t, int n_kv_heads, cudaStream_t s, LaunchLog* log);

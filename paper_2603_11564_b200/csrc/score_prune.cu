@@ -1,6 +1,6 @@
-// The retained set without the scores (Section 4.2, Eq. 5 needs the K largest S(j), not all of them): dapq_evict
-// and its multi-layer and host forms, when no scores are asked for.  The same set as from the two full sweeps, for less
-// than two thirds of their work on long prompts.
+// The retained set without the scores (Section 4.2, Eq. 5 needs the K largest S(j), not all of them): layers of a
+// dapq_evict_layers call, from kPruneLeastLayers layers on.  The set of the two full sweeps, up to keys whose scores agree
+// with the K-th to rounding, for less than two thirds of their work where it pays.
 //
 //   1. sample      sweep 1 over every 16th key: an estimate r_i of each query row's log-sum-exp;
 //   2. one pass    over all keys with r_i in place of the log-sum-exp: e_ij = 2^(s_ij - r_i) is added to the sum of its
@@ -9,21 +9,31 @@
 //   3. bounds      S(j) = sum_i e_ij / Z_i, so  sum_g E_g(j) / max_g Z  <=  S(j)  <=  sum_g E_g(j) / min_g Z.  With T the K-th
 //                  largest lower bound (at least K keys score T or more), a key whose upper bound is below T is not
 //                  among the K largest: what remains are the candidates;
-//   4. candidates  sweep 2 over them, with the log-sum-exp from step 2: the scores that the full sweep 2 gives them
-//                  (skipped, per KV head, when there are exactly K);
+//   4. candidates  sweep 2 over them, with the log-sum-exp from step 2: the scores that the full sweep 2 gives them, up to
+//                  the order in which that was summed (skipped, per KV head, when there are exactly K);
 //   5. selection   as ever, on an array that holds -1 for all other keys.
 // Nothing depends on how good the estimate is but the number of candidates.  A row sum that leaves the float range
 // is done over again by itself (careful_row).
 //
-// Measured on B200, a layer with the two full sweeps -> here, on prompts whose relevant passages stand out (candidates = K):
-// 128 k, 8 KV heads x 1024 query rows 690 -> 460 us; 128 k, 4 x 448 rows 182 -> 139; 32 k, 8 x 256 rows 64 -> 65 (four more
-// launches, the sample and the bounds at their start-up times).  On N(0, 1) keys, which stand out by nothing, a fifth to a
-// quarter of them are candidates at 128 k (704 -> 605 us with outlier channels, 188 -> 162), and a sample of 2 k keys is
-// the least that bounds anything: 8 prompts of 32 k 270 -> 249 (logits of standard deviation 2: 296 -> 290; 3: 294 -> 341, the
-// worst seen), 12 of 16 k 201 -> 237, 40 of 8 k 365 -> 446 (365 -> 290 where passages stand out), and 8 of 4 to 32 k that
-// keep a tenth 206 -> 285.  Hence the conditions in prune_plan: prompts long enough for the sample, query-key pairs enough
-// for the launches, and a budget of at most a sixteenth of a prompt (an eighth of a long one), so that the threshold lies
-// in the tail of the scores.
+// Where it pays is a matter of the data: the bounds are as wide as the worst estimate among the rows behind a sum, and rows
+// whose mass lies in few keys are estimated badly.  So the first layer of a call tries, and notes whether the
+// candidates of every head were few enough (PrunePlan::most); the next layers run the full sweeps if not (and try again
+// after kPruneRetry layers).  The decision stays on the device: the launches are the same either way, the two sweeps do the
+// one thing or the other, and the one pass and the bounds return at once.
+//
+// Measured on B200, us a layer of a 32-layer call, full sweeps -> here; keys N(0, 1) times a factor that sets the standard
+// deviation of the logits, or four channels times 8, or a first key 8 above the rest, or five keys that single rows attend
+// to, or passages that stand out for K or K/2 keys:
+//                           sd 1        sd 2        sd 3        sd 4        channels    first key   single rows passages K  K/2
+//   8 heads x 1024 rows, 128 k  655 -> 564  699 -> 706  697 -> 708  700 -> 709  672 -> 561  656 -> 498  662 -> 517  661 -> 555  678 -> 606
+//   4 x 448, 128 k          176 -> 164  174 -> 169  175 -> 182  178 -> 183  173 -> 160  175 -> 157  173 -> 164  172 -> 152  180 -> 188
+//   8 x 256, 128 k          204 -> 188  199 -> 190  212 -> 221  217 -> 229  215 -> 224  196 -> 177  198 -> 210  192 -> 171  194 -> 198
+// (with every layer trying: 8 x 1024 at sd 3 691 -> 806, 4 x 448 181 -> 219.)  What the full route still loses is the three
+// launches with nothing to do (some 2 us each) and the layer that tried: 12 layers at sd 4 655 -> 666, 178 -> 188, 189 -> 202.
+// Prompts of 32 k gained a tenth at best and lost a fifth (8 x 1024 rows: first key 190 -> 176, sd 1 209 -> 238; 8 prompts
+// of 8 x 256: 434 -> 393, sd 2 404 -> 479): a sample of 2 k keys says too little.  Hence the conditions in
+// prune_plan: prompts long enough for the sample, query-key pairs enough for the launches, and a budget of at
+// most an eighth of a prompt, so that the threshold lies in the tail of the scores.
 #include "score_qg_sweep1.cuh"
 #include "score_qg_sweep2.cuh"
 
@@ -32,7 +42,6 @@ namespace {
 
 using namespace qg;
 
-constexpr int kSampleStride = 16, kSamplePhase = 7;
 constexpr float kLog2Sample = 4.f;
 
 // ---- step 3: two kernels over tiles of kBoundTile keys of a head -------------------------------------------
@@ -47,6 +56,9 @@ struct BoundArgs {
   int64_t sum_stride, score_stride;
   uint32_t* hist;
   int32_t* cand;
+  const int* route_in;                     // this layer's route (NULL: pruned)
+  int* route_out;                          // the next one's
+  float most;                              // share of a prompt that a head's candidates may be for the next layer to be pruned
   float* scores;                           // preset: n_slots arrays [H_kv][score_stride]
   int64_t slot_stride;
   int32_t n_slots;
@@ -105,10 +117,12 @@ bound_hist_kernel(const __grid_constant__ SeqTable t, const __grid_constant__ Ch
   __shared__ uint32_t f_min[kPruneSums], f_max[kPruneSums], lse_max;
   const int tid = threadIdx.x, kvh = blockIdx.y, b = blockIdx.z, H = gridDim.y;
   pdl_trigger();
-  if ((int)blockIdx.x * kBoundTile - head_lead(t, a, b, kvh) >= t.prompt_len[b]) return;
+  const bool pruned = route_pruned(a.route_in);
+  if (pruned && (int)blockIdx.x * kBoundTile - head_lead(t, a, b, kvh) >= t.prompt_len[b]) return;
   for (int x = tid; x < kPruneBins; x += kBoundThreads) hist[x] = 0u;
   if (tid < kPruneSums) { f_min[tid] = 0x7f800000u; f_max[tid] = 0u; }
   if (tid == 0) lse_max = 0u;
+  if (!pruned) { wait_in_one_cta(); return; }
   __syncthreads();
   pdl_wait();
   const BoundSpan sp(t, a, b, kvh, blockIdx.x);
@@ -182,6 +196,7 @@ bound_list_kernel(const __grid_constant__ SeqTable t, const BoundArgs a) {
   __shared__ uint32_t list_at;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, kvh = blockIdx.y, b = blockIdx.z, H = gridDim.y;
   pdl_trigger();
+  if (!route_pruned(a.route_in)) { wait_in_one_cta(); return; }
   if ((int)blockIdx.x * kBoundTile - head_lead(t, a, b, kvh) >= t.prompt_len[b]) return;
   pdl_wait();
   const BoundSpan sp(t, a, b, kvh, blockIdx.x);
@@ -238,7 +253,11 @@ bound_list_kernel(const __grid_constant__ SeqTable t, const BoundArgs a) {
   for (int e = 0; e < kBoundKeys; ++e)
     if (e >= sp.v0 && e < sp.nv && !(hi[e] < floor_)) take |= 1u << e;   // (NaN: a candidate)
   const uint32_t n = __popc(take), upto = prefix(n, warp_sum[1], &total);
-  if (tid == 0) list_at = total ? atomicAdd(hist + kPruneBins, total) : 0u;
+  if (tid == 0) {
+    list_at = total ? atomicAdd(hist + kPruneBins, total) : 0u;
+    // (the count only grows: some block of the head sees it beyond the limit if it ends there)
+    if ((float)(list_at + total) > a.most * (float)t.prompt_len[b]) *a.route_out = kRouteFull;
+  }
   __syncthreads();
   int32_t* list = a.cand + sp.at + list_at + (upto - n);
   float preset[kBoundKeys];
@@ -248,6 +267,19 @@ bound_list_kernel(const __grid_constant__ SeqTable t, const BoundArgs a) {
     if ((take >> e) & 1u) *list++ = sp.base + e;
   }
   for (int g = 0; g < a.n_slots; ++g) sp.store(a.scores + g * a.slot_stride, preset, a.slot_stride % 4 == 0 || g == 0);
+}
+
+// Sweep 1 of a layer on the full route, its sample on the pruned one, in one launch.
+__global__ void __launch_bounds__(kThreads1, 1)
+rowstat_route_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_s, const __grid_constant__ CUtensorMap tm_q,
+                     const __grid_constant__ SeqTable t, const __grid_constant__ ChunkTable ct, const __grid_constant__ ChunkTable ct_s,
+                     const Args a) {
+  const bool sampled = route_pruned(a.route_in);
+  const ChunkTable& c = sampled ? ct_s : ct;
+  // (the grid has room for either: the CTAs with work come first)
+  const int nx = c.n_chunks * a.n_qgroups, id = blockIdx.y * gridDim.x + blockIdx.x, kvh = id / nx;
+  if (kvh >= (int)gridDim.y) return;
+  rowstat_cta<true>(sampled ? tm_s : tm_k, tm_q, t, c, a, id - kvh * nx, kvh, sampled, !sampled);
 }
 
 }  // namespace
@@ -265,23 +297,21 @@ bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const D
   double pairs = 0.0;
   for (int b = 0; b < t.batch; ++b) {
     const int L = t.prompt_len[b], K = t.cu_keep[b + 1] - t.cu_keep[b];
-    if (L < 32768 || K > L / (L < 65536 ? 16 : 8)) return false;
+    if (L < kPruneLeastLen || K > L / 8) return false;
     pairs += (double)rows * dm.n_kv_heads * L;
   }
   if (pairs < kPruneLeastPairs) return false;
   plan->qg = qg;
   plan->per_cta = kPruneSums / qg.n_qgroups;
+  // (the candidates' sweep takes the time of its largest list, a sweep of 1e9 pairs some 300 us; what the sample, the second
+  // sum of the one pass and the bounds take is 25 us, 9e7 pairs, and a third of a sweep: 0.57 for 8 x 1024 rows of 128 k,
+  // whose heads with 60 % candidates lost 3 % and with 27 % gained 15; 0.27 for 4 x 448, 33 % gained 4 and 51 % lost 20)
+  plan->most = (float)(0.65 - 9e7 / pairs);
   // ---- the sample: rows kSamplePhase, kSamplePhase + 16, ... of the cache, seen as a tensor of its own
-  SeqTable& ts = plan->ts;
-  memset(&ts, 0, sizeof(ts));
+  SeqTable ts;                                                  // (only what plan_chunks looks at)
   ts.batch = t.batch;
-  for (int b = 0; b < t.batch; ++b) {
-    const int first = (t.cu_rows[b] + kSampleStride - 1 - kSamplePhase) / kSampleStride;      // first sampled row of the sequence
-    const int end = (t.cu_rows[b] + t.prompt_len[b] - kSamplePhase + kSampleStride - 1) / kSampleStride;
-    ts.cu_rows[b] = first;
-    ts.prompt_len[b] = end - first;
-  }
-  const uint64_t rows_s = ((uint64_t)t.cu_rows[t.batch] - kSamplePhase + kSampleStride - 1) / kSampleStride;
+  for (int b = 0; b < t.batch; ++b) ts.prompt_len[b] = sample_first(t.cu_rows[b] + t.prompt_len[b]) - sample_first(t.cu_rows[b]);
+  const uint64_t rows_s = (uint64_t)sample_first(t.cu_rows[t.batch]);
   const uint64_t kd[3] = {(uint64_t)kHeadDim, rows_s, (uint64_t)dm.n_kv_heads};
   uint64_t ks[2] = {(uint64_t)cv.k_row_stride * 2 * kSampleStride, (uint64_t)cv.k_head_stride * 2};
   if (dm.n_kv_heads == 1 && ks[1] == 0) ks[1] = ks[0] * rows_s;
@@ -308,7 +338,7 @@ bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const D
 }
 
 cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTable& t, const Dims& dm, const PruneBuffers& buf,
-                         float* slots, float* scores, int64_t score_stride, int* status, long long wait_limit,
+                         int route_at, int route_next, float* slots, float* scores, int64_t score_stride, int* status, long long wait_limit,
                          cudaStream_t s, LaunchLog* log) {
   Args a = {};
   a.n_pseudo = dm.n_pseudo;
@@ -329,18 +359,19 @@ cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTab
   a.k_head_stride = cv.k_head_stride;
   a.k_row_stride = cv.k_row_stride;
   cudaError_t e;
-  // 1: the sample
-  a.sampled = 1;
+  a.route_in = route_at < 0 ? nullptr : buf.route + route_at;
+  a.route_out = buf.route + route_next;
+  // 1: the sample, or sweep 1
   a.part = buf.part_s;
   a.ref = buf.ref;
-  if ((e = cudaFuncSetAttribute(rowstat_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(rowstat_route_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes)) != cudaSuccess) return e;
+  const int n_chunks = route_at >= 0 && plan.qg.ct1.n_chunks > plan.ct_s.n_chunks ? plan.qg.ct1.n_chunks : plan.ct_s.n_chunks;
   log->begin(kKindLseMerge, s);
-  e = launch_pdl(rowstat_kernel<true>, dim3(plan.ct_s.n_chunks * a.n_qgroups, dm.n_kv_heads), dim3(kThreads1), kSmemBytes, s, 1, plan.tm_s,
-                 plan.qg.tm_q, plan.ts, plan.ct_s, a);
+  e = launch_pdl(rowstat_route_kernel, dim3(n_chunks * a.n_qgroups, dm.n_kv_heads), dim3(kThreads1), kSmemBytes, s, 1, plan.qg.tm_k1, plan.tm_s,
+                 plan.qg.tm_q, t, plan.qg.ct1, plan.ct_s, a);
   log->end(s);
   if (e != cudaSuccess) return e;
   // 2: one pass over all keys
-  a.sampled = 0;
   a.n_stages = plan.n_stages_m;
   a.log2_sample = kLog2Sample;
   a.sum_groups = plan.per_cta;
@@ -372,6 +403,9 @@ cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTab
   ba.sum_stride = a.slot_stride;
   ba.score_stride = score_stride;
   ba.hist = buf.hist;
+  ba.route_in = a.route_in;
+  ba.route_out = a.route_out;
+  ba.most = plan.most;
   ba.cand = buf.cand;
   ba.scores = out;
   ba.slot_stride = slot_stride;
@@ -389,6 +423,7 @@ cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTab
   if (e != cudaSuccess) return e;
   // 4: the candidates' scores
   a.part = buf.part_m;
+  a.part_full = buf.part_s;
   a.cand = buf.cand;
   a.n_qgroups = plan.qg.n_qgroups2;
   a.rows_g = plan.qg.rows_g2;
@@ -400,7 +435,7 @@ cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTab
     if (e2 != cudaSuccess) return e2;
     log->begin(kKindSweep2, s);
     e2 = launch_pdl(kernel, dim3(plan.ct_g.n_chunks * a.n_qgroups, dm.n_kv_heads), dim3(kThreads2), smem, s, 1, plan.qg.tm_k2, plan.qg.tm_q,
-                    t, plan.ct_g, plan.ct_m, a);
+                    t, plan.ct_g, ChunkTables2{plan.ct_m, plan.qg.ct1}, a);
     log->end(s);
     return e2;
   };

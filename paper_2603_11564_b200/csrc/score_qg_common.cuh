@@ -85,10 +85,12 @@ struct Args {
   int64_t score_stride, slot_stride;
   int* status;
   // the pruned selection (score_prune.cu)
-  int32_t sampled;           // sweep 1 over a sample of the prompt: no synthetic keys
+  const int* route_in;       // the route of this layer: kRouteFull or kRoutePruned; NULL: the pruned one
+  int* route_out;            // ... and of the next one, as far as this layer shows
   float log2_sample;         // one-pass sweep: log2 of the sample's stride
   int32_t sum_groups;        // one-pass sweep: partial column sums kept per CTA (1, 2 or 4), in slots like the scores
   float2* part_out;          // one-pass sweep: its own partials (`part` holds the sample's)
+  const float2* part_full;   // candidates' sweep: sweep 1's partials, on the full route
   float* ref_out;            // one-pass sweep: [B, H_q, N] the estimate of each row's log-sum-exp that it worked with
   uint32_t* hist;            // [B, H_kv][kPruneHist] histogram and candidate count of every head (one-pass sweep: cleared)
   const int32_t* cand;       // [H_kv][score_stride] candidate positions, sequence b's from column cu_prompt[b] on
@@ -96,23 +98,49 @@ struct Args {
   int64_t k_head_stride, k_row_stride;
 };
 
+// A layer of a multi-layer call takes the route that the layer before found worth taking (score_prune.cu).  Written by
+// kernels of the layer before that had completed before this layer's first kernel could begin: read it at any time.
+// All threads of a warp together (the shuffle lets the compiler know that they agree: without it the sweeps behind a
+// branch on the route took 5 to 10 % longer).
+enum : int { kRoutePruned = 0, kRouteFull = 1 };
+__device__ __forceinline__ bool route_pruned(const int* route) {
+  const int r = route != nullptr ? __ldcg(route) : kRoutePruned;
+  return __shfl_sync(0xffffffffu, r, 0) == kRoutePruned;
+}
+// For a grid with nothing to do: its first CTA waits, so that the grid completes, and what follows begins, behind the
+// kernel before it; the others return at once, while that one still runs.
+__device__ __forceinline__ bool wait_in_one_cta() {
+  if (blockIdx.x || blockIdx.y || blockIdx.z) return false;
+  pdl_wait();
+  return true;
+}
+
+// The sample of a prompt: rows kSamplePhase, kSamplePhase + kSampleStride, ... of the cache.
+constexpr int kSampleStride = 16, kSamplePhase = 7;
+__host__ __device__ __forceinline__ int sample_first(int row) { return (row + kSampleStride - 1 - kSamplePhase) / kSampleStride; }
+
 // This CTA's work: sequence, tile range, first cache row, its query group.
 struct Work {
   int chunk, qgrp, b, L, nt, t0, row_base, qrow_base, rows, mb;
 };
-__device__ __forceinline__ Work cta_work(const SeqTable& t, const ChunkTable& ct, const Args& a, int tile_keys,
-                                         bool with_synthetic) {
+// (bx, kvh): the CTA's place in a grid of (chunks x query groups, KV heads)
+__device__ __forceinline__ Work cta_work(const SeqTable& t, const ChunkTable& ct, const Args& a, int bx, int kvh, int tile_keys,
+                                         bool with_synthetic, bool sampled = false) {
   Work w;
-  w.chunk = blockIdx.x / a.n_qgroups;
-  w.qgrp = blockIdx.x - w.chunk * a.n_qgroups;
-  const int kvh = blockIdx.y;
+  w.chunk = bx / a.n_qgroups;
+  w.qgrp = bx - w.chunk * a.n_qgroups;
   w.b = find_segment(ct.cu_chunk, t.batch, w.chunk);
+  w.row_base = t.cu_rows[w.b];                                                    // first cache row of the sequence
   w.L = t.prompt_len[w.b];
-  const int n_keys = w.L + (with_synthetic && !a.sampled ? a.n_pseudo : 0);
+  if (sampled) {                                                                  // (rows and lengths of the sample)
+    const int first = sample_first(w.row_base);
+    w.L = sample_first(w.row_base + w.L) - first;
+    w.row_base = first;
+  }
+  const int n_keys = w.L + (with_synthetic && !sampled ? a.n_pseudo : 0);
   const int n_tiles = (n_keys + tile_keys - 1) / tile_keys;
   w.t0 = (w.chunk - ct.cu_chunk[w.b]) * ct.chunk_tiles;
   w.nt = min(n_tiles, w.t0 + ct.chunk_tiles) - w.t0;
-  w.row_base = t.cu_rows[w.b];                                                    // first cache row of the sequence
   w.qrow_base = (w.b * a.n_q_heads + kvh * a.group) * a.n_pseudo;                 // first query row of this KV head
   w.rows = min(a.rows_g, a.rows_total - w.qgrp * a.rows_g);                       // query rows of this CTA's group
   w.mb = (w.rows + 127) / 128;                                                    // blocks of 128 rows

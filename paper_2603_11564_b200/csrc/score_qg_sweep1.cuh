@@ -131,10 +131,10 @@ __device__ __forceinline__ void row_sum_cols(uint32_t* v, int col0, int lim, Row
   }
 }
 
+// sampled (score_prune.cu): tm_k shows every kSampleStride-th row; no synthetic keys.
 template <bool kConvert>
-__global__ void __launch_bounds__(kThreads1, 1)
-rowstat_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_q,
-               const __grid_constant__ SeqTable t, const __grid_constant__ ChunkTable ct, const Args a) {
+__device__ __forceinline__ void rowstat_cta(const CUtensorMap& tm_k, const CUtensorMap& tm_q, const SeqTable& t, const ChunkTable& ct,
+                                            const Args& a, int bx, int kvh, bool sampled = false, bool signal_early = false) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
   if (sbase & 1023u) {                                          // (uniform over the CTA: nothing has been set up yet)
@@ -144,8 +144,7 @@ rowstat_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   using T = TileGeo<kTile1>;
   constexpr bool kFold = kConvert;                              // the library's own fp16 queries come with reference logits
-  const int kvh = blockIdx.y;
-  const Work w = cta_work(t, ct, a, kTile1, true);
+  const Work w = cta_work(t, ct, a, bx, kvh, kTile1, true, sampled);
   const int nt = w.nt, L = w.L, N = a.n_pseudo, mb = w.mb;
   if (nt <= 0) return;
   const Bars bars{sbase + Smem::bars};
@@ -168,7 +167,7 @@ rowstat_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   });
   // (past the wait for the rotation kernel: what sweep 2 copies ahead of its own wait is complete.  Its CTAs then set up
   // as this sweep's leave: 8 k keys on 8 heads 26.8 -> 26.1 us a layer; no gain, 0.3 % lost, at 32 k, where a CTA runs longer)
-  if (!a.sampled && ct.chunk_tiles <= 8) pdl_trigger();
+  if (signal_early || (!sampled && ct.chunk_tiles <= 8)) pdl_trigger();
   const uint32_t q_half = (uint32_t)mb * 128u * 128u;           // bytes of one 64-channel half of the query group
   const int S = a.n_stages;
 
@@ -232,7 +231,7 @@ rowstat_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     float m_raw0 = -CUDART_INF_F, z0 = 0.f, m_raw1 = -CUDART_INF_F, z1 = 0.f;
     RowSum rs0, rs1;                                            // ... or, with reference logits, the rows' sums
     // pseudo-query indices (sampled: the keys end with the prompt)
-    const int i_q0 = a.sampled ? -1 : (w.qgrp * a.rows_g + r) % N, i_q1 = a.sampled ? -1 : (w.qgrp * a.rows_g + 128 + r) % N;
+    const int i_q0 = sampled ? -1 : (w.qgrp * a.rows_g + r) % N, i_q1 = sampled ? -1 : (w.qgrp * a.rows_g + 128 + r) % N;
     if (kFold) {
       // The [256 x 16] operand: row i holds -r_i as an fp16 pair in channels 0 and 1 (zeros elsewhere, also
       // for rows beyond the group); the operand of ones carries its two ones in BOTH 16-byte halves of every
@@ -325,6 +324,13 @@ rowstat_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     }
   }
   cta_epilogue(tmem_base);
+}
+
+template <bool kConvert>
+__global__ void __launch_bounds__(kThreads1, 1)
+rowstat_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_q,
+               const __grid_constant__ SeqTable t, const __grid_constant__ ChunkTable ct, const Args a) {
+  rowstat_cta<kConvert>(tm_k, tm_q, t, ct, a, blockIdx.x, blockIdx.y);
 }
 
 }  // namespace qg

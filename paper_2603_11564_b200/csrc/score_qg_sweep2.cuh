@@ -83,7 +83,8 @@ __device__ __forceinline__ float colsum_job(uint32_t taddr, const float* lse_s, 
 //   kOnePass (score_prune.cu) the log-sum-exp is an estimate from a sample of the keys.  Every exponential is added
 //            twice: to its key's sum and to its query's, so that one pass yields the exact log-sum-exp and the scores up
 //            to the estimates' errors;
-//   kGather  the keys of a candidate list instead of a chunk; rows' log-sum-exp from the one-pass sweep's partials.
+//   kGather  the keys of a candidate list instead of a chunk; rows' log-sum-exp from the one-pass sweep's partials.  On
+//            the full route: every key, log-sum-exp from sweep 1's, like kPlain.
 //            A list of most of the prompt gives way to the whole prompt, whose tiles come in larger pieces (a listed tile
 //            takes about 0.85 us to gather, a job of 256 query rows 1.1).
 enum : int { kPlain = 0, kOnePass = 1, kGather = 2 };
@@ -93,6 +94,15 @@ template <int kForm> struct Layout2 {
   static constexpr int first_epi = kForm == kOnePass ? 8 : kFirstEpiWarp, sum_warp = kForm == kOnePass ? 6 : kFirstEpiWarp + 4 * kEpiGroups;
   static constexpr int threads = kForm == kOnePass ? kThreadsOne : kThreads2;
 };
+// Chunks behind the partials that a form merges; kGather: of the one-pass sweep, and of sweep 1 on the full route.
+struct ChunkTables2 { ChunkTable pruned, full; };
+template <int kForm> struct Chunks1 { using type = ChunkTable; };
+template <> struct Chunks1<kGather> { using type = ChunkTables2; };
+template <int kForm>
+__device__ __forceinline__ const ChunkTable& chunks1(const typename Chunks1<kForm>::type& c, bool pruned) {
+  if constexpr (kForm == kGather) return pruned ? c.pruned : c.full;
+  else return c;
+}
 
 // One 16-column piece of the one-pass sweep: exponentials into the key's sum and into the columns' sums.
 __device__ __forceinline__ void both_sums_piece(const uint32_t* v, float2* z, float2& acc, float2& acc1) {
@@ -335,7 +345,7 @@ template <bool kConvert, bool kWide, int kForm = kPlain, bool kNarrow = false>
 __global__ void __launch_bounds__(Layout2<kForm>::threads, 1)
 colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_q,
               const __grid_constant__ SeqTable t, const __grid_constant__ ChunkTable ct,
-              const __grid_constant__ ChunkTable ct1, const Args a) {
+              const __grid_constant__ typename Chunks1<kForm>::type ct1s, const Args a) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
   if (sbase & 1023u) {                                          // (uniform over the CTA: nothing has been set up yet)
@@ -352,16 +362,19 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
   Work w;
   int n_cand = 0;                                               // kGather: candidates of this (sequence, head)
   bool listed = kForm == kGather;                               // ... and whether the tiles are made of them
+  bool pruned = true;                                           // this layer's route
+  if constexpr (kForm == kOnePass) pruned = route_pruned(a.route_in);
   if constexpr (kForm == kGather) {
-    pdl_wait();
+    pruned = route_pruned(a.route_in);
+    if (pruned) pdl_wait();                                     // (the full route: set-up and first copies beside sweep 1's end)
     const int cta = blockIdx.x / a.n_qgroups;
     w.qgrp = blockIdx.x - cta * a.n_qgroups;
     w.b = find_segment(ct.cu_chunk, t.batch, cta);
     w.chunk = cta - ct.cu_chunk[w.b];
     const int n_ctas = ct.cu_chunk[w.b + 1] - ct.cu_chunk[w.b];
     w.L = t.prompt_len[w.b];
-    n_cand = (int)a.hist[(w.b * a.n_kv_heads + kvh) * kPruneHist + kPruneBins];
-    if (n_cand == t.cu_keep[w.b + 1] - t.cu_keep[w.b]) return;  // as many as are kept: they need no scores
+    n_cand = pruned ? (int)a.hist[(w.b * a.n_kv_heads + kvh) * kPruneHist + kPruneBins] : w.L;
+    if (pruned && n_cand == t.cu_keep[w.b + 1] - t.cu_keep[w.b]) return;   // as many as are kept: they need no scores
     listed = kWide ? 8 * (int64_t)n_cand <= 7 * (int64_t)w.L : 3 * (int64_t)n_cand <= 2 * (int64_t)w.L;
     const int n_tiles = ((listed ? n_cand : w.L) + kTile2 - 1) / kTile2, per = (n_tiles + n_ctas - 1) / n_ctas;
     w.t0 = w.chunk * per;
@@ -371,10 +384,18 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     w.rows = min(a.rows_g, a.rows_total - w.qgrp * a.rows_g);
     w.mb = (w.rows + 127) / 128;
   } else {
-    w = cta_work(t, ct, a, kTile2, kForm == kOnePass);
+    w = cta_work(t, ct, a, blockIdx.x, kvh, kTile2, kForm == kOnePass);
   }
   const int nt = w.nt, L = w.L, b = w.b;
+  if constexpr (kForm == kOnePass) {
+    if (!pruned) {                                              // nothing to do; the next layer goes the same way
+      pdl_trigger();
+      if (wait_in_one_cta() && threadIdx.x == 0) *a.route_out = kRouteFull;
+      return;
+    }
+  }
   if (nt <= 0) return;
+  const ChunkTable& ct1 = chunks1<kForm>(ct1s, pruned);
   using Smem = SmemT<kWide>;
   const Bars bars{sbase + Smem::bars};
   const Waiter wt{reinterpret_cast<volatile int*>(smem + Smem::abort_flag), a.status, a.wait_limit};
@@ -391,7 +412,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
   const bool m_live = is_epi && m_row < w.rows && !a.lse_in;
   const int m_nc = ct1.cu_chunk[b + 1] - ct1.cu_chunk[b];
   const int64_t m_step = (int64_t)a.n_kv_heads * a.rows_pad;
-  const float2* m_p = a.part + ((int64_t)ct1.cu_chunk[b] * a.n_kv_heads + kvh) * a.rows_pad + w.qgrp * a.rows_g + m_row;
+  const float2* m_p = (pruned ? a.part : a.part_full) + ((int64_t)ct1.cu_chunk[b] * a.n_kv_heads + kvh) * a.rows_pad + w.qgrp * a.rows_g + m_row;
   float2 m_q[16];
   if (m_live) {
     pdl_wait();                                                 // (sweep 1 wrote them)
@@ -489,6 +510,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
           if (live && w.chunk == ct.cu_chunk[b]) a.ref_out[w.qrow_base + grow] = seen;
         }
       }
+      if (kForm == kOnePass && blockIdx.x == 0 && blockIdx.y == 0 && warp == kFirstEpi && lane == 0) *a.route_out = kRoutePruned;
       if (kForm == kOnePass && w.qgrp == 0 && w.chunk == ct.cu_chunk[b]) {
         uint32_t* hist = a.hist + (int64_t)(b * a.n_kv_heads + kvh) * kPruneHist;
         for (int x = (warp - kFirstEpi) * 32 + lane; x < kPruneHist; x += kEpiThreads) hist[x] = 0u;

@@ -1035,70 +1035,208 @@ def test_split_operand_scorer_wait_limit(dq):
 
 
 # --------------------------------------------------------- the retained set without the scores (pruned selection)
-# At the smallest sizes that take it (2e8 query-key pairs): 1, 2, 3 and 4 query groups with full and ragged ends, one and
-# two score slots, odd lengths, ragged batches, budgets from one row to an eighth of a prompt.
+# At the smallest sizes that take it (2e8 query-key pairs, 65536 tokens): 1, 2, 3 and 4 query groups with full and ragged
+# ends, one and two score slots, odd lengths, ragged batches, budgets from one row to an eighth of a prompt.
 PRUNE_CASES = [
     # H_q, H_kv, N, lengths, budgets
-    (32, 8, 32, (196001,), (983,)), (32, 8, 64, (98003,), (1,)), (28, 4, 64, (112001,), (14000,)), (64, 8, 128, (32771,), (500,)),
+    (32, 8, 32, (196001,), (983,)), (32, 8, 64, (98003,), (1,)), (28, 4, 64, (112001,), (14000,)), (64, 8, 128, (65537,), (500,)),
     (12, 4, 100, (167003,), (5000,)), (6, 1, 128, (262001,), (1310,)), (5, 1, 104, (390001,), (9000,)),
-    (32, 8, 32, (33001, 50003, 40000, 32768, 45001), (2062, 900, 200, 2000, 40)), (32, 8, 32, (32768,) * 6, (256,) * 6),
+    (32, 8, 32, (66001, 83003, 73000, 65536), (2062, 900, 200, 4000)), (32, 8, 32, (65536,) * 3, (256,) * 3),
 ]
 
 
+def _prune_keys(dq, ctx, kind, q, k, lens, hkv, g):
+    """Key structures of a layer's fp32 draw, in place.  plain: N(0, 1); outliers: four channels x 8; far: three keys whose
+    logit for one row of a head lies 150 above the bulk and that the sample (rows 7, 23, ...) misses, so that row sums
+    leave the float range; equal: all keys the same; wide: logits of standard deviation 4, whose row sums a sample says
+    little about; sink: the first key some 12 above the rest for every row."""
+    hq, n = q.shape[1], q.shape[2]
+    if kind == "outliers":
+        k[:, :, [3, 40, 77, 100]] *= 8
+    elif kind == "wide":
+        k *= 4
+    elif kind == "equal":
+        k[:] = k[:, :1]
+    elif kind in ("far", "sink"):
+        rot = torch.empty_like(q)
+        dq.dapq_rope_pseudo_q(ctx, q, list(lens), rot)
+        for h in range(hkv):
+            if kind == "sink":
+                u = rot[0, h * (hq // hkv):(h + 1) * (hq // hkv)].float().mean((0, 1))
+                k[h, 0] = 12.0 * 128 ** 0.5 * u / u.norm() ** 2
+            else:
+                for pos in (0, lens[0] // 2 // 16 * 16, lens[0] // 16 * 16):
+                    u = rot[0, h * (hq // hkv), pos % n].float()
+                    k[h, pos] = 150.0 * 128 ** 0.5 * u / u.norm() ** 2
+
+
+def _same_set(full, got, scores, k, v, ko, vo, lens, cu_rows, cu_keep, cu_prompt):
+    """`got`: the full sweeps' indices, up to keys whose score lies within 1e-5 of the K-th; rows copied bit for bit."""
+    for b, L in enumerate(lens):
+        o, e, p = int(cu_keep[b]), int(cu_keep[b + 1]), int(cu_prompt[b])
+        for h in range(full.shape[0]):
+            x, y = full[h, o:e].long(), got[h, o:e].long()
+            assert bool((y[1:] > y[:-1]).all()) and int(y[0]) >= 0 and int(y[-1]) < L
+            rows = y + int(cu_rows[b])
+            assert torch.equal(ko[h, o:e], k[h, rows]) and torch.equal(vo[h, o:e], v[h, rows])
+            if not torch.equal(x, y):
+                s = scores[h, p:p + L]
+                kth = s[x].min()
+                other = torch.tensor(sorted(set(x.tolist()) ^ set(y.tolist())), device="cuda")
+                assert bool(((s[other] - kth).abs() <= 1e-5 * kth).all()), (b, h, len(other))
+
+
 @pytest.mark.parametrize("hq,hkv,n,lens,keep", PRUNE_CASES)
-@pytest.mark.parametrize("keys", ["plain", "outliers", "far", "equal"])
+@pytest.mark.parametrize("keys", ["plain", "outliers", "far", "equal", "wide", "sink"])
 def test_pruned_selection_matches_the_full_sweeps(dq, hq, hkv, n, lens, keep, keys):
-    """dapq_evict without scores_out against the same call with it (both full sweeps).  The two score a candidate with
-    log-sum-exps that were summed in another order (some 1e-6 apart): the sets may differ only in keys whose
-    score lies within 1e-5 of the K-th.  keys: N(0, 1); four channels x 8; three keys whose logit for one row of a
-    head lies 150 above the bulk and that the sample misses (its row sums leave the float range); all keys equal."""
+    """dapq_evict_layers against dapq_evict with scores_out (both full sweeps) of the same layer.  The two score a candidate
+    with log-sum-exps that were summed in another order (some 1e-6 apart).  Of the twelve layers the first takes the pruned
+    selection, the others take it if that paid."""
     g = torch.Generator(device="cuda")
     g.manual_seed(hq * 1000 + n)
     w = _small(lens=lens, keep=keep, n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0)
     q = torch.randn((w.batch, hq, n, 128), generator=g, device="cuda").bfloat16()
     k = torch.randn((hkv, w.total_rows, 128), generator=g, device="cuda")
     ctx = _ctx(dq, w)
-    if keys == "outliers":
-        k[:, :, [3, 40, 77, 100]] *= 8
-    elif keys == "far":
-        rot = torch.empty_like(q)
-        dq.dapq_rope_pseudo_q(ctx, q, list(lens), rot)
-        for h in range(hkv):
-            for pos in (0, lens[0] // 2 // 16 * 16, lens[0] // 16 * 16):       # (the sample takes rows 7, 23, ...)
-                u = rot[0, h * (hq // hkv), pos % n].float()
-                k[h, pos] = 150.0 * 128 ** 0.5 * u / u.norm() ** 2
-    elif keys == "equal":
-        k[:] = k[:, :1]
+    _prune_keys(dq, ctx, keys, q, k, lens, hkv, g)
     k = k.bfloat16()
     v = torch.randn(k.shape, generator=g, device="cuda", dtype=torch.bfloat16)
     KT = int(w.cu_keep[-1])
-
-    def call(scores):
-        idx = torch.full((hkv, KT), -1, dtype=torch.int32, device="cuda")
-        ko, vo = (torch.zeros((hkv, KT, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
-        before = dq.dapq_launch_count(ctx)
-        dq.dapq_evict(ctx, q, k, v, w.cu_rows, list(lens), list(keep), ko, vo, idx, scores)
-        dq.dapq_poll_status(ctx)
-        return idx, ko, vo, dq.dapq_launch_count(ctx) - before
-
+    outs = lambda: (torch.full((hkv, KT), -1, dtype=torch.int32, device="cuda"),
+                    *(torch.zeros((hkv, KT, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2)))
+    before = dq.dapq_launch_count(ctx)
     scores = torch.empty((hkv, w.total_prompt), dtype=torch.float32, device="cuda")
-    full, _, _, n_full = call(scores)
-    idx, ko, vo, n_pruned = call(None)
-    assert n_pruned > n_full                                                   # the pruned selection ran
-    assert torch.equal(call(None)[0], idx)                                     # and gives the same set again
-    for b in range(w.batch):
-        o, e, p = int(w.cu_keep[b]), int(w.cu_keep[b + 1]), int(w.cu_prompt[b])
-        for h in range(hkv):
-            x, y = full[h, o:e].long(), idx[h, o:e].long()
-            assert bool((y[1:] > y[:-1]).all()) and int(y[0]) >= 0 and int(y[-1]) < lens[b]
-            rows = y + int(w.cu_rows[b])
-            assert torch.equal(ko[h, o:e], k[h, rows]) and torch.equal(vo[h, o:e], v[h, rows])
-            if not torch.equal(x, y):
-                s = scores[h, p:p + lens[b]]
-                kth = s[x].min()
-                other = torch.tensor(sorted(set(x.tolist()) ^ set(y.tolist())), device="cuda")
-                assert bool(((s[other] - kth).abs() <= 1e-5 * kth).all()), (b, h, len(other))
+    full, ko, vo = outs()
+    dq.dapq_evict(ctx, q, k, v, w.cu_rows, list(lens), list(keep), ko, vo, full, scores)
+    n_full = dq.dapq_launch_count(ctx) - before
+    per_layer = [outs() for _ in range(12)]
+    i_all, k_all, v_all = zip(*per_layer)
+    first = None
+    for _ in range(2):
+        before = dq.dapq_launch_count(ctx)
+        dq.dapq_evict_layers(ctx, [q] * 12, [k] * 12, [v] * 12, w.cu_rows, list(lens), list(keep), k_all, v_all, i_all)
+        dq.dapq_poll_status(ctx)
+        assert dq.dapq_launch_count(ctx) - before > 12 * n_full                 # the pruned selection was launched
+        for idx, ko, vo in per_layer:
+            _same_set(full, idx, scores, k, v, ko, vo, lens, w.cu_rows, w.cu_keep, w.cu_prompt)
+        first = first or [i.clone() for i in i_all]
+        assert all(torch.equal(x, y) for x, y in zip(first, i_all))               # ... and gives the same sets again
     dq.dapq_destroy(ctx)
+
+
+@pytest.mark.parametrize("kind,pays", [("plain", True), ("wide", False)])
+def test_pruned_selection_is_left_where_it_does_not_pay(dq, kind, pays):
+    """Twelve layers: with sums that the sample misjudges, all but the first run the full sweeps (whose first one then takes
+    longer than the pass over all keys, which returns at once)."""
+    hq, hkv, n, L, K = 28, 4, 64, 131072, 2000
+    w = _small(lens=(L,), keep=(K,), n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    own, common = (torch.randn(x, generator=g, device="cuda") for x in ((1, hkv, hq // hkv, n, 128), (1, hkv, 1, 1, 128)))
+    q = (0.5 ** 0.5 * (own + common)).reshape(1, hq, n, 128).bfloat16()
+    k = torch.randn((hkv, L + n, 128), generator=g, device="cuda")
+    ctx = _ctx(dq, w)
+    _prune_keys(dq, ctx, kind, q, k, (L,), hkv, g)
+    k = k.bfloat16()
+    ko, vo = (torch.zeros((hkv, K, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    layers = lambda: dq.dapq_evict_layers(ctx, [q] * 12, [k] * 12, [k] * 12, w.cu_rows, [L], [K], [ko] * 12, [vo] * 12)
+    layers()
+    dq.dapq_profile(ctx, True)
+    layers()
+    ms = {x: t for x, (t, _) in dq.dapq_profile_read(ctx).items()}
+    dq.dapq_poll_status(ctx)
+    dq.dapq_destroy(ctx)
+    assert (ms["sweep1"] > 2 * ms["lse_merge"]) if pays else (ms["lse_merge"] > 2 * ms["sweep1"]), ms
+
+
+def test_pruned_layers_of_different_data_and_views(dq):
+    """Twelve layers of different kinds and budgets without a poll between them, keys and values as views with strides
+    (rows of all heads interleaved, the first sequence from row 5 of the cache), twice and from a CUDA graph; every layer
+    against the full sweeps of that layer."""
+    hq, hkv, n, lens = 28, 4, 64, (66003, 65539)
+    kinds = ["plain", "far", "outliers", "plain", "sink", "plain", "nan", "inf", "plain", "wide", "plain", "far"]
+    keeps = [(1000, 700), (4000, 3), (200, 200), (8000, 8000), (1, 1), (500, 900), (300, 300), (300, 300), (77, 3000), (999, 1), (50, 50), (1000, 1000)]
+    row0, R = 5, 5 + sum(lens) + 2 * n
+    cu_rows = [row0, row0 + lens[0] + n, R]
+    ctx = dq.dapq_create(hq, hkv, n, 2, R, dq.DAPQ_BF16, 1.0e4)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(9)
+    qs, ks, vs = [], [], []
+    for kind in kinds:
+        q = torch.randn((2, hq, n, 128), generator=g, device="cuda").bfloat16()
+        k = torch.randn((hkv, R, 128), generator=g, device="cuda")
+        _prune_keys(dq, ctx, kind, q, k[:, row0:], lens, hkv, g)
+        if kind in ("nan", "inf"):
+            k[1, row0 + 4000, 7] = float(kind)                                 # one key of one head
+        kv = torch.zeros((R, hkv, 2, 136), dtype=torch.bfloat16, device="cuda")
+        kv[:, :, 0, :128] = k.bfloat16().transpose(0, 1)
+        kv[:, :, 1, :128].normal_(generator=g)
+        qs.append(q)
+        ks.append(kv[:, :, 0, :128].transpose(0, 1))
+        vs.append(kv[:, :, 1, :128].transpose(0, 1))
+    outs = [(torch.zeros((hkv, sum(kp)), dtype=torch.int32, device="cuda"),
+             *(torch.zeros((hkv, sum(kp), 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))) for kp in keeps]
+    io, ko, vo = zip(*outs)
+    call = lambda: dq.dapq_evict_layers(ctx, qs, ks, vs, cu_rows, list(lens), keeps, ko, vo, io)
+    call()
+    dq.dapq_poll_status(ctx)
+    scores = torch.empty((hkv, sum(lens)), device="cuda")
+    for l, kp in enumerate(keeps):
+        full, kf, vf = (torch.zeros_like(x) for x in outs[l])
+        dq.dapq_evict(ctx, qs[l], ks[l], vs[l], cu_rows, list(lens), kp, kf, vf, full, scores)
+        dq.dapq_poll_status(ctx)
+        cu_keep, cu_prompt = [0, kp[0], sum(kp)], [0, lens[0], sum(lens)]
+        _same_set(full, io[l], scores, ks[l], vs[l], ko[l], vo[l], lens, cu_rows, cu_keep, cu_prompt)
+    want = [tuple(x.clone() for x in o) for o in outs]
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        call()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            call()
+    for o in outs:
+        for x in o:
+            x.zero_()
+    torch.cuda.synchronize()
+    graph.replay()
+    graph.replay()
+    torch.cuda.synchronize()
+    for o, x in zip(outs, want):
+        assert all(torch.equal(a, b) for a, b in zip(o, x))
+    dq.dapq_poll_status(ctx)
+    del graph
+    dq.dapq_destroy(ctx)
+
+
+def test_pruned_layers_full_size_against_the_oracle(dq):
+    """Twelve layers of the Qwen2.5-7B-shaped 128k cache through dapq_evict_layers, sampled KV heads of the first layer (which
+    has to try) and the last (which follows) against the oracle."""
+    w = gi.workload("qwen25_7b_128k")
+    ctx = _ctx(dq, w)
+    datas = []
+    for l in range(12):
+        d = gi.draw_layer(w, l, "cuda")
+        q_rot = torch.empty_like(d["q_pre"])
+        dq.dapq_rope_pseudo_q(ctx, d["q_pre"], list(w.prompt_lens), q_rot)
+        torch.cuda.synchronize()
+        gi.plant_structure(w, d, q_rot)
+        datas.append(d)
+    KT, L, G, N = int(w.cu_keep[-1]), w.prompt_lens[0], w.group, w.n_pseudo
+    ko = [torch.empty((w.n_kv_heads, KT, 128), dtype=torch.bfloat16, device="cuda") for _ in range(12)]
+    vo = [torch.empty_like(t) for t in ko]
+    idx = [torch.empty((w.n_kv_heads, KT), dtype=torch.int32, device="cuda") for _ in range(12)]
+    dq.dapq_evict_layers(ctx, [d["q_pre"] for d in datas], [d["k"] for d in datas], [d["v"] for d in datas], w.cu_rows,
+                         w.prompt_lens, w.keep, ko, vo, idx)
+    dq.dapq_poll_status(ctx)
+    dq.dapq_destroy(ctx)
+    for l, h in ((0, 1), (11, 2)):
+        d = datas[l]
+        qr = orc.rope_pseudo_q(util.to_f64(d["q_pre"])[0, h * G:(h + 1) * G], L, w.rope_base)
+        ref = orc.score_sequence(qr, util.to_f64(d["k"][h])[None, :L + N], L, G)["scores"][0]
+        gidx = idx[l][h].cpu().numpy()
+        util.assert_index_sets_match(gidx, ref, orc.topk_select(ref, w.keep[0]), L, f"layer {l} kvh={h}")
+        rows = torch.as_tensor(gidx.astype(np.int64)).cuda()
+        assert torch.equal(ko[l][h], d["k"][h][rows]) and torch.equal(vo[l][h], d["v"][h][rows])
 
 
 def test_pruned_selection_wait_limit(dq):
@@ -1109,15 +1247,16 @@ def test_pruned_selection_wait_limit(dq):
     ctx = _ctx(dq, w)
     outs = [[torch.zeros((hkv, K, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2)] + [torch.zeros((hkv, K), dtype=torch.int32, device="cuda")]
             for _ in range(2)]
-    dq.dapq_evict(ctx, q, k, v, w.cu_rows, [L], [K], *outs[0])
+    layers = lambda o: dq.dapq_evict_layers(ctx, [q] * 12, [k] * 12, [v] * 12, w.cu_rows, [L], [K], [o[0]] * 12, [o[1]] * 12, [o[2]] * 12)
+    layers(outs[0])
     dq.dapq_poll_status(ctx)
     dq.dapq_set_wait_limit(ctx, 1)
-    dq.dapq_evict(ctx, q, k, v, w.cu_rows, [L], [K], *outs[1])
+    layers(outs[1])
     with pytest.raises(dq.DapqError) as e:
         dq.dapq_poll_status(ctx)
     assert e.value.status == dq.DAPQ_ERR_TIMEOUT
     dq.dapq_set_wait_limit(ctx, 0)
-    dq.dapq_evict(ctx, q, k, v, w.cu_rows, [L], [K], *outs[1])
+    layers(outs[1])
     dq.dapq_poll_status(ctx)
     assert all(torch.equal(x, y) for x, y in zip(*outs))
     dq.dapq_destroy(ctx)
@@ -1140,7 +1279,7 @@ def test_pruned_selection_gives_up_anywhere(dq, cycles):
     k = k.bfloat16()
     outs = [[torch.zeros((hkv, K, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2)] + [torch.zeros((hkv, K), dtype=torch.int32, device="cuda")]
             for _ in range(2)]
-    layers = lambda o: dq.dapq_evict_layers(ctx, [q] * 4, [k] * 4, [v] * 4, w.cu_rows, [L], [K], [o[0]] * 4, [o[1]] * 4, [o[2]] * 4)
+    layers = lambda o: dq.dapq_evict_layers(ctx, [q] * 12, [k] * 12, [v] * 12, w.cu_rows, [L], [K], [o[0]] * 12, [o[1]] * 12, [o[2]] * 12)
     layers(outs[0])
     dq.dapq_poll_status(ctx)
     for _ in range(3):
