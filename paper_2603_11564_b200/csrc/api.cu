@@ -378,8 +378,10 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
   ok = ok && cudaMemset(ctx->status, 0, sizeof(int)) == cudaSuccess;
   if (!ok) { cudaGetLastError(); return bail(DAPQ_ERR_CUDA, "workspace allocation failed"); }
   if (wants_umma(ctx) && !wants_lo(ctx) && !(sh->flags & DAPQ_FLAG_Q_BF16) && sh->pool_mode == DAPQ_POOL_NONE &&
-      qg_groups(ctx->dims) <= kPruneSums && (double)hq_n * rows >= kPruneLeastPairs && prune_available()) {
-    // (no room: the two full sweeps need none of these)
+      qg_groups(ctx->dims) <= kPruneSums && (double)hq_n * rows >= kPruneLeastPairs &&
+      (int64_t)rows >= (int64_t)kPruneLeastLen * sh->max_batch && prune_available()) {
+    // (some 20 bytes a row and KV head: not for contexts of many short prompts, whose calls never take the route.  No room:
+    // the two full sweeps need none of these)
     PruneBuffers& pr = ctx->prune;
     Arena pa;
     pa.add(&pr.part_m, part_elems * sizeof(float2));

@@ -1239,6 +1239,21 @@ def test_pruned_layers_full_size_against_the_oracle(dq):
         assert torch.equal(ko[l][h], d["k"][h][rows]) and torch.equal(vo[l][h], d["v"][h][rows])
 
 
+def test_contexts_of_short_prompts_hold_no_workspace_for_the_pruned_selection(dq):
+    """40 prompts of 8k tokens: the device memory of a context that cannot prune (bf16 queries), up to a block or two of
+    the driver's 2 MiB; the same rows as one prompt take more."""
+    def used(max_batch, flags):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ctx = dq.dapq_create(32, 8, 32, max_batch, 40 * 8224, dq.DAPQ_BF16, 5.0e5, flags=flags)
+        taken = before - torch.cuda.mem_get_info()[0]
+        dq.dapq_destroy(ctx)
+        return taken
+    used(40, 0)
+    assert abs(used(40, 0) - used(40, dq.DAPQ_FLAG_Q_BF16)) <= 4 << 20
+    assert used(1, 0) - used(1, dq.DAPQ_FLAG_Q_BF16) >= 20 * 8 * 40 * 8224
+
+
 def test_pruned_selection_wait_limit(dq):
     """A device-side wait of the pruned selection that runs out: status once, and the context works again."""
     hq, hkv, n, L, K = 28, 4, 64, 112001, 2000
