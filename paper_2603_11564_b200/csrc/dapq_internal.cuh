@@ -232,7 +232,8 @@ struct PrunePlan {
 };
 struct PruneBuffers {                      // device workspace
   float2 *part_s, *part_m;                 // umma_part_elems each
-  float* ref;                              // [B, H_q, N]: first the rotation's reference logits, then the estimates
+  const float* ref;                        // [B, H_q, N] the rotation's reference logits
+  float* est;                              // [B, H_q, N] the estimates
   float* sums;                             // kPruneSums * (H_kv * max_total_rows rounded up to 4)
   int32_t* cand;                           // [H_kv][max_total_rows]
   uint32_t* hist;                          // [max_batch, H_kv][kPruneHist]

@@ -2,7 +2,7 @@
 // dapq_evict_layers call, from kPruneLeastLayers layers on.  The set of the two full sweeps, up to keys whose scores agree
 // with the K-th to rounding, for less than two thirds of their work where it pays.
 //
-//   1. sample      sweep 1 over every 16th key: an estimate r_i of each query row's log-sum-exp;
+//   1. sample      sweep 1 over every 16th key: with the first key an estimate r_i of each query row's log-sum-exp;
 //   2. one pass    over all keys with r_i in place of the log-sum-exp: e_ij = 2^(s_ij - r_i) is added to the sum of its
 //                  row, Z_i, and to that of its key, E_g(j), in up to four sums g of some 64 to 256 rows each.  The row sums
 //                  are what sweep 1 yields: log-sum-exp_i = r_i + log2 Z_i, in fp32 as there;
@@ -378,7 +378,7 @@ cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTab
   a.scores = buf.sums;
   a.slot_stride = ((int64_t)dm.n_kv_heads * score_stride + 3) & ~(int64_t)3;
   a.part_out = buf.part_m;
-  a.ref_out = buf.ref;
+  a.ref_out = buf.est;
   a.hist = buf.hist;
   auto one = a.rows_g <= 128 ? colsum_kernel<true, false, kOnePass, true> : colsum_kernel<true, false, kOnePass, false>;
   if ((e = cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes)) != cudaSuccess) return e;
@@ -393,7 +393,7 @@ cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTab
   const int64_t slot_stride = (int64_t)dm.n_kv_heads * score_stride;
   BoundArgs ba = {};
   ba.part = buf.part_m;
-  ba.ref = buf.ref;
+  ba.ref = buf.est;
   ba.rows_total = a.rows_total;
   ba.rows_pad = a.rows_pad;
   ba.rows_g = a.rows_g;

@@ -88,7 +88,8 @@ __device__ __forceinline__ float2 merge_stats(float2 a, float2 b) {
 // at first.  The result stays exact for every input: a job whose sum leaves the float range (a key more
 // than ~2^127 above the reference) is redone from its registers with its own maximum and merged, which
 // moves m; once m is far from r every job takes that careful path.  Logits far BELOW r only underflow
-// against a term, the reference key's own, that is part of the same row's total.
+// against a term, the reference key's own, that is part of the same row's total (in the sweep over a sample, which does
+// not hold that key, what uses the sum adds the term).
 struct RowSum {
   float r, m, z, sc;                                            // reference, base of z, sum, 2^(r - m)
   __device__ __forceinline__ void init(float ref) { r = m = ref; z = 0.f; sc = 1.f; }

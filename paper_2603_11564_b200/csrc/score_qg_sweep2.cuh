@@ -414,8 +414,10 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
   const int64_t m_step = (int64_t)a.n_kv_heads * a.rows_pad;
   const float2* m_p = (pruned ? a.part : a.part_full) + ((int64_t)ct1.cu_chunk[b] * a.n_kv_heads + kvh) * a.rows_pad + w.qgrp * a.rows_g + m_row;
   float2 m_q[16];
+  float m_first = 0.f;                                          // kOnePass: the row's logit against the first key
   if (m_live) {
     pdl_wait();                                                 // (sweep 1 wrote them)
+    if (kForm == kOnePass) m_first = __ldg(a.ref + w.qrow_base + w.qgrp * a.rows_g + m_row);
     if (kForm != kOnePass)                                      // (the sample's partials are few: read where they are merged)
 #pragma unroll
     for (int u = 0; u < 16; ++u)
@@ -488,7 +490,14 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             const float m = fmaxf(mx, mo);
             l2 = m + log2f(z * exp2f(mx - m) + zo * exp2f(mo - m));
           }
-          if (kForm == kOnePass) l2 += a.log2_sample;
+          if (kForm == kOnePass) {
+            // the estimate: the sample's sum times its stride, and the first key, which is not in the sample and may hold
+            // most of a row's mass (its logit is the rotation's reference; it counts in full even where the sample's
+            // logits, taken relative to it, have all underflowed)
+            l2 += a.log2_sample;
+            const float first = m_first, m = fmaxf(l2, first);
+            l2 = m + log2f(exp2f(l2 - m) + exp2f(first - m));
+          }
           if (kForm == kPlain && a.lse_out && w.chunk == ct.cu_chunk[b]) a.lse_out[w.qrow_base + grow] = l2 * 0.6931471805599453f;
         }
         lse_s[row] = -l2;                                       // negated: the epilogue adds it
