@@ -128,10 +128,15 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+# The current stream without a Stream object (3 us) around it, where this torch has the two functions.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        if torch.cuda.is_initialized():            # the current stream without a Stream object (3 us) around it
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
+        if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device()) or None
         return torch.cuda.current_stream().cuda_stream or None
     return getattr(stream, "cuda_stream", stream) or None
 

@@ -1310,3 +1310,15 @@ def test_pruned_selection_gives_up_anywhere(dq, cycles):
         dq.dapq_poll_status(ctx)
         assert all(torch.equal(x, y) for x, y in zip(*outs))
     dq.dapq_destroy(ctx)
+
+
+def test_current_stream_with_and_without_the_short_way(dq, monkeypatch):
+    from paper_2603_11564_b200 import binding
+    s = torch.cuda.Stream()
+    for raw in (True, False):
+        if not raw:
+            monkeypatch.setattr(binding, "_raw_stream", None)
+        assert binding._stream(None) in (None, torch.cuda.default_stream().cuda_stream)
+        with torch.cuda.stream(s):
+            assert binding._stream(None) == s.cuda_stream
+        assert binding._stream(s) == s.cuda_stream
