@@ -244,7 +244,7 @@ DAPQ_API dapq_status dapq_evict(dapq_ctx* ctx, const void* q_pre, const dapq_cac
  * k_keep_layer_stride = 0.  Every layer uses the same workspace, so the layers run back to back;
  * only launches are issued (no copies, no synchronisation), which makes the whole call
  * capturable into a CUDA graph.  Stops at the first layer that fails and returns its status.
- * Calls of 12 layers and more on long prompts, without pooling and with budgets that are small against the prompts, compute
+ * Calls of 8 layers and more on long prompts, without pooling and with budgets that are small against the prompts, compute
  * the scores of those keys only that can be among the K largest, in layers where the layers before show that it
  * pays.  The sets are those of dapq_evict up to keys whose scores agree with the K-th to rounding (1e-5 of it), as are the
  * sets of two scorings whose log-sum-exps are summed in different orders; calls of fewer layers select dapq_evict's own,

@@ -388,7 +388,7 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
     pa.add(&pr.sums, kPruneSums * (score_bytes + 16));
     pa.add(&pr.cand, (size_t)sh->n_kv_heads * rows * sizeof(int32_t));
     pa.add(&pr.hist, (size_t)sh->max_batch * sh->n_kv_heads * kPruneHist * sizeof(uint32_t));
-    pa.add(&pr.route, 2 * sizeof(int));
+    pa.add(&pr.route, 2 * sizeof(float2));
     pa.add(&pr.est, (size_t)sh->max_batch * hq_n * sizeof(float));
     if (!pa.allocate(ctx)) {
       cudaGetLastError();

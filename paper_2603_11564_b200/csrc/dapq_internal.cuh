@@ -217,10 +217,10 @@ cudaError_t launch_score_split(const SplitPlan& plan, int q_dtype, const void* q
 
 // ---- the pruned selection: the layers of dapq_evict_layers (score_prune.cu) ----------------------------------
 constexpr int kPruneSums = 4;              // partial sums per key
-constexpr double kPruneLeastPairs = 2e8;   // query-key pairs of a layer below which the full sweeps are as fast
+constexpr double kPruneLeastPairs = 2e8;   // query-key pairs of a layer below which the full sweeps are as fast (score_prune.cu)
 constexpr int kPruneLeastLen = 65536;      // shortest prompt
-constexpr int kPruneLeastLayers = 12;      // of a call: the first one has to find out whether it pays, and loses a fifth if not
-constexpr int kPruneRetry = 32;            // layers after which a call that went back to the full sweeps tries again
+constexpr int kPruneLeastLayers = 8;       // of a call: the first has to find out whether it pays, and loses a fifth if not
+constexpr int kPruneRetry = 16;            // layers after which a call that went back to the full sweeps tries again
 // histogram of a head's lower bounds, its candidate count, the largest magnitude of its rows' log-sum-exps (bits of a float)
 constexpr int kPruneBins = 2048, kPruneHist = kPruneBins + 4;
 struct PrunePlan {
@@ -228,7 +228,7 @@ struct PrunePlan {
   CUtensorMap tm_s;                        // every 16th key
   ChunkTable ct_s, ct_m, ct_g;             // chunks of the sample's sweep and of the one-pass sweep; CTAs per candidate list
   int32_t n_stages_m, per_cta;
-  float most;                              // candidates of a head, as a share of its prompt, up to which the route pays
+  float most;                              // candidates of a head, as a share of its prompt, up to which a layer gains
 };
 struct PruneBuffers {                      // device workspace
   float2 *part_s, *part_m;                 // umma_part_elems each
@@ -237,7 +237,7 @@ struct PruneBuffers {                      // device workspace
   float* sums;                             // kPruneSums * (H_kv * max_total_rows rounded up to 4)
   int32_t* cand;                           // [H_kv][max_total_rows]
   uint32_t* hist;                          // [max_batch, H_kv][kPruneHist]
-  int* route;                              // [2] a layer's route and the next one's
+  float2* route;                           // [2] what decides a layer's route, and the next one's
 };
 bool prune_available();
 bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const Dims& dm, int n_sm, PrunePlan* plan);

@@ -16,23 +16,29 @@
 // is done over again by itself (careful_row).
 //
 // Where it pays is a matter of the data: the bounds are as wide as the worst estimate among the rows behind a sum, and rows
-// whose mass lies in few keys are estimated badly.  So the first layer of a call tries, and notes whether the
-// candidates of every head were few enough (PrunePlan::most); the next layers run the full sweeps if not (and try again
-// after kPruneRetry layers).  The decision stays on the device: the launches are the same either way, the two sweeps do the
-// one thing or the other, and the one pass and the bounds return at once.
+// whose mass lies in few keys are estimated badly.  So the first layer of a call tries, and every layer that is pruned adds
+// what its longest list of candidates gained or lost to a credit (Route); once that is used up, the next layers run the full
+// sweeps, and one tries again after kPruneRetry layers.  The decision stays on the device: the launches are the same either
+// way, the two sweeps do the one thing or the other, and the one pass and the bounds return at once.
 //
-// Measured on B200, us a layer of a 32-layer call, full sweeps -> here; keys N(0, 1) times a factor that sets the standard
-// deviation of the logits, or four channels times 8, or a first key 8 above the rest, or five keys that single rows attend
-// to, or passages that stand out for K or K/2 keys:
-//                           sd 1        sd 2        sd 3        sd 4        channels    first key   single rows passages K  K/2
-//   8 heads x 1024 rows, 128 k  655 -> 564  699 -> 706  697 -> 708  700 -> 709  672 -> 561  656 -> 498  662 -> 517  661 -> 555  678 -> 606
-//   4 x 448, 128 k          176 -> 164  174 -> 169  175 -> 182  178 -> 183  173 -> 160  175 -> 157  173 -> 164  172 -> 152  180 -> 188
-//   8 x 256, 128 k          204 -> 188  199 -> 190  212 -> 221  217 -> 229  215 -> 224  196 -> 177  198 -> 210  192 -> 171  194 -> 198
-// (with every layer trying: 8 x 1024 at sd 3 691 -> 806, 4 x 448 181 -> 219.)  What the full route still loses is the three
-// launches with nothing to do (some 2 us each) and the layer that tried: 12 layers at sd 4 655 -> 666, 178 -> 188, 189 -> 202.
-// Prompts of 32 k gained a tenth at best and lost a fifth (8 x 1024 rows: first key 190 -> 176, sd 1 209 -> 238; 8 prompts
-// of 8 x 256: 434 -> 393, sd 2 404 -> 479): a sample of 2 k keys says too little.  Hence the conditions in
-// prune_plan: prompts long enough for the sample, query-key pairs enough for the launches, and a budget of at
+// Measured on B200, us a layer of a 32-layer call, full sweeps -> here, 128 k keys:
+//                                        8 heads x 1024 rows      4 x 448       8 x 256
+//   N(0, 1) keys                             670 -> 573         177 -> 166    197 -> 184
+//   the same times 2                         694 -> 715         175 -> 170    201 -> 190
+//   times 3                                  713 -> 743         183 -> 193    209 -> 222
+//   times 4                                  712 -> 739         176 -> 183    224 -> 236
+//   four channels times 8                    683 -> 581         177 -> 165    215 -> 227
+//   a first key 8 above the rest             670 -> 507         174 -> 156    200 -> 180
+//   five keys that single rows attend to     679 -> 531         174 -> 166    214 -> 228
+//   passages that stand out, K keys          662 -> 562         172 -> 152    192 -> 171
+//   ... K/2 keys                             688 -> 621         180 -> 175    200 -> 206
+// (every layer trying whatever the others found: times 3 691 -> 806, 181 -> 219, 198 -> 222.)  What the full route still loses is
+// the three launches with nothing to do (some 2 us each) and the layers that tried: 12 layers, times 4, 671 -> 700, 184 -> 194,
+// 196 -> 211.  In a long call at the power cap (80 layers of 8 x 1024 rows, outlier channels and needles) 708 -> 603.
+// Prompts of 32 k gained a tenth at best and lost a fifth (8 x 1024 rows: first key 190 -> 176, N(0, 1) 209 -> 238; 8
+// prompts of 8 x 256: 434 -> 393, times 2 404 -> 479): a sample of 2 k keys says too little.  Fewer query-key pairs do
+// not pay for the launches: 1.3e8 pairs 130 -> 129 to 108 -> 132 (8 x 128 rows of 128 k, 8 x 256 of 64 k).  Hence the
+// conditions in prune_plan: prompts long enough for the sample, pairs enough for the launches, and a budget of at
 // most an eighth of a prompt, so that the threshold lies in the tail of the scores.
 #include "score_qg_sweep1.cuh"
 #include "score_qg_sweep2.cuh"
@@ -56,9 +62,9 @@ struct BoundArgs {
   int64_t sum_stride, score_stride;
   uint32_t* hist;
   int32_t* cand;
-  const int* route_in;                     // this layer's route (NULL: pruned)
-  int* route_out;                          // the next one's
-  float most;                              // share of a prompt that a head's candidates may be for the next layer to be pruned
+  const Route* route_in;                   // as in Args
+  Route* route_out;
+  float most;
   float* scores;                           // preset: n_slots arrays [H_kv][score_stride]
   int64_t slot_stride;
   int32_t n_slots;
@@ -117,7 +123,7 @@ bound_hist_kernel(const __grid_constant__ SeqTable t, const __grid_constant__ Ch
   __shared__ uint32_t f_min[kPruneSums], f_max[kPruneSums], lse_max;
   const int tid = threadIdx.x, kvh = blockIdx.y, b = blockIdx.z, H = gridDim.y;
   pdl_trigger();
-  const bool pruned = route_pruned(a.route_in);
+  const bool pruned = route_of(a.route_in, a.most) >= 0.f;
   if (pruned && (int)blockIdx.x * kBoundTile - head_lead(t, a, b, kvh) >= t.prompt_len[b]) return;
   for (int x = tid; x < kPruneBins; x += kBoundThreads) hist[x] = 0u;
   if (tid < kPruneSums) { f_min[tid] = 0x7f800000u; f_max[tid] = 0u; }
@@ -196,7 +202,7 @@ bound_list_kernel(const __grid_constant__ SeqTable t, const BoundArgs a) {
   __shared__ uint32_t list_at;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, kvh = blockIdx.y, b = blockIdx.z, H = gridDim.y;
   pdl_trigger();
-  if (!route_pruned(a.route_in)) { wait_in_one_cta(); return; }
+  if (!(route_of(a.route_in, a.most) >= 0.f)) { wait_in_one_cta(); return; }
   if ((int)blockIdx.x * kBoundTile - head_lead(t, a, b, kvh) >= t.prompt_len[b]) return;
   pdl_wait();
   const BoundSpan sp(t, a, b, kvh, blockIdx.x);
@@ -255,8 +261,8 @@ bound_list_kernel(const __grid_constant__ SeqTable t, const BoundArgs a) {
   const uint32_t n = __popc(take), upto = prefix(n, warp_sum[1], &total);
   if (tid == 0) {
     list_at = total ? atomicAdd(hist + kPruneBins, total) : 0u;
-    // (the count only grows: some block of the head sees it beyond the limit if it ends there)
-    if ((float)(list_at + total) > a.most * (float)t.prompt_len[b]) *a.route_out = kRouteFull;
+    // (the count only grows: the block that comes last sees all of it; positive floats order like their bit patterns)
+    atomicMax(reinterpret_cast<int*>(&a.route_out->worst), __float_as_int((float)(list_at + total) / (float)t.prompt_len[b]));
   }
   __syncthreads();
   int32_t* list = a.cand + sp.at + list_at + (upto - n);
@@ -274,7 +280,7 @@ __global__ void __launch_bounds__(kThreads1, 1)
 rowstat_route_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_s, const __grid_constant__ CUtensorMap tm_q,
                      const __grid_constant__ SeqTable t, const __grid_constant__ ChunkTable ct, const __grid_constant__ ChunkTable ct_s,
                      const Args a) {
-  const bool sampled = route_pruned(a.route_in);
+  const bool sampled = route_of(a.route_in, a.most) >= 0.f;
   const ChunkTable& c = sampled ? ct_s : ct;
   // (the grid has room for either: the CTAs with work come first)
   const int nx = c.n_chunks * a.n_qgroups, id = blockIdx.y * gridDim.x + blockIdx.x, kvh = id / nx;
@@ -303,10 +309,10 @@ bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const D
   if (pairs < kPruneLeastPairs) return false;
   plan->qg = qg;
   plan->per_cta = kPruneSums / qg.n_qgroups;
-  // (the candidates' sweep takes the time of its largest list, a sweep of 1e9 pairs some 300 us; what the sample, the second
-  // sum of the one pass and the bounds take is 25 us, 9e7 pairs, and a third of a sweep: 0.57 for 8 x 1024 rows of 128 k,
-  // whose heads with 60 % candidates lost 3 % and with 27 % gained 15; 0.27 for 4 x 448, 33 % gained 4 and 51 % lost 20)
-  plan->most = (float)(0.65 - 9e7 / pairs);
+  // (the candidates' sweep takes the time of its longest list: with two jobs a tile about its share of a full sweep, with one
+  // half as much again.  Break-even measured at 0.59 to 0.85 of a sweep's time for 8 x 1024 rows of 128 k, in bursts and at the
+  // power cap, which the full sweeps reach; 0.50 for 4 x 448; 0.43 to 0.47 for 8 x 256)
+  plan->most = (float)(qg.wide2 ? 0.78 - 6.8e7 / pairs : 0.45 - 4e7 / pairs);
   // ---- the sample: rows kSamplePhase, kSamplePhase + 16, ... of the cache, seen as a tensor of its own
   SeqTable ts;                                                  // (only what plan_chunks looks at)
   ts.batch = t.batch;
@@ -359,8 +365,9 @@ cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTab
   a.k_head_stride = cv.k_head_stride;
   a.k_row_stride = cv.k_row_stride;
   cudaError_t e;
-  a.route_in = route_at < 0 ? nullptr : buf.route + route_at;
-  a.route_out = buf.route + route_next;
+  a.route_in = route_at < 0 ? nullptr : reinterpret_cast<const Route*>(buf.route) + route_at;
+  a.route_out = reinterpret_cast<Route*>(buf.route) + route_next;
+  a.most = plan.most;
   // 1: the sample, or sweep 1
   a.part = buf.part_s;
   a.ref = buf.ref;

@@ -66,6 +66,19 @@ constexpr int kRefSlabBytes = Smem::ref_slab_bytes, kRefSlab = Smem::ref_slab;
 static_assert(kOnes1SlabBytes <= kExchDepth * kEpiGroups * 128 * 4, "sweep 1's operand of ones does not fit the exchange area");
 constexpr int kSmemBytes = Smem::total;
 
+// A layer of a multi-layer call takes the route that the layers before it found worth taking (score_prune.cu): the pruned
+// one while its credit is not negative.  A pruned layer adds `most` less the largest share of a prompt that a head's
+// candidates were (`worst`); what the layers before left is at most 1, and `most` where there are none.
+struct Route { float credit, worst; };
+__device__ __forceinline__ float route_credit(const Route& r, float most) { return fminf(r.credit + most - r.worst, 1.f); }
+// NULL: a layer that tries.  Written by kernels of the layer before that had completed before this layer's first kernel could
+// begin: read it at any time.  All threads of a warp together (the shuffle tells the compiler that they agree).
+__device__ __forceinline__ float route_of(const Route* route, float most) {
+  if (route == nullptr) return most;
+  const float2 v = __ldcg(reinterpret_cast<const float2*>(route));
+  return __shfl_sync(0xffffffffu, route_credit({v.x, v.y}, most), 0);
+}
+
 struct Args {
   int32_t n_pseudo, group, n_q_heads, n_kv_heads;
   int32_t rows_total;        // G * N query rows per KV head
@@ -85,8 +98,9 @@ struct Args {
   int64_t score_stride, slot_stride;
   int* status;
   // the pruned selection (score_prune.cu)
-  const int* route_in;       // the route of this layer: kRouteFull or kRoutePruned; NULL: the pruned one
-  int* route_out;            // ... and of the next one, as far as this layer shows
+  const Route* route_in;     // what decides this layer's route; NULL: the pruned one
+  Route* route_out;          // ... and the next one's
+  float most;                // share of a prompt up to which a head's candidates leave the pruned route the faster one
   float log2_sample;         // one-pass sweep: log2 of the sample's stride
   int32_t sum_groups;        // one-pass sweep: partial column sums kept per CTA (1, 2 or 4), in slots like the scores
   float2* part_out;          // one-pass sweep: its own partials (`part` holds the sample's)
@@ -98,15 +112,6 @@ struct Args {
   int64_t k_head_stride, k_row_stride;
 };
 
-// A layer of a multi-layer call takes the route that the layer before found worth taking (score_prune.cu).  Written by
-// kernels of the layer before that had completed before this layer's first kernel could begin: read it at any time.
-// All threads of a warp together (the shuffle lets the compiler know that they agree: without it the sweeps behind a
-// branch on the route took 5 to 10 % longer).
-enum : int { kRoutePruned = 0, kRouteFull = 1 };
-__device__ __forceinline__ bool route_pruned(const int* route) {
-  const int r = route != nullptr ? __ldcg(route) : kRoutePruned;
-  return __shfl_sync(0xffffffffu, r, 0) == kRoutePruned;
-}
 // For a grid with nothing to do: its first CTA waits, so that the grid completes, and what follows begins, behind the
 // kernel before it; the others return at once, while that one still runs.
 __device__ __forceinline__ bool wait_in_one_cta() {

@@ -363,9 +363,13 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
   int n_cand = 0;                                               // kGather: candidates of this (sequence, head)
   bool listed = kForm == kGather;                               // ... and whether the tiles are made of them
   bool pruned = true;                                           // this layer's route
-  if constexpr (kForm == kOnePass) pruned = route_pruned(a.route_in);
+  float credit = 0.f;
+  if constexpr (kForm == kOnePass) {
+    credit = route_of(a.route_in, a.most);
+    pruned = credit >= 0.f;
+  }
   if constexpr (kForm == kGather) {
-    pruned = route_pruned(a.route_in);
+    pruned = route_of(a.route_in, a.most) >= 0.f;
     if (pruned) pdl_wait();                                     // (the full route: set-up and first copies beside sweep 1's end)
     const int cta = blockIdx.x / a.n_qgroups;
     w.qgrp = blockIdx.x - cta * a.n_qgroups;
@@ -390,7 +394,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
   if constexpr (kForm == kOnePass) {
     if (!pruned) {                                              // nothing to do; the next layer goes the same way
       pdl_trigger();
-      if (wait_in_one_cta() && threadIdx.x == 0) *a.route_out = kRouteFull;
+      if (wait_in_one_cta() && threadIdx.x == 0) *a.route_out = {credit, a.most};
       return;
     }
   }
@@ -519,7 +523,7 @@ colsum_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
           if (live && w.chunk == ct.cu_chunk[b]) a.ref_out[w.qrow_base + grow] = seen;
         }
       }
-      if (kForm == kOnePass && blockIdx.x == 0 && blockIdx.y == 0 && warp == kFirstEpi && lane == 0) *a.route_out = kRoutePruned;
+      if (kForm == kOnePass && blockIdx.x == 0 && blockIdx.y == 0 && warp == kFirstEpi && lane == 0) *a.route_out = {credit, 0.f};
       if (kForm == kOnePass && w.qgrp == 0 && w.chunk == ct.cu_chunk[b]) {
         uint32_t* hist = a.hist + (int64_t)(b * a.n_kv_heads + kvh) * kPruneHist;
         for (int x = (warp - kFirstEpi) * 32 + lane; x < kPruneHist; x += kEpiThreads) hist[x] = 0u;

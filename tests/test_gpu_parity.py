@@ -1124,22 +1124,24 @@ def test_pruned_selection_matches_the_full_sweeps(dq, hq, hkv, n, lens, keep, ke
     dq.dapq_destroy(ctx)
 
 
-@pytest.mark.parametrize("kind,pays", [("plain", True), ("sink", True), ("wide", False), ("peak", False)])
+@pytest.mark.parametrize("kind,pays", [("plain", True), ("sink", True), ("one wide", True), ("wide", False), ("peak", False)])
 def test_pruned_selection_is_left_where_it_does_not_pay(dq, kind, pays):
     """Twelve layers: with sums that the sample misjudges, all but the first run the full sweeps (whose first one then takes
-    longer than the pass over all keys, which returns at once)."""
+    longer than the pass over all keys, which returns at once); one such layer among eleven others changes nothing."""
     hq, hkv, n, L, K = 28, 4, 64, 131072, 2000
     w = _small(lens=(L,), keep=(K,), n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0)
     g = torch.Generator(device="cuda")
     g.manual_seed(5)
     own, common = (torch.randn(x, generator=g, device="cuda") for x in ((1, hkv, hq // hkv, n, 128), (1, hkv, 1, 1, 128)))
-    q = (0.5 ** 0.5 * (own + common)).reshape(1, hq, n, 128).bfloat16()
+    q = (own if "wide" in kind else 0.5 ** 0.5 * (own + common)).reshape(1, hq, n, 128).bfloat16()
     k = torch.randn((hkv, L + n, 128), generator=g, device="cuda")
     ctx = _ctx(dq, w)
-    _prune_keys(dq, ctx, kind, q, k, (L,), hkv, g)
-    k = k.bfloat16()
+    _prune_keys(dq, ctx, "plain" if kind == "one wide" else kind, q, k, (L,), hkv, g)
+    ks = [k.bfloat16()] * 12
+    if kind == "one wide":
+        ks[3] = (4 * k).bfloat16()
     ko, vo = (torch.zeros((hkv, K, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
-    layers = lambda: dq.dapq_evict_layers(ctx, [q] * 12, [k] * 12, [k] * 12, w.cu_rows, [L], [K], [ko] * 12, [vo] * 12)
+    layers = lambda: dq.dapq_evict_layers(ctx, [q] * 12, ks, ks, w.cu_rows, [L], [K], [ko] * 12, [vo] * 12)
     layers()
     dq.dapq_profile(ctx, True)
     layers()
