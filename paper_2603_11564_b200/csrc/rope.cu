@@ -7,7 +7,7 @@
 // precision: at positions near 131k a float angle has only ~7 fractional bits, which alone
 // would cost half of the scorer's error budget.  The 64 angles of a query are evaluated once per block of heads.  The
 // kernel is bound by the latency of its loads, angles and stores, block by block: batches take four queries per block
-// (40 prompts of 8 k, 32 heads, 32 queries: 31 -> 23 us, two layers' eviction 599 -> 582).
+// (40 prompts of 8 k, 32 heads, 32 queries: 31 -> 23 us a layer).
 #include <cuda_fp16.h>
 
 #include "dapq_internal.cuh"

@@ -7,8 +7,8 @@
 // tile once per query head.  Measured on B200, whole eviction of a layer, CUDA cores -> here: 32 heads without
 // groups, 32 queries, 16 k bf16 keys 432 -> 70 us; 8 x 4 heads, 32 queries, 12 k fp32 keys 339 -> 66 us; 2 x 4 heads,
 // 2 k fp32 keys 48 -> 25 us of device time.  Relative error of the scores against float64 on those inputs
-// 3.1e-7 -> 1.7e-7, 1.6e-7 -> 1.5e-7, 1.3e-7 -> 1.2e-7 (the mean of three seeds each): a chain of four tensor-core
-// additions per accumulator rounds less than one of 128 FMAs.
+// 3.04e-7 -> 1.64e-7, 1.62e-7 -> 1.57e-7, 1.53e-7 -> 0.90e-7 (the mean of six seeds each): a chain of four tensor-core
+// additions per accumulator rounds less than one of 128 FMAs, and the products left out for fp32 keys are below all that.
 //
 // What bounds it.  fp32 keys: the MMAs, 2450 cycles per tile and 64 query rows (28 MMAs of 64 to 192 columns; the split
 // of a tile into its parts takes four warps somewhat less).  bf16 keys: about 1200 cycles of MMAs per tile (9 of up

@@ -913,8 +913,9 @@ SPLIT_CASES = [
 def test_split_operand_scorer(dq, dtype, hq, hkv, n, lens):
     """dapq_evict's scores against the oracle, and against the same call on the CUDA cores.  Bound: a logit is a sum
     of exact bf16 products with fp32 roundings of at most 2^-23 of its largest partial sum in some 16 steps, and
-    |q||k|/sqrt(d) log2(e) stays below 25 for these N(0, 1) operands: 16 * 2^-23 * 25 = 4.8e-5 in base 2, 3.3e-5
-    relative, plus 2^-21 for two exponentials and the sums (measured: 2e-6)."""
+    |q||k|/sqrt(d) log2(e) stays below 25 for these N(0, 1) operands: 16 * 2^-23 * 25 = 4.8e-5 in base 2, and 2^-24 * 25 =
+    1.5e-6 for the products that fp32 keys leave out: 3.4e-5 relative, plus 2^-21 for two exponentials and the sums
+    (measured: 2e-6)."""
     w = _small(lens=lens, keep=tuple(max(1, L // 3) for L in lens), dtype=dtype, n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n,
                n_needles=0, outlier_channels=0)
     data = gi.draw_layer(w, 0, "cpu")
@@ -1120,7 +1121,12 @@ def test_pruned_selection_matches_the_full_sweeps(dq, hq, hkv, n, lens, keep, ke
         for idx, ko, vo in per_layer:
             _same_set(full, idx, scores, k, v, ko, vo, lens, w.cu_rows, w.cu_keep, w.cu_prompt)
         first = first or [i.clone() for i in i_all]
-        assert all(torch.equal(x, y) for x, y in zip(first, i_all))               # ... and gives the same sets again
+        assert all(torch.equal(x, y) for x, y in zip(first, i_all))            # ... and gives the same sets again
+    # a layer by itself, and calls of few layers: the sets of the call with scores, bit for bit
+    dq.dapq_evict(ctx, q, k, v, w.cu_rows, list(lens), list(keep), k_all[0], v_all[0], i_all[0])
+    dq.dapq_evict_layers(ctx, [q] * 7, [k] * 7, [v] * 7, w.cu_rows, list(lens), list(keep), k_all[1:8], v_all[1:8], i_all[1:8])
+    dq.dapq_poll_status(ctx)
+    assert all(torch.equal(x, full) for x in i_all[:8])
     dq.dapq_destroy(ctx)
 
 
