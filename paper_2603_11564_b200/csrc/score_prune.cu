@@ -34,7 +34,8 @@
 //   ... K/2 keys                             688 -> 621         180 -> 175    200 -> 206
 // (every layer trying whatever the others found: times 3 691 -> 806, 181 -> 219, 198 -> 222.)  What the full route still loses is
 // the three launches with nothing to do (some 2 us each) and the layers that tried: 12 layers, times 4, 671 -> 700, 184 -> 194,
-// 196 -> 211.  In a long call at the power cap (80 layers of 8 x 1024 rows, outlier channels and needles) 708 -> 603.
+// 196 -> 211; the shortest calls, 8 layers, 634 -> 702, 185 -> 196, 194 -> 207 (and 646 -> 535, 181 -> 159, 191 -> 173 with
+// passages for K keys).  In a long call at the power cap (80 layers of 8 x 1024 rows, outlier channels and needles) 708 -> 603.
 // Prompts of 32 k gained a tenth at best and lost a fifth (8 x 1024 rows: first key 190 -> 176, N(0, 1) 209 -> 238; 8
 // prompts of 8 x 256: 434 -> 393, times 2 404 -> 479): a sample of 2 k keys says too little.  Fewer query-key pairs do
 // not pay for the launches: 1.3e8 pairs 130 -> 129 to 108 -> 132 (8 x 128 rows of 128 k, 8 x 256 of 64 k).  Hence the
