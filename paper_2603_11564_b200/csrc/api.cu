@@ -27,12 +27,18 @@ struct dapq_ctx {
   int* status = nullptr;         // device status word
   void* q_rot = nullptr;         // [max_batch, H_q, N, d]
   float2* part = nullptr;        // [max_chunks, H_q, N]
+  // (of these, room for flow_layers layers)
   float* lse2 = nullptr;         // [max_batch, H_q, N]
   float* scores = nullptr;       // [H_kv, max_total_rows]
   float* pooled = nullptr;       // [H_kv, max_total_rows] (pooling only)
   float* slots = nullptr;        // [query groups, H_kv, max_total_rows] (sized for groups of 256 query rows; used when sweep 2 has more than one group)
   long long wait_limit = 0;      // cycles a device-side wait may take (0: the default, about a second)
   int32_t* idx = nullptr;        // [H_kv, max_total_rows]
+  int flow_layers = 1;           // layers of the full size that one launch may cover
+  int64_t flow_chunks = 0;       // rows of `part` in the layout of score_flow.cu
+  uint32_t* sync[2] = {};        // tickets and counters of its launches, used in turn
+  int64_t sync_words = 0;
+  int sync_turn = 0;
   PruneBuffers prune = {};       // the pruned selection (sums == nullptr: not available)
   // staging for the host-buffer entry points (allocated on first use): two sets, so that the copies of one
   // layer run beside the kernels of the layer before
@@ -114,11 +120,14 @@ dapq_status cuda_fail(dapq_ctx* ctx, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail((ctx), e_, #call);      \
   } while (0)
 
+constexpr double kFlowPairs = 6e8;             // query-key pairs of a launch of score_flow.cu that make its start and end small
+constexpr size_t kFlowPartBytes = 16u << 20;   // for its partial row sums
+
 // Device buffers allocated together: as one block, cut up at 256-byte boundaries, where a block of its own for each
 // would cost up to a millisecond apiece (large ones), or each by itself, where the driver has small blocks at hand.
 struct Arena {
   struct Part { void** p; size_t bytes; };
-  Part parts[12];
+  Part parts[16];
   int n = 0;
   size_t size = 0;
   template <typename T> void add(T** p, size_t bytes) {
@@ -262,6 +271,11 @@ dapq_status run_score_qg(dapq_ctx* ctx, const QgPlan& plan, const SeqTable& t, c
   return DAPQ_OK;
 }
 
+// The scorer over several layers a launch: the eviction path's own fp16 queries, one query group per KV head.
+bool wants_flow(const dapq_ctx* ctx) {
+  return wants_umma(ctx) && !(ctx->shape.flags & (DAPQ_FLAG_Q_BF16 | DAPQ_FLAG_Q_LO_SWEEP1 | DAPQ_FLAG_Q_LO_SWEEP2));
+}
+
 // The older tensor-core kernels (a second MMA pass with the low-order bf16 part of the queries) serve
 // the contexts that ask for that part in either sweep.
 bool wants_lo(const dapq_ctx* ctx) { return (ctx->shape.flags & (DAPQ_FLAG_Q_LO_SWEEP1 | DAPQ_FLAG_Q_LO_SWEEP2)) != 0; }
@@ -283,17 +297,32 @@ dapq_status run_score(dapq_ctx* ctx, int q_dtype, const void* q_rot, const Cache
   return DAPQ_OK;
 }
 
-// Eq. 5 on the scores, or on their pooled image if the context asks for pooling.
-dapq_status run_select(dapq_ctx* ctx, const float* scores, int64_t score_stride, int32_t* idx, int64_t idx_stride,
+IndexOut one_index(const dapq_ctx* ctx, int32_t* idx) {
+  IndexOut out = {};
+  out.p[0] = idx;
+  out.heads_per_layer = ctx->dims.n_kv_heads;
+  return out;
+}
+
+RopeBatch one_rope(const dapq_ctx* ctx, const void* q_pre) {
+  RopeBatch rb = {};
+  rb.q[0] = q_pre;
+  rb.n_layers = 1;
+  rb.group = ctx->dims.group;
+  return rb;
+}
+
+// Eq. 5 on the scores ([n_layers][H_kv][score_stride]), or on their pooled image if the context asks for pooling.
+dapq_status run_select(dapq_ctx* ctx, int n_layers, const float* scores, int64_t score_stride, const IndexOut& idx, int64_t idx_stride,
                        const SeqTable& t, cudaStream_t s) {
   cudaError_t e;
   if (ctx->shape.pool_mode != DAPQ_POOL_NONE) {
-    e = launch_pool(scores, ctx->pooled, score_stride, t, ctx->dims.n_kv_heads, ctx->shape.pool_kernel,
+    e = launch_pool(scores, ctx->pooled, score_stride, t, n_layers * ctx->dims.n_kv_heads, ctx->shape.pool_kernel,
                     ctx->shape.pool_mode, s, &ctx->log);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "pooling kernel");
     scores = ctx->pooled;
   }
-  e = launch_topk(scores, score_stride, idx, idx_stride, t, ctx->dims.n_kv_heads, s, &ctx->log);
+  e = launch_topk(scores, score_stride, idx, idx_stride, t, n_layers * ctx->dims.n_kv_heads, s, &ctx->log);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "top-k kernel");
   return DAPQ_OK;
 }
@@ -361,18 +390,34 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
   const size_t part_umma = (size_t)umma_part_elems(sh->max_batch, sh->n_q_heads, sh->n_kv_heads, sh->n_pseudo);
   if (part_umma > part_elems) part_elems = part_umma;
   const size_t rows = (size_t)sh->max_total_rows;
+  const bool flow = wants_flow(ctx);
+  if (flow) {
+    // enough layers a launch for some 6e8 query-key pairs; small calls of a large context may take more
+    const double layers = kFlowPairs / ((double)hq_n * rows);
+    ctx->flow_layers = layers >= kFlowLayers ? kFlowLayers : (int)layers + 1;
+    const size_t chunk_elems = (size_t)sh->n_kv_heads * flow_rows_pad(ctx->dims);
+    const size_t extra = kFlowPartBytes / (chunk_elems * sizeof(float2));
+    const size_t want = (size_t)ctx->flow_layers * sh->max_batch + (extra < 640 ? extra : 640);
+    const size_t need = want * chunk_elems * 3 / 2;                // (a float2 and a float each)
+    if (need > part_elems) part_elems = need;
+    ctx->flow_chunks = (int64_t)(part_elems * 2 / 3 / chunk_elems);
+    ctx->sync_words = (int64_t)ctx->flow_layers * sh->max_batch * sh->n_kv_heads * qg_groups(ctx->dims) + 1;
+  }
+  const size_t nl = (size_t)ctx->flow_layers;
   const int n_slots = wants_umma(ctx) ? qg_groups(ctx->dims) : (wants_split(ctx) ? split_groups(ctx->dims) : 1);
   const size_t score_bytes = (size_t)sh->n_kv_heads * rows * sizeof(float);
   Arena ar;
   ar.add(&ctx->inv_freq, sizeof(freq));
   ar.add(&ctx->status, sizeof(int));
-  ar.add(&ctx->q_rot, (size_t)sh->max_batch * hq_n * kHeadDim * sizeof(float));
+  ar.add(&ctx->q_rot, (size_t)sh->max_batch * hq_n * kHeadDim * (nl > 1 ? nl * sizeof(__half) : sizeof(float)));
   ar.add(&ctx->part, part_elems * sizeof(float2));
-  ar.add(&ctx->lse2, ((size_t)sh->max_batch * hq_n + 32) * sizeof(float));
-  ar.add(&ctx->scores, score_bytes);
-  ar.add(&ctx->idx, (size_t)sh->n_kv_heads * rows * sizeof(int32_t));
-  if (sh->pool_mode != DAPQ_POOL_NONE) ar.add(&ctx->pooled, score_bytes);
-  if (n_slots > 1) ar.add(&ctx->slots, n_slots * score_bytes);
+  ar.add(&ctx->lse2, (nl * sh->max_batch * hq_n + 32) * sizeof(float));
+  ar.add(&ctx->scores, nl * score_bytes);
+  ar.add(&ctx->idx, nl * sh->n_kv_heads * rows * sizeof(int32_t));
+  if (sh->pool_mode != DAPQ_POOL_NONE) ar.add(&ctx->pooled, nl * score_bytes);
+  if (n_slots > 1) ar.add(&ctx->slots, nl * n_slots * score_bytes);
+  if (flow)
+    for (auto& w : ctx->sync) ar.add(&w, ctx->sync_words * sizeof(uint32_t));
   bool ok = ar.allocate(ctx);
   ok = ok && cudaMemcpy(ctx->inv_freq, freq, sizeof(freq), cudaMemcpyHostToDevice) == cudaSuccess;
   ok = ok && cudaMemset(ctx->status, 0, sizeof(int)) == cudaSuccess;
@@ -384,7 +429,7 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
     // the two full sweeps need none of these)
     PruneBuffers& pr = ctx->prune;
     Arena pa;
-    pa.add(&pr.part_m, part_elems * sizeof(float2));
+    pa.add(&pr.part_m, part_umma * sizeof(float2));
     pa.add(&pr.sums, kPruneSums * (score_bytes + 16));
     pa.add(&pr.cand, (size_t)sh->n_kv_heads * rows * sizeof(int32_t));
     pa.add(&pr.hist, (size_t)sh->max_batch * sh->n_kv_heads * kPruneHist * sizeof(uint32_t));
@@ -507,8 +552,8 @@ dapq_status dapq_rope_pseudo_q(dapq_ctx* ctx, const void* q_pre, const int32_t* 
   dapq_status st = build_table(ctx, batch, nullptr, nullptr, nullptr, nullptr, pos_start_host, &t);
   if (st != DAPQ_OK) return st;
   DeviceGuard guard(ctx->device);
-  cudaError_t e = launch_rope(ctx->shape.dtype, ctx->shape.dtype, 0, q_pre, q_rot, ctx->inv_freq, t, ctx->dims, false, (cudaStream_t)stream,
-                              &ctx->log);
+  cudaError_t e = launch_rope(ctx->shape.dtype, ctx->shape.dtype, 0, one_rope(ctx, q_pre), q_rot, ctx->inv_freq, t, ctx->dims, false,
+                              (cudaStream_t)stream, &ctx->log);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "rope kernel");
   return DAPQ_OK;
 }
@@ -550,7 +595,7 @@ dapq_status dapq_topk_select(dapq_ctx* ctx, const float* scores, const int32_t* 
   dapq_status st = build_table(ctx, batch, nullptr, nullptr, cu_prompt_host, k_keep_host, nullptr, &t);
   if (st != DAPQ_OK) return st;
   DeviceGuard guard(ctx->device);
-  return run_select(ctx, scores, t.cu_prompt[batch], idx_out, t.cu_keep[batch], t, (cudaStream_t)stream);
+  return run_select(ctx, 1, scores, t.cu_prompt[batch], one_index(ctx, idx_out), t.cu_keep[batch], t, (cudaStream_t)stream);
 }
 
 dapq_status dapq_compact_kv(dapq_ctx* ctx, const dapq_cache_view* cache, const int32_t* idx,
@@ -565,8 +610,10 @@ dapq_status dapq_compact_kv(dapq_ctx* ctx, const dapq_cache_view* cache, const i
   st = build_table(ctx, cache->batch, cache->cu_rows_host, cache->prompt_len_host, nullptr, k_keep_host, nullptr, &t);
   if (st != DAPQ_OK) return st;
   DeviceGuard guard(ctx->device);
-  cudaError_t e = launch_compact(ctx->shape.dtype, cd, idx, t.cu_keep[t.batch], k_out, v_out, t,
-                                 ctx->dims.n_kv_heads, ctx->status, (cudaStream_t)stream, &ctx->log);
+  CompactBatch cb = {};
+  cb.l[0] = {cd, idx, k_out, v_out};
+  cudaError_t e = launch_compact(ctx->shape.dtype, cb, 1, t.cu_keep[t.batch], t, ctx->dims.n_kv_heads, ctx->status, (cudaStream_t)stream,
+                                 &ctx->log);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "compaction kernel");
   return DAPQ_OK;
 }
@@ -593,43 +640,131 @@ namespace {
 // before it had found, and which of the two route words holds what the next one is to do.
 struct PruneRoute { int32_t last_try = -1, at = 0; };
 
+// One layer's arguments, checked.
+struct Layer {
+  const void* q_pre;
+  CacheDev cd;
+  void *k_out, *v_out;
+  int32_t* idx_out;
+};
+dapq_status check_layer(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* cache, const int32_t* k_keep_host, void* k_out, void* v_out,
+                        int32_t* idx_out, Layer* y, SeqTable* t) {
+  if (!q_pre || !k_keep_host || !k_out || !v_out) return fail(ctx, DAPQ_ERR_INVALID_ARG, "dapq_evict: NULL argument");
+  if (!aligned16(k_out) || !aligned16(v_out)) return fail(ctx, DAPQ_ERR_UNSUPPORTED, "k_out / v_out must be 16-byte aligned");
+  *y = {q_pre, {}, k_out, v_out, idx_out};
+  const dapq_status st = check_view(ctx, cache, true, false, &y->cd);
+  if (st != DAPQ_OK) return st;
+  return build_table(ctx, cache->batch, cache->cu_rows_host, cache->prompt_len_host, nullptr, k_keep_host, nullptr, t);
+}
+
+// What a layer's step reads and writes: [lo, hi) of its arrays.
+struct Span {
+  uintptr_t lo, hi;
+  bool meets(const Span& o) const { return lo < o.hi && o.lo < hi; }
+};
+Span span_of(const void* p, size_t bytes) { return {(uintptr_t)p, p ? (uintptr_t)p + bytes : (uintptr_t)p}; }
+
+// Layers may share launches if nothing that one of them writes is written or read by another, so that their order does
+// not matter.
+struct LayerSpans {
+  Span out[3], in[3];
+  LayerSpans() = default;
+  LayerSpans(const dapq_ctx* ctx, const Layer& y, const SeqTable& t) {
+    const size_t eb = (size_t)ctx->elem_bytes, H = (size_t)ctx->dims.n_kv_heads, kt = (size_t)t.cu_keep[t.batch];
+    auto cache = [&](const void* p, int64_t head, int64_t row) {
+      return span_of(p, ((H - 1) * (size_t)head + (size_t)(t.cu_rows[t.batch] - 1) * (size_t)row + kHeadDim) * eb);
+    };
+    out[0] = span_of(y.k_out, H * kt * kHeadDim * eb);
+    out[1] = span_of(y.v_out, H * kt * kHeadDim * eb);
+    out[2] = span_of(y.idx_out, H * kt * sizeof(int32_t));
+    in[0] = cache(y.cd.k, y.cd.k_head_stride, y.cd.k_row_stride);
+    in[1] = cache(y.cd.v, y.cd.v_head_stride, y.cd.v_row_stride);
+    in[2] = span_of(y.q_pre, (size_t)t.batch * ctx->dims.n_q_heads * ctx->dims.n_pseudo * kHeadDim * eb);
+  }
+  bool apart(const LayerSpans& o) const {
+    for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j)
+        if (out[i].meets(o.out[j]) || out[i].meets(o.in[j]) || in[i].meets(o.out[j])) return false;
+    return true;
+  }
+};
+
+// Layers of this geometry whose workspace fits the context's.
+int layers_that_fit(const dapq_ctx* ctx, const SeqTable& t) {
+  const int64_t rows = ctx->shape.max_total_rows * ctx->flow_layers / t.cu_prompt[t.batch];
+  const int64_t seqs = (int64_t)ctx->shape.max_batch * ctx->flow_layers / t.batch;
+  const int64_t n = rows < seqs ? rows : seqs;
+  return n < 1 ? 1 : (n > kFlowLayers ? kFlowLayers : (int)n);
+}
+
+// n layers of one geometry and one row of budgets; *taken says how many of them were done (more than one only by score_flow.cu).
 // after_own_compaction: the kernel before this call in `stream` is the compaction kernel of an
 // earlier evict on the same context (the layers of dapq_evict_layers); the rotation then does
 // not wait for it before it starts.
-// route: the call's layers may take the pruned selection (NULL: they may not); layer: this one's number.
-dapq_status evict_impl(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* cache, const int32_t* k_keep_host,
-                       void* k_out, void* v_out, int32_t* idx_out, float* scores_out, void* stream,
-                       bool after_own_compaction, PruneRoute* route = nullptr, int32_t layer = 0) {
-  if (!ctx) return DAPQ_ERR_INVALID_ARG;
-  if (!q_pre || !k_keep_host || !k_out || !v_out) return fail(ctx, DAPQ_ERR_INVALID_ARG, "dapq_evict: NULL argument");
-  if (!aligned16(k_out) || !aligned16(v_out)) return fail(ctx, DAPQ_ERR_UNSUPPORTED, "k_out / v_out must be 16-byte aligned");
-  CacheDev cd;
-  dapq_status st = check_view(ctx, cache, true, false, &cd);
-  if (st != DAPQ_OK) return st;
-  SeqTable t;
-  st = build_table(ctx, cache->batch, cache->cu_rows_host, cache->prompt_len_host, nullptr, k_keep_host, nullptr, &t);
-  if (st != DAPQ_OK) return st;
-  DeviceGuard guard(ctx->device);
-  cudaStream_t s = (cudaStream_t)stream;
+// route: the call's layers may take the pruned selection (NULL: they may not); layer: the first one's number.
+dapq_status evict_impl(dapq_ctx* ctx, const Layer* y, int n, const SeqTable& t, float* scores_out, cudaStream_t s, bool after_own_compaction,
+                       PruneRoute* route, int32_t layer, int* taken) {
+  const CacheDev& cd = y[0].cd;
   float* scores = scores_out ? scores_out : ctx->scores;
-  int32_t* idx = idx_out ? idx_out : ctx->idx;
   const int64_t score_stride = t.cu_prompt[t.batch], idx_stride = t.cu_keep[t.batch];
   UmmaPlan plan;
   QgPlan qplan;
+  FlowPlan fplan;
+  PrunePlan pplan;
   const int64_t lo_rows = ctx->q_rows_max;
   const int flags = ctx->shape.flags;
   cudaError_t e;
-  if (wants_umma(ctx) && !wants_lo(ctx) && qg_plan(ctx->q_rot, (flags & DAPQ_FLAG_Q_BF16) ? 0 : 1, cd, t, ctx->dims, ctx->n_sm, &qplan)) {
-    // tensor-core scorer: rotated queries rounded to fp16, K tiles converted to fp16 on their way to the MMAs
-    // (DAPQ_FLAG_Q_BF16: queries rounded to bf16, no conversion)
+  dapq_status st = DAPQ_OK;
+  CompactBatch cb = {};
+  IndexOut idx = {};
+  idx.heads_per_layer = ctx->dims.n_kv_heads;
+  for (int l = 0; l < n; ++l) {
+    idx.p[l] = y[l].idx_out ? y[l].idx_out : ctx->idx + (int64_t)l * ctx->dims.n_kv_heads * idx_stride;
+    cb.l[l] = {y[l].cd, idx.p[l], y[l].k_out, y[l].v_out};
+  }
+  RopeBatch rb = one_rope(ctx, y[0].q_pre);
+  auto with_references = [&](int layers) {
     // (with fp16 queries the rotation also leaves, in lse2, every query's logit against the first key of its
     // sequence: the reference that sweep 1 measures the row's other logits against)
-    const RopeRef ref = {(const __nv_bfloat16*)cd.k, cd.k_head_stride, cd.k_row_stride, ctx->lse2, ctx->dims.group};
-    e = launch_rope(ctx->shape.dtype, qplan.q_is_f16 ? kRopeOutF16 : kRopeOutBf16, 0, q_pre, ctx->q_rot, ctx->inv_freq, t,
-                    ctx->dims, after_own_compaction, s, &ctx->log, &ref);
+    for (int l = 0; l < layers; ++l) {
+      rb.q[l] = y[l].q_pre;
+      rb.k[l] = (const __nv_bfloat16*)y[l].cd.k;
+      rb.head_stride[l] = y[l].cd.k_head_stride;
+      rb.row_stride[l] = y[l].cd.k_row_stride;
+    }
+    rb.n_layers = layers;
+    rb.ref = ctx->lse2;
+  };
+  const bool qg = wants_umma(ctx) && !wants_lo(ctx) &&
+                  qg_plan(ctx->q_rot, (flags & DAPQ_FLAG_Q_BF16) ? 0 : 1, cd, t, ctx->dims, ctx->n_sm, &qplan);
+  const bool prune = qg && route && ctx->prune.sums && prune_plan(qplan, cd, t, ctx->dims, ctx->n_sm, &pplan);
+  bool flow = false;
+  *taken = 1;
+  if (wants_flow(ctx) && !prune) {
+    CacheDev cds[kFlowLayers];
+    for (int l = 0; l < n; ++l) cds[l] = y[l].cd;
+    while (n > 1 && !flow_plan(ctx->q_rot, cds, n, t, ctx->dims, ctx->n_sm, ctx->flow_chunks, &fplan)) --n;
+    flow = n > 1;
+  }
+  if (flow) {
+    // rotated queries rounded to fp16, K tiles converted to fp16 on their way to the MMAs; both sweeps of all n layers in one launch
+    with_references(n);
+    uint32_t* sync = ctx->sync[ctx->sync_turn ^= 1];
+    rb.clear = sync;
+    rb.n_clear = fplan.n_items + 1;
+    e = launch_rope(ctx->shape.dtype, kRopeOutF16, 0, rb, ctx->q_rot, ctx->inv_freq, t, ctx->dims, after_own_compaction, s, &ctx->log);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "rope kernel");
-    PrunePlan pplan;
-    if (route && ctx->prune.sums && prune_plan(qplan, cd, t, ctx->dims, ctx->n_sm, &pplan)) {
+    e = launch_score_flow(fplan, t, ctx->dims, ctx->part, ctx->flow_chunks, ctx->lse2, ctx->slots, scores, score_stride, sync, ctx->n_sm, ctx->status,
+                          ctx->wait_limit, s, &ctx->log);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "tensor-core score kernel");
+    *taken = n;
+  } else if (qg) {
+    // tensor-core scorer, a launch per sweep (DAPQ_FLAG_Q_BF16: queries rounded to bf16, no conversion)
+    with_references(1);
+    e = launch_rope(ctx->shape.dtype, qplan.q_is_f16 ? kRopeOutF16 : kRopeOutBf16, 0, rb, ctx->q_rot, ctx->inv_freq, t,
+                    ctx->dims, after_own_compaction, s, &ctx->log);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "rope kernel");
+    if (prune) {
       // nobody reads the scores: only those that can be among the K largest are computed
       const bool attempt = route->last_try < 0 || layer - route->last_try >= kPruneRetry;
       if (attempt) route->last_try = layer;
@@ -645,21 +780,21 @@ dapq_status evict_impl(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* 
     // pass in the sweeps that the flags name
     plan.lo_sweep1 = (flags & DAPQ_FLAG_Q_LO_SWEEP1) ? 1 : 0;
     plan.lo_sweep2 = (flags & DAPQ_FLAG_Q_LO_SWEEP2) ? 1 : 0;
-    e = launch_rope(ctx->shape.dtype, kRopeOutSplitBf16, lo_rows * kHeadDim, q_pre, ctx->q_rot, ctx->inv_freq, t,
+    e = launch_rope(ctx->shape.dtype, kRopeOutSplitBf16, lo_rows * kHeadDim, rb, ctx->q_rot, ctx->inv_freq, t,
                     ctx->dims, after_own_compaction, s, &ctx->log);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "rope kernel");
     st = run_score_umma(ctx, plan, t, nullptr, scores, score_stride, nullptr, s);
   } else {
     // the rotated queries unrounded (fp32)
-    e = launch_rope(ctx->shape.dtype, kRopeOutF32, 0, q_pre, ctx->q_rot, ctx->inv_freq, t, ctx->dims, after_own_compaction, s,
+    e = launch_rope(ctx->shape.dtype, kRopeOutF32, 0, rb, ctx->q_rot, ctx->inv_freq, t, ctx->dims, after_own_compaction, s,
                     &ctx->log);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "rope kernel");
     st = run_score(ctx, DAPQ_F32, ctx->q_rot, cd, t, nullptr, scores, score_stride, nullptr, nullptr, true, s);
   }
   if (st != DAPQ_OK) return st;
-  st = run_select(ctx, scores, score_stride, idx, idx_stride, t, s);
+  st = run_select(ctx, *taken, scores, score_stride, idx, idx_stride, t, s);
   if (st != DAPQ_OK) return st;
-  e = launch_compact(ctx->shape.dtype, cd, idx, idx_stride, k_out, v_out, t, ctx->dims.n_kv_heads, ctx->status, s, &ctx->log);
+  e = launch_compact(ctx->shape.dtype, cb, *taken, idx_stride, t, ctx->dims.n_kv_heads, ctx->status, s, &ctx->log);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "compaction kernel");
   return DAPQ_OK;
 }
@@ -669,7 +804,14 @@ dapq_status evict_impl(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* 
 dapq_status dapq_evict(dapq_ctx* ctx, const void* q_pre, const dapq_cache_view* cache,
                        const int32_t* k_keep_host, void* k_out, void* v_out, int32_t* idx_out,
                        float* scores_out, void* stream) {
-  return evict_impl(ctx, q_pre, cache, k_keep_host, k_out, v_out, idx_out, scores_out, stream, false);
+  if (!ctx) return DAPQ_ERR_INVALID_ARG;
+  Layer y;
+  SeqTable t;
+  const dapq_status st = check_layer(ctx, q_pre, cache, k_keep_host, k_out, v_out, idx_out, &y, &t);
+  if (st != DAPQ_OK) return st;
+  DeviceGuard guard(ctx->device);
+  int taken;
+  return evict_impl(ctx, &y, 1, t, scores_out, (cudaStream_t)stream, false, nullptr, 0, &taken);
 }
 
 dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const* q_pre,
@@ -680,12 +822,34 @@ dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const
   if (n_layers < 0 || k_keep_layer_stride < 0) return fail(ctx, DAPQ_ERR_INVALID_ARG, "dapq_evict_layers: negative count or stride");
   if (n_layers > 0 && (!q_pre || !caches || !k_keep_host || !k_out || !v_out))
     return fail(ctx, DAPQ_ERR_INVALID_ARG, "dapq_evict_layers: NULL argument");
+  DeviceGuard guard(ctx->device);
   PruneRoute route;
-  for (int32_t l = 0; l < n_layers; ++l) {
-    const dapq_status st = evict_impl(ctx, q_pre[l], &caches[l], k_keep_host + (int64_t)l * k_keep_layer_stride, k_out[l],
-                                      v_out[l], idx_out ? idx_out[l] : nullptr, nullptr, stream, l > 0,
-                                      n_layers >= kPruneLeastLayers ? &route : nullptr, l);
+  auto check = [&](int32_t m, Layer* y, SeqTable* t) {
+    return check_layer(ctx, q_pre[m], &caches[m], k_keep_host + (int64_t)m * k_keep_layer_stride, k_out[m], v_out[m], idx_out ? idx_out[m] : nullptr, y, t);
+  };
+  for (int32_t l = 0; l < n_layers;) {
+    Layer y[kFlowLayers];
+    SeqTable t, other;
+    dapq_status st = check(l, &y[0], &t);
     if (st != DAPQ_OK) return st;
+    // The layers behind it that may share its launches: of the same geometry and budgets, as many as fit the workspace, none of them
+    // touching another's outputs; in launches of equal size.  (A layer that is not in order says so when its own turn comes.)
+    int n = 1;
+    if (wants_flow(ctx)) {
+      const int fit = layers_that_fit(ctx, t), left = n_layers - l, launches = (left + fit - 1) / fit, most = (left + launches - 1) / launches;
+      LayerSpans spans[kFlowLayers];
+      spans[0] = LayerSpans(ctx, y[0], t);
+      for (; n < most && check(l + n, &y[n], &other) == DAPQ_OK && memcmp(&other, &t, sizeof(t)) == 0; ++n) {
+        spans[n] = LayerSpans(ctx, y[n], t);
+        bool apart = true;
+        for (int i = 0; i < n; ++i) apart = apart && spans[n].apart(spans[i]);
+        if (!apart) break;
+      }
+    }
+    int taken = 1;
+    st = evict_impl(ctx, y, n, t, nullptr, (cudaStream_t)stream, l > 0, n_layers >= kPruneLeastLayers ? &route : nullptr, l, &taken);
+    if (st != DAPQ_OK) return st;
+    l += taken;
   }
   return DAPQ_OK;
 }

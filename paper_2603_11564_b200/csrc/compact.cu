@@ -15,14 +15,17 @@ constexpr int kRowsPerThread = 2;
 // flight per thread (the gather is bound by how many bytes the SMs keep in flight, not by instructions).
 template <int kPieces>   // 16-byte pieces per row
 __global__ void __launch_bounds__(kCompactThreads)
-compact_kv_kernel(const CacheDev cv, int elem_bytes, const int32_t* __restrict__ idx, int64_t idx_stride,
-                  uint4* __restrict__ k_out, uint4* __restrict__ v_out,
-                  const __grid_constant__ SeqTable t, int* __restrict__ status) {
+compact_kv_kernel(const __grid_constant__ CompactBatch cb, int elem_bytes, int64_t idx_stride, const __grid_constant__ SeqTable t,
+                  int* __restrict__ status) {
   pdl_trigger();                     // whatever follows may be set up (or, if it does not depend on this copy, run) beside it
   const int kt = t.cu_keep[t.batch];
   const int64_t gid = (int64_t)blockIdx.x * kCompactThreads + threadIdx.x;
   const int r0 = (int)(gid / kPieces) * kRowsPerThread, piece = (int)(gid % kPieces);
   const int kvh = blockIdx.y;
+  const CacheDev& cv = cb.l[blockIdx.z].cv;
+  const int32_t* __restrict__ idx = cb.l[blockIdx.z].idx;
+  uint4* __restrict__ k_out = reinterpret_cast<uint4*>(cb.l[blockIdx.z].k_out);
+  uint4* __restrict__ v_out = reinterpret_cast<uint4*>(cb.l[blockIdx.z].v_out);
   int seg[kRowsPerThread];
 #pragma unroll
   for (int i = 0; i < kRowsPerThread; ++i) seg[i] = r0 + i < kt ? find_segment(t.cu_keep, t.batch, r0 + i) : 0;
@@ -58,22 +61,17 @@ compact_kv_kernel(const CacheDev cv, int elem_bytes, const int32_t* __restrict__
 
 }  // namespace
 
-cudaError_t launch_compact(int dtype, const CacheDev& cv, const int32_t* idx, int64_t idx_stride,
-                           void* k_out, void* v_out, const SeqTable& t, int n_kv_heads, int* status,
+cudaError_t launch_compact(int dtype, const CompactBatch& cb, int n_layers, int64_t idx_stride, const SeqTable& t, int n_kv_heads, int* status,
                            cudaStream_t s, LaunchLog* log) {
   log->begin(kKindCompact, s);
-  const int kt = t.cu_keep[t.batch];
-  if (dtype == DAPQ_BF16) {
-    constexpr int P = kHeadDim * 2 / 16;
-    const dim3 grid((unsigned)(((int64_t)((kt + kRowsPerThread - 1) / kRowsPerThread) * P + kCompactThreads - 1) / kCompactThreads), n_kv_heads);
-    launch_pdl(compact_kv_kernel<P>, grid, dim3(kCompactThreads), 0, s, 1, cv, 2, idx, idx_stride, (uint4*)k_out,
-               (uint4*)v_out, t, status);
-  } else {
-    constexpr int P = kHeadDim * 4 / 16;
-    const dim3 grid((unsigned)(((int64_t)((kt + kRowsPerThread - 1) / kRowsPerThread) * P + kCompactThreads - 1) / kCompactThreads), n_kv_heads);
-    launch_pdl(compact_kv_kernel<P>, grid, dim3(kCompactThreads), 0, s, 1, cv, 4, idx, idx_stride, (uint4*)k_out,
-               (uint4*)v_out, t, status);
-  }
+  const int kt = t.cu_keep[t.batch], threads = (kt + kRowsPerThread - 1) / kRowsPerThread;   // (per piece of a row)
+  auto run = [&](auto kernel, int pieces, int elem_bytes) {
+    const dim3 grid((unsigned)(((int64_t)threads * pieces + kCompactThreads - 1) / kCompactThreads), n_kv_heads, n_layers);
+    launch_pdl(kernel, grid, dim3(kCompactThreads), 0, s, 1, cb, elem_bytes, idx_stride, t, status);
+  };
+  constexpr int P16 = kHeadDim * 2 / 16, P32 = kHeadDim * 4 / 16;
+  if (dtype == DAPQ_BF16) run(compact_kv_kernel<P16>, P16, 2);
+  else run(compact_kv_kernel<P32>, P32, 4);
   log->end(s);
   return cudaGetLastError();
 }

@@ -123,17 +123,21 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // q_pre has element type `dtype`; q_rot is written as `out_mode`: bf16, fp32 (unrounded, for
 // the CUDA-core scorer) or a bf16 pair hi + lo with lo = bf16(q - hi) stored `lo_offset`
 // elements after hi (for the tensor-core scorer).
-// ref (fp16 output mode only, may be NULL): the bf16 key cache and where to write, per rotated query, its base-2
-// logit against the first key of its sequence (see rope.cu).
-struct RopeRef {
-  const __nv_bfloat16* k;
-  int64_t head_stride, row_stride;   // elements
-  float* out;                        // [B, H_q, N]
-  int32_t group;
+// Layers that one launch of the rotation, the scorer, the selection and the compaction may cover (dapq_evict_layers).
+constexpr int kFlowLayers = 8;
+// q_rot: [layers][B, H_q, N, d].  ref (fp16 output mode only, may be NULL): where to write, per rotated query, its base-2
+// logit against the first key of its sequence in the layer's bf16 key cache (see rope.cu).  clear: words set to 0.
+struct RopeBatch {
+  const void* q[kFlowLayers];
+  const __nv_bfloat16* k[kFlowLayers];
+  int64_t head_stride[kFlowLayers], row_stride[kFlowLayers];   // of k, elements
+  int32_t n_layers, group;
+  float* ref;                                                  // [layers][B, H_q, N]
+  uint32_t* clear;
+  int32_t n_clear;
 };
-cudaError_t launch_rope(int dtype, int out_mode, int64_t lo_offset, const void* q_pre, void* q_rot, const double* inv_freq_dev,
-                        const SeqTable& t, const Dims& dm, bool late_wait, cudaStream_t s, LaunchLog* log,
-                        const RopeRef* ref = nullptr);
+cudaError_t launch_rope(int dtype, int out_mode, int64_t lo_offset, const RopeBatch& rb, void* q_rot, const double* inv_freq_dev,
+                        const SeqTable& t, const Dims& dm, bool late_wait, cudaStream_t s, LaunchLog* log);
 
 // Generic CUDA-core scorer (any N <= 128, both dtypes).
 //   part  : [n_chunks, H_q, N] float2 (running max, sum) in base-2 logits, room for max_chunks
@@ -196,6 +200,23 @@ cudaError_t launch_score_qg(const QgPlan& plan, const SeqTable& t, const Dims& d
                             float* slots, float* scores, int64_t score_stride, float* lse_out, const float* ref, int* status,
                             long long wait_limit, bool after_own_kernel, cudaStream_t s, LaunchLog* log);
 
+// The same scorer over several layers of the same geometry in one launch (score_flow.cu), for fp16 queries of the rotation
+// ([layers][B, H_q, N, d]).  flow_plan returns false when a view cannot be described to TMA or the partials do not fit
+// max_chunks rows of [H_kv][flow_rows_pad].  part: that many rows, and as many of floats behind them; ref: [layers][B, H_q, N];
+// scores: [layers][H_kv][score_stride]; slots (more than one query group): n_qgroups arrays like scores; sync: 1 + n_items
+// words, cleared.
+struct FlowPlan {
+  CUtensorMap tm_k[kFlowLayers], tm_q;
+  ChunkTable ct;                          // runs of key pairs
+  int32_t n_layers, n_qgroups, rows_g, rows_pad, two;
+  int32_t n_units, n_items, block;
+};
+int flow_rows_pad(const Dims& dm);
+bool flow_plan(const void* q, const CacheDev* cv, int n_layers, const SeqTable& t, const Dims& dm, int n_sm, int64_t max_chunks, FlowPlan* plan);
+cudaError_t launch_score_flow(const FlowPlan& plan, const SeqTable& t, const Dims& dm, float2* part, int64_t max_chunks, const float* ref, float* slots,
+                              float* scores, int64_t score_stride, uint32_t* sync, int n_sm, int* status, long long wait_limit, cudaStream_t s,
+                              LaunchLog* log);
+
 // Sum of n_slots score arrays of `count` values that lie one behind the other, in slot order.
 cudaError_t launch_slots_sum(const float* slots, int n_slots, float* scores, int64_t count, cudaStream_t s, LaunchLog* log);
 
@@ -247,8 +268,10 @@ bool prune_plan(const QgPlan& qg, const CacheDev& cv, const SeqTable& t, const D
 cudaError_t launch_prune(const PrunePlan& plan, const CacheDev& cv, const SeqTable& t, const Dims& dm, const PruneBuffers& buf,
                          int route_at, int route_next, float* slots, float* scores, int64_t score_stride, int* status, long long wait_limit,
                          cudaStream_t s, LaunchLog* log);
-cudaError_t launch_topk(const float* scores, int64_t score_stride, int32_t* idx, int64_t idx_stride,
-                        const SeqTable& t, int n_kv_heads, cudaStream_t s, LaunchLog* log);
+// n_heads: heads of all layers, heads_per_layer of them to each of the index arrays.
+struct IndexOut { int32_t* p[kFlowLayers]; int32_t heads_per_layer; };
+cudaError_t launch_topk(const float* scores, int64_t score_stride, const IndexOut& idx, int64_t idx_stride,
+                        const SeqTable& t, int n_heads, cudaStream_t s, LaunchLog* log);
 
 // pooled[kvh, j] = max / mean of scores[kvh, j - kernel/2 .. j + kernel/2] within each sequence.
 cudaError_t launch_pool(const float* scores, float* pooled, int64_t stride, const SeqTable& t, int n_kv_heads,
@@ -258,8 +281,9 @@ cudaError_t launch_pool(const float* scores, float* pooled, int64_t stride, cons
 cudaError_t launch_recall(const int32_t* gold, const int32_t* pred, int64_t idx_stride, const SeqTable& t,
                           int n_kv_heads, float* recall, cudaStream_t s, LaunchLog* log);
 
-cudaError_t launch_compact(int dtype, const CacheDev& cv, const int32_t* idx, int64_t idx_stride,
-                           void* k_out, void* v_out, const SeqTable& t, int n_kv_heads, int* status,
+struct CompactLayer { CacheDev cv; const int32_t* idx; void *k_out, *v_out; };
+struct CompactBatch { CompactLayer l[kFlowLayers]; };
+cudaError_t launch_compact(int dtype, const CompactBatch& cb, int n_layers, int64_t idx_stride, const SeqTable& t, int n_kv_heads, int* status,
                            cudaStream_t s, LaunchLog* log);
 
 }  // namespace dapq

@@ -2,7 +2,7 @@
 // tokens take positions L_p .. L_p+N-1, so their queries carry the positional encodings of
 // the first N decoding steps).
 //
-// Grid (pseudo queries i, sequence b, block of query heads); thread (c, hy) owns the channel
+// Grid (pseudo queries i, layer and sequence b, block of query heads); thread (c, hy) owns the channel
 // pair of frequency c of one head: (c, c + d/2), or (2c, 2c + 1) for the interleaved layout.  The angle pos * theta_c is formed and reduced in double
 // precision: at positions near 131k a float angle has only ~7 fractional bits, which alone
 // would cost half of the scorer's error budget.  The 64 angles of a query are evaluated once per block of heads.  The
@@ -35,16 +35,16 @@ template <> __device__ __forceinline__ __half from_double<__half>(double x) {
 }
 
 // kSplit: TO is bf16 and the rounding residual is stored as a second bf16 lo_offset elements on.
-// ref (optional, bf16 caches): also the logit of every rotated query against the FIRST key of its
-// sequence, ref.out[b, h, i] = out_scale * q_rot . K[h / G, cu_rows[b], :]: the first sweep of the
+// rb.ref (optional, bf16 caches): also the logit of every rotated query against the FIRST key of its
+// sequence, ref[layer, b, h, i] = out_scale * q_rot . K[h / G, cu_rows[b], :]: the first sweep of the
 // tensor-core scorer measures every other logit of the row against it.
 // kQ: consecutive pseudo queries per block.
 template <typename T, typename TO, bool kSplit, int kQ>
 __global__ void __launch_bounds__(kHeadDim / 2 * kHeadsPerBlock)
-rope_pseudo_q_kernel(const T* __restrict__ q_pre, TO* __restrict__ q_rot,
+rope_pseudo_q_kernel(const __grid_constant__ RopeBatch rb, TO* __restrict__ q_rot,
                      const double* __restrict__ inv_freq, const __grid_constant__ SeqTable t,
                      int n_q_heads, int n_pseudo, int64_t lo_offset, int late_wait,
-                     int interleaved, double out_scale, const RopeRef ref) {
+                     int interleaved, double out_scale) {
   // late_wait: the kernel before this one in the stream neither writes q_pre nor still reads q_rot
   // (it is the compaction of the layer before), so the rotation runs beside it; the wait at the end
   // keeps this grid, and with it everything launched after it, ordered behind that kernel.
@@ -53,13 +53,20 @@ rope_pseudo_q_kernel(const T* __restrict__ q_pre, TO* __restrict__ q_rot,
   // its wait.)
   if (!late_wait) pdl_wait();
   pdl_trigger();
-  const int i0 = blockIdx.x * kQ, b = blockIdx.y, c = threadIdx.x;
+  const int layer = blockIdx.y / t.batch, b = blockIdx.y - layer * t.batch;
+  const int i0 = blockIdx.x * kQ, c = threadIdx.x;
+  // (the counters of the scorer behind this kernel; their last user completed before the kernel before this one could begin)
+  for (int i = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * blockDim.x * blockDim.y + threadIdx.y * blockDim.x + c;
+       i < rb.n_clear; i += gridDim.x * gridDim.y * gridDim.z * blockDim.x * blockDim.y)
+    rb.clear[i] = 0u;
+  const T* __restrict__ q_pre = reinterpret_cast<const T*>(rb.q[layer]);
   const int h = blockIdx.z * kHeadsPerBlock + threadIdx.y, n = min(kQ, n_pseudo - i0);
   const bool active = h < n_q_heads;
   constexpr int half = kHeadDim / 2;
   static_assert(kQ <= kHeadsPerBlock, "row y of the block evaluates the angles of query y");
   const int c0 = interleaved ? 2 * c : c, c1 = interleaved ? 2 * c + 1 : c + half;
-  const size_t base = (((size_t)b * n_q_heads + h) * n_pseudo + i0) * kHeadDim;
+  const size_t base = (((size_t)b * n_q_heads + h) * n_pseudo + i0) * kHeadDim;         // of a layer's queries
+  const size_t row0 = ((size_t)blockIdx.y * n_q_heads + h) * n_pseudo + i0, out = row0 * kHeadDim;
   double lo[kQ], hi[kQ];
 #pragma unroll
   for (int u = 0; u < kQ; ++u) {
@@ -76,8 +83,8 @@ rope_pseudo_q_kernel(const T* __restrict__ q_pre, TO* __restrict__ q_rot,
     angle[threadIdx.y][c] = make_double2(sn, cs);
   }
   float key0 = 0.f, key1 = 0.f;
-  if (active && ref.out != nullptr) {
-    const __nv_bfloat16* k0 = ref.k + (int64_t)(h / ref.group) * ref.head_stride + (int64_t)t.cu_rows[b] * ref.row_stride;
+  if (active && rb.ref != nullptr) {
+    const __nv_bfloat16* k0 = rb.k[layer] + (int64_t)(h / rb.group) * rb.head_stride[layer] + (int64_t)t.cu_rows[b] * rb.row_stride[layer];
     key0 = __bfloat162float(k0[c0]);
     key1 = __bfloat162float(k0[c1]);
   }
@@ -89,7 +96,7 @@ rope_pseudo_q_kernel(const T* __restrict__ q_pre, TO* __restrict__ q_rot,
     const double r0 = (lo[u] * cs - hi[u] * sn) * out_scale, r1 = (hi[u] * cs + lo[u] * sn) * out_scale;
     part[u] = (float)r0 * key0 + (float)r1 * key1;
     if (active && u < n) {
-      const size_t e0 = base + u * kHeadDim + c0, e1 = base + u * kHeadDim + c1;
+      const size_t e0 = out + u * kHeadDim + c0, e1 = out + u * kHeadDim + c1;
       const TO h0 = from_double<TO>(r0), h1 = from_double<TO>(r1);
       q_rot[e0] = h0;
       q_rot[e1] = h1;
@@ -99,7 +106,7 @@ rope_pseudo_q_kernel(const T* __restrict__ q_pre, TO* __restrict__ q_rot,
       }
     }
   }
-  if (ref.out != nullptr) {                                     // (uniform over the grid)
+  if (rb.ref != nullptr) {                                      // (uniform over the grid)
     __shared__ float red[kHeadsPerBlock][kQ][2];
 #pragma unroll
     for (int u = 0; u < kQ; ++u) {
@@ -108,40 +115,38 @@ rope_pseudo_q_kernel(const T* __restrict__ q_pre, TO* __restrict__ q_rot,
       if ((c & 31) == 0) red[threadIdx.y][u][c >> 5] = part[u];   // the 64 threads of a head are two whole warps
     }
     __syncthreads();
-    if (active && c < n) ref.out[((size_t)b * n_q_heads + h) * n_pseudo + i0 + c] = red[threadIdx.y][c][0] + red[threadIdx.y][c][1];
+    if (active && c < n) rb.ref[row0 + c] = red[threadIdx.y][c][0] + red[threadIdx.y][c][1];
   }
   if (late_wait) pdl_wait();
 }
 
 }  // namespace
 
-cudaError_t launch_rope(int dtype, int out_mode, int64_t lo_offset, const void* q_pre, void* q_rot,
-                        const double* inv_freq_dev, const SeqTable& t, const Dims& dm, bool late_wait,
-                        cudaStream_t s, LaunchLog* log, const RopeRef* ref_in) {
-  RopeRef none = {nullptr, 0, 0, nullptr, 1};
-  const RopeRef ref = (ref_in && out_mode == kRopeOutF16) ? *ref_in : none;
+cudaError_t launch_rope(int dtype, int out_mode, int64_t lo_offset, const RopeBatch& rb, void* q_rot, const double* inv_freq_dev,
+                        const SeqTable& t, const Dims& dm, bool late_wait, cudaStream_t s, LaunchLog* log) {
   const int lw = late_wait ? 1 : 0;
   log->begin(kKindRope, s);
   // One query per block keeps a short call's latency lowest; four where a block each would take several waves.
-  const int heads = (dm.n_q_heads + kHeadsPerBlock - 1) / kHeadsPerBlock;
-  const bool many = (int64_t)dm.n_pseudo * t.batch * heads > 2048;
-  auto run = [&](auto kernel1, auto kernel4, auto* in, auto* out, int64_t offset, double scale, const RopeRef& r) {
-    const dim3 block(kHeadDim / 2, kHeadsPerBlock), grid1(dm.n_pseudo, t.batch, heads), grid4((dm.n_pseudo + 3) / 4, t.batch, heads);
-    return launch_pdl(many ? kernel4 : kernel1, many ? grid4 : grid1, block, 0, s, 1, in, out, inv_freq_dev, t, dm.n_q_heads, dm.n_pseudo, offset,
-                      lw, dm.rope_interleaved, scale, r);
+  const int heads = (dm.n_q_heads + kHeadsPerBlock - 1) / kHeadsPerBlock, seqs = t.batch * rb.n_layers;
+  const bool many = (int64_t)dm.n_pseudo * seqs * heads > 2048;
+  auto run = [&](auto kernel1, auto kernel4, auto* out, int64_t offset, double scale, bool with_ref) {
+    const dim3 block(kHeadDim / 2, kHeadsPerBlock), grid1(dm.n_pseudo, seqs, heads), grid4((dm.n_pseudo + 3) / 4, seqs, heads);
+    RopeBatch r = rb;
+    if (!with_ref) r.ref = nullptr;
+    return launch_pdl(many ? kernel4 : kernel1, many ? grid4 : grid1, block, 0, s, 1, r, out, inv_freq_dev, t, dm.n_q_heads, dm.n_pseudo, offset, lw,
+                      dm.rope_interleaved, scale);
   };
   using bf16 = __nv_bfloat16;
-  const bf16* in16 = (const bf16*)q_pre;
   if (dtype == DAPQ_BF16 && out_mode == kRopeOutSplitBf16)
-    run(rope_pseudo_q_kernel<bf16, bf16, true, 1>, rope_pseudo_q_kernel<bf16, bf16, true, 4>, in16, (bf16*)q_rot, lo_offset, 1.0, none);
+    run(rope_pseudo_q_kernel<bf16, bf16, true, 1>, rope_pseudo_q_kernel<bf16, bf16, true, 4>, (bf16*)q_rot, lo_offset, 1.0, false);
   else if (dtype == DAPQ_BF16 && out_mode == kRopeOutF16)
-    run(rope_pseudo_q_kernel<bf16, __half, false, 1>, rope_pseudo_q_kernel<bf16, __half, false, 4>, in16, (__half*)q_rot, 0, (double)dm.scale_log2e, ref);
+    run(rope_pseudo_q_kernel<bf16, __half, false, 1>, rope_pseudo_q_kernel<bf16, __half, false, 4>, (__half*)q_rot, 0, (double)dm.scale_log2e, true);
   else if (dtype == DAPQ_BF16 && out_mode == kRopeOutBf16)
-    run(rope_pseudo_q_kernel<bf16, bf16, false, 1>, rope_pseudo_q_kernel<bf16, bf16, false, 4>, in16, (bf16*)q_rot, 0, 1.0, none);
+    run(rope_pseudo_q_kernel<bf16, bf16, false, 1>, rope_pseudo_q_kernel<bf16, bf16, false, 4>, (bf16*)q_rot, 0, 1.0, false);
   else if (dtype == DAPQ_BF16)
-    run(rope_pseudo_q_kernel<bf16, float, false, 1>, rope_pseudo_q_kernel<bf16, float, false, 4>, in16, (float*)q_rot, 0, 1.0, none);
+    run(rope_pseudo_q_kernel<bf16, float, false, 1>, rope_pseudo_q_kernel<bf16, float, false, 4>, (float*)q_rot, 0, 1.0, false);
   else
-    run(rope_pseudo_q_kernel<float, float, false, 1>, rope_pseudo_q_kernel<float, float, false, 4>, (const float*)q_pre, (float*)q_rot, 0, 1.0, none);
+    run(rope_pseudo_q_kernel<float, float, false, 1>, rope_pseudo_q_kernel<float, float, false, 4>, (float*)q_rot, 0, 1.0, false);
   log->end(s);
   return cudaGetLastError();
 }

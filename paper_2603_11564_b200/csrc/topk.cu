@@ -48,6 +48,11 @@ __device__ __forceinline__ uint32_t order_key(float f) {
 constexpr int kMaxLead = 3;
 __device__ __forceinline__ int lead(const float* x) { return (int)((reinterpret_cast<uintptr_t>(x) & 15u) >> 2); }
 
+__device__ __forceinline__ int32_t* index_list(const IndexOut& idx, int head, int64_t stride) {
+  const int layer = head / idx.heads_per_layer;
+  return idx.p[layer] + (int64_t)(head - layer * idx.heads_per_layer) * stride;
+}
+
 struct TopkTables {
   uint32_t merged[3][kBins];   // cluster-wide histogram of each pass (every CTA holds a copy)
   uint32_t hist[kBins];        // this CTA's histogram (all zero between passes)
@@ -152,7 +157,7 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 __global__ void __launch_bounds__(kTopkThreads)
-topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, int32_t* __restrict__ idx,
+topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, const __grid_constant__ IndexOut idx,
                    int64_t idx_stride, const __grid_constant__ SeqTable t, int cache_keys) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   TopkSmem& sm = *reinterpret_cast<TopkSmem*>(smem_raw);
@@ -169,7 +174,7 @@ topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, int32
   const int L = t.prompt_len[b];
   const int K = t.cu_keep[b + 1] - t.cu_keep[b];
   const float* x = scores + (int64_t)kvh * score_stride + t.cu_prompt[b];
-  int32_t* out = idx + (int64_t)kvh * idx_stride + t.cu_keep[b];
+  int32_t* out = index_list(idx, kvh, idx_stride) + t.cu_keep[b];
 
   // slice of this CTA: [j0, j1), a multiple of 32 keys long so that warps stay converged
   const int slice = (((L + n_cta - 1) / n_cta) + 31) & ~31;
@@ -278,7 +283,7 @@ topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, int32
 // keys) the later passes merge histograms across the cluster like the general kernel.
 template <int kKpt, int kMinCtas>
 __global__ void __launch_bounds__(kTopkThreads, kMinCtas)
-topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, int32_t* __restrict__ idx,
+topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, const __grid_constant__ IndexOut idx,
                        int64_t idx_stride, const __grid_constant__ SeqTable t) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   TopkRegSmem& sm = *reinterpret_cast<TopkRegSmem*>(smem_raw);
@@ -293,7 +298,7 @@ topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, i
   const int L = t.prompt_len[b];
   const int K = t.cu_keep[b + 1] - t.cu_keep[b];
   const float* x = scores + (int64_t)kvh * score_stride + t.cu_prompt[b];
-  int32_t* out = idx + (int64_t)kvh * idx_stride + t.cu_keep[b];
+  int32_t* out = index_list(idx, kvh, idx_stride) + t.cu_keep[b];
   const int base = (rank * kTopkThreads + tid) * kKpt - lead(x);   // position of this thread's first key
   const int v0 = max(0, -base), nv = max(0, min(kKpt, L - base));  // its keys v0 .. nv - 1 exist
 
@@ -466,7 +471,7 @@ topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, i
 // (batches): the same steps as topk_select_reg_kernel without any exchange: the three tables are local histograms.
 template <int kKpt>
 __global__ void __launch_bounds__(kTopkThreads)
-topk_select_solo_kernel(const float* __restrict__ scores, int64_t score_stride, int32_t* __restrict__ idx,
+topk_select_solo_kernel(const float* __restrict__ scores, int64_t score_stride, const __grid_constant__ IndexOut idx,
                         int64_t idx_stride, const __grid_constant__ SeqTable t) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   TopkRegSmem& sm = *reinterpret_cast<TopkRegSmem*>(smem_raw);
@@ -478,7 +483,7 @@ topk_select_solo_kernel(const float* __restrict__ scores, int64_t score_stride, 
   const int L = t.prompt_len[b];
   const int K = t.cu_keep[b + 1] - t.cu_keep[b];
   const float* x = scores + (int64_t)kvh * score_stride + t.cu_prompt[b];
-  int32_t* out = idx + (int64_t)kvh * idx_stride + t.cu_keep[b];
+  int32_t* out = index_list(idx, kvh, idx_stride) + t.cu_keep[b];
   const int base = tid * kKpt - lead(x);
   const int v0 = max(0, -base), nv = max(0, min(kKpt, L - base));
 
@@ -598,8 +603,8 @@ TopkShape plan_topk(int heads, int max_len, int n_sm, int max_lead) {
 
 }  // namespace
 
-cudaError_t launch_topk(const float* scores, int64_t score_stride, int32_t* idx, int64_t idx_stride,
-                        const SeqTable& t, int n_kv_heads, cudaStream_t s, LaunchLog* log) {
+cudaError_t launch_topk(const float* scores, int64_t score_stride, const IndexOut& idx, int64_t idx_stride,
+                        const SeqTable& t, int n_heads, cudaStream_t s, LaunchLog* log) {
   int max_len = 1;
   for (int b = 0; b < t.batch; ++b) max_len = t.prompt_len[b] > max_len ? t.prompt_len[b] : max_len;
   // (every head begins on a 16-byte boundary: nothing is lost in front of it)
@@ -609,10 +614,10 @@ cudaError_t launch_topk(const float* scores, int64_t score_stride, int32_t* idx,
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const TopkShape shape = plan_topk(t.batch * n_kv_heads, max_len, n_sm, aligned ? 0 : kMaxLead);
+  const TopkShape shape = plan_topk(t.batch * n_heads, max_len, n_sm, aligned ? 0 : kMaxLead);
   if (shape.n_cta > 0) {                                              // keys in registers: 4, 8, 16 or 32 per thread
     const int n_cta = shape.n_cta;
-    const dim3 grid(t.batch * n_cta, n_kv_heads), block(kTopkThreads);
+    const dim3 grid(t.batch * n_cta, n_heads), block(kTopkThreads);
     auto launch = [&](auto kernel) {
       cudaError_t le = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TopkRegSmem));
       if (le != cudaSuccess) return le;
@@ -637,9 +642,9 @@ cudaError_t launch_topk(const float* scores, int64_t score_stride, int32_t* idx,
     }
   }
   int n_cta = kCluster;
-  while (n_cta > 1 && t.batch * n_kv_heads * n_cta > kWaveCtas && (int64_t)(n_cta / 2) * 4 * kKeysPerCta >= max_len) n_cta /= 2;
+  while (n_cta > 1 && t.batch * n_heads * n_cta > kWaveCtas && (int64_t)(n_cta / 2) * 4 * kKeysPerCta >= max_len) n_cta /= 2;
   const int slice = (((max_len + n_cta - 1) / n_cta) + 31) & ~31;
-  const dim3 grid(t.batch * n_cta, n_kv_heads), block(kTopkThreads);
+  const dim3 grid(t.batch * n_cta, n_heads), block(kTopkThreads);
   const int cache_keys = slice <= kMaxSliceSmem ? slice : 0;          // 0: every pass re-reads global memory
   const size_t smem = sizeof(TopkSmem) + (size_t)cache_keys * sizeof(uint32_t);
   e = cudaFuncSetAttribute(topk_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
