@@ -35,6 +35,7 @@ struct dapq_ctx {
   long long wait_limit = 0;      // cycles a device-side wait may take (0: the default, about a second)
   int32_t* idx = nullptr;        // [H_kv, max_total_rows]
   int flow_layers = 1;           // layers of the full size that one launch may cover
+  int score_slots = 2;           // layers of the full size that `scores` has room for, that of `idx` included
   int64_t flow_chunks = 0;       // rows of `part` in the layout of score_flow.cu
   uint32_t* sync[2] = {};        // tickets and counters of its launches, used in turn
   int64_t sync_words = 0;
@@ -121,7 +122,8 @@ dapq_status cuda_fail(dapq_ctx* ctx, cudaError_t e, const char* what) {
   } while (0)
 
 constexpr double kFlowPairs = 6e8;             // query-key pairs of a launch of score_flow.cu that make its start and end small
-constexpr size_t kFlowPartBytes = 16u << 20;   // for its partial row sums
+constexpr int kFlowLongest = 65536;            // prompts of this length and more: a launch per sweep and layer
+constexpr size_t kFlowLeastPairs = 16;         // key pairs of a unit for which its partial row sums have room in any call
 
 // Device buffers allocated together: as one block, cut up at 256-byte boundaries, where a block of its own for each
 // would cost up to a millisecond apiece (large ones), or each by itself, where the driver has small blocks at hand.
@@ -395,9 +397,9 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
     // enough layers a launch for some 6e8 query-key pairs; small calls of a large context may take more
     const double layers = kFlowPairs / ((double)hq_n * rows);
     ctx->flow_layers = layers >= kFlowLayers ? kFlowLayers : (int)layers + 1;
-    const size_t chunk_elems = (size_t)sh->n_kv_heads * flow_rows_pad(ctx->dims);
-    const size_t extra = kFlowPartBytes / (chunk_elems * sizeof(float2));
-    const size_t want = (size_t)ctx->flow_layers * sh->max_batch + (extra < 640 ? extra : 640);
+    const size_t chunk_elems = (size_t)sh->n_kv_heads * flow_rows_pad(ctx->dims), nl_full = (size_t)ctx->flow_layers;
+    const size_t runs = nl_full * (rows / (256 * kFlowLeastPairs) + 1), few = 4 * (size_t)ctx->n_sm / ((size_t)sh->n_kv_heads * qg_groups(ctx->dims)) + 1;
+    const size_t want = nl_full * sh->max_batch + (runs > few ? runs : few);
     const size_t need = want * chunk_elems * 3 / 2;                // (a float2 and a float each)
     if (need > part_elems) part_elems = need;
     ctx->flow_chunks = (int64_t)(part_elems * 2 / 3 / chunk_elems);
@@ -412,13 +414,15 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
   ar.add(&ctx->q_rot, (size_t)sh->max_batch * hq_n * kHeadDim * (nl > 1 ? nl * sizeof(__half) : sizeof(float)));
   ar.add(&ctx->part, part_elems * sizeof(float2));
   ar.add(&ctx->lse2, (nl * sh->max_batch * hq_n + 32) * sizeof(float));
-  ar.add(&ctx->scores, nl * score_bytes);
-  ar.add(&ctx->idx, nl * sh->n_kv_heads * rows * sizeof(int32_t));
+  // (the indices have the last of the score slots, which launches whose caller takes the indices fill with scores too)
+  ctx->score_slots = nl > 2 ? (int)nl : 2;
+  ar.add(&ctx->scores, ctx->score_slots * score_bytes);
   if (sh->pool_mode != DAPQ_POOL_NONE) ar.add(&ctx->pooled, nl * score_bytes);
   if (n_slots > 1) ar.add(&ctx->slots, nl * n_slots * score_bytes);
   if (flow)
     for (auto& w : ctx->sync) ar.add(&w, ctx->sync_words * sizeof(uint32_t));
   bool ok = ar.allocate(ctx);
+  if (ok) ctx->idx = reinterpret_cast<int32_t*>(ctx->scores + (size_t)(ctx->score_slots - 1) * sh->n_kv_heads * rows);
   ok = ok && cudaMemcpy(ctx->inv_freq, freq, sizeof(freq), cudaMemcpyHostToDevice) == cudaSuccess;
   ok = ok && cudaMemset(ctx->status, 0, sizeof(int)) == cudaSuccess;
   if (!ok) { cudaGetLastError(); return bail(DAPQ_ERR_CUDA, "workspace allocation failed"); }
@@ -689,11 +693,18 @@ struct LayerSpans {
   }
 };
 
-// Layers of this geometry whose workspace fits the context's.
-int layers_that_fit(const dapq_ctx* ctx, const SeqTable& t) {
-  const int64_t rows = ctx->shape.max_total_rows * ctx->flow_layers / t.cu_prompt[t.batch];
-  const int64_t seqs = (int64_t)ctx->shape.max_batch * ctx->flow_layers / t.batch;
-  const int64_t n = rows < seqs ? rows : seqs;
+// Layers of this geometry that one launch may cover: their workspace fits the context's (own_idx: the indices take a part of
+// it too), and the prompts are so short that a launch per sweep and layer would cost much of their time.  Us a
+// layer, a launch per sweep -> one for several layers: 8 k tokens on 8 heads x 128 query rows 27.7 -> 10.5, x 1024 68.5 -> 48.9;
+// 30 k x 512 96 -> 83, x 1024 170 -> 155; 60 k x 128 72.7 -> 56.4, x 256 99 -> 85, x 1024 302 -> 303.
+int layers_that_fit(const dapq_ctx* ctx, const SeqTable& t, bool own_idx) {
+  for (int b = 0; b < t.batch; ++b)
+    if (t.prompt_len[b] >= kFlowLongest) return 1;
+  const int64_t room = ctx->shape.max_total_rows, seqs = (int64_t)ctx->shape.max_batch * ctx->flow_layers / t.batch;
+  const int slots = ctx->score_slots < ctx->flow_layers ? ctx->score_slots : ctx->flow_layers;
+  int64_t n = room * (own_idx && slots == ctx->score_slots ? slots - 1 : slots) / t.cu_prompt[t.batch];
+  if (own_idx && room / t.cu_keep[t.batch] < n) n = room / t.cu_keep[t.batch];
+  if (seqs < n) n = seqs;
   return n < 1 ? 1 : (n > kFlowLayers ? kFlowLayers : (int)n);
 }
 
@@ -836,7 +847,9 @@ dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const
     // touching another's outputs; in launches of equal size.  (A layer that is not in order says so when its own turn comes.)
     int n = 1;
     if (wants_flow(ctx)) {
-      const int fit = layers_that_fit(ctx, t), left = n_layers - l, launches = (left + fit - 1) / fit, most = (left + launches - 1) / launches;
+      bool own_idx = false;
+      for (int32_t m = l; m < n_layers && m < l + kFlowLayers; ++m) own_idx = own_idx || !idx_out || !idx_out[m];
+      const int fit = layers_that_fit(ctx, t, own_idx), left = n_layers - l, launches = (left + fit - 1) / fit, most = (left + launches - 1) / launches;
       LayerSpans spans[kFlowLayers];
       spans[0] = LayerSpans(ctx, y[0], t);
       for (; n < most && check(l + n, &y[n], &other) == DAPQ_OK && memcmp(&other, &t, sizeof(t)) == 0; ++n) {

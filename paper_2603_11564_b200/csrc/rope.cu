@@ -120,6 +120,94 @@ rope_pseudo_q_kernel(const __grid_constant__ RopeBatch rb, TO* __restrict__ q_ro
   if (late_wait) pdl_wait();
 }
 
+// The same for many queries (bf16 in, fp16 out): a warp per query head, a lane the channel pairs 2 l, 2 l + 1 of either half, so
+// that a row moves in four-byte pieces, and a block evaluates the angles of its kRowsQ queries once for all heads.  The next head's
+// rows are requested before this one's are computed.  Two layers of 40 prompts of 8 k, 32 heads, 32 queries: 37 -> 15 us.
+constexpr int kRowsQ = 4, kRowsWarps = 8;
+__global__ void __launch_bounds__(kRowsWarps * 32)
+rope_rows_kernel(const __grid_constant__ RopeBatch rb, __half2* __restrict__ q_rot, const double* __restrict__ inv_freq,
+                 const __grid_constant__ SeqTable t, int n_q_heads, int n_pseudo, int late_wait, int interleaved, double out_scale) {
+  if (!late_wait) pdl_wait();                                    // (as above)
+  pdl_trigger();
+  constexpr int half = kHeadDim / 2;
+  const int layer = blockIdx.y / t.batch, b = blockIdx.y - layer * t.batch, i0 = blockIdx.x * kRowsQ;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = min(kRowsQ, n_pseudo - i0);
+  for (int i = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < rb.n_clear; i += gridDim.x * gridDim.y * blockDim.x)
+    rb.clear[i] = 0u;
+  const __nv_bfloat162* q_pre = reinterpret_cast<const __nv_bfloat162*>(rb.q[layer]);
+  const __nv_bfloat162* key = reinterpret_cast<const __nv_bfloat162*>(rb.k[layer] + (int64_t)t.cu_rows[b] * rb.row_stride[layer]);
+  const int64_t key_step = rb.head_stride[layer] / 2;
+  const size_t in_seq = (size_t)b * n_q_heads, out_seq = (size_t)blockIdx.y * n_q_heads;
+  __nv_bfloat162 x[kRowsQ], y[kRowsQ], kx, ky;
+  auto load = [&](int h) {
+    const size_t row = ((in_seq + h) * n_pseudo + i0) * half;
+#pragma unroll
+    for (int u = 0; u < kRowsQ; ++u) {
+      const size_t at = row + (size_t)min(u, n - 1) * half + lane;
+      x[u] = q_pre[at];
+      y[u] = q_pre[at + half / 2];
+    }
+    kx = key[(h / rb.group) * key_step + lane];
+    ky = key[(h / rb.group) * key_step + half / 2 + lane];
+  };
+  if (warp < n_q_heads) load(warp);
+  __shared__ double2 angle[kRowsQ][half];
+  static_assert(kRowsQ * half == kRowsWarps * 32, "an angle per thread");
+  {
+    const int u = threadIdx.x / half, c = threadIdx.x % half;
+    double sn, cs;
+    sincos((double)(t.pos_start[b] + i0 + u) * inv_freq[c], &sn, &cs);
+    angle[u][c] = make_double2(sn, cs);
+  }
+  __syncthreads();
+  // the frequencies of a lane: pairs (c, c + d/2) of channels 2 l, 2 l + 1, or the pairs (2 l, 2 l + 1), (64 + 2 l, 65 + 2 l) themselves
+  const int c0 = interleaved ? lane : 2 * lane, c1 = interleaved ? half / 2 + lane : 2 * lane + 1;
+  for (int h = warp; h < n_q_heads; h += kRowsWarps) {
+    float2 xs[kRowsQ], ys[kRowsQ];
+#pragma unroll
+    for (int u = 0; u < kRowsQ; ++u) {
+      xs[u] = __bfloat1622float2(x[u]);
+      ys[u] = __bfloat1622float2(y[u]);
+    }
+    const float2 fx = __bfloat1622float2(kx), fy = __bfloat1622float2(ky);
+    if (h + kRowsWarps < n_q_heads) load(h + kRowsWarps);
+    const size_t row0 = (out_seq + h) * n_pseudo + i0;
+    float part[kRowsQ];
+#pragma unroll
+    for (int u = 0; u < kRowsQ; ++u) {
+      const double2 s0 = angle[u][c0], s1 = angle[u][c1];
+      // (lo, hi) of the two rotations
+      const double lo0 = xs[u].x, hi0 = interleaved ? xs[u].y : ys[u].x, lo1 = interleaved ? ys[u].x : xs[u].y, hi1 = ys[u].y;
+      const double r0 = (lo0 * s0.y - hi0 * s0.x) * out_scale, r1 = (hi0 * s0.y + lo0 * s0.x) * out_scale;
+      const double r2 = (lo1 * s1.y - hi1 * s1.x) * out_scale, r3 = (hi1 * s1.y + lo1 * s1.x) * out_scale;
+      // channels 2 l, 2 l + 1 of the first half, of the second
+      const double a0 = r0, a1 = interleaved ? r1 : r2, b0 = interleaved ? r2 : r1, b1 = r3;
+      part[u] = ((float)a0 * fx.x + (float)b0 * fy.x) + ((float)a1 * fx.y + (float)b1 * fy.y);
+      if (u < n) {
+        __half2* out = q_rot + (row0 + u) * half + lane;
+        out[0] = __halves2half2(from_double<__half>(a0), from_double<__half>(a1));
+        out[half / 2] = __halves2half2(from_double<__half>(b0), from_double<__half>(b1));
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < kRowsQ; ++u) part[u] += __shfl_xor_sync(0xffffffffu, part[u], o);
+    float mine = part[0];
+#pragma unroll
+    for (int u = 1; u < kRowsQ; ++u) mine = lane == u ? part[u] : mine;
+    if (lane < n) rb.ref[row0 + lane] = mine;
+  }
+  if (late_wait) pdl_wait();
+}
+
+// The queries may begin anywhere that an element may (the keys lie on 16-byte boundaries, like their strides).
+bool aligned4(const RopeBatch& rb) {
+  for (int l = 0; l < rb.n_layers; ++l)
+    if ((uintptr_t)rb.q[l] & 3u) return false;
+  return true;
+}
+
 }  // namespace
 
 cudaError_t launch_rope(int dtype, int out_mode, int64_t lo_offset, const RopeBatch& rb, void* q_rot, const double* inv_freq_dev,
@@ -139,6 +227,9 @@ cudaError_t launch_rope(int dtype, int out_mode, int64_t lo_offset, const RopeBa
   using bf16 = __nv_bfloat16;
   if (dtype == DAPQ_BF16 && out_mode == kRopeOutSplitBf16)
     run(rope_pseudo_q_kernel<bf16, bf16, true, 1>, rope_pseudo_q_kernel<bf16, bf16, true, 4>, (bf16*)q_rot, lo_offset, 1.0, false);
+  else if (dtype == DAPQ_BF16 && out_mode == kRopeOutF16 && many && rb.ref != nullptr && aligned4(rb))
+    launch_pdl(rope_rows_kernel, dim3((dm.n_pseudo + kRowsQ - 1) / kRowsQ, seqs), dim3(kRowsWarps * 32), 0, s, 1, rb, (__half2*)q_rot, inv_freq_dev, t,
+               dm.n_q_heads, dm.n_pseudo, lw, dm.rope_interleaved, (double)dm.scale_log2e);
   else if (dtype == DAPQ_BF16 && out_mode == kRopeOutF16)
     run(rope_pseudo_q_kernel<bf16, __half, false, 1>, rope_pseudo_q_kernel<bf16, __half, false, 4>, (__half*)q_rot, 0, (double)dm.scale_log2e, true);
   else if (dtype == DAPQ_BF16 && out_mode == kRopeOutBf16)

@@ -20,24 +20,24 @@ bool flow_plan(const void* q, const CacheDev* cv, int n_layers, const SeqTable& 
   plan->two = plan->rows_g > 128 ? 1 : 0;
   const int per_chunk = dm.n_kv_heads * plan->n_qgroups;
   int64_t pairs = 0;
-  int max_pairs = 0;
-  for (int b = 0; b < t.batch; ++b) {
-    const int p = (t.prompt_len[b] + dm.n_pseudo + kPair - 1) / kPair;
-    pairs += p;
-    max_pairs = p > max_pairs ? p : max_pairs;
-  }
+  for (int b = 0; b < t.batch; ++b) pairs += (t.prompt_len[b] + dm.n_pseudo + kPair - 1) / kPair;
   auto chunks = [&](int ct) {
     int64_t n = 0;
     for (int b = 0; b < t.batch; ++b) n += ((t.prompt_len[b] + dm.n_pseudo + kPair - 1) / kPair + ct - 1) / ct;
     return n;
   };
-  // Pairs of a unit: three to four units a CTA and sweep, and at most 16 pairs.
-  const double load = (double)n_layers * per_chunk * pairs / n_sm;
-  int ct = (int)(load / 3.5 + 0.5);
-  ct = ct < 3 ? 3 : (ct > 16 ? 16 : ct);
-  if (ct > max_pairs) ct = max_pairs;
-  while (ct < max_pairs && n_layers * chunks(ct) > max_chunks) ++ct;
-  if (n_layers * chunks(ct) > max_chunks) return false;
+  // Pairs of a unit: units go to the CTAs one by one, so a sweep takes about as many rounds of them as units / CTAs, rounded up,
+  // each of a unit's pairs and some half a pair of set-up.  Below four pairs the next unit's ticket, queries and
+  // log-sum-exps no longer hide behind this one.
+  int ct = 0;
+  double best = 0.0;
+  for (int c = 4; c <= 16; ++c) {
+    const int64_t n = n_layers * chunks(c), units = n * per_chunk;
+    if (n > max_chunks) continue;
+    const double cost = (double)((2 * units + n_sm - 1) / n_sm) * ((double)n_layers * per_chunk * pairs / units + 0.4);
+    if (ct == 0 || cost < best) { ct = c; best = cost; }
+  }
+  if (ct == 0) return false;
   plan->ct.chunk_tiles = ct;
   int32_t n = 0, most_chunks = 0;
   for (int b = 0; b < t.batch; ++b) {

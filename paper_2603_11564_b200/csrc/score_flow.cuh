@@ -142,15 +142,9 @@ __device__ __forceinline__ void make_unit(Unit& u, int x, const SeqTable& t, con
   u.item = ((u.layer * t.batch + u.b) * a.n_kv_heads + u.kvh) * a.n_qgroups + u.qgrp;
 }
 
-// 32 key columns of an accumulator row into the row's sum (RowSum, score_qg_sweep1.cuh).  lim: last visible column.
-template <bool kMasked>
-__device__ __forceinline__ void row_sum32(uint32_t* v, int col0, int lim, RowSum& st) {
-  float* x = reinterpret_cast<float*>(v);
-  if (kMasked) {
-#pragma unroll
-    for (int e = 0; e < 32; ++e)
-      if (col0 + e > lim) x[e] = -CUDART_INF_F;
-  }
+// 32 key columns of an accumulator row into the row's sum (RowSum, score_qg_sweep1.cuh).
+__device__ __forceinline__ void row_sum32(const uint32_t* v, RowSum& st) {
+  const float* x = reinterpret_cast<const float*>(v);
   if (st.m - st.r < 100.f) {
     float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
 #pragma unroll
@@ -184,6 +178,25 @@ __device__ __forceinline__ void row_sum32(uint32_t* v, int col0, int lim, RowSum
   }
 }
 
+__device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, long long limit) {
+  return mbar_wait_limit(bar, parity, abort_flag, status, limit);
+}
+struct Waiter {
+  volatile int* abort_flag;
+  int* status;
+  long long limit;
+  __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity) const {
+    return mbar_try(bar, parity) || wait_slow(bar, parity, abort_flag, status, limit);
+  }
+  __device__ __forceinline__ bool aborting() const { return *abort_flag != 0; }
+};
+
+__device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5}], [%2], %6;"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z), "l"(policy) : "memory");
+}
+
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -197,6 +210,13 @@ __device__ __forceinline__ uint32_t half_pair(float v) {
 }
 __device__ __forceinline__ float half_pair_value(uint32_t w) {
   return __half2float(__ushort_as_half((uint16_t)(w & 0xffffu))) + __half2float(__ushort_as_half((uint16_t)(w >> 16)));
+}
+
+__device__ __noinline__ float merge_row(const float2* part, int64_t step, int n) {
+  float2 s = make_float2(-CUDART_INF_F, 0.f);
+#pragma unroll 1
+  for (int c = 0; c < n; ++c) s = qg::merge_stats(s, __ldcg(part + c * step));
+  return s.x + log2f(s.y);
 }
 
 // Base-2 log-sum-exps of four neighbouring query rows from the sums of the item's n runs, in order; l holds the rows' references
@@ -220,11 +240,7 @@ __device__ __forceinline__ void merge_rows(const Args& a, int64_t at, int64_t st
     return;
   }
 #pragma unroll
-  for (int x = 0; x < 4; ++x) {
-    float2 s = make_float2(-CUDART_INF_F, 0.f);
-    for (int c = 0; c < n; ++c) s = qg::merge_stats(s, __ldcg(a.part + at + x + c * step));
-    l[x] = s.x + log2f(s.y);
-  }
+  for (int x = 0; x < 4; ++x) l[x] = merge_row(a.part + at + x, step, n);
 }
 
 constexpr int kMaxLayers = kFlowLayers;
@@ -264,7 +280,7 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
   tc_fence_after();
   pdl_wait();                                                    // (queries, references and cleared counters: the rotation's)
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + S::tmem_ptr);
-  const qg::Waiter wt{reinterpret_cast<volatile int*>(smem + S::abort_flag), a.status, a.wait_limit};
+  const Waiter wt{reinterpret_cast<volatile int*>(smem + S::abort_flag), a.status, a.wait_limit};
   // Unit n for a role of one thread, or of whole warps (lane 0 reports the read).
   auto next_unit = [&](int n, Unit& u, bool whole_warp) -> bool {
     const int at = n % kUnitRing;
@@ -280,10 +296,13 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
     // ================================================================================ keys, by TMA
     if (lane == 0) {
       int si = 0;                                                // sub-tiles issued
+      uint64_t last_use;
+      asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(last_use));
       bool ok = true;
       Unit u;
       for (int n = 0; ok && next_unit(n, u, false); ++n) {
         const CUtensorMap* map = &tm_k.m[u.layer];
+#pragma unroll 1
         for (int j = 0; j < 2 * u.n_pairs; ++j, ++si) {
           const int s = si & 3;
           if (si >= kSubs) ok = wt.wait(bar(S::k_empty + s), ((si >> 2) - 1) & 1);
@@ -291,8 +310,13 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
           const uint32_t dst = sbase + S::ring + (s >> 1) * kPairBytes + (s & 1) * kSubHalf;
           const int row = u.row_base + u.pair0 * kPair + j * kSub;
           mbar_expect_tx(bar(S::k_full + s), 2 * kSubHalf);
-          tma_load_3d(dst, map, bar(S::k_full + s), 0, row, u.kvh);
-          tma_load_3d(dst + kPairHalf, map, bar(S::k_full + s), 64, row, u.kvh);
+          if (u.kind == kSweep1) {
+            tma_load_3d(dst, map, bar(S::k_full + s), 0, row, u.kvh);
+            tma_load_3d(dst + kPairHalf, map, bar(S::k_full + s), 64, row, u.kvh);
+          } else {                                               // (nobody reads these keys again: L2 may drop them first)
+            tma_load_3d_hint(dst, map, bar(S::k_full + s), 0, row, u.kvh, last_use);
+            tma_load_3d_hint(dst + kPairHalf, map, bar(S::k_full + s), 64, row, u.kvh, last_use);
+          }
         }
       }
       // every copy issued lands before this thread, and with it the CTA, returns
@@ -312,6 +336,7 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
         if (ok && u.new_q) ok = wt.wait(bar(S::q_full), q_loads++ & 1);
         const int mb = kTwo ? (u.rows + 127) / 128 : 1, ncols = (u.rows + 15) & ~15;
         const uint32_t id1 = umma_idesc_f16(128, kPair), id2 = umma_idesc_f16(128, ncols);
+#pragma unroll 1
         for (int p = 0; p < u.n_pairs && ok; ++p) {
           // (the next ticket is drawn when four pairs are left: late enough for a short launch's first units to go round the
           // CTAs, early enough for the next unit's keys and log-sum-exps)
@@ -321,6 +346,7 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
           const uint32_t ph = (si >> 2) & 1;
           if (u.kind == kSweep1) {
             ok = wt.wait(bar(S::k_conv + s), ph) && wt.wait(bar(S::k_conv + s + 1), ph);
+#pragma unroll 1
             for (int m = 0; m < mb && ok; ++m, ++job) {
               if (!(ok = acc_free())) break;
               tc_fence_after();
@@ -337,6 +363,7 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
             tc_commit(bar(S::k_empty + s));
             tc_commit(bar(S::k_empty + s + 1));
           } else {
+#pragma unroll 1
             for (int j = 0; j < 2 && ok; ++j) {
               ok = wt.wait(bar(S::k_conv + s + j), ph);
               if (ok && (kTwo || j == 0)) ok = acc_free();
@@ -377,13 +404,13 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
         if (!__all_sync(0xffffffffu, wt.wait(bar(S::k_full + s), (si >> 2) & 1))) { ok = false; break; }
         // this warp: 64 channels of 64 keys
         const uint32_t p0 = sbase + S::ring + (s >> 1) * kPairBytes + (s & 1) * kSubHalf + (cw >> 1) * kPairHalf + (cw & 1) * (kSubHalf / 2) + lane * 16;
+#pragma unroll 1
+        for (int it = 0; it < 16; it += 8) {
+          uint4 v[8];
 #pragma unroll
-        for (int it = 0; it < 16; it += 4) {
-          uint4 v[4];
+          for (int x = 0; x < 8; ++x) v[x] = lds128(p0 + (it + x) * 512);
 #pragma unroll
-          for (int x = 0; x < 4; ++x) v[x] = lds128(p0 + (it + x) * 512);
-#pragma unroll
-          for (int x = 0; x < 4; ++x) {
+          for (int x = 0; x < 8; ++x) {
             v[x].x = qg::bf16x2_to_f16x2(v[x].x);
             v[x].y = qg::bf16x2_to_f16x2(v[x].y);
             v[x].z = qg::bf16x2_to_f16x2(v[x].z);
@@ -417,44 +444,56 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
       if (!ok) break;
       if (u.kind == kSweep1) {
         const int mb = kTwo ? (u.rows + 127) / 128 : 1;
-        RowSum rs0, rs1;
+        // (the row of query block 0 and, kTwo, that of block 1: they change places after every job, so that there is one body)
+        RowSum now, other;
         auto reference = [&](int row) {                          // as the MMAs see it
           return -half_pair_value(*reinterpret_cast<const volatile uint32_t*>(smem + S::slab + (n & 1) * S::slab_bytes + (row >> 3) * 256 + (row & 7) * 32));
         };
-        rs0.init(reference(r));
-        rs1.init(kTwo ? reference(128 + r) : 0.f);
+        now.init(reference(r));
+        other.init(kTwo ? reference(128 + r) : 0.f);
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(S::slab_empty + (n & 1)));
-        const int i0 = (u.qgrp * a.rows_g + r) % a.n_pseudo, i1 = (u.qgrp * a.rows_g + 128 + r) % a.n_pseudo;
-        for (int p = 0; p < u.n_pairs && ok; ++p) {
-          const int base = (u.pair0 + p) * kPair;
-          const bool masked = base + kPair > u.L;                // holds synthetic (or foreign) rows
-          auto one = [&](RowSum& rs, int i) {
-            const int b = job & 1;
-            if (!take_job(b)) { ok = false; return; }
-            tc_fence_after();
-            const int lim = u.L + i - base;
+        int i_now = (u.qgrp * a.rows_g + r) % a.n_pseudo, i_other = (u.qgrp * a.rows_g + 128 + r) % a.n_pseudo;
+        auto change = [&] {
+          const RowSum x = now;
+          now = other;
+          other = x;
+          const int i = i_now;
+          i_now = i_other;
+          i_other = i;
+        };
+        int base = u.pair0 * kPair;
+#pragma unroll 1
+        for (int j = 0; j < u.n_pairs * mb; ++j, ++job) {
+          const int b = job & 1;
+          if (!(ok = take_job(b))) break;
+          tc_fence_after();
+          const uint32_t taddr = lane_addr + b * 256 + eg * 64;
+#pragma unroll 1
+          for (int h = 0; h < 2; ++h) {
+            uint32_t v[32];
+            tmem_ld32(taddr + h * 32, v);
+            tmem_ld_wait_for(v);
+            if (h == 1) release(b);
+            if (base + kPair > u.L) {                            // holds synthetic (or foreign) rows
+              const int last = u.L + i_now - base - eg * 64 - h * 32;   // visible columns: up to this one
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              uint32_t v[32];
-              const int col = eg * 64 + h * 32;
-              tmem_ld32(lane_addr + b * 256 + col, v);
-              tmem_ld_wait_for(v);
-              if (h == 1) release(b);
-              if (masked) row_sum32<true>(v, col, lim, rs);
-              else row_sum32<false>(v, col, lim, rs);
+              for (int e = 0; e < 32; ++e)
+                if (e > last) v[e] = 0xff800000u;                // -inf
             }
-            ++job;
-          };
-          one(rs0, i0);
-          if (kTwo && mb == 2 && ok) one(rs1, i1);
+            row_sum32(v, now);
+          }
+          if (kTwo && mb == 2) change();
+          if (!kTwo || mb == 1 || (j & 1)) base += kPair;
         }
         // the four groups' sums of the same rows over different keys, 64 rows to a post; negative: not relative to the reference
+#pragma unroll 1
         for (int h = 0; h < 2 * mb && ok; ++h, ++post) {
           if (!(ok = slot_free())) break;
           if ((quad >> 1) == (h & 1)) {
-            const RowSum& rs = kTwo && h >= 2 ? rs1 : rs0;
-            reinterpret_cast<float2*>(exch + (post & 3) * 512)[eg * 64 + (r & 63)] = make_float2(rs.m, rs.m == rs.r ? rs.z : -rs.z);
+            const bool second = kTwo && h >= 2;
+            const float m = second ? other.m : now.m, z = second ? other.z : now.z, ref = second ? other.r : now.r;
+            reinterpret_cast<float2*>(exch + (post & 3) * 512)[eg * 64 + (r & 63)] = make_float2(m, m == ref ? z : -z);
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(bar(S::part_full + (post & 3)));
@@ -465,16 +504,34 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
         const int nch = (u.rows + 15) >> 4;
         const int part = kTwo ? eg : (eg & 1), parts = kTwo ? 4 : 2;
         const int p0 = (part * nch) / parts, np = ((part + 1) * nch) / parts - p0;
-        const bool full = (p0 + np) * 16 <= u.rows;
-        const uint32_t col_addr = lane_addr + (kTwo ? 0 : (eg >> 1) * 128);
+        const uint32_t col_addr = lane_addr + (kTwo ? 0 : (eg >> 1) * 128) + p0 * 16;
+        const int cols = min(np * 16, u.rows - p0 * 16);         // this thread's columns
+#pragma unroll 1
         for (int j = 0; j < (kTwo ? 2 : 1) * u.n_pairs; ++j, ++job, ++post) {
           const int b = job & 1;
           if (!(ok = take_job(b))) break;
           tc_fence_after();
-          const float sum = full ? qg::colsum_job<true, true>(col_addr + b * 256, nullptr, p0, np, u.rows, 1.f, [&] { release(b); })
-                                 : qg::colsum_job<false, true>(col_addr + b * 256, nullptr, p0, np, u.rows, 1.f, [&] { release(b); });
+          float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+          if (np == 0) release(b);
+#pragma unroll 1
+          for (int c = 0; c < cols; c += 32) {
+            uint32_t v[32];
+            tmem_ld16(col_addr + b * 256 + c, v);
+            if (c + 16 < np * 16) tmem_ld16(col_addr + b * 256 + c + 16, v + 16);
+            tmem_ld_wait_for(v);
+            if (c + 32 >= cols) {
+              release(b);
+              if (c + 32 > cols) {
+#pragma unroll
+                for (int e = 0; e < 32; ++e)
+                  if (c + e >= cols) v[e] = 0xff800000u;
+              }
+            }
+            qg::colsum_piece<true, true>(v, nullptr, 16, 1.f, acc0, acc1);
+            if (c + 16 < cols) qg::colsum_piece<true, true>(v + 16, nullptr, 16, 1.f, acc0, acc1);
+          }
           if (!(ok = slot_free())) break;
-          exch[(post & 3) * 512 + eg * 128 + r] = sum;
+          exch[(post & 3) * 512 + eg * 128 + r] = (acc0.x + acc0.y) + (acc1.x + acc1.y);
           __syncwarp();
           if (lane == 0) mbar_arrive(bar(S::part_full + (post & 3)));
         }
@@ -498,7 +555,7 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
         for (int h = 0; h < 2 * mb; ++h, ++post) {
           if (!(ok = take())) break;
           const float2* e = reinterpret_cast<const float2*>(exch + (post & 3) * 512);
-#pragma unroll
+#pragma unroll 1
           for (int x = 0; x < 2; ++x) {
             const int row = x * 32 + lane;
             // (a fixed order: the result does not depend on timing)
