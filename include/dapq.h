@@ -241,14 +241,14 @@ DAPQ_API dapq_status dapq_evict(dapq_ctx* ctx, const void* q_pre, const dapq_cac
  * q_pre, caches, k_out, v_out, idx_out: HOST arrays of n_layers entries holding what dapq_evict
  * takes for one layer (idx_out, or any entry of it, may be NULL).  k_keep_host: host
  * [n_layers, batch] when k_keep_layer_stride = batch, or one row shared by all layers when
- * k_keep_layer_stride = 0.  Every layer uses the same workspace, so the layers run back to back;
- * only launches are issued (no copies, no synchronisation), which makes the whole call
+ * k_keep_layer_stride = 0.  Layers of the same lengths and budgets whose arrays do not overlap share launches, up to eight at a
+ * time; otherwise the layers run back to back; only launches are issued (no copies, no synchronisation), which makes the whole call
  * capturable into a CUDA graph.  Stops at the first layer that fails and returns its status.
  * Calls of 8 layers and more on long prompts, without pooling and with budgets that are small against the prompts, compute
  * the scores of those keys only that can be among the K largest, in layers where the layers before show that it
  * pays.  The sets are those of dapq_evict up to keys whose scores agree with the K-th to rounding (1e-5 of it), as are the
- * sets of two scorings whose log-sum-exps are summed in different orders; calls of fewer layers select dapq_evict's own,
- * bit for bit. */
+ * sets of two scorings whose log-sum-exps are summed in different orders; so are those of layers that share launches.  Layers
+ * that do neither select dapq_evict's own, bit for bit. */
 DAPQ_API dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const* q_pre,
                               const dapq_cache_view* caches, const int32_t* k_keep_host,
                               int64_t k_keep_layer_stride, void* const* k_out, void* const* v_out,

@@ -122,7 +122,6 @@ dapq_status cuda_fail(dapq_ctx* ctx, cudaError_t e, const char* what) {
   } while (0)
 
 constexpr double kFlowPairs = 6e8;             // query-key pairs of a launch of score_flow.cu that make its start and end small
-constexpr int kFlowLongest = 65536;            // prompts of this length and more: a launch per sweep and layer
 constexpr size_t kFlowLeastPairs = 16;         // key pairs of a unit for which its partial row sums have room in any call
 
 // Device buffers allocated together: as one block, cut up at 256-byte boundaries, where a block of its own for each
@@ -694,12 +693,14 @@ struct LayerSpans {
 };
 
 // Layers of this geometry that one launch may cover: their workspace fits the context's (own_idx: the indices take a part of
-// it too), and the prompts are so short that a launch per sweep and layer would cost much of their time.  Us a
-// layer, a launch per sweep -> one for several layers: 8 k tokens on 8 heads x 128 query rows 27.7 -> 10.5, x 1024 68.5 -> 48.9;
-// 30 k x 512 96 -> 83, x 1024 170 -> 155; 60 k x 128 72.7 -> 56.4, x 256 99 -> 85, x 1024 302 -> 303.
+// it too).  Us a layer, a launch per sweep -> one for several layers: 8 k tokens on 8 heads x 128 query rows 27.7 -> 10.5,
+// x 1024 68.5 -> 48.9; 30 k x 512 96 -> 83, x 1024 170 -> 155; 60 k x 128 72.7 -> 56.4, x 256 99 -> 85, x 1024 302 -> 303; 100 k x 128
+// 106 -> 92, x 256 147 -> 147, x 512 262 -> 268.  So layers of long prompts and the size from which the pruned selection
+// pays go by themselves; there a sweep is long enough.
 int layers_that_fit(const dapq_ctx* ctx, const SeqTable& t, bool own_idx) {
-  for (int b = 0; b < t.batch; ++b)
-    if (t.prompt_len[b] >= kFlowLongest) return 1;
+  int longest = 0;
+  for (int b = 0; b < t.batch; ++b) longest = t.prompt_len[b] > longest ? t.prompt_len[b] : longest;
+  if (longest >= kPruneLeastLen && (double)t.cu_prompt[t.batch] * ctx->dims.n_q_heads * ctx->dims.n_pseudo >= kPruneLeastPairs) return 1;
   const int64_t room = ctx->shape.max_total_rows, seqs = (int64_t)ctx->shape.max_batch * ctx->flow_layers / t.batch;
   const int slots = ctx->score_slots < ctx->flow_layers ? ctx->score_slots : ctx->flow_layers;
   int64_t n = room * (own_idx && slots == ctx->score_slots ? slots - 1 : slots) / t.cu_prompt[t.batch];

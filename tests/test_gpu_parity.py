@@ -1330,3 +1330,104 @@ def test_current_stream_with_and_without_the_short_way(dq, monkeypatch):
         with torch.cuda.stream(s):
             assert binding._stream(None) == s.cuda_stream
         assert binding._stream(s) == s.cuda_stream
+
+
+# ------------------------------------------------------------------------------- layers that share launches
+SHARED_CASES = [
+    # H_q, H_kv, N, lengths, budgets, layers: edges of 128- and 256-key tiles, query blocks of 64 .. 1024 rows of 16 and of none,
+    # one run a head and many, more layers than a launch takes, more units than CTAs
+    (4, 2, 32, (1,), (1,), 2), (8, 2, 25, (255, 256, 257), (9, 256, 30), 3), (8, 2, 32, (127, 129, 513), (20, 1, 500), 9),
+    (4, 1, 33, (767, 224), (50, 60), 2), (14, 2, 32, (1025, 3), (100, 2), 11), (10, 2, 52, (2049,), (64,), 2),
+    (16, 2, 128, (1500, 4100), (200, 41), 3), (7, 1, 100, (9001,), (333,), 5), (32, 8, 32, (12001, 700, 5003), (600, 35, 250), 8),
+    (32, 8, 64, (30000,), (900,), 3),
+]
+
+
+def _layers(dq, hq, hkv, n, lens, keep, layers, keys="plain"):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(hq * 1000 + n + layers)
+    w = _small(lens=lens, keep=keep, n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0)
+    ctx = _ctx(dq, w)
+    qs, ks, vs = [], [], []
+    for _ in range(layers):
+        qs.append(torch.randn((w.batch, hq, n, 128), generator=g, device="cuda").bfloat16())
+        k = torch.randn((hkv, w.total_rows, 128), generator=g, device="cuda")
+        _prune_keys(dq, ctx, keys, qs[-1], k, lens, hkv, g)
+        ks.append(k.bfloat16())
+        vs.append(torch.randn(k.shape, generator=g, device="cuda", dtype=torch.bfloat16))
+    KT = int(w.cu_keep[-1])
+    idx = [torch.full((hkv, KT), -1, dtype=torch.int32, device="cuda") for _ in range(layers)]
+    ko, vo = ([torch.zeros((hkv, KT, 128), dtype=torch.bfloat16, device="cuda") for _ in range(layers)] for _ in range(2))
+    return w, ctx, qs, ks, vs, idx, ko, vo
+
+
+def _one_by_one(dq, ctx, w, q, k, v):
+    KT = int(w.cu_keep[-1])
+    idx = torch.full((w.n_kv_heads, KT), -1, dtype=torch.int32, device="cuda")
+    ko, vo = (torch.zeros((w.n_kv_heads, KT, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    scores = torch.empty((w.n_kv_heads, w.total_prompt), dtype=torch.float32, device="cuda")
+    dq.dapq_evict(ctx, q, k, v, w.cu_rows, list(w.prompt_lens), list(w.keep), ko, vo, idx, scores)
+    return idx, scores
+
+
+@pytest.mark.parametrize("keys", ["plain", "far", "wide"])
+@pytest.mark.parametrize("hq,hkv,n,lens,keep,layers", SHARED_CASES)
+def test_layers_that_share_launches(dq, hq, hkv, n, lens, keep, layers, keys):
+    """Layers of different data scored in one launch against dapq_evict of each (two scorings of the same logits, whose
+    log-sum-exps are summed in another order: the tolerance of _same_set).  Twice: the counters start from 0 again."""
+    w, ctx, qs, ks, vs, idx, ko, vo = _layers(dq, hq, hkv, n, lens, keep, layers, keys)
+    before = dq.dapq_launch_count(ctx)
+    alone = [_one_by_one(dq, ctx, w, *x) for x in zip(qs, ks, vs)]
+    n_alone = dq.dapq_launch_count(ctx) - before
+    for _ in range(2):
+        before = dq.dapq_launch_count(ctx)
+        dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(keep), ko, vo, idx)
+        dq.dapq_poll_status(ctx)
+        assert dq.dapq_launch_count(ctx) - before < n_alone
+        for l in range(layers):
+            _same_set(alone[l][0], idx[l], alone[l][1], ks[l], vs[l], ko[l], vo[l], lens, w.cu_rows, w.cu_keep, w.cu_prompt)
+            ko[l].zero_(), vo[l].zero_(), idx[l].fill_(-1)
+    dq.dapq_destroy(ctx)
+
+
+def test_layers_whose_arrays_overlap_keep_their_order(dq):
+    """Outputs of one layer that are another's outputs or inputs: as if the layers ran one after the other.  And without index
+    arrays, or with some."""
+    hq, hkv, n, lens, keep, layers = 8, 2, 32, (600, 300), (64, 30), 5
+    w, ctx, qs, ks, vs, idx, ko, vo = _layers(dq, hq, hkv, n, lens, keep, layers)
+    KT = int(w.cu_keep[-1])
+    alone = [_one_by_one(dq, ctx, w, *x) for x in zip(qs, ks, vs)]
+    dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(keep), [ko[0]] * layers, [vo[0]] * layers, [idx[0]] * layers)
+    dq.dapq_poll_status(ctx)
+    _same_set(alone[-1][0], idx[0], alone[-1][1], ks[-1], vs[-1], ko[0], vo[0], lens, w.cu_rows, w.cu_keep, w.cu_prompt)
+    # layer 3 reads what layers 1 and 2 leave at the start of its keys and values
+    dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(keep), ko, vo)
+    dq.dapq_poll_status(ctx)
+    k3, v3 = ks[3].clone(), vs[3].clone()
+    k3.view(-1)[:hkv * KT * 128] = ko[1].view(-1)
+    v3.view(-1)[:hkv * KT * 128] = vo[2].view(-1)
+    want, scores = _one_by_one(dq, ctx, w, qs[3], k3, v3)
+    chained_k, chained_v = list(ko), list(vo)
+    chained_k[1], chained_v[2] = (x.view(-1)[:hkv * KT * 128].view(hkv, KT, 128) for x in (ks[3], vs[3]))
+    dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(keep), chained_k, chained_v, idx)
+    dq.dapq_poll_status(ctx)
+    _same_set(want, idx[3], scores, k3, v3, ko[3], vo[3], lens, w.cu_rows, w.cu_keep, w.cu_prompt)
+    dq.dapq_destroy(ctx)
+
+
+def test_layers_that_share_launches_wait_limit(dq):
+    """A wait that runs out in the shared launch: reported once, and the next call is right again."""
+    hq, hkv, n, lens, keep, layers = 8, 2, 32, (3000, 900), (64, 30), 4
+    w, ctx, qs, ks, vs, idx, ko, vo = _layers(dq, hq, hkv, n, lens, keep, layers)
+    alone = [_one_by_one(dq, ctx, w, *x) for x in zip(qs, ks, vs)]
+    dq.dapq_set_wait_limit(ctx, 1)
+    dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(keep), ko, vo, idx)
+    with pytest.raises(dq.DapqError) as e:
+        dq.dapq_poll_status(ctx)
+    assert e.value.status == dq.DAPQ_ERR_TIMEOUT
+    dq.dapq_set_wait_limit(ctx, 0)
+    dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(keep), ko, vo, idx)
+    dq.dapq_poll_status(ctx)
+    for l in range(layers):
+        _same_set(alone[l][0], idx[l], alone[l][1], ks[l], vs[l], ko[l], vo[l], lens, w.cu_rows, w.cu_keep, w.cu_prompt)
+    dq.dapq_destroy(ctx)
