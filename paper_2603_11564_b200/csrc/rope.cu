@@ -53,7 +53,7 @@ rope_pseudo_q_kernel(const __grid_constant__ RopeBatch rb, TO* __restrict__ q_ro
   // its wait.)
   if (!late_wait) pdl_wait();
   pdl_trigger();
-  const int layer = blockIdx.y / t.batch, b = blockIdx.y - layer * t.batch;
+  const int layer = rb.n_layers == 1 ? 0 : blockIdx.y / t.batch, b = blockIdx.y - layer * t.batch;
   const int i0 = blockIdx.x * kQ, c = threadIdx.x;
   // (the counters of the scorer behind this kernel; their last user completed before the kernel before this one could begin)
   for (int i = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * blockDim.x * blockDim.y + threadIdx.y * blockDim.x + c;

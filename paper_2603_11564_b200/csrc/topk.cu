@@ -49,7 +49,7 @@ constexpr int kMaxLead = 3;
 __device__ __forceinline__ int lead(const float* x) { return (int)((reinterpret_cast<uintptr_t>(x) & 15u) >> 2); }
 
 __device__ __forceinline__ int32_t* index_list(const IndexOut& idx, int head, int64_t stride) {
-  const int layer = head / idx.heads_per_layer;
+  const int layer = head < idx.heads_per_layer ? 0 : head / idx.heads_per_layer;
   return idx.p[layer] + (int64_t)(head - layer * idx.heads_per_layer) * stride;
 }
 
@@ -174,7 +174,7 @@ topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, const
   const int L = t.prompt_len[b];
   const int K = t.cu_keep[b + 1] - t.cu_keep[b];
   const float* x = scores + (int64_t)kvh * score_stride + t.cu_prompt[b];
-  int32_t* out = index_list(idx, kvh, idx_stride) + t.cu_keep[b];
+  auto list = [&] { return index_list(idx, kvh, idx_stride) + t.cu_keep[b]; };   // (formed where it is used: no registers until then)
 
   // slice of this CTA: [j0, j1), a multiple of 32 keys long so that warps stay converged
   const int slice = (((L + n_cta - 1) / n_cta) + 31) & ~31;
@@ -182,6 +182,7 @@ topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, const
   const int n_own = j1 - j0;
 
   if (K >= L) {                      // keep everything (uniform over the cluster: no barrier is skipped by a part of it)
+    int32_t* out = list();
     for (int j = j0 + tid; j < j1; j += kTopkThreads) out[j] = j;
     return;
   }
@@ -258,6 +259,7 @@ topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, const
   for (int w = 0; w < warp; ++w) { gt_before += tb.cnt_gt[w]; eq_before += tb.cnt_eq[w]; }
   uint32_t pos = gt_before + min(eq_before, n_ties);
   const uint32_t lt_mask = (1u << lane) - 1u;
+  int32_t* out = list();
   for (int j = s0 + lane; j < s0 + span; j += 32) {
     const uint32_t key = (j < s1) ? (cached ? keys[j] : order_key(x[j0 + j])) : 0u;
     const bool gt = j < s1 && key > thr;
@@ -298,7 +300,7 @@ topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, c
   const int L = t.prompt_len[b];
   const int K = t.cu_keep[b + 1] - t.cu_keep[b];
   const float* x = scores + (int64_t)kvh * score_stride + t.cu_prompt[b];
-  int32_t* out = index_list(idx, kvh, idx_stride) + t.cu_keep[b];
+  auto list = [&] { return index_list(idx, kvh, idx_stride) + t.cu_keep[b]; };   // (formed where it is used: no registers until then)
   const int base = (rank * kTopkThreads + tid) * kKpt - lead(x);   // position of this thread's first key
   const int v0 = max(0, -base), nv = max(0, min(kKpt, L - base));  // its keys v0 .. nv - 1 exist
 
@@ -312,6 +314,7 @@ topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, c
 
   if (K >= L) {                      // keep everything (uniform over the cluster)
     cluster_wait();
+    int32_t* out = list();
     for (int e = v0; e < nv; ++e) out[base + e] = base + e;
     return;
   }
@@ -457,6 +460,7 @@ topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, c
   gt_before += before & 0xffffu;
   eq_before += before >> 16;
   uint32_t pos = gt_before + min(eq_before, n_ties);
+  int32_t* out = list();
 #pragma unroll
   for (int e = 0; e < kKpt; ++e) {
     if (e >= v0 && e < nv) {
@@ -483,7 +487,7 @@ topk_select_solo_kernel(const float* __restrict__ scores, int64_t score_stride, 
   const int L = t.prompt_len[b];
   const int K = t.cu_keep[b + 1] - t.cu_keep[b];
   const float* x = scores + (int64_t)kvh * score_stride + t.cu_prompt[b];
-  int32_t* out = index_list(idx, kvh, idx_stride) + t.cu_keep[b];
+  auto list = [&] { return index_list(idx, kvh, idx_stride) + t.cu_keep[b]; };   // (formed where it is used: no registers until then)
   const int base = tid * kKpt - lead(x);
   const int v0 = max(0, -base), nv = max(0, min(kKpt, L - base));
 
@@ -493,6 +497,7 @@ topk_select_solo_kernel(const float* __restrict__ scores, int64_t score_stride, 
   pdl_wait();                        // the scores are written, and the index buffer's last reader is done
 
   if (K >= L) {
+    int32_t* out = list();
     for (int e = v0; e < nv; ++e) out[base + e] = base + e;
     return;
   }
@@ -562,6 +567,7 @@ topk_select_solo_kernel(const float* __restrict__ scores, int64_t score_stride, 
   const uint32_t before = packed_prefix(tb, mine, lane, warp, &total);
   uint32_t eq_before = before >> 16;
   uint32_t pos = (before & 0xffffu) + min(eq_before, n_ties);
+  int32_t* out = list();
 #pragma unroll
   for (int e = 0; e < kKpt; ++e) {
     if (e >= v0 && e < nv) {
