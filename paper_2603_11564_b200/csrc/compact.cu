@@ -13,19 +13,23 @@ constexpr int kRowsPerThread = 2;
 
 // One thread moves piece `piece` of kRowsPerThread kept rows, of K and of V: four independent 16-byte loads in
 // flight per thread (the gather is bound by how many bytes the SMs keep in flight, not by instructions).
-template <int kPieces>   // 16-byte pieces per row
+// Batch: CompactLayer for one layer, CompactBatch for several (blockIdx.z).
+__device__ __forceinline__ const CompactLayer& layer_of(const CompactLayer& one) { return one; }
+__device__ __forceinline__ const CompactLayer& layer_of(const CompactBatch& cb) { return cb.l[blockIdx.z]; }
+template <int kPieces, class Batch>   // 16-byte pieces per row
 __global__ void __launch_bounds__(kCompactThreads)
-compact_kv_kernel(const __grid_constant__ CompactBatch cb, int elem_bytes, int64_t idx_stride, const __grid_constant__ SeqTable t,
+compact_kv_kernel(const __grid_constant__ Batch batch, int elem_bytes, int64_t idx_stride, const __grid_constant__ SeqTable t,
                   int* __restrict__ status) {
   pdl_trigger();                     // whatever follows may be set up (or, if it does not depend on this copy, run) beside it
   const int kt = t.cu_keep[t.batch];
   const int64_t gid = (int64_t)blockIdx.x * kCompactThreads + threadIdx.x;
   const int r0 = (int)(gid / kPieces) * kRowsPerThread, piece = (int)(gid % kPieces);
   const int kvh = blockIdx.y;
-  const CacheDev& cv = cb.l[blockIdx.z].cv;
-  const int32_t* __restrict__ idx = cb.l[blockIdx.z].idx;
-  uint4* __restrict__ k_out = reinterpret_cast<uint4*>(cb.l[blockIdx.z].k_out);
-  uint4* __restrict__ v_out = reinterpret_cast<uint4*>(cb.l[blockIdx.z].v_out);
+  const CompactLayer& y = layer_of(batch);
+  const CacheDev& cv = y.cv;
+  const int32_t* __restrict__ idx = y.idx;
+  uint4* __restrict__ k_out = reinterpret_cast<uint4*>(y.k_out);
+  uint4* __restrict__ v_out = reinterpret_cast<uint4*>(y.v_out);
   int seg[kRowsPerThread];
 #pragma unroll
   for (int i = 0; i < kRowsPerThread; ++i) seg[i] = r0 + i < kt ? find_segment(t.cu_keep, t.batch, r0 + i) : 0;
@@ -65,13 +69,14 @@ cudaError_t launch_compact(int dtype, const CompactBatch& cb, int n_layers, int6
                            cudaStream_t s, LaunchLog* log) {
   log->begin(kKindCompact, s);
   const int kt = t.cu_keep[t.batch], threads = (kt + kRowsPerThread - 1) / kRowsPerThread;   // (per piece of a row)
-  auto run = [&](auto kernel, int pieces, int elem_bytes) {
+  auto run = [&](auto kernel, const auto& batch, int pieces, int elem_bytes) {
     const dim3 grid((unsigned)(((int64_t)threads * pieces + kCompactThreads - 1) / kCompactThreads), n_kv_heads, n_layers);
-    launch_pdl(kernel, grid, dim3(kCompactThreads), 0, s, 1, cb, elem_bytes, idx_stride, t, status);
+    launch_pdl(kernel, grid, dim3(kCompactThreads), 0, s, 1, batch, elem_bytes, idx_stride, t, status);
   };
   constexpr int P16 = kHeadDim * 2 / 16, P32 = kHeadDim * 4 / 16;
-  if (dtype == DAPQ_BF16) run(compact_kv_kernel<P16>, P16, 2);
-  else run(compact_kv_kernel<P32>, P32, 4);
+  if (dtype == DAPQ_BF16 && n_layers > 1) run(compact_kv_kernel<P16, CompactBatch>, cb, P16, 2);
+  else if (dtype == DAPQ_BF16) run(compact_kv_kernel<P16, CompactLayer>, cb.l[0], P16, 2);
+  else run(compact_kv_kernel<P32, CompactLayer>, cb.l[0], P32, 4);   // (fp32 layers go by themselves)
   log->end(s);
   return cudaGetLastError();
 }

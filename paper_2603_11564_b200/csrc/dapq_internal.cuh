@@ -127,15 +127,17 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 constexpr int kFlowLayers = 8;
 // q_rot: [layers][B, H_q, N, d].  ref (fp16 output mode only, may be NULL): where to write, per rotated query, its base-2
 // logit against the first key of its sequence in the layer's bf16 key cache (see rope.cu).  clear: words set to 0.
-struct RopeBatch {
-  const void* q[kFlowLayers];
-  const __nv_bfloat16* k[kFlowLayers];
-  int64_t head_stride[kFlowLayers], row_stride[kFlowLayers];   // of k, elements
+template <int kLayers>
+struct RopeLayers {
+  const void* q[kLayers];
+  const __nv_bfloat16* k[kLayers];
+  int64_t head_stride[kLayers], row_stride[kLayers];           // of k, elements
   int32_t n_layers, group;
   float* ref;                                                  // [layers][B, H_q, N]
   uint32_t* clear;
   int32_t n_clear;
 };
+using RopeBatch = RopeLayers<kFlowLayers>;
 cudaError_t launch_rope(int dtype, int out_mode, int64_t lo_offset, const RopeBatch& rb, void* q_rot, const double* inv_freq_dev,
                         const SeqTable& t, const Dims& dm, bool late_wait, cudaStream_t s, LaunchLog* log);
 

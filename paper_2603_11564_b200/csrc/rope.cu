@@ -39,9 +39,10 @@ template <> __device__ __forceinline__ __half from_double<__half>(double x) {
 // sequence, ref[layer, b, h, i] = out_scale * q_rot . K[h / G, cu_rows[b], :]: the first sweep of the
 // tensor-core scorer measures every other logit of the row against it.
 // kQ: consecutive pseudo queries per block.
-template <typename T, typename TO, bool kSplit, int kQ>
+// kLayers: 1, or up to kFlowLayers of them.
+template <typename T, typename TO, bool kSplit, int kQ, int kLayers>
 __global__ void __launch_bounds__(kHeadDim / 2 * kHeadsPerBlock)
-rope_pseudo_q_kernel(const __grid_constant__ RopeBatch rb, TO* __restrict__ q_rot,
+rope_pseudo_q_kernel(const __grid_constant__ RopeLayers<kLayers> rb, TO* __restrict__ q_rot,
                      const double* __restrict__ inv_freq, const __grid_constant__ SeqTable t,
                      int n_q_heads, int n_pseudo, int64_t lo_offset, int late_wait,
                      int interleaved, double out_scale) {
@@ -53,11 +54,11 @@ rope_pseudo_q_kernel(const __grid_constant__ RopeBatch rb, TO* __restrict__ q_ro
   // its wait.)
   if (!late_wait) pdl_wait();
   pdl_trigger();
-  const int layer = rb.n_layers == 1 ? 0 : blockIdx.y / t.batch, b = blockIdx.y - layer * t.batch;
+  const int layer = kLayers == 1 ? 0 : blockIdx.y / t.batch, b = blockIdx.y - layer * t.batch;
   const int i0 = blockIdx.x * kQ, c = threadIdx.x;
   // (the counters of the scorer behind this kernel; their last user completed before the kernel before this one could begin)
   for (int i = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * blockDim.x * blockDim.y + threadIdx.y * blockDim.x + c;
-       i < rb.n_clear; i += gridDim.x * gridDim.y * gridDim.z * blockDim.x * blockDim.y)
+       kLayers > 1 && i < rb.n_clear; i += gridDim.x * gridDim.y * gridDim.z * blockDim.x * blockDim.y)
     rb.clear[i] = 0u;
   const T* __restrict__ q_pre = reinterpret_cast<const T*>(rb.q[layer]);
   const int h = blockIdx.z * kHeadsPerBlock + threadIdx.y, n = min(kQ, n_pseudo - i0);
@@ -217,27 +218,32 @@ cudaError_t launch_rope(int dtype, int out_mode, int64_t lo_offset, const RopeBa
   // One query per block keeps a short call's latency lowest; four where a block each would take several waves.
   const int heads = (dm.n_q_heads + kHeadsPerBlock - 1) / kHeadsPerBlock, seqs = t.batch * rb.n_layers;
   const bool many = (int64_t)dm.n_pseudo * seqs * heads > 2048;
-  auto run = [&](auto kernel1, auto kernel4, auto* out, int64_t offset, double scale, bool with_ref) {
+  RopeLayers<1> one = {{rb.q[0]}, {rb.k[0]}, {rb.head_stride[0]}, {rb.row_stride[0]}, 1, rb.group, nullptr, nullptr, 0};   // (no reference)
+  auto launch = [&](auto kernel1, auto kernel4, auto* out, int64_t offset, double scale, const auto& layers) {
     const dim3 block(kHeadDim / 2, kHeadsPerBlock), grid1(dm.n_pseudo, seqs, heads), grid4((dm.n_pseudo + 3) / 4, seqs, heads);
-    RopeBatch r = rb;
-    if (!with_ref) r.ref = nullptr;
-    return launch_pdl(many ? kernel4 : kernel1, many ? grid4 : grid1, block, 0, s, 1, r, out, inv_freq_dev, t, dm.n_q_heads, dm.n_pseudo, offset, lw,
-                      dm.rope_interleaved, scale);
+    launch_pdl(many ? kernel4 : kernel1, many ? grid4 : grid1, block, 0, s, 1, layers, out, inv_freq_dev, t, dm.n_q_heads, dm.n_pseudo, offset, lw,
+               dm.rope_interleaved, scale);
   };
   using bf16 = __nv_bfloat16;
-  if (dtype == DAPQ_BF16 && out_mode == kRopeOutSplitBf16)
-    run(rope_pseudo_q_kernel<bf16, bf16, true, 1>, rope_pseudo_q_kernel<bf16, bf16, true, 4>, (bf16*)q_rot, lo_offset, 1.0, false);
-  else if (dtype == DAPQ_BF16 && out_mode == kRopeOutF16 && many && rb.ref != nullptr && aligned4(rb))
-    launch_pdl(rope_rows_kernel, dim3((dm.n_pseudo + kRowsQ - 1) / kRowsQ, seqs), dim3(kRowsWarps * 32), 0, s, 1, rb, (__half2*)q_rot, inv_freq_dev, t,
-               dm.n_q_heads, dm.n_pseudo, lw, dm.rope_interleaved, (double)dm.scale_log2e);
-  else if (dtype == DAPQ_BF16 && out_mode == kRopeOutF16)
-    run(rope_pseudo_q_kernel<bf16, __half, false, 1>, rope_pseudo_q_kernel<bf16, __half, false, 4>, (__half*)q_rot, 0, (double)dm.scale_log2e, true);
-  else if (dtype == DAPQ_BF16 && out_mode == kRopeOutBf16)
-    run(rope_pseudo_q_kernel<bf16, bf16, false, 1>, rope_pseudo_q_kernel<bf16, bf16, false, 4>, (bf16*)q_rot, 0, 1.0, false);
-  else if (dtype == DAPQ_BF16)
-    run(rope_pseudo_q_kernel<bf16, float, false, 1>, rope_pseudo_q_kernel<bf16, float, false, 4>, (float*)q_rot, 0, 1.0, false);
-  else
-    run(rope_pseudo_q_kernel<float, float, false, 1>, rope_pseudo_q_kernel<float, float, false, 4>, (float*)q_rot, 0, 1.0, false);
+  if (dtype == DAPQ_BF16 && out_mode == kRopeOutSplitBf16) {
+    launch(rope_pseudo_q_kernel<bf16, bf16, true, 1, 1>, rope_pseudo_q_kernel<bf16, bf16, true, 4, 1>, (bf16*)q_rot, lo_offset, 1.0, one);
+  } else if (dtype == DAPQ_BF16 && out_mode == kRopeOutF16) {
+    one.ref = rb.ref;
+    if (many && rb.ref != nullptr && aligned4(rb))
+      launch_pdl(rope_rows_kernel, dim3((dm.n_pseudo + kRowsQ - 1) / kRowsQ, seqs), dim3(kRowsWarps * 32), 0, s, 1, rb, (__half2*)q_rot, inv_freq_dev, t,
+                 dm.n_q_heads, dm.n_pseudo, lw, dm.rope_interleaved, (double)dm.scale_log2e);
+    else if (rb.n_layers > 1)
+      launch(rope_pseudo_q_kernel<bf16, __half, false, 1, kFlowLayers>, rope_pseudo_q_kernel<bf16, __half, false, 4, kFlowLayers>, (__half*)q_rot, 0,
+             (double)dm.scale_log2e, rb);
+    else
+      launch(rope_pseudo_q_kernel<bf16, __half, false, 1, 1>, rope_pseudo_q_kernel<bf16, __half, false, 4, 1>, (__half*)q_rot, 0, (double)dm.scale_log2e, one);
+  } else if (dtype == DAPQ_BF16 && out_mode == kRopeOutBf16) {
+    launch(rope_pseudo_q_kernel<bf16, bf16, false, 1, 1>, rope_pseudo_q_kernel<bf16, bf16, false, 4, 1>, (bf16*)q_rot, 0, 1.0, one);
+  } else if (dtype == DAPQ_BF16) {
+    launch(rope_pseudo_q_kernel<bf16, float, false, 1, 1>, rope_pseudo_q_kernel<bf16, float, false, 4, 1>, (float*)q_rot, 0, 1.0, one);
+  } else {
+    launch(rope_pseudo_q_kernel<float, float, false, 1, 1>, rope_pseudo_q_kernel<float, float, false, 4, 1>, (float*)q_rot, 0, 1.0, one);
+  }
   log->end(s);
   return cudaGetLastError();
 }

@@ -48,8 +48,11 @@ __device__ __forceinline__ uint32_t order_key(float f) {
 constexpr int kMaxLead = 3;
 __device__ __forceinline__ int lead(const float* x) { return (int)((reinterpret_cast<uintptr_t>(x) & 15u) >> 2); }
 
+// Where a head's indices go: the array of its layer, or (one layer) the array.
+struct OneIndex { int32_t* p; };
+__device__ __forceinline__ int32_t* index_list(const OneIndex& idx, int head, int64_t stride) { return idx.p + (int64_t)head * stride; }
 __device__ __forceinline__ int32_t* index_list(const IndexOut& idx, int head, int64_t stride) {
-  const int layer = head < idx.heads_per_layer ? 0 : head / idx.heads_per_layer;
+  const int layer = head / idx.heads_per_layer;
   return idx.p[layer] + (int64_t)(head - layer * idx.heads_per_layer) * stride;
 }
 
@@ -156,8 +159,9 @@ __device__ __forceinline__ uint32_t packed_prefix(TopkTables& tb, uint32_t mine,
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
+template <class Out>
 __global__ void __launch_bounds__(kTopkThreads)
-topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, const __grid_constant__ IndexOut idx,
+topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, const __grid_constant__ Out idx,
                    int64_t idx_stride, const __grid_constant__ SeqTable t, int cache_keys) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   TopkSmem& sm = *reinterpret_cast<TopkSmem*>(smem_raw);
@@ -283,9 +287,9 @@ topk_select_kernel(const float* __restrict__ scores, int64_t score_stride, const
 // on its copy of the candidates and derives the other CTAs' totals from them: two cluster barriers in all, none
 // after the exchange, so no CTA waits for another at the end.  Otherwise (a bin that holds thousands of a CTA's
 // keys) the later passes merge histograms across the cluster like the general kernel.
-template <int kKpt, int kMinCtas>
+template <int kKpt, int kMinCtas, class Out>
 __global__ void __launch_bounds__(kTopkThreads, kMinCtas)
-topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, const __grid_constant__ IndexOut idx,
+topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, const __grid_constant__ Out idx,
                        int64_t idx_stride, const __grid_constant__ SeqTable t) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   TopkRegSmem& sm = *reinterpret_cast<TopkRegSmem*>(smem_raw);
@@ -473,9 +477,9 @@ topk_select_reg_kernel(const float* __restrict__ scores, int64_t score_stride, c
 
 // One CTA per (sequence, KV head), for sequences of up to 16k keys when a cluster per head would not fit one wave
 // (batches): the same steps as topk_select_reg_kernel without any exchange: the three tables are local histograms.
-template <int kKpt>
+template <int kKpt, class Out>
 __global__ void __launch_bounds__(kTopkThreads)
-topk_select_solo_kernel(const float* __restrict__ scores, int64_t score_stride, const __grid_constant__ IndexOut idx,
+topk_select_solo_kernel(const float* __restrict__ scores, int64_t score_stride, const __grid_constant__ Out idx,
                         int64_t idx_stride, const __grid_constant__ SeqTable t) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   TopkRegSmem& sm = *reinterpret_cast<TopkRegSmem*>(smem_raw);
@@ -609,8 +613,11 @@ TopkShape plan_topk(int heads, int max_len, int n_sm, int max_lead) {
 
 }  // namespace
 
-cudaError_t launch_topk(const float* scores, int64_t score_stride, const IndexOut& idx, int64_t idx_stride,
-                        const SeqTable& t, int n_heads, cudaStream_t s, LaunchLog* log) {
+namespace {
+
+template <class Out>
+cudaError_t select(const float* scores, int64_t score_stride, const Out& idx, int64_t idx_stride, const SeqTable& t, int n_heads, cudaStream_t s,
+                   LaunchLog* log) {
   int max_len = 1;
   for (int b = 0; b < t.batch; ++b) max_len = t.prompt_len[b] > max_len ? t.prompt_len[b] : max_len;
   // (every head begins on a 16-byte boundary: nothing is lost in front of it)
@@ -635,16 +642,16 @@ cudaError_t launch_topk(const float* scores, int64_t score_stride, const IndexOu
     const bool two = shape.per_sm == 2;
     if (n_cta == 1) {
       switch (shape.kpt) {
-        case 4: return launch(topk_select_solo_kernel<4>);
-        case 8: return launch(topk_select_solo_kernel<8>);
-        default: return launch(topk_select_solo_kernel<16>);
+        case 4: return launch(topk_select_solo_kernel<4, Out>);
+        case 8: return launch(topk_select_solo_kernel<8, Out>);
+        default: return launch(topk_select_solo_kernel<16, Out>);
       }
     }
     switch (shape.kpt) {
-      case 4: return two ? launch(topk_select_reg_kernel<4, 2>) : launch(topk_select_reg_kernel<4, 1>);
-      case 8: return two ? launch(topk_select_reg_kernel<8, 2>) : launch(topk_select_reg_kernel<8, 1>);
-      case 16: return two ? launch(topk_select_reg_kernel<16, 2>) : launch(topk_select_reg_kernel<16, 1>);
-      default: return launch(topk_select_reg_kernel<32, 1>);
+      case 4: return two ? launch(topk_select_reg_kernel<4, 2, Out>) : launch(topk_select_reg_kernel<4, 1, Out>);
+      case 8: return two ? launch(topk_select_reg_kernel<8, 2, Out>) : launch(topk_select_reg_kernel<8, 1, Out>);
+      case 16: return two ? launch(topk_select_reg_kernel<16, 2, Out>) : launch(topk_select_reg_kernel<16, 1, Out>);
+      default: return launch(topk_select_reg_kernel<32, 1, Out>);
     }
   }
   int n_cta = kCluster;
@@ -653,13 +660,21 @@ cudaError_t launch_topk(const float* scores, int64_t score_stride, const IndexOu
   const dim3 grid(t.batch * n_cta, n_heads), block(kTopkThreads);
   const int cache_keys = slice <= kMaxSliceSmem ? slice : 0;          // 0: every pass re-reads global memory
   const size_t smem = sizeof(TopkSmem) + (size_t)cache_keys * sizeof(uint32_t);
-  e = cudaFuncSetAttribute(topk_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  e = cudaFuncSetAttribute(topk_select_kernel<Out>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(sizeof(TopkSmem) + (size_t)kMaxSliceSmem * sizeof(uint32_t)));
   if (e != cudaSuccess) return e;
   log->begin(kKindTopk, s);
-  e = launch_pdl(topk_select_kernel, grid, block, smem, s, n_cta, scores, score_stride, idx, idx_stride, t, cache_keys);
+  e = launch_pdl(topk_select_kernel<Out>, grid, block, smem, s, n_cta, scores, score_stride, idx, idx_stride, t, cache_keys);
   log->end(s);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_topk(const float* scores, int64_t score_stride, const IndexOut& idx, int64_t idx_stride,
+                        const SeqTable& t, int n_heads, cudaStream_t s, LaunchLog* log) {
+  if (n_heads <= idx.heads_per_layer) return select(scores, score_stride, OneIndex{idx.p[0]}, idx_stride, t, n_heads, s, log);
+  return select(scores, score_stride, idx, idx_stride, t, n_heads, s, log);
 }
 
 }  // namespace dapq
