@@ -369,7 +369,7 @@ def measure(env: Env, w: gi.Workload, n_layers: int, steps: int, warmup: int, re
     dq.dapq_profile(ctx, True)
     for _ in range(min(steps, 8)):
         step()
-    prof = dq.dapq_profile_read(ctx)
+    prof, prof_layers = dq.dapq_profile_read(ctx), min(steps, 8) * n_layers
     dq.dapq_profile(ctx, False)
     if sampler:
         # short runs end before nvidia-smi has sampled a few times: keep the same load on for ~0.5 s
@@ -395,14 +395,19 @@ def measure(env: Env, w: gi.Workload, n_layers: int, steps: int, warmup: int, re
     total_prof_ms = sum(v[0] for v in kinds.values())
     dom = max(kinds, key=lambda k: kinds[k][0])
     dom_ms = kinds[dom][0] / kinds[dom][1]
+    # layers that share launches: both sweeps of several layers in one launch (counted as sweep1); its figures are per layer
+    stream = dom == "sweep1" and "sweep2" not in kinds
+    n_work = 1.0
+    if stream:
+        dom_ms, n_work = kinds[dom][0] / prof_layers, 2.0
     if dom in ("sweep1", "sweep2", "lse_merge") and w.dtype == "bf16":
         # Two pipes bound a score sweep: the tensor pipe (2 * pairs * d flops) and the MUFU pipe (one exponential per
         # visible (query, key) pair, 16 per clock and SM).  The line reports the one that is closer to its peak.
-        tflops = work["flops_per_sweep"] / (dom_ms * 1e-3) / 1e12
+        tflops = n_work * work["flops_per_sweep"] / (dom_ms * 1e-3) / 1e12
         tensor = {"achieved": tflops, "peak": tensor_peak, "unit": "TFLOP/s", "frac": tflops / tensor_peak,
                   "frac_of_burst": tflops / peaks["bf16_burst"], "frac_of_sustained": tflops / peaks["bf16_sustained"],
                   "peak_source": peaks["source"] + " (%s bf16: timed region %.2f s)" % (tensor_kind, timed_s)}
-        exp_rate = work["exps_per_sweep"] / (dom_ms * 1e-3) / 1e9
+        exp_rate = n_work * work["exps_per_sweep"] / (dom_ms * 1e-3) / 1e9
         exp_peak = 16.0 * env.n_sm * sm_max * 1e6 / 1e9
         exp = {"achieved": exp_rate, "peak": exp_peak, "unit": "Gexp/s", "frac": exp_rate / exp_peak,
                "peak_source": "16 ex2 per clock and SM x %d SMs x %.0f MHz (the part's maximum SM clock)" % (env.n_sm, sm_max)}
@@ -420,11 +425,12 @@ def measure(env: Env, w: gi.Workload, n_layers: int, steps: int, warmup: int, re
                 "frac": achieved / peaks["hbm_gbs"]}
     roof.setdefault("peak_source", peaks["source"])
     roof.update({"kernel": dom, "avg_launch_us": dom_ms * 1e3,
-                 "traffic": ncu_traffic(dom, w.name),
+                 "traffic": None if stream else ncu_traffic(dom, w.name), "both_sweeps": stream,
                  "algorithmic_bytes": work["k_read_bytes"] if dom in ("sweep1", "sweep2") else None,
                  "share_of_step": kinds[dom][0] / total_prof_ms,
-                 # per layer (a kind may be launched several times a layer: the bounds of the pruned selection count as topk)
-                 "kernels_us": {k: round(v[0] / kinds["compact"][1] * 1e3, 2) for k, v in kinds.items()}})
+                 # per layer (a kind may be launched several times a layer: the bounds of the pruned selection count as topk;
+                 # or once for several layers)
+                 "kernels_us": {k: round(v[0] / prof_layers * 1e3, 2) for k, v in kinds.items()}})
     hbm_bytes = work["k_read_bytes"] + work["score_write_bytes"] + work["gather_bytes"]
     frac = hbm_bytes / (layer_ms * 1e-3) / 1e9 / peaks["hbm_gbs"]
     n_sweeps = sweeps_that_ran(kinds)
