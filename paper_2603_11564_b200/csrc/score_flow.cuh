@@ -4,7 +4,7 @@
 // A unit is one sweep over a run of key pairs (256 keys) of one (layer, sequence, KV head, query group): sweep 1 leaves
 // the run's partial row sums, sweep 2 the scores of its keys.  The CTAs, one per SM, take units in a fixed order from a
 // ticket counter.  The order alternates blocks of units, sweep 2 two blocks behind sweep 1, so that a unit of sweep 2 finds
-// the row sums of its item complete (they are counted per item).  A unit depends on units with lower tickets only, which
+// the row sums of its item complete (they are counted per item) and, with short units, its keys still in L2.  A unit depends on units with lower tickets only, which
 // other CTAs are already working on: whatever number of CTAs is resident, the lowest unfinished unit can always finish.
 //
 // Why one launch: two launches per layer spent a third (32 k keys, 8 heads x 256 query rows) to a half (8 k keys) of their
@@ -16,6 +16,12 @@
 // pair as one operand of 256 columns (a job is [128 query rows x 256 keys]), sweep 2 a sub-tile at a time (a job is
 // [128 keys x 256 query rows]; with at most 128 query rows, both sub-tiles side by side, [2 x 128 keys x 128 rows]).
 // So a job is always one accumulator of 256 columns of which every epilogue thread adds up 64.
+//
+// What bounds it: instruction issue (0.55 to 0.6 a cycle and scheduler) and, under a sustained load, power (1.62 GHz); the
+// exponential pipe is 57 (128 query rows) to 70 % busy (256), the tensor pipe 36 to 45 %.  Us a layer in short runs, two launches a
+// layer -> here: 32 k keys on 8 heads x 256 rows 65 -> 46, a ragged batch of 150 k keys x 128 rows 177 -> 158, 40 prompts of 8 k
+// 350 -> 305.  The code has one body per role on purpose: with all variants inlined (118 to 142 KB against 67 to 71) units of three
+// pairs ran at 0.75 of this pace, waiting for instructions.
 #pragma once
 #include "score_qg_sweep1.cuh"
 #include "score_qg_sweep2.cuh"
