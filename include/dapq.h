@@ -29,7 +29,7 @@
  *     (staging buffers, a copy stream, events).
  *   - Argument errors are returned synchronously and launch nothing.  A bounded
  *     device-side wait that gives up sets a status word that dapq_poll_status reads.
- *   - Outputs must not alias inputs.
+ *   - Outputs must not alias inputs (of the same layer; dapq_evict_layers says what holds between layers).
  *
  * Layouts (d = head_dim = 128, G = n_q_heads / n_kv_heads, query head h reads KV head h / G)
  *   q_pre, q_rot  [B, H_q, N, d]   contiguous, element type = dapq_shape.dtype
@@ -242,7 +242,8 @@ DAPQ_API dapq_status dapq_evict(dapq_ctx* ctx, const void* q_pre, const dapq_cac
  * takes for one layer (idx_out, or any entry of it, may be NULL).  k_keep_host: host
  * [n_layers, batch] when k_keep_layer_stride = batch, or one row shared by all layers when
  * k_keep_layer_stride = 0.  Layers of the same lengths and budgets whose arrays do not overlap share launches, up to eight at a
- * time; otherwise the layers run back to back; only launches are issued (no copies, no synchronisation), which makes the whole call
+ * time; otherwise the layers run back to back, and a layer whose queries or cache lie in outputs of an earlier layer of the
+ * call reads what that layer wrote.  Only launches are issued (no copies, no synchronisation), which makes the whole call
  * capturable into a CUDA graph.  Stops at the first layer that fails and returns its status.
  * Calls of 8 layers and more on long prompts, without pooling and with budgets that are small against the prompts, compute
  * the scores of those keys only that can be among the K largest, in layers where the layers before show that it

@@ -668,7 +668,7 @@ struct Span {
 Span span_of(const void* p, size_t bytes) { return {(uintptr_t)p, p ? (uintptr_t)p + bytes : (uintptr_t)p}; }
 
 // Layers may share launches if nothing that one of them writes is written or read by another, so that their order does
-// not matter.
+// not matter; and a rotation may begin beside the compaction of the layers before if none of its own layers reads what they write.
 struct LayerSpans {
   Span out[3], in[3];
   LayerSpans() = default;
@@ -689,6 +689,12 @@ struct LayerSpans {
       for (int j = 0; j < 3; ++j)
         if (out[i].meets(o.out[j]) || out[i].meets(o.in[j]) || in[i].meets(o.out[j])) return false;
     return true;
+  }
+  bool reads(const LayerSpans& o) const {
+    for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j)
+        if (in[i].meets(o.out[j])) return true;
+    return false;
   }
 };
 
@@ -711,8 +717,8 @@ int layers_that_fit(const dapq_ctx* ctx, const SeqTable& t, bool own_idx) {
 
 // n layers of one geometry and one row of budgets; *taken says how many of them were done (more than one only by score_flow.cu).
 // after_own_compaction: the kernel before this call in `stream` is the compaction kernel of an
-// earlier evict on the same context (the layers of dapq_evict_layers); the rotation then does
-// not wait for it before it starts.
+// earlier evict on the same context (the layers of dapq_evict_layers), which writes nothing that these layers read; the rotation
+// then does not wait for it before it starts, and the first sweep's first keys are copied beside it too.
 // route: the call's layers may take the pruned selection (NULL: they may not); layer: the first one's number.
 dapq_status evict_impl(dapq_ctx* ctx, const Layer* y, int n, const SeqTable& t, float* scores_out, cudaStream_t s, bool after_own_compaction,
                        PruneRoute* route, int32_t layer, int* taken) {
@@ -839,6 +845,10 @@ dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const
   auto check = [&](int32_t m, Layer* y, SeqTable* t) {
     return check_layer(ctx, q_pre[m], &caches[m], k_keep_host + (int64_t)m * k_keep_layer_stride, k_out[m], v_out[m], idx_out ? idx_out[m] : nullptr, y, t);
   };
+  // what the launches before this one write: they have the layers before `l` and wait for the compaction before them, so nothing
+  // older is still being written when this one's rotation begins
+  LayerSpans before[kFlowLayers];
+  int n_before = 0;
   for (int32_t l = 0; l < n_layers;) {
     Layer y[kFlowLayers];
     SeqTable t, other;
@@ -847,12 +857,12 @@ dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const
     // The layers behind it that may share its launches: of the same geometry and budgets, as many as fit the workspace, none of them
     // touching another's outputs; in launches of equal size.  (A layer that is not in order says so when its own turn comes.)
     int n = 1;
+    LayerSpans spans[kFlowLayers];
+    spans[0] = LayerSpans(ctx, y[0], t);
     if (wants_flow(ctx)) {
       bool own_idx = false;
       for (int32_t m = l; m < n_layers && m < l + kFlowLayers; ++m) own_idx = own_idx || !idx_out || !idx_out[m];
       const int fit = layers_that_fit(ctx, t, own_idx), left = n_layers - l, launches = (left + fit - 1) / fit, most = (left + launches - 1) / launches;
-      LayerSpans spans[kFlowLayers];
-      spans[0] = LayerSpans(ctx, y[0], t);
       for (; n < most && check(l + n, &y[n], &other) == DAPQ_OK && memcmp(&other, &t, sizeof(t)) == 0; ++n) {
         spans[n] = LayerSpans(ctx, y[n], t);
         bool apart = true;
@@ -860,10 +870,15 @@ dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const
         if (!apart) break;
       }
     }
+    bool beside = l > 0;
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n_before; ++j) beside = beside && !spans[i].reads(before[j]);
     int taken = 1;
-    st = evict_impl(ctx, y, n, t, nullptr, (cudaStream_t)stream, l > 0, n_layers >= kPruneLeastLayers ? &route : nullptr, l, &taken);
+    st = evict_impl(ctx, y, n, t, nullptr, (cudaStream_t)stream, beside, n_layers >= kPruneLeastLayers ? &route : nullptr, l, &taken);
     if (st != DAPQ_OK) return st;
     l += taken;
+    n_before = taken;
+    for (int i = 0; i < taken; ++i) before[i] = spans[i];
   }
   return DAPQ_OK;
 }

@@ -1364,7 +1364,7 @@ def _layers(dq, hq, hkv, n, lens, keep, layers, keys="plain"):
 def _one_by_one(dq, ctx, w, q, k, v):
     KT = int(w.cu_keep[-1])
     idx = torch.full((w.n_kv_heads, KT), -1, dtype=torch.int32, device="cuda")
-    ko, vo = (torch.zeros((w.n_kv_heads, KT, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    ko, vo = (torch.zeros((w.n_kv_heads, KT, 128), dtype=k.dtype, device="cuda") for _ in range(2))
     scores = torch.empty((w.n_kv_heads, w.total_prompt), dtype=torch.float32, device="cuda")
     dq.dapq_evict(ctx, q, k, v, w.cu_rows, list(w.prompt_lens), list(w.keep), ko, vo, idx, scores)
     return idx, scores
@@ -1412,6 +1412,37 @@ def test_layers_whose_arrays_overlap_keep_their_order(dq):
     dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(keep), chained_k, chained_v, idx)
     dq.dapq_poll_status(ctx)
     _same_set(want, idx[3], scores, k3, v3, ko[3], vo[3], lens, w.cu_rows, w.cu_keep, w.cu_prompt)
+    dq.dapq_destroy(ctx)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("read", ["queries", "keys", "keys two apart"])
+def test_layers_that_read_what_an_earlier_one_wrote(dq, read, dtype):
+    """The layers behind one whose kept rows are their queries (each layer the next one's), or whose kept keys lie in the cache
+    of the last layer, which goes alone: directly behind that layer, or behind a launch that it shares with another.  Long copies,
+    so that a rotation or a first copy of keys that did not wait for them would see what was there before."""
+    hq, hkv, n, L, K = 8, 2, 32, 6000, 3000
+    w = _small(lens=(L,), keep=(K,), n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0, dtype=dtype)
+    ctx, layers = _ctx(dq, w), {"queries": 5, "keys": 2, "keys two apart": 3}[read]
+    g = torch.Generator(device="cuda").manual_seed(layers)
+    draw = lambda *shape: torch.randn(shape, generator=g, device="cuda").to(w.torch_dtype())
+    qs, ks, vs = [draw(1, hq, n, 128) for _ in range(layers)], [draw(hkv, L + n, 128) for _ in range(layers)], [draw(hkv, L + n, 128) for _ in range(layers)]
+    ko, vo = ([torch.zeros((hkv, K, 128), dtype=w.torch_dtype(), device="cuda") for _ in range(layers)] for _ in range(2))
+    idx = [torch.full((hkv, K), -1, dtype=torch.int32, device="cuda") for _ in range(layers)]
+    if read == "queries":
+        qs[1:] = [x.view(-1)[:hq * n * 128].view(1, hq, n, 128) for x in ko[:-1]]
+    else:
+        ko[0] = ks[-1].view(-1)[:hkv * K * 128].view(hkv, K, 128)
+    for turn in range(3):
+        for x in ko:
+            x.normal_(generator=g)                              # what a layer must not see
+        dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, [L], [K], ko, vo, idx)
+        dq.dapq_poll_status(ctx)
+        for l in range(1 if read == "queries" else layers - 1, layers):
+            want, _ = _one_by_one(dq, ctx, w, qs[l], ks[l], vs[l])
+            assert torch.equal(want, idx[l]), (turn, l)
+            rows = want.long()[..., None].expand(-1, -1, 128)
+            assert torch.equal(ko[l], ks[l].gather(1, rows)) and torch.equal(vo[l], vs[l].gather(1, rows))
     dq.dapq_destroy(ctx)
 
 
