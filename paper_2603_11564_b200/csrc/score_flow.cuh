@@ -629,6 +629,7 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
         }
       }
       if (!__all_sync(0xffffffffu, ok)) break;
+      __syncwarp();                                              // (a vote orders no memory: what lane 0 has announced)
       const Unit u = read_unit(smem, S::unit + n % kUnitRing * (int)sizeof(Unit));   // (stays until unit n + 2 is announced)
       if (u.kind == kEndUnit) break;
       last_q = u.qrow;
@@ -650,6 +651,7 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
           }
         }
         ok = __all_sync(0xffffffffu, there);
+        __syncwarp();                                            // (lane 0 has acquired the row sums: for all lanes)
       }
       if (!ok) break;
 #pragma unroll 1

@@ -1446,6 +1446,21 @@ def test_layers_that_read_what_an_earlier_one_wrote(dq, read, dtype):
     dq.dapq_destroy(ctx)
 
 
+@pytest.mark.parametrize("hq,hkv,n,lens", [(32, 8, 32, (20001, 9000)), (14, 2, 25, (5000, 300, 2500)), (16, 2, 128, (9000,))])
+def test_layers_that_share_launches_repeat(dq, hq, hkv, n, lens):
+    """Bit for bit the same sets and rows however the units fall to the CTAs."""
+    w, ctx, qs, ks, vs, idx, ko, vo = _layers(dq, hq, hkv, n, lens, tuple(L // 2 for L in lens), 4)
+    first = None
+    for _ in range(20):
+        for x in (*ko, *vo, *idx):
+            x.fill_(-1)
+        dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(w.keep), ko, vo, idx)
+        dq.dapq_poll_status(ctx)
+        first = first or [x.clone() for x in (*ko, *vo, *idx)]
+        assert all(torch.equal(x, y) for x, y in zip(first, (*ko, *vo, *idx)))
+    dq.dapq_destroy(ctx)
+
+
 def test_layers_that_share_launches_wait_limit(dq):
     """A wait that runs out in the shared launch: reported once, and the next call is right again."""
     hq, hkv, n, lens, keep, layers = 8, 2, 32, (3000, 900), (64, 30), 4
