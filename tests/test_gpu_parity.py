@@ -1391,8 +1391,9 @@ def test_layers_that_share_launches(dq, hq, hkv, n, lens, keep, layers, keys):
 
 
 def test_layers_whose_arrays_overlap_keep_their_order(dq):
-    """Outputs of one layer that are another's outputs or inputs: as if the layers ran one after the other.  And without index
-    arrays, or with some."""
+    """Outputs of one layer that are another's outputs or inputs, the reading layer in a shared launch: as if the layers ran one after
+    the other.  (Reading layers that go alone: test_layers_that_read_what_an_earlier_one_wrote; index arrays that are missing:
+    test_layers_that_share_launches_in_other_forms.)"""
     hq, hkv, n, lens, keep, layers = 8, 2, 32, (600, 300), (64, 30), 5
     w, ctx, qs, ks, vs, idx, ko, vo = _layers(dq, hq, hkv, n, lens, keep, layers)
     KT = int(w.cu_keep[-1])
@@ -1476,4 +1477,126 @@ def test_layers_that_share_launches_wait_limit(dq):
     dq.dapq_poll_status(ctx)
     for l in range(layers):
         _same_set(alone[l][0], idx[l], alone[l][1], ks[l], vs[l], ko[l], vo[l], lens, w.cu_rows, w.cu_keep, w.cu_prompt)
+    dq.dapq_destroy(ctx)
+
+
+# (form, H_q, H_kv, N, lengths, layers): what a layer may look like beside the plain one of the cases above.  views: rows of all
+# heads interleaved, the first sequence from row 5 of the cache, every second layer contiguous instead; nan, inf: one such key of
+# one head of one layer; max, avg: pooling; room: a context of 50 times the call's rows and 8 times its
+# prompts (more layers a launch than layers of its full size); budgets: two rows of budgets; some indices, no indices: without some or all index arrays, the call as large as the context,
+# which leaves the scores a slot less; interleaved, odd queries: the rotation of many queries, heads and queries that its blocks do
+# not divide, with paired neighbours, and with queries off four-byte boundaries; graph: three launches captured, so that a replay
+# takes the counters that the launch before it took
+FORMS = [("views", 8, 2, 25, (700, 2300), 5), ("nan", 8, 2, 32, (900, 1400), 4), ("inf", 8, 2, 32, (900, 1400), 4), ("max", 8, 2, 32, (3001, 517), 4),
+         ("avg", 16, 2, 64, (3001, 517), 4), ("room", 32, 8, 64, (4000,), 8), ("room", 64, 8, 128, (2000, 1000), 8), ("budgets", 8, 2, 32, (900, 1400), 7),
+         ("some indices", 8, 2, 32, (900, 1400), 8), ("no indices", 8, 2, 32, (900, 1400), 8), ("no indices", 32, 8, 128, (9000,), 8),
+         ("interleaved", 12, 3, 21, (300, 40, 500, 33, 64, 257, 129), 8), ("odd queries", 12, 3, 21, (300, 40, 500, 33, 64, 257, 129), 8),
+         ("odd queries", 12, 3, 21, (300, 40), 3), ("graph", 8, 2, 32, (900, 1400), 17)]
+
+
+@pytest.mark.parametrize("form,hq,hkv,n,lens,layers", FORMS)
+def test_layers_that_share_launches_in_other_forms(dq, form, hq, hkv, n, lens, layers):
+    """Against dapq_evict of each layer (the tolerance of _same_set, on pooled scores where they are pooled)."""
+    g = torch.Generator(device="cuda").manual_seed(hq + n + layers)
+    B, row0, pool = len(lens), 5 if form == "views" else 0, {"max": 7, "avg": 5}.get(form, 0)
+    cu_rows = [row0 + sum(lens[:b]) + b * n for b in range(B + 1)]
+    cu_prompt = [sum(lens[:b]) for b in range(B + 1)]
+    keeps = [tuple(L // (4 if form == "budgets" and 2 <= l < 5 else 9) for L in lens) for l in range(layers)]
+    more = (8 * B, 50 * cu_rows[-1]) if form == "room" else (B, cu_rows[-1])
+    ctx = dq.dapq_create(hq, hkv, n, *more, dq.DAPQ_BF16, 1.0e4, flags=dq.DAPQ_FLAG_ROPE_INTERLEAVED if form == "interleaved" else 0,
+                         pool_mode={"max": dq.DAPQ_POOL_MAX, "avg": dq.DAPQ_POOL_AVG}.get(form, dq.DAPQ_POOL_NONE), pool_kernel=pool or 1)
+    draw = lambda *shape: torch.randn(shape, generator=g, device="cuda").bfloat16()
+    qs, ks, vs = [], [], []
+    for l in range(layers):
+        if form == "odd queries":
+            x = torch.empty(B * hq * n * 128 + 1, dtype=torch.bfloat16, device="cuda")[1:]
+            qs.append(x.copy_(draw(x.numel())).view(B, hq, n, 128))
+            assert qs[-1].data_ptr() % 4 == 2
+        else:
+            qs.append(draw(B, hq, n, 128))
+        if form == "views" and l % 2 == 0:
+            kv = draw(cu_rows[-1], hkv, 2, 136)
+            ks.append(kv[:, :, 0, :128].transpose(0, 1))
+            vs.append(kv[:, :, 1, :128].transpose(0, 1))
+        else:
+            ks.append(draw(hkv, cu_rows[-1], 128))
+            vs.append(draw(hkv, cu_rows[-1], 128))
+    if form in ("nan", "inf"):
+        ks[1][1, 400, 7] = float(form)
+    alone, scores = [], torch.empty((hkv, sum(lens)), device="cuda")
+    for l in range(layers):
+        full = torch.full((hkv, sum(keeps[l])), -1, dtype=torch.int32, device="cuda")
+        a, b = (torch.zeros((hkv, sum(keeps[l]), 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        before = dq.dapq_launch_count(ctx)
+        dq.dapq_evict(ctx, qs[l], ks[l], vs[l], cu_rows, list(lens), keeps[l], a, b, full, scores)
+        n_alone = dq.dapq_launch_count(ctx) - before
+        alone.append((full, a, b, scores.clone()))
+    io, ko, vo = ([torch.full_like(x[i], -1) for x in alone] for i in range(3))
+    missing = [form == "no indices" or form == "some indices" and l % 3 != 1 for l in range(layers)]
+
+    class Null:
+        def data_ptr(self):
+            return 0
+    call = lambda: dq.dapq_evict_layers(ctx, qs, ks, vs, cu_rows, list(lens), keeps, ko, vo, [Null() if m else x for m, x in zip(missing, io)])
+    run = call
+    if form == "graph":
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            call()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                call()
+        torch.cuda.synchronize()
+        run = lambda: (graph.replay(), graph.replay(), call(), graph.replay())
+    for turn in range(2):
+        for x in (*io, *ko, *vo):
+            x.fill_(-1)
+        before = dq.dapq_launch_count(ctx)
+        run()
+        dq.dapq_poll_status(ctx)
+        assert dq.dapq_launch_count(ctx) - before < layers * n_alone         # (some layers shared)
+        for l, (full, a, b, s) in enumerate(alone):
+            cu_keep = [sum(keeps[l][:x]) for x in range(B + 1)]
+            if missing[l]:                                                     # the copies say which rows they are
+                assert bool((io[l] == -1).all())
+                got = torch.empty_like(full)
+                for h in range(hkv):
+                    for x in range(B):
+                        rows, at = ks[l][h, cu_rows[x]:cu_rows[x + 1]], slice(cu_keep[x], cu_keep[x + 1])
+                        got[h, at] = (ko[l][h, at, None] == rows).all(-1).int().argmax(1)
+                _same_set(full, got, s, ks[l], vs[l], ko[l], vo[l], lens, cu_rows, cu_keep, cu_prompt)
+                continue
+            if form == "nan" and l == 1:                                       # (head 1: a row with NaN has no score to compare)
+                assert torch.equal(full, io[l])
+                assert all(torch.equal(x.view(torch.int16), y.view(torch.int16)) for x, y in ((a, ko[l]), (b, vo[l])))
+                continue
+            for x in range(B if pool else 0):
+                y = s[:, cu_prompt[x]:cu_prompt[x + 1]]
+                f = torch.nn.functional
+                s[:, cu_prompt[x]:cu_prompt[x + 1]] = (f.max_pool1d(y[None], pool, 1, pool // 2) if form == "max" else
+                                                       f.avg_pool1d(y[None], pool, 1, pool // 2, count_include_pad=False))[0] if turn == 0 else y
+            _same_set(full, io[l], s, ks[l], vs[l], ko[l], vo[l], lens, cu_rows, cu_keep, cu_prompt)
+    dq.dapq_destroy(ctx)
+
+
+@pytest.mark.parametrize("cycles", [1, 30, 100, 1000, 5000, 30000])
+def test_layers_that_share_launches_give_up_anywhere(dq, cycles):
+    """Limits at which some waits run out and others do not: no role hangs on another that gave up, and the context works again."""
+    hq, hkv, n, lens, layers = 32, 8, 64, (9000, 3000), 6
+    w, ctx, qs, ks, vs, idx, ko, vo = _layers(dq, hq, hkv, n, lens, (900, 64), layers)
+    call = lambda: dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(w.keep), ko, vo, idx)
+    call()
+    dq.dapq_poll_status(ctx)
+    want = [x.clone() for x in (*idx, *ko, *vo)]
+    for _ in range(3):
+        dq.dapq_set_wait_limit(ctx, cycles)
+        call()
+        try:
+            dq.dapq_poll_status(ctx)
+        except dq.DapqError as e:
+            assert e.status == dq.DAPQ_ERR_TIMEOUT
+        dq.dapq_set_wait_limit(ctx, 0)
+        call()
+        dq.dapq_poll_status(ctx)
+        assert all(torch.equal(x, y) for x, y in zip(want, (*idx, *ko, *vo)))
     dq.dapq_destroy(ctx)
