@@ -122,6 +122,7 @@ dapq_status cuda_fail(dapq_ctx* ctx, cudaError_t e, const char* what) {
   } while (0)
 
 constexpr double kFlowPairs = 6e8;             // query-key pairs of a launch of score_flow.cu that make its start and end small
+constexpr double kAlonePairs = 3.3e8;          // query-key pairs of one prompt from which a layer goes by itself
 constexpr size_t kFlowLeastPairs = 16;         // key pairs of a unit for which its partial row sums have room in any call
 
 // Device buffers allocated together: as one block, cut up at 256-byte boundaries, where a block of its own for each
@@ -699,14 +700,18 @@ struct LayerSpans {
 };
 
 // Layers of this geometry that one launch may cover: their workspace fits the context's (own_idx: the indices take a part of
-// it too).  Us a layer, a launch per sweep -> one for several layers: 8 k tokens on 8 heads x 128 query rows 27.7 -> 10.5,
-// x 1024 68.5 -> 48.9; 30 k x 512 96 -> 83, x 1024 170 -> 155; 60 k x 128 72.7 -> 56.4, x 256 99 -> 85, x 1024 302 -> 303; 100 k x 128
-// 106 -> 92, x 256 147 -> 147, x 512 262 -> 268.  So layers of long prompts and the size from which the pruned selection
-// pays go by themselves; there a sweep is long enough.
+// it too).  Us a layer on 8 heads, a launch per sweep -> shared launches of 7 layers, in bursts of 10 ms | over seconds (power cap):
+// 8 k tokens x 128 query rows 26.9 -> 10.3 | 26.8 -> 10.1, x 1024 68 -> 48 | 68 -> 50; 30 k x 512 97 -> 83 | 98 -> 93, x 1024 173 -> 163
+// | 177 -> 176; 60 k x 128 80 -> 56 | 81 -> 64, x 256 108 -> 91 | 110 -> 99; 100 k x 128 115 -> 97 | 122 -> 109, x 256 168 -> 159 | 171 -> 168,
+// x 512 279 -> 280 | 293 -> 303.  So layers of long prompts and the size from which the pruned selection pays go by themselves.
+// From 3.3e8 pairs of one prompt on a sweep of its own is long enough whatever the length, and where it holds 512 query rows a CTA
+// it fetches and converts keys half as often: 40 k x 1024 227 -> 225 | 231 -> 236, 48 k 263 -> 265 | 271 -> 278, 60 k 329 -> 327 | 335 -> 342
+// (36 k, 3e8: 206 -> 195 | 210 -> 209).  A batch of as many pairs in short prompts gains (8 x 8 k x 1024 377 -> 329 | 402 -> 375).
 int layers_that_fit(const dapq_ctx* ctx, const SeqTable& t, bool own_idx) {
   int longest = 0;
   for (int b = 0; b < t.batch; ++b) longest = t.prompt_len[b] > longest ? t.prompt_len[b] : longest;
-  if (longest >= kPruneLeastLen && (double)t.cu_prompt[t.batch] * ctx->dims.n_q_heads * ctx->dims.n_pseudo >= kPruneLeastPairs) return 1;
+  const double rows = (double)ctx->dims.n_q_heads * ctx->dims.n_pseudo;
+  if ((longest >= kPruneLeastLen && t.cu_prompt[t.batch] * rows >= kPruneLeastPairs) || longest * rows >= kAlonePairs) return 1;
   const int64_t room = ctx->shape.max_total_rows, seqs = (int64_t)ctx->shape.max_batch * ctx->flow_layers / t.batch;
   const int slots = ctx->score_slots < ctx->flow_layers ? ctx->score_slots : ctx->flow_layers;
   int64_t n = room * (own_idx && slots == ctx->score_slots ? slots - 1 : slots) / t.cu_prompt[t.batch];

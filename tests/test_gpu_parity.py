@@ -1390,6 +1390,21 @@ def test_layers_that_share_launches(dq, hq, hkv, n, lens, keep, layers, keys):
     dq.dapq_destroy(ctx)
 
 
+@pytest.mark.parametrize("n,lens,shared", [(128, (40200,), True), (128, (40400,), False), (128, (30000, 20000), True), (127, (40600,), True)])
+def test_layers_of_many_pairs_go_alone(dq, n, lens, shared):
+    """64 heads: 8192 query rows from 3.3e8 / 8192 = 40283 tokens of one prompt on; dapq_evict's own sets there, bit for bit."""
+    w, ctx, qs, ks, vs, idx, ko, vo = _layers(dq, 64, 8, n, lens, tuple(L // 50 for L in lens), 2)
+    before = dq.dapq_launch_count(ctx)
+    alone = [_one_by_one(dq, ctx, w, *x) for x in zip(qs, ks, vs)]
+    n_alone = dq.dapq_launch_count(ctx) - before
+    dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(w.keep), ko, vo, idx)
+    dq.dapq_poll_status(ctx)
+    n_layers = dq.dapq_launch_count(ctx) - before - n_alone
+    assert n_layers < n_alone if shared else n_layers == n_alone
+    assert shared or all(torch.equal(a[0], i) for a, i in zip(alone, idx))
+    dq.dapq_destroy(ctx)
+
+
 def test_layers_whose_arrays_overlap_keep_their_order(dq):
     """Outputs of one layer that are another's outputs or inputs, the reading layer in a shared launch: as if the layers ran one after
     the other.  (Reading layers that go alone: test_layers_that_read_what_an_earlier_one_wrote; index arrays that are missing:
