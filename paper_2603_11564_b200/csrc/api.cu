@@ -388,40 +388,51 @@ dapq_status dapq_create(dapq_ctx** out, const dapq_shape* sh, int device) {
                     (2LL * ctx->n_sm + sh->n_kv_heads - 1) / sh->n_kv_heads;
   const size_t hq_n = (size_t)sh->n_q_heads * sh->n_pseudo;
   ctx->q_rows_max = (int64_t)sh->max_batch * hq_n;
-  size_t part_elems = (size_t)ctx->max_chunks * hq_n;
   const size_t part_umma = (size_t)umma_part_elems(sh->max_batch, sh->n_q_heads, sh->n_kv_heads, sh->n_pseudo);
-  if (part_umma > part_elems) part_elems = part_umma;
   const size_t rows = (size_t)sh->max_total_rows;
   const bool flow = wants_flow(ctx);
   if (flow) {
     // enough layers a launch for some 6e8 query-key pairs; small calls of a large context may take more
     const double layers = kFlowPairs / ((double)hq_n * rows);
     ctx->flow_layers = layers >= kFlowLayers ? kFlowLayers : (int)layers + 1;
-    const size_t chunk_elems = (size_t)sh->n_kv_heads * flow_rows_pad(ctx->dims), nl_full = (size_t)ctx->flow_layers;
-    const size_t runs = nl_full * (rows / (256 * kFlowLeastPairs) + 1), few = 4 * (size_t)ctx->n_sm / ((size_t)sh->n_kv_heads * qg_groups(ctx->dims)) + 1;
-    const size_t want = nl_full * sh->max_batch + (runs > few ? runs : few);
-    const size_t need = want * chunk_elems * 3 / 2;                // (a float2 and a float each)
-    if (need > part_elems) part_elems = need;
-    ctx->flow_chunks = (int64_t)(part_elems * 2 / 3 / chunk_elems);
-    ctx->sync_words = (int64_t)ctx->flow_layers * sh->max_batch * sh->n_kv_heads * qg_groups(ctx->dims) + 1;
   }
-  const size_t nl = (size_t)ctx->flow_layers;
   const int n_slots = wants_umma(ctx) ? qg_groups(ctx->dims) : (wants_split(ctx) ? split_groups(ctx->dims) : 1);
   const size_t score_bytes = (size_t)sh->n_kv_heads * rows * sizeof(float);
-  Arena ar;
-  ar.add(&ctx->inv_freq, sizeof(freq));
-  ar.add(&ctx->status, sizeof(int));
-  ar.add(&ctx->q_rot, (size_t)sh->max_batch * hq_n * kHeadDim * (nl > 1 ? nl * sizeof(__half) : sizeof(float)));
-  ar.add(&ctx->part, part_elems * sizeof(float2));
-  ar.add(&ctx->lse2, (nl * sh->max_batch * hq_n + 32) * sizeof(float));
-  // (the indices have the last of the score slots, which launches whose caller takes the indices fill with scores too)
-  ctx->score_slots = nl > 2 ? (int)nl : 2;
-  ar.add(&ctx->scores, ctx->score_slots * score_bytes);
-  if (sh->pool_mode != DAPQ_POOL_NONE) ar.add(&ctx->pooled, nl * score_bytes);
-  if (n_slots > 1) ar.add(&ctx->slots, nl * n_slots * score_bytes);
-  if (flow)
-    for (auto& w : ctx->sync) ar.add(&w, ctx->sync_words * sizeof(uint32_t));
-  bool ok = ar.allocate(ctx);
+  auto allocate = [&] {
+    const size_t nl = (size_t)ctx->flow_layers, part_fma = (size_t)ctx->max_chunks * hq_n;
+    size_t part_elems = part_umma > part_fma ? part_umma : part_fma;
+    if (flow) {
+      const size_t chunk_elems = (size_t)sh->n_kv_heads * flow_rows_pad(ctx->dims);
+      const size_t runs = nl * (rows / (256 * kFlowLeastPairs) + 1), few = 4 * (size_t)ctx->n_sm / ((size_t)sh->n_kv_heads * qg_groups(ctx->dims)) + 1;
+      const size_t want = nl * sh->max_batch + (runs > few ? runs : few);
+      const size_t need = want * chunk_elems * 3 / 2;                // (a float2 and a float each)
+      if (need > part_elems) part_elems = need;
+      ctx->flow_chunks = (int64_t)(part_elems * 2 / 3 / chunk_elems);
+      ctx->sync_words = (int64_t)nl * sh->max_batch * sh->n_kv_heads * qg_groups(ctx->dims) + 1;
+    }
+    Arena ar;
+    ar.add(&ctx->inv_freq, sizeof(freq));
+    ar.add(&ctx->status, sizeof(int));
+    ar.add(&ctx->q_rot, (size_t)sh->max_batch * hq_n * kHeadDim * (nl > 1 ? nl * sizeof(__half) : sizeof(float)));
+    ar.add(&ctx->part, part_elems * sizeof(float2));
+    ar.add(&ctx->lse2, (nl * sh->max_batch * hq_n + 32) * sizeof(float));
+    // (the indices have the last of the score slots, which launches whose caller takes the indices fill with scores too)
+    ctx->score_slots = nl > 2 ? (int)nl : 2;
+    ar.add(&ctx->scores, ctx->score_slots * score_bytes);
+    if (sh->pool_mode != DAPQ_POOL_NONE) ar.add(&ctx->pooled, nl * score_bytes);
+    if (n_slots > 1) ar.add(&ctx->slots, nl * n_slots * score_bytes);
+    if (flow)
+      for (auto& w : ctx->sync) ar.add(&w, ctx->sync_words * sizeof(uint32_t));
+    return ar.allocate(ctx);
+  };
+  bool ok = allocate();
+  if (!ok && ctx->flow_layers > 1) {
+    // no room for several layers of the full size: what one takes will do (64 prompts of 130 tokens on 64 heads: 290 of 696 MB)
+    cudaGetLastError();
+    while (ctx->n_owned > 0) cudaFree(ctx->owned[--ctx->n_owned]);
+    ctx->flow_layers = 1;
+    ok = allocate();
+  }
   if (ok) ctx->idx = reinterpret_cast<int32_t*>(ctx->scores + (size_t)(ctx->score_slots - 1) * sh->n_kv_heads * rows);
   ok = ok && cudaMemcpy(ctx->inv_freq, freq, sizeof(freq), cudaMemcpyHostToDevice) == cudaSuccess;
   ok = ok && cudaMemset(ctx->status, 0, sizeof(int)) == cudaSuccess;

@@ -1263,6 +1263,28 @@ def test_contexts_of_short_prompts_hold_no_workspace_for_the_pruned_selection(dq
     assert used(1, 0) - used(1, dq.DAPQ_FLAG_Q_BF16) >= 20 * 8 * 40 * 8224
 
 
+def test_contexts_fit_where_one_layer_fits(dq):
+    """64 prompts of 130 tokens on 64 heads: 696 MB with room for five layers in a launch, some 290 for one.  With 480 left a context
+    is made, and its layers' sets are right."""
+    hq, hkv, n, lens = 64, 8, 128, (130,) * 64
+    w, ctx, qs, ks, vs, idx, ko, vo = _layers(dq, hq, hkv, n, lens, (9,) * 64, 2)
+    alone = [_one_by_one(dq, ctx, w, *x) for x in zip(qs, ks, vs)]
+    dq.dapq_destroy(ctx)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    ballast = torch.empty(torch.cuda.mem_get_info()[0] - (480 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        ctx = _ctx(dq, w)
+        dq.dapq_evict_layers(ctx, qs, ks, vs, w.cu_rows, list(lens), list(w.keep), ko, vo, idx)
+        dq.dapq_poll_status(ctx)
+        dq.dapq_destroy(ctx)
+    finally:
+        del ballast
+        torch.cuda.empty_cache()
+    for l in range(2):
+        _same_set(alone[l][0], idx[l], alone[l][1], ks[l], vs[l], ko[l], vo[l], lens, w.cu_rows, w.cu_keep, w.cu_prompt)
+
+
 def test_pruned_selection_wait_limit(dq):
     """A device-side wait of the pruned selection that runs out: status once, and the context works again."""
     hq, hkv, n, L, K = 28, 4, 64, 112001, 2000
