@@ -122,6 +122,7 @@ dapq_status cuda_fail(dapq_ctx* ctx, cudaError_t e, const char* what) {
   } while (0)
 
 constexpr double kFlowPairs = 6e8;             // query-key pairs of a launch of score_flow.cu that make its start and end small
+constexpr int kMaxGridY = 65535;
 constexpr double kAlonePairs = 3.3e8;          // query-key pairs of one prompt from which a layer goes by itself
 constexpr size_t kFlowLeastPairs = 16;         // key pairs of a unit for which its partial row sums have room in any call
 
@@ -728,6 +729,7 @@ int layers_that_fit(const dapq_ctx* ctx, const SeqTable& t, bool own_idx) {
   int64_t n = room * (own_idx && slots == ctx->score_slots ? slots - 1 : slots) / t.cu_prompt[t.batch];
   if (own_idx && room / t.cu_keep[t.batch] < n) n = room / t.cu_keep[t.batch];
   if (seqs < n) n = seqs;
+  if (kMaxGridY / ctx->dims.n_kv_heads < n) n = kMaxGridY / ctx->dims.n_kv_heads;   // (selection and pooling: a row of the grid per head)
   return n < 1 ? 1 : (n > kFlowLayers ? kFlowLayers : (int)n);
 }
 

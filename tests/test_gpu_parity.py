@@ -1616,6 +1616,28 @@ def test_layers_that_share_launches_in_other_forms(dq, form, hq, hkv, n, lens, l
     dq.dapq_destroy(ctx)
 
 
+def test_layers_of_more_heads_than_a_grid_has_rows(dq):
+    """Eight layers of 8200 heads: 65600 rows of a grid, of which there are 65535."""
+    h, n, L, K, layers = 8200, 64, 20, 3, 8
+    ctx = dq.dapq_create(h, h, n, 1, L + n, dq.DAPQ_BF16, 1.0e4)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    draw = lambda *shape: torch.randn(shape, generator=g, device="cuda").bfloat16()
+    qs, ks = [draw(1, h, n, 128) for _ in range(layers)], [draw(h, L + n, 128) for _ in range(layers)]
+    ko, vo = ([torch.zeros((h, K, 128), dtype=torch.bfloat16, device="cuda") for _ in range(layers)] for _ in range(2))
+    idx = [torch.full((h, K), -1, dtype=torch.int32, device="cuda") for _ in range(layers)]
+    dq.dapq_evict_layers(ctx, qs, ks, ks, [0, L + n], [L], [K], ko, vo, idx)
+    dq.dapq_poll_status(ctx)
+    full, scores = torch.empty_like(idx[0]), torch.empty((h, L), device="cuda")
+    for l in (0, layers - 1):
+        dq.dapq_evict(ctx, qs[l], ks[l], ks[l], [0, L + n], [L], [K], torch.empty_like(ko[l]), torch.empty_like(vo[l]), full, scores)
+        dq.dapq_poll_status(ctx)
+        differ = (full != idx[l]).any(1)
+        assert int(differ.sum()) <= h // 1000                       # (keys whose scores agree with the K-th to rounding)
+        rows = idx[l].long()[..., None].expand(-1, -1, 128)
+        assert torch.equal(ko[l], ks[l].gather(1, rows)) and torch.equal(vo[l], ks[l].gather(1, rows))
+    dq.dapq_destroy(ctx)
+
+
 @pytest.mark.parametrize("cycles", [1, 30, 100, 1000, 5000, 30000])
 def test_layers_that_share_launches_give_up_anywhere(dq, cycles):
     """Limits at which some waits run out and others do not: no role hangs on another that gave up, and the context works again."""
