@@ -1616,6 +1616,36 @@ def test_layers_that_share_launches_in_other_forms(dq, form, hq, hkv, n, lens, l
     dq.dapq_destroy(ctx)
 
 
+@pytest.mark.parametrize("flags", [0, 2])
+def test_evict_of_a_large_batch_by_sequence(dq, flags):
+    """The rotation of many queries in a call of one layer (60 prompts, 21 queries, 12 heads; flags: DAPQ_FLAG_ROPE_INTERLEAVED),
+    every prompt against a call of its own, which takes the other kernel: scores up to sums in another order (1e-6; measured 5.5e-7)
+    and an fp16 query rounded the other way (2^-11 of one product of 128 in one of 84 rows: 2e-6), sets by the tolerance of _same_set."""
+    hq, hkv, n = 12, 3, 21
+    lens = [64 + 37 * b % 500 for b in range(60)]
+    keep = [L // 8 for L in lens]
+    w = _small(lens=lens, keep=keep, n_q_heads=hq, n_kv_heads=hkv, n_pseudo=n, n_needles=0, outlier_channels=0)
+    ctx = _ctx(dq, w, flags=flags)
+    g = torch.Generator(device="cuda").manual_seed(flags)
+    q, k, v = (torch.randn(s, generator=g, device="cuda").bfloat16() for s in ((60, hq, n, 128), (hkv, w.total_rows, 128), (hkv, w.total_rows, 128)))
+    idx, scores = _one_by_one(dq, ctx, w, q, k, v)
+    dq.dapq_poll_status(ctx)
+    for b, L in enumerate(lens):
+        one = torch.full((hkv, keep[b]), -1, dtype=torch.int32, device="cuda")
+        ko, vo = (torch.zeros((hkv, keep[b], 128), dtype=k.dtype, device="cuda") for _ in range(2))
+        s = torch.empty((hkv, L), device="cuda")
+        rows = slice(int(w.cu_rows[b]), int(w.cu_rows[b + 1]))
+        kb, vb = k[:, rows].contiguous(), v[:, rows].contiguous()
+        dq.dapq_evict(ctx, q[b:b + 1].contiguous(), kb, vb, [0, L + n], [L], [keep[b]], ko, vo, one, s)
+        dq.dapq_poll_status(ctx)
+        got = scores[:, int(w.cu_prompt[b]):int(w.cu_prompt[b + 1])]
+        assert float(((got - s).abs() / s).max()) <= 5e-6
+        mine = idx[:, int(w.cu_keep[b]):int(w.cu_keep[b + 1])]
+        r = mine.long()[..., None].expand(-1, -1, 128)
+        _same_set(one, mine, s, kb, vb, kb.gather(1, r), vb.gather(1, r), [L], [0], [0, keep[b]], [0])
+    dq.dapq_destroy(ctx)
+
+
 def test_layers_of_more_heads_than_a_grid_has_rows(dq):
     """Eight layers of 8200 heads: 65600 rows of a grid, of which there are 65535."""
     h, n, L, K, layers = 8200, 64, 20, 3, 8
