@@ -50,13 +50,15 @@ FALLBACK_BF16_TFLOPS_SUSTAINED = 1400.0
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum, bytes) of the score sweeps
 # from ncu captures of this program, keyed by (kernel, workload); "sweep1" of the two 128k workloads is the
-# pass over all keys of the pruned selection (their "sweep2" depends on the candidates).  Every entry carries the digest of
+# pass over all keys of the pruned selection (their "sweep2" depends on the candidates); "stream": a layer's share of a launch
+# that makes both sweeps of several layers (the other two workloads; their "sweep1" and "sweep2" serve runs of one layer).  Every entry carries the digest of
 # the kernel's sources that it was captured with: once those change, the entry no longer describes
 # the kernel that runs and the bench reports `traffic: null` until the capture is redone.
 _MB = 1000 * 1000
 _KERNEL_SOURCES = {"sweep1": ("umma_ptx.cuh", "score_qg_common.cuh", "score_qg_sweep1.cuh"),
-                   "sweep2": ("umma_ptx.cuh", "score_qg_common.cuh", "score_qg_sweep2.cuh")}
-_ROWSTAT, _COLSUM = "b987fcea74afc429", "509d6568e5e36724"
+                   "sweep2": ("umma_ptx.cuh", "score_qg_common.cuh", "score_qg_sweep2.cuh"),
+                   "stream": ("umma_ptx.cuh", "score_qg_common.cuh", "score_qg_sweep1.cuh", "score_qg_sweep2.cuh", "score_flow.cuh")}
+_ROWSTAT, _COLSUM, _STREAM = "b987fcea74afc429", "509d6568e5e36724", "778259dbc095464c"
 NCU_TRAFFIC = {
     ("sweep1", "llama3_70b_128k"): {"bytes": int((271.84 + 13.90) * _MB), "digest": _COLSUM},
     ("sweep1", "qwen25_7b_128k"): {"bytes": int((135.23 + 3.42) * _MB), "digest": _COLSUM},
@@ -64,6 +66,8 @@ NCU_TRAFFIC = {
     ("sweep2", "llama3_8b_32k"): {"bytes": int((67.99 + 0.02) * _MB), "digest": _COLSUM},
     ("sweep1", "batched_serving"): {"bytes": int((313.05 + 1.90) * _MB), "digest": _ROWSTAT},
     ("sweep2", "batched_serving"): {"bytes": int((311.89 + 3.26) * _MB), "digest": _COLSUM},
+    ("stream", "llama3_8b_32k"): {"bytes": int((471.02 + 3.97) / 4 * _MB), "digest": _STREAM},
+    ("stream", "batched_serving"): {"bytes": int((1175.39 + 10.22) / 2 * _MB), "digest": _STREAM},
 }
 
 
@@ -425,8 +429,8 @@ def measure(env: Env, w: gi.Workload, n_layers: int, steps: int, warmup: int, re
                 "frac": achieved / peaks["hbm_gbs"]}
     roof.setdefault("peak_source", peaks["source"])
     roof.update({"kernel": dom, "avg_launch_us": dom_ms * 1e3,
-                 "traffic": None if stream else ncu_traffic(dom, w.name), "both_sweeps": stream,
-                 "algorithmic_bytes": work["k_read_bytes"] if dom in ("sweep1", "sweep2") else None,
+                 "traffic": ncu_traffic("stream" if stream else dom, w.name), "both_sweeps": stream,
+                 "algorithmic_bytes": n_work * work["k_read_bytes"] if dom in ("sweep1", "sweep2") else None,   # (K once a sweep)
                  "share_of_step": kinds[dom][0] / total_prof_ms,
                  # per layer (a kind may be launched several times a layer: the bounds of the pruned selection count as topk;
                  # or once for several layers)

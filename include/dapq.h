@@ -248,8 +248,10 @@ DAPQ_API dapq_status dapq_evict(dapq_ctx* ctx, const void* q_pre, const dapq_cac
  * Calls of 8 layers and more on long prompts, without pooling and with budgets that are small against the prompts, compute
  * the scores of those keys only that can be among the K largest, in layers where the layers before show that it
  * pays.  The sets are those of dapq_evict up to keys whose scores agree with the K-th to rounding (1e-5 of it), as are the
- * sets of two scorings whose log-sum-exps are summed in different orders; so are those of layers that share launches.  Layers
- * that do neither select dapq_evict's own, bit for bit. */
+ * sets of two scorings whose log-sum-exps are summed in different orders.  So are those of layers that share launches: over which
+ * runs of keys their sums are formed depends on the lengths, the number of layers that share a launch and the size of the
+ * context, so within that tolerance a layer's set may depend on the layers it is called with; the same call on the same context
+ * gives the same sets bit for bit.  Layers that do neither select dapq_evict's own, bit for bit. */
 DAPQ_API dapq_status dapq_evict_layers(dapq_ctx* ctx, int32_t n_layers, const void* const* q_pre,
                               const dapq_cache_view* caches, const int32_t* k_keep_host,
                               int64_t k_keep_layer_stride, void* const* k_out, void* const* v_out,

@@ -274,7 +274,8 @@ dapq_status run_score_qg(dapq_ctx* ctx, const QgPlan& plan, const SeqTable& t, c
   return DAPQ_OK;
 }
 
-// The scorer over several layers a launch: the eviction path's own fp16 queries, one query group per KV head.
+// The scorer over several layers a launch: the eviction path's own fp16 queries (more than 256 query rows a KV head: in groups, each
+// with its own score slot).
 bool wants_flow(const dapq_ctx* ctx) {
   return wants_umma(ctx) && !(ctx->shape.flags & (DAPQ_FLAG_Q_BF16 | DAPQ_FLAG_Q_LO_SWEEP1 | DAPQ_FLAG_Q_LO_SWEEP2));
 }

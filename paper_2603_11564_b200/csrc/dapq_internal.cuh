@@ -120,13 +120,13 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 // ---- launchers (each returns the cudaError_t of its launch) -------------------------------
-// q_pre has element type `dtype`; q_rot is written as `out_mode`: bf16, fp32 (unrounded, for
-// the CUDA-core scorer) or a bf16 pair hi + lo with lo = bf16(q - hi) stored `lo_offset`
-// elements after hi (for the tensor-core scorer).
 // Layers that one launch of the rotation, the scorer, the selection and the compaction may cover (dapq_evict_layers).
 constexpr int kFlowLayers = 8;
-// q_rot: [layers][B, H_q, N, d].  ref (fp16 output mode only, may be NULL): where to write, per rotated query, its base-2
-// logit against the first key of its sequence in the layer's bf16 key cache (see rope.cu).  clear: words set to 0.
+// The rotation of the layers' queries q (element type `dtype`) to q_rot, [layers][B, H_q, N, d] as `out_mode` says: fp16 (times
+// scale * log2 e, for the tensor-core scorer), bf16, fp32 (unrounded, for the CUDA-core scorer) or a bf16 pair hi + lo with
+// lo = bf16(q - hi) stored `lo_offset` elements after hi.  Only the fp16 mode takes more than one layer.
+// ref (fp16 mode only, may be NULL): where to write, per rotated query, its base-2 logit against the first key of its sequence in
+// the layer's bf16 key cache (see rope.cu).  clear: words set to 0.
 template <int kLayers>
 struct RopeLayers {
   const void* q[kLayers];

@@ -17,10 +17,10 @@
 // [128 keys x 256 query rows]; with at most 128 query rows, both sub-tiles side by side, [2 x 128 keys x 128 rows]).
 // So a job is always one accumulator of 256 columns of which every epilogue thread adds up 64.
 //
-// What bounds it: instruction issue (0.55 to 0.6 a cycle and scheduler) and, under a sustained load, power (1.62 GHz); the
-// exponential pipe is 57 (128 query rows) to 70 % busy (256), the tensor pipe 36 to 45 %.  Us a layer in short runs, two launches a
-// layer -> here: 32 k keys on 8 heads x 256 rows 65 -> 46, a ragged batch of 150 k keys x 128 rows 177 -> 158, 40 prompts of 8 k
-// 350 -> 305.  The code has one body per role on purpose: with all variants inlined (118 to 142 KB against 67 to 71) units of three
+// What bounds it: instruction issue (0.57 to 0.59 a cycle and scheduler) and, under a sustained load, power (1.62 GHz); the
+// exponential pipe is 57 (128 query rows) to 69 % busy (256), the tensor pipe 34 to 40 %, DRAM 55 to 30 %.  Us a layer with selection
+// and compaction, two launches a layer -> here, in bursts of 10 ms | over seconds: 32 k keys on 8 heads x 256 rows 71 -> 47 | 71 -> 54,
+// a ragged batch of 150 k keys x 128 rows 189 -> 158 | 198 -> 176, 40 prompts of 8 k 371 -> 309 | 404 -> 357.  The code has one body per role on purpose: with all variants inlined (118 to 142 KB against 67 to 71) units of three
 // pairs ran at 0.75 of this pace, waiting for instructions.
 #pragma once
 #include "score_qg_sweep1.cuh"
@@ -319,7 +319,9 @@ flow_kernel(const __grid_constant__ KeyMaps tm_k, const __grid_constant__ CUtens
           if (u.kind == kSweep1) {
             tma_load_3d(dst, map, bar(S::k_full + s), 0, row, u.kvh);
             tma_load_3d(dst + kPairHalf, map, bar(S::k_full + s), 64, row, u.kvh);
-          } else {                                               // (nobody reads these keys again: L2 may drop them first)
+          } else {
+            // (nobody but the next query group, at once, and the compaction of the kept rows reads these keys again: L2 may drop them
+            // first.  A plain policy for all groups but the last: +- 0.5 % on 448 to 1024 query rows, in bursts and over seconds)
             tma_load_3d_hint(dst, map, bar(S::k_full + s), 0, row, u.kvh, last_use);
             tma_load_3d_hint(dst + kPairHalf, map, bar(S::k_full + s), 64, row, u.kvh, last_use);
           }
